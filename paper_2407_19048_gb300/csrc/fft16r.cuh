@@ -99,10 +99,9 @@ __device__ __forceinline__ float2 rot16(float2 x) {
 // 16-point DFT in registers, natural order in and out: v[k] <- sum_m v[m] e^{-+2 pi i m k/16}.
 // With m = 4a + b and k = c + 4d: four 4-point DFTs over a, the factors e^{-+2 pi i b c/16},
 // four 4-point DFTs over b; the result V[c + 4d] lands in v[4c + d] and is renamed back.
+// The part after the first four 4-point DFTs (their results V_b[c] in v[4c + b]).
 template <bool INV>
-__device__ __forceinline__ void dft16(float2* v) {
-#pragma unroll
-  for (int b = 0; b < 4; ++b) dft4<INV>(v[b], v[4 + b], v[8 + b], v[12 + b]);
+__device__ __forceinline__ void dft16_tail(float2* v) {
   v[5] = rot16<1, INV>(v[5]);
   v[9] = rot16<2, INV>(v[9]);
   v[13] = rot16<3, INV>(v[13]);
@@ -122,6 +121,46 @@ __device__ __forceinline__ void dft16(float2* v) {
   }
 #pragma unroll
   for (int k = 0; k < 16; ++k) v[k] = o[k];
+}
+
+template <bool INV>
+__device__ __forceinline__ void dft16(float2* v) {
+#pragma unroll
+  for (int b = 0; b < 4; ++b) dft4<INV>(v[b], v[4 + b], v[8 + b], v[12 + b]);
+  dft16_tail<INV>(v);
+}
+
+// The same for inputs that are zero except v[m], m < M, and v[m], m >= 16 - M (M <= 4; the
+// others are not read): a column b then holds at most its first element A = v[b] (b < M)
+// and its last D = v[12 + b] (b >= 4 - M), and its 4-point DFT is what dft4 makes of
+// (A, 0, 0, D) with the additions of zero left out, so the result is dft16's bit for bit
+// (up to the sign of a zero).
+template <bool INV, int M>
+__device__ __forceinline__ void dft16_ends(float2* v) {
+  static_assert(M >= 1 && M <= 4, "at most four inputs at each end");
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const bool has_a = b < M, has_d = b >= 4 - M;
+    const float2 A = v[b], D = v[12 + b];
+    if (has_a && has_d) {
+      const float2 t = mul_mi<INV>(make_float2(-D.x, -D.y));
+      v[b] = cadd(A, D);
+      v[8 + b] = csub(A, D);
+      v[4 + b] = cadd(A, t);
+      v[12 + b] = csub(A, t);
+    } else if (has_a) {
+      v[4 + b] = v[8 + b] = v[12 + b] = A;
+    } else if (has_d) {
+      const float2 t = mul_mi<INV>(make_float2(-D.x, -D.y));
+      v[b] = D;
+      v[8 + b] = make_float2(-D.x, -D.y);
+      v[4 + b] = t;
+      v[12 + b] = make_float2(-t.x, -t.y);
+    } else {
+      v[b] = v[4 + b] = v[8 + b] = v[12 + b] = make_float2(0.f, 0.f);
+    }
+  }
+  dft16_tail<INV>(v);
 }
 
 // ---------------------------------------------------------------- shared memory

@@ -307,7 +307,7 @@ cudaError_t launch_loglike_full(const float* ydata, const float2* Ydata, const f
 // evaluated by Horner's rule in e^{2 pi i (j + r/(2u))/n}, otherwise the butterfly runs in
 // full.
 //
-// A block takes 32 consecutive samples: its first warp does their FP64 set-up (one lane
+// A block takes up to 32 consecutive samples: its first warp does their FP64 set-up (one lane
 // per sample); per sample all threads build P and Q in shared memory, then G groups of
 // n/16 threads (16 values each) run the u transforms G at a time, each group on its own
 // barrier (in-place passes where that fits more blocks on an SM, two buffers otherwise).
@@ -370,12 +370,13 @@ constexpr int TM_U_MAX = 64;
 
 size_t tm_rows_bytes() { return (size_t)TM_U_MAX * TM_ROW * sizeof(float2); }
 
-// The u rows (one block, before the likelihood kernel; the blocks of that kernel copy them
-// into shared memory).
+// The u rows (one block each, before the likelihood kernel; the blocks of that kernel copy
+// them into shared memory).  FP64 sincospi latency: one block over all rows took 12.3 us at
+// u = 16.
 __global__ void k_tm_rows(int n, int u, float2* __restrict__ rows) {
   const int64_t Nu = 2LL * n * u;
-  for (int i = threadIdx.x; i < u * TM_ROW; i += blockDim.x) {
-    const int r = i / TM_ROW, k = i - r * TM_ROW;
+  const int r = blockIdx.x;
+  for (int k = threadIdx.x; k < TM_ROW; k += blockDim.x) {
     int64_t m = 0;                                            // the entry is e^{2 pi i m/(N u)}
     if (k < 16) m = (int64_t)k * (n / 16) * r;
     else if (k == 16) m = -(int64_t)n * r;
@@ -385,7 +386,7 @@ __global__ void k_tm_rows(int n, int u, float2* __restrict__ rows) {
     if (m < 0) m += Nu;
     double sn, cs;
     sincospi(2.0 * (double)m / (double)Nu, &sn, &cs);
-    rows[i] = make_float2((float)cs, (float)sn);
+    rows[r * TM_ROW + k] = make_float2((float)cs, (float)sn);
   }
 }
 
@@ -470,20 +471,33 @@ __device__ __forceinline__ float2 tm_band_product(const DrawCoef& c, int k, int 
 }
 
 // First pass (radix 16, Ns = 1): butterfly t reads Z_{t + q n/16} from the tables (without
-// the factor a^t, which the later passes carry) and writes buffer dst.
-template <int LOGN>
+// the factor a^t, which the later passes carry) and writes buffer dst.  With M < 8 only
+// the q < M and q >= 16 - M are read, the others being zero (tm_band_reach).
+template <int LOGN, int M>
 __device__ __forceinline__ void tm_first_pass(uint32_t pq, uint32_t row, uint32_t dst, int t) {
   constexpr int T = (1 << LOGN) / 16;
   const float2 crb = lds2(row + 8u * 16u);   // e^{-i pi r/u}
   float2 v[16];
 #pragma unroll
   for (int q = 0; q < 16; ++q) {
+    if (q >= M && q < 16 - M) continue;
     const float4 e = lds4(pq + 16u * (uint32_t)(t + q * T));
     const float2 z = make_float2(fmaf(crb.x, e.z, fmaf(-crb.y, e.w, e.x)), fmaf(crb.x, e.w, fmaf(crb.y, e.z, e.y)));
     v[q] = q ? cmul(z, lds2(row + 8u * (uint32_t)q)) : z;
   }
-  dft16<true>(v);
+  if constexpr (M < 8) dft16_ends<true, M>(v);
+  else dft16<true>(v);
   store_pass16<16, 1>(dst, t, v);
+}
+
+// How many of the 16 input blocks of n/16 points, at each end, hold a nonzero Z_j when the
+// template's last bin is kend: c_k is zero above kend, so Z_j is zero for
+// kend < j < n - kend, and block q = j/(n/16) is empty unless q < M or q >= 16 - M with
+// M = kend/(n/16) + 1.  2, 3 and 4 have first passes of their own (a 20 + 20 Msun template
+// at 1024 Hz ends at 0.21 of the band, M = 4); 8 stands for the full pass.
+__device__ __forceinline__ int tm_band_reach(int kend, int T) {
+  const int m = kend < 0 ? 1 : kend / T + 1;
+  return m <= 2 ? 2 : (m <= 4 ? m : 8);
 }
 
 // Middle pass of radix 16 and stride Ns: twiddles (e^{2 pi i (t mod Ns)/(16 Ns)} a^W)^l,
@@ -598,7 +612,7 @@ __global__ void __launch_bounds__(TmPlan<LOGN>::THREADS, TmPlan<LOGN>::MIN_BLOCK
 k_loglike_tmarg(const double* __restrict__ theta, SetupConsts kc, double fs, DetParams dp, double gmst, double tc_lo,
                 const float2* __restrict__ Y, const float* __restrict__ W, const int64_t* __restrict__ ev_off,
                 const double* __restrict__ yy_part, const float2* __restrict__ g_rows, int64_t E, int k_lo, int n_tc,
-                int u, int nq, int64_t S, double invN, double log_J, double* __restrict__ lnl) {
+                int u, int nq, int spb, int64_t S, double invN, double log_J, double* __restrict__ lnl) {
   using PL = TmPlan<LOGN>;
   constexpr int n = PL::n;
   constexpr int F = n + 1;
@@ -618,8 +632,8 @@ k_loglike_tmarg(const double* __restrict__ theta, SetupConsts kc, double fs, Det
   const uint32_t buf0 = pq + 16u * n + 8u * (uint32_t)(g * NBUF * n);
   const uint32_t buf1 = buf0 + 8u * n;
   const uint32_t rows = pq + 16u * n + 8u * (uint32_t)(PL::G * NBUF * n);
-  const int64_t base = (int64_t)blockIdx.x * TM_SAMPLES;
-  const int cnt = (int)min((int64_t)TM_SAMPLES, S - base);
+  const int64_t base = (int64_t)blockIdx.x * spb;
+  const int cnt = (int)min((int64_t)spb, S - base);
   if (wid == 0 && lane < cnt) {
     const int64_t s_own = base + lane;
     int64_t lo = 0, hi = E;                                   // event: largest e with ev_off[e] <= s
@@ -643,7 +657,11 @@ k_loglike_tmarg(const double* __restrict__ theta, SetupConsts kc, double fs, Det
     // P, Q of the pair (k, n - k) and this thread's part of sum |H|^2 (Kahan); item 0 also
     // takes the middle bin n/2 (its own pair), so the n/2 items split evenly
     float hs = 0.f, hcmp = 0.f;
-    for (int k = tid; k < n / 2; k += NT) {
+    // only the blocks that the first pass reads (and entry n - TPR M, its lowest, which
+    // pairs with no bin below TPR M)
+    const int M = tm_band_reach(kend, TPR);
+    if (M < 8 && tid == 0) sts4(pq + 16u * (uint32_t)(n - TPR * M), make_float4(0.f, 0.f, 0.f, 0.f));
+    for (int k = tid; k < min(n / 2, TPR * M); k += NT) {
 #pragma unroll 1
       for (int h = 0; h < (k == 0 ? 2 : 1); ++h) {
         const int kk = h ? n / 2 : k;
@@ -668,7 +686,12 @@ k_loglike_tmarg(const double* __restrict__ theta, SetupConsts kc, double fs, Det
       const int r = r0 + g;
       if (r < u) {                                            // uniform over the group
         const uint32_t row = rows + 8u * (uint32_t)(r * TM_ROW);
-        tm_first_pass<LOGN>(pq, row, buf0, t);
+        switch (M) {                                          // uniform over the block
+          case 2: tm_first_pass<LOGN, 2>(pq, row, buf0, t); break;
+          case 3: tm_first_pass<LOGN, 3>(pq, row, buf0, t); break;
+          case 4: tm_first_pass<LOGN, 4>(pq, row, buf0, t); break;
+          default: tm_first_pass<LOGN, 8>(pq, row, buf0, t); break;
+        }
         tm_group_sync<TPR>(g);
         const uint32_t xl = TmMid<LOGN, 0>::run(buf0, buf1, row, t, g);
         tm_last_pass<LOGN>(xl, t, row, n_tc, nq, mx, sm);
@@ -720,12 +743,15 @@ cudaError_t launch_loglike_tmarg(const float* ydata, const float2* Ydata, const 
   }
   if (S <= 0) return cudaSuccess;
   if (u < 1 || u > TM_U_MAX || n_tc < 1) return cudaErrorInvalidValue;
-  k_tm_rows<<<1, 256, 0, s>>>(n, u, rows);
+  k_tm_rows<<<(unsigned)u, 64, 0, s>>>(n, u, rows);
   {
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
-  const unsigned grid = (unsigned)((S + TM_SAMPLES - 1) / TM_SAMPLES);
+  int dev = 0, sms = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (err != cudaSuccess) return err;
   const double invN = 1.0 / (double)N;
   const double log_J = log((double)u * (double)n_tc);
   const SetupConsts kc = make_setup_consts(df);
@@ -735,11 +761,19 @@ cudaError_t launch_loglike_tmarg(const float* ydata, const float2* Ydata, const 
     constexpr int NB = PL::n / PL::RS;
     const int nq = min(PL::RS, (n_tc + 2 * NB - 1) / (2 * NB));   // outputs q of the last pass with 2 q NB < n_tc
     const size_t smem = PL::smem(u);
+    // Samples per block: as few whole waves of resident blocks as 32 samples a block need,
+    // evenly filled.  (7001 samples: 219 blocks of 32 left half of the 456 block slots
+    // empty, 375 us; 438 blocks of 16, 276 us.  2.03 M samples: 61.9 ms at 32 a block,
+    // 63.4 at 16, 67.4 at 8: each block's FP64 set-up is one warp's latency.)
+    const int64_t slots = (int64_t)sms * PL::MIN_BLOCKS;
+    const int64_t waves = (S + TM_SAMPLES * slots - 1) / (TM_SAMPLES * slots);
+    const int spb = (int)((S + slots * waves - 1) / (slots * waves));
+    const unsigned grid = (unsigned)((S + spb - 1) / spb);
     auto run = [&](auto kern) -> cudaError_t {
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::smem(TM_U_MAX));
       if (e != cudaSuccess) return e;
       kern<<<grid, PL::THREADS, smem, s>>>(theta, kc, fs, dp, gmst, tc_lo, Ydata, W, ev_off, yy_part, rows, E, k_lo,
-                                           n_tc, u, nq, S, invN, log_J, lnl);
+                                           n_tc, u, nq, spb, S, invN, log_J, lnl);
       return cudaGetLastError();
     };
     switch (D) {
