@@ -104,11 +104,28 @@ cudaError_t launch_importance_weights(const double* lnl, const double* ratio, co
 // group: tile-rows per raster band (0 = the default).
 cudaError_t launch_gemm_bf16(const void* A, const void* B, void* C, int64_t M, int64_t N, int64_t K, bool out_bf16,
                              const float* bias, int act, int group, cudaStream_t s);
-// Split-K product C [M][N] (FP32) = A B^T for few tiles and a long K: the slices' partial
-// products go to `part` (gemm_splitk_ws bytes), then one kernel sums them in order.
+// dZ = dY act'(Z) (bfloat16 [M][N]) of the layer Z = X W^T + bias, and the FP32 column sums of
+// every 32 rows of it before rounding (colsum [ceil(M/32)][N]); act 1 or 2.
+cudaError_t launch_gemm_dact(const void* X, const void* W, const float* bias, const float* dY, int act, int64_t M,
+                             int64_t N, int64_t K, void* dZ, float* colsum, int group, cudaStream_t s);
+// C [M][N] (FP32) = A B with A [M][K] and B [K][N] bfloat16, read as they lie.
+cudaError_t launch_gemm_nn(const void* A, const void* B, float* C, int64_t M, int64_t N, int64_t K, cudaStream_t s);
+// Weight gradients dW [M][N] (FP32) = dZ^T X from dZ [K][M] and X [K][N] bfloat16, read as
+// they lie; `groups` products whose operands and results lie dz_stride, x_stride and
+// dw_stride elements apart.  Few tiles and a long K: K slices, whose partial products go to
+// `part` (wgrad_ws bytes) and are summed in order by a second kernel.
+int wgrad_splits(int64_t M, int64_t N, int64_t K, int64_t groups);
+size_t wgrad_ws(int64_t M, int64_t N, int64_t K, int64_t groups);
+cudaError_t launch_wgrad(const void* dZ, const void* X, float* dW, int64_t M, int64_t N, int64_t K, float* part,
+                         cudaStream_t s, int64_t groups = 1, int64_t dz_stride = 0, int64_t x_stride = 0,
+                         int64_t dw_stride = 0);
+// The same for a stride-1 convolution: dW [O][k C] from dz [Bn][T][O] and x [Bn][T][C].
+cudaError_t launch_conv_wgrad(const void* dz, const void* x, float* dW, int64_t Bn, int64_t T, int64_t C, int64_t O,
+                              int k, float* part, cudaStream_t s);
 // Implicit-GEMM 1-D convolution (stride 1, zero "same" padding): out [Bn][T][N] FP32 =
-// sum_{j < k, c < C} x[b][t + dir (j - (k-1)/2)][c] W[o][j C + c] (+ addend); x bfloat16
-// channels last, W bfloat16 [N][k C].  T % 128 == 0, C % 64 == 0, 16-byte aligned x, W.
+// sum_{j < k, c < C} x[b][t + dir (j - (k-1)/2)][c] Wj[c][o] (+ addend); x bfloat16 channels
+// last; W bfloat16 [N][k C] with dir 1, [C][k N] with dir -1 (k_gemm.cu).  T % 128 == 0,
+// C % 64 == 0 (and N % 64 == 0 with dir -1), 16-byte aligned x, W.
 cudaError_t launch_conv_gemm(const void* x, int64_t Bn, int64_t T, int64_t C, int k, int dir, const void* W, int64_t N,
                              float* out, const float* addend, cudaStream_t s);
 // The ResNet's stride-1 convolutions (k_conv.cu): forward z [Bn][T][O] = conv(x, W)
@@ -119,13 +136,12 @@ cudaError_t launch_conv_forward(const void* x, int64_t Bn, int64_t T, int C, int
                                 const float* addend, float* z, cudaStream_t s);
 cudaError_t launch_conv_backward(const float* dz, const void* x, const void* W, int64_t Bn, int64_t T, int C, int O,
                                  int k, const float* addend, float* dx, float* dW, void* ws, cudaStream_t s);
-int gemm_splits(int64_t M, int64_t N, int64_t K);
-size_t gemm_splitk_ws(int64_t M, int64_t N, int64_t K);
-cudaError_t launch_gemm_splitk(const void* A, const void* B, float* C, int64_t M, int64_t N, int64_t K, float* part,
-                               cudaStream_t s);
 cudaError_t gemm_status(int* status);
 
-// Dense-layer backward (k_dense.cu): workspace bytes and the launcher.
+// Dense-layer backward (k_dense.cu): workspace bytes and the launcher.  dz_rows: dZ in
+// bfloat16 from FP32 dY (masked by Y > 0 when Y, the layer's bfloat16 ReLU output, is given)
+// and, with part, the column sums of every 32 rows; N even.
+cudaError_t launch_dz_rows(const float* dY, const void* Y, int64_t M, int N, void* dZ, float* part, cudaStream_t s);
 size_t dense_backward_ws(int64_t M, int64_t N, int64_t K);
 cudaError_t launch_dense_backward(const void* X, const void* W, const float* bias, const float* dY, int64_t M,
                                   int64_t N, int64_t K, int act, float* dX, float* dW, float* db, void* ws, int group,

@@ -27,6 +27,11 @@
 // the next tile's products (~2 % at K = 8192); the eight draining warps take one
 // accumulator half each.
 //
+// Operand layouts (OPS): besides A [M][K] and B [N][K] (both K-major), B or both operands
+// can be read as they lie when K is their row index ("MN-major": boxes of 64 columns x 64
+// rows, transposed by the tensor core's operand descriptors), so that the products of a
+// dense layer's backward, dX = dZ W and dW = dZ^T X, need no transposed copies.
+//
 // Split K: a product with few tiles and a long K (the weight gradients dW = dZ^T X, whose
 // K is the batch) would run on a handful of SMs.  There the work list is (tile, K slice)
 // pairs: slice s covers K blocks [s kbs, (s + 1) kbs) and stores its FP32 partial product
@@ -63,7 +68,6 @@ struct Tile {
   static constexpr int NSTAGE = MW == 1 ? STAGES : 3;
   static constexpr int NACC = MW == 1 ? 2 : 1;             // accumulator sets in tensor memory
   static constexpr uint32_t TMEM_COLS = TN_;              // FP32 columns of one accumulator
-  static constexpr uint32_t IDESC = idesc_bf16(GM, TN_);
   static constexpr size_t SMEM = (size_t)NSTAGE * STAGE_BYTES + (size_t)EPI_WARPS * EPI_BUF_BYTES + 1024;
 };
 
@@ -77,6 +81,30 @@ struct ConvGeo {
   int pad;   // (k - 1) / 2
   int dir;   // +1: convolution; -1: its input gradient (taps mirrored)
 };
+
+// Operand layouts of the kernel.
+enum : int {
+  OP_KK = 0,       // A [M][K], B [N][K]
+  OP_NN = 1,       // A [M][K], B [K][N]
+  OP_TN = 2,       // A [groups][K][M], B [groups][K][N]
+  OP_CONV = 3,     // A an implicit im2col tile (ConvGeo), B [N][K]
+  OP_CONV_NN = 4,  // A an implicit im2col tile, B [K / k][k N] (tap-major columns: the input gradient's weights)
+  OP_CONV_TN = 5   // A [K][M] rows of times, B the implicit im2col rows [K][N], N = k Cin (the weight gradient)
+};
+constexpr bool op_a_mn(int op) { return op == OP_TN || op == OP_CONV_TN; }
+constexpr bool op_b_mn(int op) { return op == OP_NN || op == OP_TN || op == OP_CONV_NN || op == OP_CONV_TN; }
+constexpr bool op_conv_a(int op) { return op == OP_CONV || op == OP_CONV_NN; }
+
+// What the epilogue writes: FP32, bfloat16, or dZ = dY act'(Z) in bfloat16 for the product
+// Z = A B^T + bias, with the FP32 column sums of every 32 rows.
+enum : int { OUT_F32 = 0, OUT_BF16 = 1, OUT_DACT = 2 };
+
+__device__ __forceinline__ float act_grad(float z, int act) {
+  if (act == 1) return z > 0.f ? 1.f : 0.f;
+  if (act == 2)   // GELU: Phi(z) + z phi(z)
+    return 0.5f * erfcf(-0.70710678118654752f * z) + z * 0.39894228040143268f * expf(-0.5f * z * z);
+  return 1.f;
+}
 
 __device__ int g_gemm_status;
 
@@ -113,14 +141,21 @@ __device__ __forceinline__ void tile_coords(int t, int TM, int TN, int group, in
 // tile's main loop; MW = 2 (256 x 256 tiles): the two accumulators are the tile's two
 // 128-row halves and the next tile waits for both to drain.  "tfull" (MMA commit) and
 // "tempty" (one arrival per epilogue warp) hand them over.
-// TN_: tile width; CONV: A is loaded as an implicit im2col tile (ConvGeo).  addend
-// (optional; N % 32 == 0, 16-byte aligned): C = (A B^T + addend), then bias and activation.
-template <bool OUT_BF16, int TN_, bool CONV, int MW = 1>
+// TN_: tile width; OPS: operand layouts.  extra: with OUT_DACT the dY of C = dY act'(Z)
+// (any N); else an optional addend (N % 32 == 0, 16-byte aligned): C = (A B^T + addend),
+// then bias and activation.  colsum (OUT_DACT): [ceil(M/32)][N].
+// groups: independent products (OP_TN; map coordinate z), group g's C at + g cstride; with
+// splits > 1 the slice's partial product of group g at C + (slice groups + g) M N.
+template <int OUT, int TN_, int OPS, int MW = 1>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     k_gemm_bf16(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, void* __restrict__ C,
                 const float* __restrict__ bias, int act, int group, int M, int N, int K, int kbs, int splits,
-                const float* __restrict__ addend, ConvGeo geo) {
-  static_assert(MW == 1 || !CONV, "wide tiles are for plain products");
+                const float* __restrict__ extra, float* __restrict__ colsum, int groups, int64_t cstride,
+                ConvGeo geo) {
+  static_assert(MW == 1 || OPS == OP_KK, "wide tiles are for plain products");
+  constexpr bool A_MN = op_a_mn(OPS), B_MN = op_b_mn(OPS);
+  constexpr uint32_t CHUNK = 64 * GK * 2;   // one 64-column box of an MN-major operand
+  const float* addend = OUT == OUT_DACT ? nullptr : extra;
   constexpr int GN = TN_;
   using TL = Tile<TN_, MW>;
   constexpr int GMT = TL::ROWS;
@@ -129,7 +164,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   constexpr uint32_t A_BYTES = TL::A_TILE;
   constexpr uint32_t STAGE_BYTES = TL::STAGE_BYTES;
   constexpr uint32_t TMEM_COLS = TL::TMEM_COLS;
-  constexpr uint32_t IDESC = TL::IDESC;
+  constexpr uint32_t IDESC = idesc_bf16(GM, TN_, A_MN, B_MN);
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], tfull[2], tempty[2];
   __shared__ uint32_t tmem_slot;
@@ -139,7 +174,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   const int KB = (K + GK - 1) / GK;
   const int TM = (M + GMT - 1) / GMT, TN = (N + GN - 1) / GN;
   const int tiles = TM * TN;
-  const int work = tiles * splits;   // (tile, K slice) pairs, tile fastest
+  const int per = tiles * groups;
+  const int work = per * splits;   // (tile, group, K slice) triples, tile fastest
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -170,7 +206,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       for (int w = blockIdx.x; w < work && !*(volatile int*)&abort_flag; w += gridDim.x) {
         int tm, tn;
         tile_coords(w % tiles, TM, TN, group, tm, tn);
-        const int kb0 = (w / tiles) * kbs, kb1 = min(KB, kb0 + kbs);
+        const int z = (w % per) / tiles;
+        const int kb0 = (w / per) * kbs, kb1 = min(KB, kb0 + kbs);
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const uint32_t s = it % STAGES;
           if (it >= STAGES && !mbar_wait(su32(&empty[s]), ((it / STAGES) - 1) & 1u, WAIT_POLLS)) {
@@ -179,14 +216,41 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           }
           const uint32_t sa = base + s * STAGE_BYTES, sb = sa + A_BYTES;
           mbar_expect_tx(su32(&full[s]), STAGE_BYTES);
-          if constexpr (CONV) {
+          if constexpr (op_conv_a(OPS)) {
             const int tpb = geo.T / GM;   // M tiles per sample
             const int tap = kb / geo.KC, cb = kb - tap * geo.KC;
             tma_load_3d(sa, &ta, cb * GK, (tm % tpb) * GM + geo.dir * (tap - geo.pad), tm / tpb, su32(&full[s]));
+            if constexpr (B_MN) {   // rows cb GK .. of [K / k][k N], columns of tap `tap`
+#pragma unroll
+              for (int c = 0; c < TN_ / 64; ++c)
+                tma_load_2d(sb + c * CHUNK, &tb, tap * N + min(tn * GN + 64 * c, N - 64), cb * GK, su32(&full[s]));
+            }
+          } else if constexpr (A_MN) {
+#pragma unroll
+            for (int c = 0; c < GM / 64; ++c)
+              tma_load_3d(sa + c * CHUNK, &ta, tm * GM + 64 * c, kb * GK, z, su32(&full[s]));
           } else {
             tma_load_2d(sa, &ta, kb * GK, tm * GMT, su32(&full[s]));   // one box of GMT rows
           }
-          tma_load_2d(sb, &tb, kb * GK, tn * GN, su32(&full[s]));
+          if constexpr (OPS == OP_CONV_TN) {
+            // 64 times of one sample (T % 128 == 0); columns past N repeat the last 64
+            const int row = kb * GK, b = row / geo.T, t0 = row - b * geo.T;
+#pragma unroll
+            for (int c = 0; c < TN_ / 64; ++c) {
+              const int col = min(tn * GN + 64 * c, N - 64) / 64, tap = col / geo.KC;
+              tma_load_3d(sb + c * CHUNK, &tb, (col - tap * geo.KC) * 64, t0 + tap - geo.pad, b, su32(&full[s]));
+            }
+          } else if constexpr (OPS == OP_TN) {
+#pragma unroll
+            for (int c = 0; c < TN_ / 64; ++c)
+              tma_load_3d(sb + c * CHUNK, &tb, tn * GN + 64 * c, kb * GK, z, su32(&full[s]));
+          } else if constexpr (OPS == OP_NN) {
+#pragma unroll
+            for (int c = 0; c < TN_ / 64; ++c)
+              tma_load_2d(sb + c * CHUNK, &tb, tn * GN + 64 * c, kb * GK, su32(&full[s]));
+          } else if constexpr (!B_MN) {
+            tma_load_2d(sb, &tb, kb * GK, tn * GN, su32(&full[s]));
+          }
         }
       }
     }
@@ -195,7 +259,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       uint32_t it = 0, tl = 0;
       for (int w = blockIdx.x; w < work && !*(volatile int*)&abort_flag; w += gridDim.x, ++tl) {
         const uint32_t acc = tl % NACC;
-        const int kb0 = (w / tiles) * kbs, kb1 = min(KB, kb0 + kbs);
+        const int kb0 = (w / per) * kbs, kb1 = min(KB, kb0 + kbs);
         if (tl >= NACC && !mbar_wait(su32(&tempty[acc]), ((tl / NACC) - 1) & 1u, WAIT_POLLS)) {
           atomicExch(&abort_flag, 1);
           break;
@@ -216,8 +280,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             // M-tile m: rows 128 m .. of the A box (16 KiB apart), accumulator columns m TN_ ..
 #pragma unroll
             for (int m = 0; m < MW; ++m)
-              mma_bf16(d + (uint32_t)m * TMEM_COLS, sw128_desc(sa + (uint32_t)m * (GM * GK * 2) + 32u * kk),
-                       sw128_desc(sb + 32u * kk), IDESC, kb != kb0 || kk != 0);
+              mma_bf16(d + (uint32_t)m * TMEM_COLS,
+                       A_MN ? sw128_mn_desc(sa + 2048u * kk, CHUNK)
+                            : sw128_desc(sa + (uint32_t)m * (GM * GK * 2) + 32u * kk),
+                       B_MN ? sw128_mn_desc(sb + 2048u * kk, CHUNK) : sw128_desc(sb + 32u * kk), IDESC,
+                       kb != kb0 || kk != 0);
           }
           mma_commit(su32(&empty[s]));
         }
@@ -239,7 +306,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     for (int w = blockIdx.x; w < work; w += gridDim.x, ++tl) {
       int tm, tn;
       tile_coords(w % tiles, TM, TN, group, tm, tn);
-      const size_t slice = (size_t)(w / tiles) * (size_t)M * (size_t)N;   // 0 unless split
+      const size_t slice = splits > 1 ? (size_t)(w / tiles) * (size_t)M * (size_t)N
+                                      : (size_t)((w % per) / tiles) * (size_t)cstride;
       const uint32_t acc = tl % NACC;
       const bool have = mbar_wait(su32(&tfull[acc]), (tl / NACC) & 1u, WAIT_POLLS);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -265,6 +333,14 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 #pragma unroll
           for (int j = 0; j < 8; ++j) ad[j] = in ? __ldg(ap + j) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        // dY of this lane's column (OUT_DACT), fetched early for the same reason
+        float dy[32];
+        if constexpr (OUT == OUT_DACT) {
+          const float* yp = extra + (int64_t)row0 * N + col0 + lane;
+#pragma unroll
+          for (int r = 0; r < 32; ++r)
+            dy[r] = row0 + r < M && col0 + lane < N ? __ldg(yp + (int64_t)r * N) : 0.f;
+        }
         tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (acc + (uint32_t)msel) * TMEM_COLS + (uint32_t)(32 * c), v);
         if (row0 >= M || col0 >= N) continue;   // warp-uniform
         if (addend != nullptr) {
@@ -276,11 +352,23 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             v[4 * j + 3] += ad[j].w;
           }
         }
-        epilogue_ops(v, bias, act, col0, N);
+        epilogue_ops(v, bias, OUT == OUT_DACT ? 0 : act, col0, N);
 #pragma unroll
         for (int j = 0; j < 32; ++j) ebuf[lane * 32 + (j ^ lane)] = v[j];
         __syncwarp();
-        if constexpr (OUT_BF16) {
+        if constexpr (OUT == OUT_DACT) {
+          __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(C);
+          const int col = col0 + lane;
+          float sum = 0.f;
+#pragma unroll
+          for (int r = 0; r < 32; ++r) {
+            float a = dy[r];
+            if (act != 0) a *= act_grad(ebuf[r * 32 + (lane ^ r)], act);
+            sum += a;
+            if (row0 + r < M && col < N) out[(int64_t)(row0 + r) * N + col] = __float2bfloat16_rn(a);
+          }
+          if (col < N) colsum[(int64_t)(row0 / 32) * N + col] = sum;
+        } else if constexpr (OUT == OUT_BF16) {
           __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(C) + slice;
           const int w = lane & 15, col = col0 + 2 * w;
 #pragma unroll 4
@@ -335,6 +423,20 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
+// Row-major bfloat16 [groups][rows][cols], groups gstride elements apart, as a 3-D tensor
+// map with boxes of 64 columns x 64 rows (an MN-major operand).
+bool make_map_mn(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, int64_t groups, int64_t gstride) {
+  auto enc = encode_fn();
+  if (!enc) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)groups};
+  cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)gstride * 2};
+  cuuint32_t box[3] = {64, (cuuint32_t)GK, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Row-major bfloat16 [rows][K] as a 2-D tensor map with boxes of box_rows x 64.
 bool make_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t K, uint32_t box_rows) {
   auto enc = encode_fn();
@@ -348,41 +450,66 @@ bool make_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t K, uint32
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// out[i] = sum over s of part[s][i] for i < n (slices in order: deterministic).
-__global__ void k_split_reduce(const float* __restrict__ part, int splits, int64_t n, float* __restrict__ out) {
+// out[g][i] = sum over s of part[s][g][i] for i < n (slices in order: deterministic); groups
+// of out ostride apart.
+__global__ void k_split_reduce(const float* __restrict__ part, int splits, int64_t n, int64_t ostride,
+                               float* __restrict__ out) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  const int64_t total = n * gridDim.y;
+  const float* p = part + (int64_t)blockIdx.y * n + i;
   float acc = 0.f;
-  for (int s = 0; s < splits; ++s) acc += __ldg(&part[(int64_t)s * n + i]);
-  out[i] = acc;
+#pragma unroll 4
+  for (int s = 0; s < splits; ++s) acc += __ldg(p + (int64_t)s * total);
+  out[(int64_t)blockIdx.y * ostride + i] = acc;
 }
 
-template <int TN_, int MW = 1>
-cudaError_t launch_gemm_tn(const CUtensorMap& ta, const CUtensorMap& tb, void* C, int64_t M, int64_t N, int64_t K,
-                           bool out_bf16, const float* bias, int act, int group, int splits, int sms,
-                           cudaStream_t s) {
-  const int KB = (int)((K + GK - 1) / GK);
-  const int kbs = (KB + splits - 1) / splits;   // every slice has at least one K block
-  splits = (KB + kbs - 1) / kbs;
-  const int64_t work = ((M + Tile<TN_, MW>::ROWS - 1) / Tile<TN_, MW>::ROWS) * ((N + TN_ - 1) / TN_) * splits;
+// Everything of a launch but the operands.
+struct GemmCall {
+  void* C;
+  int64_t M, N, K;
+  const float* bias = nullptr;
+  int act = 0;
+  int group = DEFAULT_GROUP;
+  int splits = 1;
+  const float* extra = nullptr;
+  float* colsum = nullptr;
+  int groups = 1;
+  int64_t cstride = 0;
+  ConvGeo geo{0, 0, 0, 0};
+};
+
+cudaError_t sm_count(int* sms) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+  return e;
+}
+
+template <int OUT, int TN_, int OPS, int MW = 1>
+cudaError_t run_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmCall& c, int sms, cudaStream_t s) {
+  const int KB = (int)((c.K + GK - 1) / GK);
+  const int kbs = (KB + c.splits - 1) / c.splits;   // every slice has at least one K block
+  const int splits = (KB + kbs - 1) / kbs;
+  const int64_t work = ((c.M + Tile<TN_, MW>::ROWS - 1) / Tile<TN_, MW>::ROWS) * ((c.N + TN_ - 1) / TN_) * splits *
+                       c.groups;
   const unsigned grid = (unsigned)(work < sms ? work : sms);   // persistent: one CTA per SM
   constexpr size_t smem = Tile<TN_, MW>::SMEM;
-  const ConvGeo none{0, 0, 0, 0};
-  cudaError_t e;
-  if (out_bf16) {
-    e = cudaFuncSetAttribute(k_gemm_bf16<true, TN_, false, MW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return e;
-    k_gemm_bf16<true, TN_, false, MW><<<grid, GEMM_THREADS, smem, s>>>(ta, tb, C, bias, act, group, (int)M, (int)N,
-                                                                       (int)K, kbs, splits, nullptr, none);
-  } else {
-    e = cudaFuncSetAttribute(k_gemm_bf16<false, TN_, false, MW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return e;
-    k_gemm_bf16<false, TN_, false, MW><<<grid, GEMM_THREADS, smem, s>>>(ta, tb, C, bias, act, group, (int)M, (int)N,
-                                                                        (int)K, kbs, splits, nullptr, none);
-  }
+  auto kern = k_gemm_bf16<OUT, TN_, OPS, MW>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, GEMM_THREADS, smem, s>>>(ta, tb, c.C, c.bias, c.act, c.group, (int)c.M, (int)c.N, (int)c.K, kbs, splits,
+                                        c.extra, c.colsum, c.groups, c.cstride, c.geo);
   return cudaGetLastError();
+}
+
+// The same at a tile width chosen at run time.
+template <int OUT, int OPS>
+cudaError_t run_gemm_at(int tn, const CUtensorMap& ta, const CUtensorMap& tb, const GemmCall& c, int sms,
+                        cudaStream_t s) {
+  if (tn == 64) return run_gemm<OUT, 64, OPS>(ta, tb, c, sms, s);
+  if (tn == 128) return run_gemm<OUT, 128, OPS>(ta, tb, c, sms, s);
+  return run_gemm<OUT, 256, OPS>(ta, tb, c, sms, s);
 }
 
 // Tile width of a product: 256 columns unless the 128 x 256 tiles would leave more than half
@@ -404,103 +531,158 @@ bool gemm_wide(int64_t M, int64_t N, int64_t K, int splits, int act, int sms) {
   return splits == 1 && K >= 1024 && act != GWX_ACT_GELU && ((M + 255) / 256) * ((N + 255) / 256) >= sms;
 }
 
-cudaError_t launch_gemm(const void* A, const void* B, void* C, int64_t M, int64_t N, int64_t K, bool out_bf16,
-                        const float* bias, int act, int group, int splits, cudaStream_t s) {
-  if (group < 1) group = DEFAULT_GROUP;
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+// C = A B^T with A [M][K], B [N][K]; OUT as in the kernel.
+template <int OUT>
+cudaError_t launch_gemm(const void* A, const void* B, GemmCall c, cudaStream_t s) {
+  if (c.group < 1) c.group = DEFAULT_GROUP;
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
   CUtensorMap ta, tb;
-  if (gemm_wide(M, N, K, splits, act, sms)) {
-    if (!make_map(&ta, A, M, K, 2 * GM) || !make_map(&tb, B, N, K, 256)) return cudaErrorInvalidValue;
-    return launch_gemm_tn<256, 2>(ta, tb, C, M, N, K, out_bf16, bias, act, group, splits, sms, s);
+  if constexpr (OUT != OUT_DACT) {
+    if (gemm_wide(c.M, c.N, c.K, c.splits, c.act, sms)) {
+      if (!make_map(&ta, A, c.M, c.K, 2 * GM) || !make_map(&tb, B, c.N, c.K, 256)) return cudaErrorInvalidValue;
+      return run_gemm<OUT, 256, OP_KK, 2>(ta, tb, c, sms, s);
+    }
   }
-  const int tn = gemm_tile_width(M, N, splits, sms);
-  if (!make_map(&ta, A, M, K, GM) || !make_map(&tb, B, N, K, (uint32_t)tn)) return cudaErrorInvalidValue;
-  if (tn == 64) return launch_gemm_tn<64>(ta, tb, C, M, N, K, out_bf16, bias, act, group, splits, sms, s);
-  if (tn == 128) return launch_gemm_tn<128>(ta, tb, C, M, N, K, out_bf16, bias, act, group, splits, sms, s);
-  return launch_gemm_tn<256>(ta, tb, C, M, N, K, out_bf16, bias, act, group, splits, sms, s);
+  const int tn = gemm_tile_width(c.M, c.N, c.splits, sms);
+  if (!make_map(&ta, A, c.M, c.K, GM) || !make_map(&tb, B, c.N, c.K, (uint32_t)tn)) return cudaErrorInvalidValue;
+  return run_gemm_at<OUT, OP_KK>(tn, ta, tb, c, sms, s);
 }
 
-// Channels-last bfloat16 x [Bn][T][C] as a 3-D tensor map with boxes of 64 channels x 128 times.
-bool make_map_3d(CUtensorMap* map, const void* ptr, int64_t Bn, int64_t T, int64_t C) {
+// Channels-last bfloat16 x [Bn][T][C] as a 3-D tensor map with boxes of 64 channels x
+// box_t times.
+bool make_map_3d(CUtensorMap* map, const void* ptr, int64_t Bn, int64_t T, int64_t C, uint32_t box_t) {
   auto enc = encode_fn();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)T, (cuuint64_t)Bn};
   cuuint64_t strides[2] = {(cuuint64_t)C * 2, (cuuint64_t)T * C * 2};
-  cuuint32_t box[3] = {(cuuint32_t)GK, (cuuint32_t)GM, 1};
+  cuuint32_t box[3] = {(cuuint32_t)GK, box_t, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int TN_>
-cudaError_t launch_conv_tn(const CUtensorMap& ta, const CUtensorMap& tb, float* out, const float* addend, int M, int N,
-                           int K, ConvGeo geo, cudaStream_t s) {
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  const int KB = K / GK;
-  const int64_t work = (int64_t)(M / GM) * ((N + TN_ - 1) / TN_);
-  const unsigned grid = (unsigned)(work < sms ? work : sms);
-  constexpr size_t smem = Tile<TN_>::SMEM;
-  e = cudaFuncSetAttribute(k_gemm_bf16<false, TN_, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_gemm_bf16<false, TN_, true><<<grid, GEMM_THREADS, smem, s>>>(ta, tb, out, nullptr, GWX_ACT_NONE, DEFAULT_GROUP, M,
-                                                                 N, K, KB, 1, addend, geo);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 // Implicit-GEMM 1-D convolution, stride 1, "same" zero padding: out [Bn][T][N] (FP32) =
-// sum over taps j < k and channels c of x[b][t + dir (j - (k-1)/2)][c] W[o][j C + c], plus
-// addend if given.  Tile width 64 / 128 / 256 by N.  Shapes checked by the caller.
+// sum over taps j < k and channels c of x[b][t + dir (j - (k-1)/2)][c] Wj[c][o], plus addend
+// if given.  dir +1: Wj[c][o] = W[o][j C + c] for W [N][k C] (the convolution); dir -1:
+// Wj[c][o] = W[c][j N + o] for W [C][k N] (its input gradient, C the output channels of the
+// convolution, whose weights are read as they lie).  Tile width 64 / 128 / 256 by N.
+// Shapes checked by the caller.
 cudaError_t launch_conv_gemm(const void* x, int64_t Bn, int64_t T, int64_t C, int k, int dir, const void* W, int64_t N,
                              float* out, const float* addend, cudaStream_t s) {
   CUtensorMap ta, tb;
-  const int64_t K = (int64_t)k * C;
+  GemmCall c{out, Bn * T, N, (int64_t)k * C};
+  c.extra = addend;
+  c.geo = ConvGeo{(int)T, (int)(C / GK), (k - 1) / 2, dir};
   const int tn = N <= 64 ? 64 : (N <= 128 ? 128 : 256);
-  if (!make_map_3d(&ta, x, Bn, T, C) || !make_map(&tb, W, N, K, (uint32_t)tn)) return cudaErrorInvalidValue;
-  const ConvGeo geo{(int)T, (int)(C / GK), (k - 1) / 2, dir};
-  const int M = (int)(Bn * T);
-  if (tn == 64) return launch_conv_tn<64>(ta, tb, out, addend, M, (int)N, (int)K, geo, s);
-  if (tn == 128) return launch_conv_tn<128>(ta, tb, out, addend, M, (int)N, (int)K, geo, s);
-  return launch_conv_tn<256>(ta, tb, out, addend, M, (int)N, (int)K, geo, s);
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  if (!make_map_3d(&ta, x, Bn, T, C, GM)) return cudaErrorInvalidValue;
+  if (dir > 0) {
+    if (!make_map(&tb, W, N, c.K, (uint32_t)tn)) return cudaErrorInvalidValue;
+    return run_gemm_at<OUT_F32, OP_CONV>(tn, ta, tb, c, sms, s);
+  }
+  if (!make_map(&tb, W, C, (int64_t)k * N, GK)) return cudaErrorInvalidValue;   // boxes of 64 x 64
+  return run_gemm_at<OUT_F32, OP_CONV_NN>(tn, ta, tb, c, sms, s);
 }
 
 cudaError_t launch_gemm_bf16(const void* A, const void* B, void* C, int64_t M, int64_t N, int64_t K, bool out_bf16,
                              const float* bias, int act, int group, cudaStream_t s) {
-  return launch_gemm(A, B, C, M, N, K, out_bf16, bias, act, group, 1, s);
+  GemmCall c{C, M, N, K};
+  c.bias = bias;
+  c.act = act;
+  c.group = group;
+  return out_bf16 ? launch_gemm<OUT_BF16>(A, B, c, s) : launch_gemm<OUT_F32>(A, B, c, s);
 }
 
-int gemm_splits(int64_t M, int64_t N, int64_t K) {
-  const int64_t tiles = ((M + GM - 1) / GM) * ((N + GN - 1) / GN);
+cudaError_t launch_gemm_dact(const void* X, const void* W, const float* bias, const float* dY, int act, int64_t M,
+                             int64_t N, int64_t K, void* dZ, float* colsum, int group, cudaStream_t s) {
+  GemmCall c{dZ, M, N, K};
+  c.bias = bias;
+  c.act = act;
+  c.group = group;
+  c.extra = dY;
+  c.colsum = colsum;
+  return launch_gemm<OUT_DACT>(X, W, c, s);
+}
+
+cudaError_t launch_gemm_nn(const void* A, const void* B, float* C, int64_t M, int64_t N, int64_t K, cudaStream_t s) {
+  GemmCall c{C, M, N, K};
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  CUtensorMap ta, tb;
+  const int tn = gemm_tile_width(M, N, 1, sms);
+  if (!make_map(&ta, A, M, K, GM) || !make_map(&tb, B, K, N, GK)) return cudaErrorInvalidValue;
+  return run_gemm_at<OUT_F32, OP_NN>(tn, ta, tb, c, sms, s);
+}
+
+// K slices of a weight gradient with `tiles` output tiles: ~128 work items, at least four K
+// blocks per slice.
+static int wgrad_splits_of(int64_t tiles, int64_t K) {
   const int64_t KB = (K + GK - 1) / GK;
   if (tiles >= 64) return 1;
-  int64_t sp = std::min<int64_t>(128 / tiles, KB / 4);   // ~128 work items, >= 4 K blocks per slice
+  const int64_t sp = std::min<int64_t>(128 / tiles, KB / 4);
   if (sp <= 1) return 1;
   const int64_t kbs = (KB + sp - 1) / sp;
   return (int)((KB + kbs - 1) / kbs);
 }
 
-size_t gemm_splitk_ws(int64_t M, int64_t N, int64_t K) {
-  const int sp = gemm_splits(M, N, K);
-  return sp > 1 ? (size_t)sp * (size_t)M * (size_t)N * 4 : 0;
+static int wgrad_width(int64_t N) { return N <= 64 ? 64 : (N <= 128 ? 128 : GN); }
+
+int wgrad_splits(int64_t M, int64_t N, int64_t K, int64_t groups) {
+  const int tn = wgrad_width(N);
+  return wgrad_splits_of(((M + GM - 1) / GM) * ((N + tn - 1) / tn) * groups, K);
 }
 
-cudaError_t launch_gemm_splitk(const void* A, const void* B, float* C, int64_t M, int64_t N, int64_t K, float* part,
-                               cudaStream_t s) {
-  const int sp = gemm_splits(M, N, K);
-  if (sp <= 1) return launch_gemm(A, B, C, M, N, K, false, nullptr, GWX_ACT_NONE, 0, 1, s);
-  cudaError_t e = launch_gemm(A, B, part, M, N, K, false, nullptr, GWX_ACT_NONE, 0, sp, s);
-  if (e != cudaSuccess) return e;
-  const int64_t n = M * N;
-  k_split_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(part, sp, n, C);
+size_t wgrad_ws(int64_t M, int64_t N, int64_t K, int64_t groups) {
+  const int sp = wgrad_splits(M, N, K, groups);
+  return sp > 1 ? (size_t)sp * (size_t)groups * (size_t)M * (size_t)N * 4 : 0;
+}
+
+static cudaError_t wgrad_finish(const GemmCall& c, float* C, int64_t cstride, const float* part, cudaStream_t s) {
+  if (c.splits <= 1) return cudaSuccess;
+  const int64_t n = c.M * c.N;
+  k_split_reduce<<<dim3((unsigned)((n + 255) / 256), (unsigned)c.groups), 256, 0, s>>>(part, c.splits, n, cstride, C);
   return cudaGetLastError();
+}
+
+cudaError_t launch_wgrad(const void* dZ, const void* X, float* dW, int64_t M, int64_t N, int64_t K, float* part,
+                         cudaStream_t s, int64_t groups, int64_t dz_stride, int64_t x_stride, int64_t dw_stride) {
+  GemmCall c{dW, M, N, K};
+  c.groups = (int)groups;
+  c.cstride = dw_stride;
+  c.splits = wgrad_splits(M, N, K, groups);
+  if (c.splits > 1) c.C = part;
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  CUtensorMap ta, tb;
+  if (!make_map_mn(&ta, dZ, K, M, groups, groups > 1 ? dz_stride : K * M) ||
+      !make_map_mn(&tb, X, K, N, groups, groups > 1 ? x_stride : K * N))
+    return cudaErrorInvalidValue;
+  e = run_gemm_at<OUT_F32, OP_TN>(wgrad_width(N), ta, tb, c, sms, s);
+  return e != cudaSuccess ? e : wgrad_finish(c, dW, dw_stride, part, s);
+}
+
+cudaError_t launch_conv_wgrad(const void* dz, const void* x, float* dW, int64_t Bn, int64_t T, int64_t C, int64_t O,
+                              int k, float* part, cudaStream_t s) {
+  GemmCall c{dW, O, (int64_t)k * C, Bn * T};
+  c.splits = wgrad_splits(c.M, c.N, c.K, 1);
+  if (c.splits > 1) c.C = part;
+  c.geo = ConvGeo{(int)T, (int)(C / GK), (k - 1) / 2, +1};
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  CUtensorMap ta, tb;
+  if (!make_map_mn(&ta, dz, c.K, O, 1, c.K * O) || !make_map_3d(&tb, x, Bn, T, C, GK)) return cudaErrorInvalidValue;
+  e = run_gemm_at<OUT_F32, OP_CONV_TN>(wgrad_width(c.N), ta, tb, c, sms, s);
+  return e != cudaSuccess ? e : wgrad_finish(c, dW, 0, part, s);
 }
 
 // Self-test of the bounded waits: one thread waits on an mbarrier that nothing arrives at,
