@@ -823,11 +823,12 @@ int gwx_debug_status(uint64_t* first_bad) {
 
 int gwx_device_status(void) {
   GWX_TRY(ensure_init());
-  int st = 0, st2 = 0, st3 = 0;
+  int st = 0, st2 = 0, st3 = 0, st4 = 0;
   GWX_TRY(launched(gemm_status(&st), "device status"));
   GWX_TRY(launched(flow_fused_status(&st2), "device status"));
+  GWX_TRY(launched(flow_train_status(&st4), "device status"));
   GWX_TRY(launched(sim_status(&st3), "device status"));
-  if (st != 0 || st2 != 0 || st3 != 0)
+  if (st != 0 || st2 != 0 || st3 != 0 || st4 != 0)
     return fail(GWX_ETIMEOUT, "a kernel gave up waiting for its own copies; its output is incomplete");
   return GWX_OK;
 }

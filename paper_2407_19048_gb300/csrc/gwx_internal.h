@@ -211,6 +211,25 @@ cudaError_t launch_flow_sample_fused(const void* params_bf16, const float* param
                                      int K, const float* z, const void* ctx, const int64_t* ev_off, int64_t E,
                                      int64_t row0, int64_t n, float* x_out, float* ss_out, cudaStream_t s);
 cudaError_t flow_fused_status(int* status);
+
+// Fused density and training passes (k_flow_train.cu), for the sampler's widths with C <= 64.
+// The density of x [n][8] under ctx rows (a row's own, or its event's with ev_off) writes z and
+// sum s; the training pass runs forward and backward of all layers on the standardised
+// targets xs + K n 8, filling the conditioners' gradients, dctx [n][C] and the mean loss.
+struct FlowTrainBufs {   // all carved from the caller's workspace
+  void *X, *g1, *g2, *dz1, *dz2, *dO, *m1, *m2;
+  float *o, *p1, *p2, *p3, *kpart;
+  double* loss_part;
+};
+bool flow_fused_train_supported(int C, int H, int K);
+FlowTrainBufs flow_train_bufs(int64_t n, int C, int H, int K, void* base, size_t* bytes);
+cudaError_t launch_flow_density(const void* params_bf16, const float* params, const int64_t* off_t, int C, int H, int K,
+                                const float* x, const void* ctx, const int64_t* ev_off, int64_t E, int64_t row0,
+                                int64_t n, float* z_out, float* ss_out, cudaStream_t s);
+cudaError_t launch_flow_train_fused(const void* params_bf16, const float* params, const int64_t* off_t, int C, int H,
+                                    int K, float* xs, const void* ctx, int64_t n, float* grads, float* dctx,
+                                    double* loss_mean, const FlowTrainBufs& f, cudaStream_t s);
+cudaError_t flow_train_status(int* status);
 size_t flow_train_ws(const gwx_flow_shape& sh, int64_t B, int D, int64_t N);
 cudaError_t flow_train_step(const gwx_flow_shape& sh, float* params, void* params_bf16, float* grads, float* m,
                             float* v, int64_t step, int64_t* step_counter, double lr, double b1, double b2, double eps, double wd, double clip,

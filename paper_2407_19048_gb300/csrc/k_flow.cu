@@ -479,28 +479,37 @@ struct TrainWs {
   __nv_bfloat16 *feat, *h1, *h2, *ctx, *X, *g1, *g2;
   float *xs, *o, *sum_s, *loss, *G, *Gu, *d_o, *dA, *dB, *dctx;
   void *fws, *dws, *clip;
+  FlowTrainBufs fused;
   size_t bytes;
 };
 
+bool train_is_fused(const FlowDims& d) { return flow_fused_train_supported((int)d.C, (int)d.H, (int)d.K); }
+
 TrainWs carve_train(const FlowDims& d, int64_t B, int D, int64_t N, void* base) {
   Carve c(base);
-  TrainWs w;
+  TrainWs w{};
   const int64_t maxw = std::max(std::max(d.H, 8 + d.C), std::max(d.He, d.C));
   w.fws = c.take<char>((int64_t)((size_t)B * D * (size_t)(N / 2 + 1) * sizeof(float2)));
   w.feat = c.take<__nv_bfloat16>(B * d.F);
   w.h1 = c.take<__nv_bfloat16>(B * d.He);
   w.h2 = c.take<__nv_bfloat16>(B * d.He);
   w.ctx = c.take<__nv_bfloat16>(B * d.C);
-  w.X = c.take<__nv_bfloat16>(d.K * B * (8 + d.C));
-  w.g1 = c.take<__nv_bfloat16>(d.K * B * d.H);
-  w.g2 = c.take<__nv_bfloat16>(d.K * B * d.H);
   w.xs = c.take<float>((d.K + 1) * B * 8);
-  w.o = c.take<float>(d.K * B * 8);
-  w.sum_s = c.take<float>(B);
-  w.loss = c.take<float>(B);
-  w.G = c.take<float>(B * 8);
-  w.Gu = c.take<float>(B * 8);
-  w.d_o = c.take<float>(B * 8);
+  if (train_is_fused(d)) {
+    size_t bytes = 0;
+    flow_train_bufs(B, (int)d.C, (int)d.H, (int)d.K, nullptr, &bytes);
+    w.fused = flow_train_bufs(B, (int)d.C, (int)d.H, (int)d.K, c.take<char>((int64_t)bytes), nullptr);
+  } else {
+    w.X = c.take<__nv_bfloat16>(d.K * B * (8 + d.C));
+    w.g1 = c.take<__nv_bfloat16>(d.K * B * d.H);
+    w.g2 = c.take<__nv_bfloat16>(d.K * B * d.H);
+    w.o = c.take<float>(d.K * B * 8);
+    w.sum_s = c.take<float>(B);
+    w.loss = c.take<float>(B);
+    w.G = c.take<float>(B * 8);
+    w.Gu = c.take<float>(B * 8);
+    w.d_o = c.take<float>(B * 8);
+  }
   w.dA = c.take<float>(B * maxw);
   w.dB = c.take<float>(B * maxw);
   w.dctx = c.take<float>(B * d.C);
@@ -527,6 +536,21 @@ ChainWs carve_chain(const FlowDims& d, int64_t R, Carve& c) {
   return w;
 }
 
+// The density direction of rows row0 .. row0 + n - 1 in place on w.v, sum s to w.sum_s: one
+// kernel for the widths it covers, else layer by layer (the same values bit for bit).
+cudaError_t density_chain(const FlowDims& d, const Params& P, const __nv_bfloat16* ctx, const int64_t* off, int64_t E,
+                          int64_t row0, int64_t n, const ChainWs& w, cudaStream_t s) {
+  if (flow_fused_supported((int)d.C, (int)d.H, (int)d.K))
+    return launch_flow_density(P.p16, P.p, P.off.data(), (int)d.C, (int)d.H, (int)d.K, w.v, ctx, off, E, row0, n, w.v,
+                               w.sum_s, s);
+  for (int l = (int)d.K - 1; l >= 0; --l) {
+    FL_TRY(launch_flow_input(l, w.v, ctx, (int)d.C, off, E, row0, n, w.X, s));
+    FL_TRY(conditioner_forward(d, P, l, n, w.X, w.g1, w.g2, w.o, s));
+    FL_TRY(launch_flow_coupling(l, -1, w.v, w.o, n, w.v, w.sum_s, l == (int)d.K - 1, s));
+  }
+  return cudaSuccess;
+}
+
 constexpr int64_t kSampleChunk = (int64_t)1 << 17;
 
 }  // namespace
@@ -550,35 +574,40 @@ cudaError_t flow_train_step(const gwx_flow_shape& sh, float* params, void* param
   const __nv_bfloat16* ctx = ctx_in ? reinterpret_cast<const __nv_bfloat16*>(ctx_in) : w.ctx;
   if (!ctx_in) FL_TRY(embed_forward(d, P, y, B, D, N, k_lo, w.fws, w.feat, w.h1, w.h2, w.ctx, s));
   FL_TRY(launch_flow_targets(theta, B, mean8, scale8, w.xs + d.K * rows8, s));
-  for (int l = (int)d.K - 1; l >= 0; --l) {
-    __nv_bfloat16* X = w.X + l * B * (8 + d.C);
-    __nv_bfloat16* g1 = w.g1 + l * B * d.H;
-    __nv_bfloat16* g2 = w.g2 + l * B * d.H;
-    float* o = w.o + l * rows8;
-    FL_TRY(launch_flow_input(l, w.xs + (l + 1) * rows8, ctx, (int)d.C, nullptr, B, 0, B, X, s));
-    FL_TRY(conditioner_forward(d, P, l, B, X, g1, g2, o, s));
-    FL_TRY(launch_flow_coupling(l, -1, w.xs + (l + 1) * rows8, o, B, w.xs + l * rows8, w.sum_s,
-                                l == (int)d.K - 1, s));
-  }
-  FL_TRY(launch_flow_nll(w.xs, w.sum_s, B, w.loss, loss_mean, w.G, s));
   FL_TRY(cudaMemsetAsync(grads, 0, (size_t)n_params * sizeof(float), s));
-  float* G = w.G;
-  float* Gu = w.Gu;
-  for (int l = 0; l < (int)d.K; ++l) {
-    const int t = 6 + 6 * l;
-    const __nv_bfloat16* X = w.X + l * B * (8 + d.C);
-    const __nv_bfloat16* g1 = w.g1 + l * B * d.H;
-    const __nv_bfloat16* g2 = w.g2 + l * B * d.H;
-    FL_TRY(launch_flow_coupling_backward(l, w.xs + l * rows8, w.o + l * rows8, G, B, 1.f / (float)B, w.d_o, Gu, s));
-    FL_TRY(launch_dense_backward(g2, P.W(t + 4), P.b(t + 5), w.d_o, B, 8, d.H, GWX_ACT_NONE, w.dA,
-                                 grads + P.off[t + 4], grads + P.off[t + 5], w.dws, 0, s));
-    // the ReLU layers' masks from their stored outputs (g2, g1)
-    FL_TRY(launch_dense_backward(g1, P.W(t + 2), P.b(t + 3), w.dA, B, d.H, d.H, GWX_ACT_RELU, w.dB,
-                                 grads + P.off[t + 2], grads + P.off[t + 3], w.dws, 0, s, g2));
-    FL_TRY(launch_dense_backward(X, P.W(t), P.b(t + 1), w.dB, B, d.H, 8 + d.C, GWX_ACT_RELU, w.dA,
-                                 grads + P.off[t], grads + P.off[t + 1], w.dws, 0, s, g1));
-    FL_TRY(launch_flow_input_backward(l, w.dA, (int)d.C, B, Gu, w.dctx, l == 0, s));
-    std::swap(G, Gu);
+  if (train_is_fused(d)) {
+    FL_TRY(launch_flow_train_fused(params_bf16, params, P.off.data(), (int)d.C, (int)d.H, (int)d.K, w.xs, ctx, B,
+                                   grads, w.dctx, loss_mean, w.fused, s));
+  } else {
+    for (int l = (int)d.K - 1; l >= 0; --l) {
+      __nv_bfloat16* X = w.X + l * B * (8 + d.C);
+      __nv_bfloat16* g1 = w.g1 + l * B * d.H;
+      __nv_bfloat16* g2 = w.g2 + l * B * d.H;
+      float* o = w.o + l * rows8;
+      FL_TRY(launch_flow_input(l, w.xs + (l + 1) * rows8, ctx, (int)d.C, nullptr, B, 0, B, X, s));
+      FL_TRY(conditioner_forward(d, P, l, B, X, g1, g2, o, s));
+      FL_TRY(launch_flow_coupling(l, -1, w.xs + (l + 1) * rows8, o, B, w.xs + l * rows8, w.sum_s,
+                                  l == (int)d.K - 1, s));
+    }
+    FL_TRY(launch_flow_nll(w.xs, w.sum_s, B, w.loss, loss_mean, w.G, s));
+    float* G = w.G;
+    float* Gu = w.Gu;
+    for (int l = 0; l < (int)d.K; ++l) {
+      const int t = 6 + 6 * l;
+      const __nv_bfloat16* X = w.X + l * B * (8 + d.C);
+      const __nv_bfloat16* g1 = w.g1 + l * B * d.H;
+      const __nv_bfloat16* g2 = w.g2 + l * B * d.H;
+      FL_TRY(launch_flow_coupling_backward(l, w.xs + l * rows8, w.o + l * rows8, G, B, 1.f / (float)B, w.d_o, Gu, s));
+      FL_TRY(launch_dense_backward(g2, P.W(t + 4), P.b(t + 5), w.d_o, B, 8, d.H, GWX_ACT_NONE, w.dA,
+                                   grads + P.off[t + 4], grads + P.off[t + 5], w.dws, 0, s));
+      // the ReLU layers' masks from their stored outputs (g2, g1)
+      FL_TRY(launch_dense_backward(g1, P.W(t + 2), P.b(t + 3), w.dA, B, d.H, d.H, GWX_ACT_RELU, w.dB,
+                                   grads + P.off[t + 2], grads + P.off[t + 3], w.dws, 0, s, g2));
+      FL_TRY(launch_dense_backward(X, P.W(t), P.b(t + 1), w.dB, B, d.H, 8 + d.C, GWX_ACT_RELU, w.dA,
+                                   grads + P.off[t], grads + P.off[t + 1], w.dws, 0, s, g1));
+      FL_TRY(launch_flow_input_backward(l, w.dA, (int)d.C, B, Gu, w.dctx, l == 0, s));
+      std::swap(G, Gu);
+    }
   }
   if (ctx_in) {
     FL_TRY(cudaMemcpyAsync(d_ctx_out, w.dctx, (size_t)B * d.C * sizeof(float), cudaMemcpyDeviceToDevice, s));
@@ -637,11 +666,7 @@ cudaError_t flow_log_prob(const gwx_flow_shape& sh, const float* params, const v
   const __nv_bfloat16* ctx = ctx_in ? reinterpret_cast<const __nv_bfloat16*>(ctx_in) : e.ctx;
   if (!ctx_in) FL_TRY(embed_forward(d, P, y, B, D, N, k_lo, e.fws, e.feat, e.h1, e.h2, e.ctx, s));
   FL_TRY(launch_flow_targets(theta, B, mean8, scale8, w.v, s));
-  for (int l = (int)d.K - 1; l >= 0; --l) {
-    FL_TRY(launch_flow_input(l, w.v, ctx, (int)d.C, nullptr, B, 0, B, w.X, s));
-    FL_TRY(conditioner_forward(d, P, l, B, w.X, w.g1, w.g2, w.o, s));
-    FL_TRY(launch_flow_coupling(l, -1, w.v, w.o, B, w.v, w.sum_s, l == (int)d.K - 1, s));
-  }
+  FL_TRY(density_chain(d, P, ctx, nullptr, B, 0, B, w, s));
   const Std8 st = make_std(mean8, scale8);
   k_flow_logq<<<blocks(B, 128), 128, 0, s>>>(w.v, w.sum_s, B, -4.0 * LN_2PI - st.ln_scale_sum, log_q);
   return cudaGetLastError();
@@ -868,11 +893,7 @@ cudaError_t flow_skymap(const gwx_flow_shape& sh, const float* params, const voi
     const int64_t n = std::min(kSampleChunk, npix - row0);
     k_sky_rows<<<blocks(n, 128), 128, 0, s>>>(nside, row0, n, r8, st, w.v);
     FL_TRY(cudaGetLastError());
-    for (int l = (int)d.K - 1; l >= 0; --l) {
-      FL_TRY(launch_flow_input(l, w.v, ctx, (int)d.C, off, 1, row0, n, w.X, s));
-      FL_TRY(conditioner_forward(d, P, l, n, w.X, w.g1, w.g2, w.o, s));
-      FL_TRY(launch_flow_coupling(l, -1, w.v, w.o, n, w.v, w.sum_s, l == (int)d.K - 1, s));
-    }
+    FL_TRY(density_chain(d, P, ctx, off, 1, row0, n, w, s));
     k_flow_logq<<<blocks(n, 128), 128, 0, s>>>(w.v, w.sum_s, n, -4.0 * LN_2PI - st.ln_scale_sum, lnq + row0);
     FL_TRY(cudaGetLastError());
   }

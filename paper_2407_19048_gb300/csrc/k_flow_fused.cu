@@ -19,42 +19,15 @@
 // The activations never go to global memory: per draw and layer only the weights (shared
 // by all draws, L2-resident) move.  Every mbarrier wait is bounded; on expiry the CTA
 // records a status, stops and frees its tensor memory.
-#include <cuda.h>
-#include <cudaTypedefs.h>
-#include <cuda_bf16.h>
-
-#include "gwx_internal.h"
-#include "tc05.cuh"
+#include "flow_tile.cuh"
 
 namespace gwx {
 
 namespace {
 
-using namespace tc;
+using namespace flowt;
 
-constexpr int FM = 128;                                  // draws per tile
-constexpr int F_THREADS = 320;                           // warp 0 TMA, warp 1 MMA, warps 2-9 rows
-constexpr uint32_t KB_BYTES = FM * 128;                  // one 128-row x 64-column bfloat16 K-block: 16 KiB
-constexpr uint32_t X_BYTES = 2 * KB_BYTES;               // conditioner input, 8 + C <= 128 columns
-constexpr uint32_t G_BYTES = 4 * KB_BYTES;               // hidden activations, H <= 256 columns
-constexpr uint32_t SLOT_BYTES = 2 * 256 * 128;           // two K-blocks of a 256-row weight tile
-constexpr uint32_t F_WAIT = 1u << 22;
 constexpr size_t FUSED_SMEM = (size_t)X_BYTES + G_BYTES + 2 * SLOT_BYTES + 1024;
-constexpr float S_MAX = 3.f;
-
-// Split p of the eight coordinates: conditioning half a_j = A(p, j), transformed half
-// b_j = Bc(p, j) (the flow's four fixed splits; compile-time so v[] stays in registers).
-__host__ __device__ constexpr int A(int p, int j) {
-  return p == 0 ? j : p == 1 ? 4 + j : p == 2 ? 2 * j : 2 * j + 1;
-}
-__host__ __device__ constexpr int Bc(int p, int j) {
-  return p == 0 ? 4 + j : p == 1 ? j : p == 2 ? 2 * j + 1 : 2 * j;
-}
-
-template <int P>
-__device__ __forceinline__ void pack_half(const float* v, uint32_t& w0, uint32_t& w1);
-template <int P>
-__device__ __forceinline__ void couple(float* v, const float* o, const float* b3, float& ss);
 
 __device__ int g_flow_status;
 
@@ -71,28 +44,6 @@ struct FusedArgs {
   float* x_out;                   // [n][8]
   float* ss_out;                  // [n]
 };
-
-// Byte offset of 16-byte chunk j of row r inside a 128-row K-block (128-byte swizzle).
-__device__ __forceinline__ uint32_t swz(int r, int j) {
-  return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((j ^ (r & 7)) << 4));
-}
-
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-  __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-
-__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-
-__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-template <int P>
-__device__ __forceinline__ void pack_half(const float* v, uint32_t& w0, uint32_t& w1) {
-  w0 = pack2(v[A(P, 0)], v[A(P, 1)]);
-  w1 = pack2(v[A(P, 2)], v[A(P, 3)]);
-}
 
 // v_b <- v_b e^s + mu with mu_j = o_j + b3_j, s_j = 3 tanh((o_{4+j} + b3_{4+j}) / 3);
 // b3: the layer's eight output biases, in registers
@@ -395,33 +346,6 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   if (threadIdx.x == 0 && *(volatile int*)&abort_flag) atomicExch(&g_flow_status, 1);
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-}
-
-PFN_cuTensorMapEncodeTiled_v12000 encoder() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
-  return fn;
-}
-
-// bfloat16 weights of every layer as a 3-D tensor [layers][rows][cols] with the layers
-// lstride elements apart; boxes of 64 columns x box_rows rows x one layer.
-bool layer_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int64_t layers, int64_t lstride,
-               uint32_t box_rows) {
-  auto enc = encoder();
-  if (!enc) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)layers};
-  cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)lstride * 2};
-  cuuint32_t box[3] = {64, box_rows, 1};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace
