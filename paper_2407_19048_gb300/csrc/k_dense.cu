@@ -22,7 +22,7 @@ constexpr int TT = 32;   // rows of a column-sum partial; columns of a k_colsum 
 // dZ = dY (masked by Y > 0 when Y, the layer's bfloat16 ReLU output, is given: that is Z > 0,
 // since a positive float never rounds to a bfloat16 zero short of 1e-40) in bfloat16, and the
 // FP32 column sums of every 32 rows into part.  HBM bound: a warp takes 32 rows x 64 columns,
-// 256-byte row segments in (eight in flight), 128-byte segments out.
+// 256-byte row segments in (sixteen in flight), 128-byte segments out.
 __global__ void __launch_bounds__(256) k_dz_rows(const float* __restrict__ dY, const __nv_bfloat16* __restrict__ Y,
                                                  int64_t M, int N, __nv_bfloat16* __restrict__ dZ,
                                                  float* __restrict__ part) {
@@ -35,18 +35,26 @@ __global__ void __launch_bounds__(256) k_dz_rows(const float* __restrict__ dY, c
   const int rows = (int)(M - m0 < TT ? M - m0 : TT);
   const bool pairs = ((uintptr_t)dY & 7u) == 0;   // dY comes with 4-byte alignment only
   float s0 = 0.f, s1 = 0.f;
-#pragma unroll 8
-  for (int r = 0; r < rows; ++r) {
-    const int64_t at = (m0 + r) * N + col;
-    float2 v = pairs ? __ldg(reinterpret_cast<const float2*>(dY + at)) : make_float2(__ldg(dY + at), __ldg(dY + at + 1));
-    if (Y != nullptr) {
-      const __nv_bfloat162 y = *reinterpret_cast<const __nv_bfloat162*>(Y + at);
-      v.x = __low2float(y) > 0.f ? v.x : 0.f;
-      v.y = __high2float(y) > 0.f ? v.y : 0.f;
+  for (int r0 = 0; r0 < rows; r0 += 16) {
+    float2 v[16];
+    __nv_bfloat162 y[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int64_t at = (m0 + min(r0 + i, rows - 1)) * N + col;
+      v[i] = pairs ? __ldg(reinterpret_cast<const float2*>(dY + at)) : make_float2(__ldg(dY + at), __ldg(dY + at + 1));
+      if (Y != nullptr) y[i] = *reinterpret_cast<const __nv_bfloat162*>(Y + at);
     }
-    *reinterpret_cast<__nv_bfloat162*>(dZ + at) = __floats2bfloat162_rn(v.x, v.y);
-    s0 += v.x;
-    s1 += v.y;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (r0 + i >= rows) break;
+      if (Y != nullptr) {
+        v[i].x = __low2float(y[i]) > 0.f ? v[i].x : 0.f;
+        v[i].y = __high2float(y[i]) > 0.f ? v[i].y : 0.f;
+      }
+      *reinterpret_cast<__nv_bfloat162*>(dZ + (m0 + r0 + i) * N + col) = __floats2bfloat162_rn(v[i].x, v[i].y);
+      s0 += v[i].x;
+      s1 += v[i].y;
+    }
   }
   if (part != nullptr) *reinterpret_cast<float2*>(part + p * N + col) = make_float2(s0, s1);
 }

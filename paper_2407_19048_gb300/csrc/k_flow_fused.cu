@@ -100,112 +100,99 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   const uint32_t tmem = tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
-        for (int l = 0; l < K && ok; ++l)
-          for (int p = 0; p < NP; ++p, ++it) {
-            const uint32_t s = it & 1u;
-            if (it >= 2 && !mbar_wait(su32(&empty[s]), ((it >> 1) - 1) & 1u, F_WAIT)) {
-              ok = false;
-              break;
-            }
-            if (*(volatile int*)&abort_flag) {
-              ok = false;
-              break;
-            }
-            const uint32_t dst = sw + s * SLOT_BYTES, bar = su32(&full[s]);
-            if (p == 0) {
-              mbar_expect_tx(bar, (uint32_t)H * 256u);
-              tma_load_3d(dst, &mv1, 0, 0, l, bar);
-              tma_load_3d(dst + (uint32_t)H * 128u, &mv1, 64, 0, l, bar);
-            } else if (p < NP - 1) {
-              const int kb0 = 2 * (p - 1);
-              mbar_expect_tx(bar, (uint32_t)H * 256u);
-              tma_load_3d(dst, &mv2, 64 * kb0, 0, l, bar);
-              tma_load_3d(dst + (uint32_t)H * 128u, &mv2, 64 * (kb0 + 1), 0, l, bar);
-            } else {
+    uint32_t it = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
+      for (int l = 0; l < K && ok; ++l)
+        for (int p = 0; p < NP; ++p, ++it) {
+          const uint32_t s = it & 1u;
+          if (!mbar_wait_warp(su32(&empty[s]), ((it >> 1) & 1u) ^ 1u, F_WAIT) ||
+              __any_sync(0xffffffffu, *(volatile int*)&abort_flag)) {
+            ok = false;
+            break;
+          }
+          const uint32_t dst = sw + s * SLOT_BYTES, bar = su32(&full[s]);
+          if (elect_one()) {
+            if (p == NP - 1) {
               mbar_expect_tx(bar, (uint32_t)H * 32u);
               for (int kb = 0; kb < H / 64; ++kb) tma_load_3d(dst + 2048u * kb, &mv3, 64 * kb, 0, l, bar);
+            } else {
+              const CUtensorMap* m = p == 0 ? &mv1 : &mv2;
+              const int kb0 = p == 0 ? 0 : 2 * (p - 1);
+              mbar_expect_tx(bar, (uint32_t)H * 256u);
+              tma_load_3d(dst, m, 64 * kb0, 0, l, bar);
+              tma_load_3d(dst + (uint32_t)H * 128u, m, 64 * (kb0 + 1), 0, l, bar);
             }
           }
-      if (!ok) atomicExch(&abort_flag, 1);
-    }
+          __syncwarp();
+        }
+    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else if (warp == 1) {
-    if (lane == 0) {
-      uint32_t it = 0, li = 0;
-      bool ok = true;
-      auto take = [&](uint32_t& slot) -> bool {
-        slot = it & 1u;
-        if (!mbar_wait(su32(&full[slot]), (it >> 1) & 1u, F_WAIT)) return false;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        return true;
-      };
-      auto wait_on = [&](uint64_t* bar, uint32_t parity) -> bool {
-        if (!mbar_wait(su32(bar), parity, F_WAIT)) return false;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        return true;
-      };
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
-        for (int l = 0; l < K && ok; ++l, ++li) {
-          uint32_t slot;
-          // acc1 = X V1^T (two K-blocks of the input row), one 128-column part at a time
-          if (!(ok = wait_on(&xready, li & 1u)) || !(ok = take(slot))) break;
-          {
-            const uint32_t wb = sw + slot * SLOT_BYTES;
-            for (int np = 0; np < NR; ++np) {
-              for (int kb = 0; kb < 2; ++kb)
+    uint32_t it = 0, li = 0;
+    bool ok = true;
+    auto wait_on = [&](uint64_t* bar, uint32_t parity) -> bool {
+      const bool got = mbar_wait_warp(su32(bar), parity, F_WAIT);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      return got;
+    };
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
+      for (int l = 0; l < K && ok; ++l, ++li) {
+        // acc1 = X V1^T, one 128-column part at a time
+        uint32_t slot = it & 1u, wb = sw + slot * SLOT_BYTES;
+        if (!(ok = wait_on(&full[slot], (it >> 1) & 1u) && wait_on(&xready, li & 1u))) break;
+        if (elect_one()) {
+          for (int np = 0; np < NR; ++np) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  mma_bf16(tmem + 128u * np, sw128_desc(sx + KB_BYTES * kb + 32u * kk),
-                           sw128_desc(wb + (uint32_t)H * 128u * kb + 16384u * np + 32u * kk), id_128,
-                           (kb | kk) != 0);
-              mma_commit(su32(&acc1f[np]));
-            }
-            mma_commit(su32(&empty[slot]));
-            ++it;
+            for (int kk = 0; kk < 8; ++kk)
+              mma_bf16(tmem + 128u * np, sw128_desc(sx + KB_BYTES * (kk >> 2) + 32u * (kk & 3)),
+                       sw128_desc(wb + (uint32_t)H * 128u * (kk >> 2) + 16384u * np + 32u * (kk & 3)), id_128, kk != 0);
+            mma_commit(su32(&acc1f[np]));
           }
-          // acc2 = g1 V2^T: K round pr (g1 columns 128 pr .. + 127, weight part pr) once the
-          // rows have written it, both 128-column output parts per round
-          for (int pr = 0; pr < NR && ok; ++pr) {
-            if (!(ok = wait_on(&gready[pr], 0u)) || !(ok = take(slot))) break;
-            const uint32_t wb = sw + slot * SLOT_BYTES;
+          mma_commit(su32(&empty[slot]));
+        }
+        __syncwarp();
+        ++it;
+        // acc2 = g1 V2^T: K round pr (g1 columns 128 pr ..) once the rows have written it
+        for (int pr = 0; pr < NR; ++pr) {
+          slot = it & 1u, wb = sw + slot * SLOT_BYTES;
+          if (!(ok = wait_on(&full[slot], (it >> 1) & 1u) && wait_on(&gready[pr], 0u))) break;
+          if (elect_one()) {
             for (int np = 0; np < NR; ++np) {
-              for (int kb = 0; kb < 2; ++kb) {
-                const int kg = 2 * pr + kb;
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  mma_bf16(tmem + 256u + 128u * np, sw128_desc(sg + KB_BYTES * kg + 32u * kk),
-                           sw128_desc(wb + (uint32_t)H * 128u * kb + 16384u * np + 32u * kk), id_128,
-                           (kg | kk) != 0);
-              }
+              for (int kk = 0; kk < 8; ++kk)
+                mma_bf16(tmem + 256u + 128u * np, sw128_desc(sg + KB_BYTES * (2 * pr + (kk >> 2)) + 32u * (kk & 3)),
+                         sw128_desc(wb + (uint32_t)H * 128u * (kk >> 2) + 16384u * np + 32u * (kk & 3)), id_128,
+                         (pr | kk) != 0);
               if (pr == NR - 1) mma_commit(su32(&acc2f[np]));
             }
             mma_commit(su32(&empty[slot]));
-            ++it;
           }
-          if (!ok) break;
-          // acc3 = g2 V3^T (16 rows, 8 of them the conditioner's outputs), K round by round
-          if (!(ok = take(slot))) break;
-          {
-            const uint32_t wb = sw + slot * SLOT_BYTES;
-            for (int r = 0; r < NR && ok; ++r) {
-              if (!(ok = wait_on(&gready[r], 1u))) break;
-              for (int kb = 2 * r; kb < 2 * r + 2; ++kb)
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  mma_bf16(tmem, sw128_desc(sg + KB_BYTES * kb + 32u * kk), sw128_desc(wb + 2048u * kb + 32u * kk),
-                           id_16, (kb | kk) != 0);
-            }
-            if (!ok) break;
-            mma_commit(su32(&empty[slot]));
-            ++it;
-            mma_commit(su32(&acc3f));
-          }
+          __syncwarp();
+          ++it;
         }
-      if (!ok) atomicExch(&abort_flag, 1);
-    }
+        if (!ok) break;
+        // acc3 = g2 V3^T (16 rows, 8 of them the conditioner's outputs)
+        slot = it & 1u, wb = sw + slot * SLOT_BYTES;
+        if (!(ok = wait_on(&full[slot], (it >> 1) & 1u))) break;
+        for (int r = 0; r < NR; ++r) {
+          if (!(ok = wait_on(&gready[r], 1u))) break;
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+              const int kb = 2 * r + (kk >> 2);
+              mma_bf16(tmem, sw128_desc(sg + KB_BYTES * kb + 32u * (kk & 3)), sw128_desc(wb + 2048u * kb + 32u * (kk & 3)),
+                       id_16, (r | kk) != 0);
+            }
+            if (r == NR - 1) {
+              mma_commit(su32(&acc3f));
+              mma_commit(su32(&empty[slot]));
+            }
+          }
+          __syncwarp();
+        }
+        ++it;
+      }
+    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else {
     const int q = warp & 3;
     const int h = (warp - 2) >> 2;                             // which half of the columns

@@ -148,10 +148,10 @@ __device__ __forceinline__ void ring_init(Ring* r, int* abort_flag) {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-__device__ __forceinline__ bool wait_mma(uint64_t* bar, uint32_t parity) {   // a single thread's wait
-  if (!mbar_wait(su32(bar), parity, F_WAIT)) return false;
+__device__ __forceinline__ bool wait_mma(uint64_t* bar, uint32_t parity) {   // the issuing warp's wait
+  const bool got = mbar_wait_warp(su32(bar), parity, F_WAIT);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  return true;
+  return got;
 }
 
 // A row warp's wait (all lanes) and arrival (its shared-memory writes made visible to the
@@ -199,19 +199,19 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   const uint32_t tmem = tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
-        for (int l = K - 1; l >= 0 && ok; --l)
-          for (int p = 0; p < NP; ++p, ++it) {
-            const uint32_t s = it & 1u;
-            if ((it >= 2 && !mbar_wait(su32(&rg.empty[s]), ((it >> 1) - 1) & 1u, F_WAIT)) ||
-                *(volatile int*)&abort_flag) {
-              ok = false;
-              break;
-            }
-            const uint32_t dst = sw + s * SLOT_BYTES, bar = su32(&rg.full[s]);
+    uint32_t it = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
+      for (int l = K - 1; l >= 0 && ok; --l)
+        for (int p = 0; p < NP; ++p, ++it) {
+          const uint32_t s = it & 1u;
+          if (!mbar_wait_warp(su32(&rg.empty[s]), ((it >> 1) & 1u) ^ 1u, F_WAIT) ||
+              __any_sync(0xffffffffu, *(volatile int*)&abort_flag)) {
+            ok = false;
+            break;
+          }
+          const uint32_t dst = sw + s * SLOT_BYTES, bar = su32(&rg.full[s]);
+          if (elect_one()) {
             if (p == NP - 1) {
               mbar_expect_tx(bar, (uint32_t)H * 32u);
               for (int kb = 0; kb < H / 64; ++kb) tma_load_3d(dst + 2048u * kb, &mv3, 64 * kb, 0, l, bar);
@@ -223,72 +223,70 @@ __global__ void __launch_bounds__(F_THREADS, 1)
               tma_load_3d(dst + (uint32_t)H * 128u, m, 64 * (kb0 + 1), 0, l, bar);
             }
           }
-      if (!ok) atomicExch(&abort_flag, 1);
-    }
+          __syncwarp();
+        }
+    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else if (warp == 1) {
-    if (lane == 0) {
-      uint32_t it = 0, li = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
-        for (int l = K - 1; l >= 0 && ok; --l, ++li) {
-          // acc1 = X V1^T, one 128-column part at a time
-          uint32_t slot = it & 1u;
-          if (!(ok = wait_mma(&rg.in_ready, li & 1u) && wait_mma(&rg.full[slot], (it >> 1) & 1u))) break;
-          {
-            const uint32_t wb = sw + slot * SLOT_BYTES;
-            for (int np = 0; np < NR; ++np) {
-              for (int kb = 0; kb < 2; ++kb)
+    uint32_t it = 0, li = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
+      for (int l = K - 1; l >= 0 && ok; --l, ++li) {
+        // acc1 = X V1^T, one 128-column part at a time
+        uint32_t slot = it & 1u, wb = sw + slot * SLOT_BYTES;
+        if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u) && wait_mma(&rg.in_ready, li & 1u))) break;
+        if (elect_one()) {
+          for (int np = 0; np < NR; ++np) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  mma_bf16(tmem + 128u * np, sw128_desc(sx + KB_BYTES * kb + 32u * kk),
-                           sw128_desc(wb + (uint32_t)H * 128u * kb + 16384u * np + 32u * kk), id_128,
-                           (kb | kk) != 0);
-              mma_commit(su32(&rg.acc1f[np]));
-            }
-            mma_commit(su32(&rg.empty[slot]));
-            ++it;
+            for (int kk = 0; kk < 8; ++kk)
+              mma_bf16(tmem + 128u * np, sw128_desc(sx + KB_BYTES * (kk >> 2) + 32u * (kk & 3)),
+                       sw128_desc(wb + (uint32_t)H * 128u * (kk >> 2) + 16384u * np + 32u * (kk & 3)), id_128, kk != 0);
+            mma_commit(su32(&rg.acc1f[np]));
           }
-          // acc2 = g1 V2^T: K round pr (g1 columns 128 pr ..) once the rows have written it
-          for (int pr = 0; pr < NR && ok; ++pr) {
-            slot = it & 1u;
-            if (!(ok = wait_mma(&rg.gready[pr], 0u) && wait_mma(&rg.full[slot], (it >> 1) & 1u))) break;
-            const uint32_t wb = sw + slot * SLOT_BYTES;
+          mma_commit(su32(&rg.empty[slot]));
+        }
+        __syncwarp();
+        ++it;
+        // acc2 = g1 V2^T: K round pr (g1 columns 128 pr ..) once the rows have written it
+        for (int pr = 0; pr < NR; ++pr) {
+          slot = it & 1u, wb = sw + slot * SLOT_BYTES;
+          if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u) && wait_mma(&rg.gready[pr], 0u))) break;
+          if (elect_one()) {
             for (int np = 0; np < NR; ++np) {
-              for (int kb = 0; kb < 2; ++kb) {
-                const int kg = 2 * pr + kb;
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  mma_bf16(tmem + 256u + 128u * np, sw128_desc(sg + KB_BYTES * kg + 32u * kk),
-                           sw128_desc(wb + (uint32_t)H * 128u * kb + 16384u * np + 32u * kk), id_128,
-                           (kg | kk) != 0);
-              }
+              for (int kk = 0; kk < 8; ++kk)
+                mma_bf16(tmem + 256u + 128u * np, sw128_desc(sg + KB_BYTES * (2 * pr + (kk >> 2)) + 32u * (kk & 3)),
+                         sw128_desc(wb + (uint32_t)H * 128u * (kk >> 2) + 16384u * np + 32u * (kk & 3)), id_128,
+                         (pr | kk) != 0);
               if (pr == NR - 1) mma_commit(su32(&rg.acc2f[np]));
             }
             mma_commit(su32(&rg.empty[slot]));
-            ++it;
           }
-          if (!ok) break;
-          // acc3 = g2 V3^T (16 rows, 8 of them the conditioner's outputs)
-          slot = it & 1u;
-          if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u))) break;
-          {
-            const uint32_t wb = sw + slot * SLOT_BYTES;
-            for (int r = 0; r < NR && ok; ++r) {
-              if (!(ok = wait_mma(&rg.gready[r], 1u))) break;
-              for (int kb = 2 * r; kb < 2 * r + 2; ++kb)
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  mma_bf16(tmem, sw128_desc(sg + KB_BYTES * kb + 32u * kk), sw128_desc(wb + 2048u * kb + 32u * kk),
-                           id_16, (kb | kk) != 0);
-            }
-            if (!ok) break;
-            mma_commit(su32(&rg.empty[slot]));
-            ++it;
-            mma_commit(su32(&rg.acc3f));
-          }
+          __syncwarp();
+          ++it;
         }
-      if (!ok) atomicExch(&abort_flag, 1);
-    }
+        if (!ok) break;
+        // acc3 = g2 V3^T (16 rows, 8 of them the conditioner's outputs)
+        slot = it & 1u, wb = sw + slot * SLOT_BYTES;
+        if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u))) break;
+        for (int r = 0; r < NR; ++r) {
+          if (!(ok = wait_mma(&rg.gready[r], 1u))) break;
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+              const int kb = 2 * r + (kk >> 2);
+              mma_bf16(tmem, sw128_desc(sg + KB_BYTES * kb + 32u * (kk & 3)), sw128_desc(wb + 2048u * kb + 32u * (kk & 3)),
+                       id_16, (r | kk) != 0);
+            }
+            if (r == NR - 1) {
+              mma_commit(su32(&rg.acc3f));
+              mma_commit(su32(&rg.empty[slot]));
+            }
+          }
+          __syncwarp();
+        }
+        ++it;
+      }
+    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else {
     const int q = warp & 3;
     const int h = (warp - 2) >> 2;                             // which half of the columns
@@ -506,19 +504,19 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   const uint32_t tmem = tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
-        for (int l = 0; l < K && ok; ++l)
-          for (int p = 0; p < NP; ++p, ++it) {
-            const uint32_t s = it & 1u;
-            if ((it >= 2 && !mbar_wait(su32(&rg.empty[s]), ((it >> 1) - 1) & 1u, F_WAIT)) ||
-                *(volatile int*)&abort_flag) {
-              ok = false;
-              break;
-            }
-            const uint32_t dst = sw + s * SLOT_BYTES, bar = su32(&rg.full[s]);
+    uint32_t it = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
+      for (int l = 0; l < K && ok; ++l)
+        for (int p = 0; p < NP; ++p, ++it) {
+          const uint32_t s = it & 1u;
+          if (!mbar_wait_warp(su32(&rg.empty[s]), ((it >> 1) & 1u) ^ 1u, F_WAIT) ||
+              __any_sync(0xffffffffu, *(volatile int*)&abort_flag)) {
+            ok = false;
+            break;
+          }
+          const uint32_t dst = sw + s * SLOT_BYTES, bar = su32(&rg.full[s]);
+          if (elect_one()) {
             if (p == 0) {                                      // V3: 8 rows (16 with the zero fill) x H columns
               mbar_expect_tx(bar, (uint32_t)H * 32u);
               for (int c = 0; c < H / 64; ++c) tma_load_3d(dst + 2048u * c, &mv3, 64 * c, 0, l, bar);
@@ -531,59 +529,66 @@ __global__ void __launch_bounds__(F_THREADS, 1)
               for (int c = 0; c < nc; ++c) tma_load_3d(dst + (uint32_t)H * 128u * c, &mv1, 64 * c, 0, l, bar);
             }
           }
-      if (!ok) atomicExch(&abort_flag, 1);
-    }
+          __syncwarp();
+        }
+    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else if (warp == 1) {
-    if (lane == 0) {
-      uint32_t it = 0, li = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
-        for (int l = 0; l < K && ok; ++l, ++li) {
-          // acc1 = dO V3: one K = 16 step (8 outputs and 8 zeros)
-          uint32_t slot = it & 1u;
-          if (!(ok = wait_mma(&rg.in_ready, li & 1u) && wait_mma(&rg.full[slot], (it >> 1) & 1u))) break;
+    uint32_t it = 0, li = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
+      for (int l = 0; l < K && ok; ++l, ++li) {
+        // acc1 = dO V3: one K = 16 step (8 outputs and 8 zeros)
+        uint32_t slot = it & 1u, wb = sw + slot * SLOT_BYTES;
+        if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u) && wait_mma(&rg.in_ready, li & 1u))) break;
+        if (elect_one()) {
           for (int np = 0; np < NR; ++np) {
-            mma_bf16(tmem + 128u * np, sw128_desc(so), sw128_mn_desc(sw + slot * SLOT_BYTES + 4096u * np, 2048u), id_128,
-                     0u);
+            mma_bf16(tmem + 128u * np, sw128_desc(so), sw128_mn_desc(wb + 4096u * np, 2048u), id_128, 0u);
             mma_commit(su32(&rg.acc1f[np]));
           }
           mma_commit(su32(&rg.empty[slot]));
-          ++it;
-          // acc2 = dZ2 V2: K round pr (dZ2 columns 128 pr .., rows of V2) once the rows have written it
-          for (int pr = 0; pr < NR && ok; ++pr) {
-            slot = it & 1u;
-            if (!(ok = wait_mma(&rg.gready[pr], 0u) && wait_mma(&rg.full[slot], (it >> 1) & 1u))) break;
-            const uint32_t wb = sw + slot * SLOT_BYTES;
+        }
+        __syncwarp();
+        ++it;
+        // acc2 = dZ2 V2: K round pr (dZ2 columns 128 pr .., rows of V2) once the rows have written it
+        for (int pr = 0; pr < NR; ++pr) {
+          slot = it & 1u, wb = sw + slot * SLOT_BYTES;
+          if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u) && wait_mma(&rg.gready[pr], 0u))) break;
+          if (elect_one()) {
             for (int np = 0; np < NR; ++np) {
 #pragma unroll
-              for (int ks = 0; ks < 8; ++ks)
-                mma_bf16(tmem + 256u + 128u * np, sw128_desc(sg + KB_BYTES * (2 * pr + (ks >> 2)) + 32u * (ks & 3)),
-                         sw128_mn_desc(wb + 32768u * np + 2048u * ks, 16384u), id_128, (pr | ks) != 0);
+              for (int kk = 0; kk < 8; ++kk)
+                mma_bf16(tmem + 256u + 128u * np, sw128_desc(sg + KB_BYTES * (2 * pr + (kk >> 2)) + 32u * (kk & 3)),
+                         sw128_mn_desc(wb + 32768u * np + 2048u * kk, 16384u), id_128, (pr | kk) != 0);
               if (pr == NR - 1) mma_commit(su32(&rg.acc2f[np]));
             }
             mma_commit(su32(&rg.empty[slot]));
-            ++it;
           }
-          if (!ok) break;
-          // acc3 = dZ1 V1
-          slot = it & 1u;
-          if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u))) break;
-          {
-            const uint32_t wb = sw + slot * SLOT_BYTES;
-            for (int r = 0; r < NR && ok; ++r) {
-              if (!(ok = wait_mma(&rg.gready[r], 1u))) break;
-              for (int ks = 8 * r; ks < 8 * r + 8; ++ks)
-                mma_bf16(tmem, sw128_desc(sg + KB_BYTES * (ks >> 2) + 32u * (ks & 3)),
-                         sw128_mn_desc(wb + 2048u * ks, (uint32_t)H * 128u), id_x, ks != 0);
-            }
-            if (!ok) break;
-            mma_commit(su32(&rg.empty[slot]));
-            ++it;
-            mma_commit(su32(&rg.acc3f));
-          }
+          __syncwarp();
+          ++it;
         }
-      if (!ok) atomicExch(&abort_flag, 1);
-    }
+        if (!ok) break;
+        // acc3 = dZ1 V1
+        slot = it & 1u, wb = sw + slot * SLOT_BYTES;
+        if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u))) break;
+        for (int r = 0; r < NR; ++r) {
+          if (!(ok = wait_mma(&rg.gready[r], 1u))) break;
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+              const int ks = 8 * r + kk;
+              mma_bf16(tmem, sw128_desc(sg + KB_BYTES * (ks >> 2) + 32u * (ks & 3)),
+                       sw128_mn_desc(wb + 2048u * ks, (uint32_t)H * 128u), id_x, ks != 0);
+            }
+            if (r == NR - 1) {
+              mma_commit(su32(&rg.acc3f));
+              mma_commit(su32(&rg.empty[slot]));
+            }
+          }
+          __syncwarp();
+        }
+        ++it;
+      }
+    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else {
     const int q = warp & 3;
     const int h = (warp - 2) >> 2;

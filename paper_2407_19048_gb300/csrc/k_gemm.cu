@@ -4,7 +4,7 @@
 //
 // Persistent CTAs (one per SM) walk the 128 x 256 tiles of C; per CTA:
 // - warp 0 streams 128 x 64 (A) and 256 x 64 (B) bfloat16 tiles into shared memory with
-//   TMA (cp.async.bulk.tensor, 128-byte swizzle), four stages deep, each stage completing
+//   TMA (cp.async.bulk.tensor, 128-byte swizzle), 192 KiB of stages deep, each stage completing
 //   on a "full" mbarrier;
 // - warp 1 allocates 512 tensor-memory columns and issues tcgen05.mma (M 128, N 256,
 //   K 16; four per stage) into one of two 256-column FP32 accumulators, committing each
@@ -49,7 +49,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int GM = 128, GN = 256, GK = 64, STAGES = 4;   // GN: the dense products' tile width
+constexpr int GM = 128, GN = 256, GK = 64;               // GN: the dense products' tile width
 constexpr int EPI_WARPS = 8;                            // two per tensor-memory lane quarter
 constexpr int GEMM_THREADS = 64 + 32 * EPI_WARPS;
 constexpr uint32_t WAIT_POLLS = 1u << 22;
@@ -64,8 +64,15 @@ struct Tile {
   static constexpr int ROWS = GM * MW;                     // rows of C per tile
   static constexpr uint32_t A_TILE = (uint32_t)ROWS * GK * 2;
   static constexpr uint32_t B_BYTES = TN_ * GK * 2;
-  static constexpr uint32_t STAGE_BYTES = A_TILE + B_BYTES;
-  static constexpr int NSTAGE = MW == 1 ? STAGES : 3;
+  static constexpr uint32_t BLOCK_BYTES = A_TILE + B_BYTES;
+  // K blocks per stage: a stage costs the issuing warp ~250 cycles of wait, poll and commit
+  // besides its MMAs (~130 cycles a K block at 64 columns), so the narrowest tiles take two at
+  // a time (128 x 64 tiles at K = 3968: 22.4 us with lane-wise issue, 17.6, 14.6)
+  static constexpr int KPS = TN_ == 64 ? 2 : 1;
+  static constexpr uint32_t STAGE_BYTES = KPS * BLOCK_BYTES;
+  // 192 KiB of stages: a narrow tile's K blocks are small, and a product with few tiles and a
+  // long K is bound by the latency of its stages, so it keeps more of them in flight
+  static constexpr int NSTAGE = 192 * 1024 / (int)STAGE_BYTES;
   static constexpr int NACC = MW == 1 ? 2 : 1;             // accumulator sets in tensor memory
   static constexpr uint32_t TMEM_COLS = TN_;              // FP32 columns of one accumulator
   static constexpr size_t SMEM = (size_t)NSTAGE * STAGE_BYTES + (size_t)EPI_WARPS * EPI_BUF_BYTES + 1024;
@@ -162,7 +169,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   constexpr int STAGES = TL::NSTAGE;
   constexpr int NACC = TL::NACC;
   constexpr uint32_t A_BYTES = TL::A_TILE;
-  constexpr uint32_t STAGE_BYTES = TL::STAGE_BYTES;
+  constexpr uint32_t STAGE_BYTES = TL::STAGE_BYTES, BLOCK_BYTES = TL::BLOCK_BYTES;
+  constexpr int KPS = TL::KPS;
   constexpr uint32_t TMEM_COLS = TL::TMEM_COLS;
   constexpr uint32_t IDESC = idesc_bf16(GM, TN_, A_MN, B_MN);
   extern __shared__ uint8_t smem_raw[];
@@ -201,98 +209,130 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   const uint32_t tmem = tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t it = 0;
-      for (int w = blockIdx.x; w < work && !*(volatile int*)&abort_flag; w += gridDim.x) {
-        int tm, tn;
-        tile_coords(w % tiles, TM, TN, group, tm, tn);
-        const int z = (w % per) / tiles;
-        const int kb0 = (w / per) * kbs, kb1 = min(KB, kb0 + kbs);
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const uint32_t s = it % STAGES;
-          if (it >= STAGES && !mbar_wait(su32(&empty[s]), ((it / STAGES) - 1) & 1u, WAIT_POLLS)) {
-            atomicExch(&abort_flag, 1);
-            break;
-          }
-          const uint32_t sa = base + s * STAGE_BYTES, sb = sa + A_BYTES;
-          mbar_expect_tx(su32(&full[s]), STAGE_BYTES);
-          if constexpr (op_conv_a(OPS)) {
-            const int tpb = geo.T / GM;   // M tiles per sample
-            const int tap = kb / geo.KC, cb = kb - tap * geo.KC;
-            tma_load_3d(sa, &ta, cb * GK, (tm % tpb) * GM + geo.dir * (tap - geo.pad), tm / tpb, su32(&full[s]));
-            if constexpr (B_MN) {   // rows cb GK .. of [K / k][k N], columns of tap `tap`
+    uint32_t s = 0, ph = 1;   // stage and the parity of its "empty" phase (the first round finds them free)
+    bool ok = true, ready = true;
+    for (int w = blockIdx.x; w < work && ok; w += gridDim.x) {
+      int tm, tn;
+      tile_coords(w % tiles, TM, TN, group, tm, tn);
+      const int z = (w % per) / tiles;
+      const int kb0 = (w / per) * kbs, kb1 = min(KB, kb0 + kbs);
+      for (int k0 = kb0; k0 < kb1; k0 += KPS) {
+        if (!__all_sync(0xffffffffu, ready) && !mbar_wait_warp(su32(&empty[s]), ph, WAIT_POLLS)) {
+          ok = false;
+          break;
+        }
+        const uint32_t st = base + s * STAGE_BYTES, bar = su32(&full[s]);
+        const int nk = min(KPS, kb1 - k0);
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
+        }
+        // the next stage's poll overlaps the copies' issue (not with the wide tiles, whose
+        // 1024 cycles of MMAs a stage hide it)
+        ready = MW == 1 && mbar_test(su32(&empty[s]), ph);
+        if (elect_one()) {
+          mbar_expect_tx(bar, (uint32_t)nk * BLOCK_BYTES);
+#pragma unroll
+          for (int j = 0; j < KPS; ++j) {
+            if (j >= nk) break;
+            const int kb = k0 + j;
+            const uint32_t sa = st + (uint32_t)j * BLOCK_BYTES, sb = sa + A_BYTES;
+            if constexpr (op_conv_a(OPS)) {
+              const int tpb = geo.T / GM;   // M tiles per sample
+              const int tap = kb / geo.KC, cb = kb - tap * geo.KC;
+              tma_load_3d(sa, &ta, cb * GK, (tm % tpb) * GM + geo.dir * (tap - geo.pad), tm / tpb, bar);
+              if constexpr (B_MN) {   // rows cb GK .. of [K / k][k N], columns of tap `tap`
+#pragma unroll
+                for (int c = 0; c < TN_ / 64; ++c)
+                  tma_load_2d(sb + c * CHUNK, &tb, tap * N + min(tn * GN + 64 * c, N - 64), cb * GK, bar);
+              }
+            } else if constexpr (A_MN) {
+#pragma unroll
+              for (int c = 0; c < GM / 64; ++c)
+                tma_load_3d(sa + c * CHUNK, &ta, tm * GM + 64 * c, kb * GK, z, bar);
+            } else {
+              tma_load_2d(sa, &ta, kb * GK, tm * GMT, bar);   // one box of GMT rows
+            }
+            if constexpr (OPS == OP_CONV_TN) {
+              // 64 times of one sample (T % 128 == 0); columns past N repeat the last 64
+              const int row = kb * GK, b = row / geo.T, t0 = row - b * geo.T;
+#pragma unroll
+              for (int c = 0; c < TN_ / 64; ++c) {
+                const int col = min(tn * GN + 64 * c, N - 64) / 64, tap = col / geo.KC;
+                tma_load_3d(sb + c * CHUNK, &tb, (col - tap * geo.KC) * 64, t0 + tap - geo.pad, b, bar);
+              }
+            } else if constexpr (OPS == OP_TN) {
 #pragma unroll
               for (int c = 0; c < TN_ / 64; ++c)
-                tma_load_2d(sb + c * CHUNK, &tb, tap * N + min(tn * GN + 64 * c, N - 64), cb * GK, su32(&full[s]));
+                tma_load_3d(sb + c * CHUNK, &tb, tn * GN + 64 * c, kb * GK, z, bar);
+            } else if constexpr (OPS == OP_NN) {
+#pragma unroll
+              for (int c = 0; c < TN_ / 64; ++c)
+                tma_load_2d(sb + c * CHUNK, &tb, tn * GN + 64 * c, kb * GK, bar);
+            } else if constexpr (!B_MN) {
+              tma_load_2d(sb, &tb, kb * GK, tn * GN, bar);
             }
-          } else if constexpr (A_MN) {
-#pragma unroll
-            for (int c = 0; c < GM / 64; ++c)
-              tma_load_3d(sa + c * CHUNK, &ta, tm * GM + 64 * c, kb * GK, z, su32(&full[s]));
-          } else {
-            tma_load_2d(sa, &ta, kb * GK, tm * GMT, su32(&full[s]));   // one box of GMT rows
-          }
-          if constexpr (OPS == OP_CONV_TN) {
-            // 64 times of one sample (T % 128 == 0); columns past N repeat the last 64
-            const int row = kb * GK, b = row / geo.T, t0 = row - b * geo.T;
-#pragma unroll
-            for (int c = 0; c < TN_ / 64; ++c) {
-              const int col = min(tn * GN + 64 * c, N - 64) / 64, tap = col / geo.KC;
-              tma_load_3d(sb + c * CHUNK, &tb, (col - tap * geo.KC) * 64, t0 + tap - geo.pad, b, su32(&full[s]));
-            }
-          } else if constexpr (OPS == OP_TN) {
-#pragma unroll
-            for (int c = 0; c < TN_ / 64; ++c)
-              tma_load_3d(sb + c * CHUNK, &tb, tn * GN + 64 * c, kb * GK, z, su32(&full[s]));
-          } else if constexpr (OPS == OP_NN) {
-#pragma unroll
-            for (int c = 0; c < TN_ / 64; ++c)
-              tma_load_2d(sb + c * CHUNK, &tb, tn * GN + 64 * c, kb * GK, su32(&full[s]));
-          } else if constexpr (!B_MN) {
-            tma_load_2d(sb, &tb, kb * GK, tn * GN, su32(&full[s]));
           }
         }
+        __syncwarp();
       }
+      if (*(volatile int*)&abort_flag) ok = false;
+      ok = __all_sync(0xffffffffu, ok);
     }
+    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else if (warp == 1) {
-    if (lane == 0) {
-      uint32_t it = 0, tl = 0;
-      for (int w = blockIdx.x; w < work && !*(volatile int*)&abort_flag; w += gridDim.x, ++tl) {
-        const uint32_t acc = tl % NACC;
-        const int kb0 = (w / per) * kbs, kb1 = min(KB, kb0 + kbs);
-        if (tl >= NACC && !mbar_wait(su32(&tempty[acc]), ((tl / NACC) - 1) & 1u, WAIT_POLLS)) {
-          atomicExch(&abort_flag, 1);
+    uint32_t s = 0, ph = 0, tl = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; w < work && ok; w += gridDim.x, ++tl) {
+      const uint32_t acc = tl % NACC;
+      const int kb0 = (w / per) * kbs, kb1 = min(KB, kb0 + kbs);
+      if (tl >= NACC && !mbar_wait_warp(su32(&tempty[acc]), ((tl / NACC) - 1) & 1u, WAIT_POLLS)) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d = tmem + acc * TMEM_COLS;
+      bool ready = false;   // the coming stage's poll, taken while the MMAs before it are issued
+      for (int k0 = kb0; k0 < kb1; k0 += KPS) {
+        if (!__all_sync(0xffffffffu, ready) && !mbar_wait_warp(su32(&full[s]), ph, WAIT_POLLS)) {
+          ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d = tmem + acc * TMEM_COLS;
-        bool ok = true;
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const uint32_t s = it % STAGES;
-          if (!mbar_wait(su32(&full[s]), (it / STAGES) & 1u, WAIT_POLLS)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t sa = base + s * STAGE_BYTES, sb = sa + A_BYTES;
-#pragma unroll
-          for (int kk = 0; kk < GK / 16; ++kk) {   // 16 bfloat16 = 32 bytes along K per instruction
-            // M-tile m: rows 128 m .. of the A box (16 KiB apart), accumulator columns m TN_ ..
-#pragma unroll
-            for (int m = 0; m < MW; ++m)
-              mma_bf16(d + (uint32_t)m * TMEM_COLS,
-                       A_MN ? sw128_mn_desc(sa + 2048u * kk, CHUNK)
-                            : sw128_desc(sa + (uint32_t)m * (GM * GK * 2) + 32u * kk),
-                       B_MN ? sw128_mn_desc(sb + 2048u * kk, CHUNK) : sw128_desc(sb + 32u * kk), IDESC,
-                       kb != kb0 || kk != 0);
-          }
-          mma_commit(su32(&empty[s]));
+        const uint32_t st = base + s * STAGE_BYTES, done = su32(&empty[s]);
+        const int nk = min(KPS, kb1 - k0);
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
         }
-        if (!ok) atomicExch(&abort_flag, 1);
-        mma_commit(su32(&tfull[acc]));   // arrives once the tile's MMAs have completed
-        if (!ok) break;
+        ready = MW == 1 && k0 + KPS < kb1 && mbar_test(su32(&full[s]), ph);
+        if (elect_one()) {
+#pragma unroll
+          for (int j = 0; j < KPS; ++j) {
+            if (j >= nk) break;
+            const uint32_t sa = st + (uint32_t)j * BLOCK_BYTES, sb = sa + A_BYTES;
+#pragma unroll
+            for (int kk = 0; kk < GK / 16; ++kk) {   // 16 bfloat16 = 32 bytes along K per instruction
+              // M-tile m: rows 128 m .. of the A box (16 KiB apart), accumulator columns m TN_ ..
+#pragma unroll
+              for (int m = 0; m < MW; ++m)
+                mma_bf16(d + (uint32_t)m * TMEM_COLS,
+                         A_MN ? sw128_mn_desc(sa + 2048u * kk, CHUNK)
+                              : sw128_desc(sa + (uint32_t)m * (GM * GK * 2) + 32u * kk),
+                         B_MN ? sw128_mn_desc(sb + 2048u * kk, CHUNK) : sw128_desc(sb + 32u * kk), IDESC,
+                         k0 + j != kb0 || kk != 0);
+            }
+          }
+          mma_commit(done);
+        }
+        __syncwarp();
       }
+      if (elect_one()) mma_commit(su32(&tfull[acc]));   // arrives once the tile's MMAs have completed
+      __syncwarp();
+      if (*(volatile int*)&abort_flag) ok = false;
+      ok = __all_sync(0xffffffffu, ok);
     }
+    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else {
     // epilogue warps 2-9; tensor-memory lane quarter (warp % 4) = tile rows 32 q .. 32 q + 31;
     // (warp - 2) / 4 picks the column half (MW = 1) or the M-tile (MW = 2, all columns)
