@@ -406,6 +406,10 @@ int gwx_dense_bf16(const void* X, const void* W, const float* bias, void* Y, int
  * db sums the FP32 dZ.  dX, dW or db may be NULL to skip it.  M, N, K multiples of 8 in
  * [8, 65535 * 32]; X, W, dX, dW 16-byte aligned, dY, bias, db 4-byte aligned.
  * Workspace: gwx_dense_bf16_backward_workspace(M, N, K) bytes. */
+/* dX and dW alone, from dZ already in bfloat16 [M][N] (16-byte aligned); the same sizes and
+ * workspace. */
+int gwx_dense_bf16_backward_dz(const void* dZ16, const void* X, const void* W, int64_t M, int64_t N, int64_t K,
+                               float* dX, float* dW, void* workspace, size_t workspace_bytes, void* stream);
 size_t gwx_dense_bf16_backward_workspace(int64_t M, int64_t N, int64_t K);
 int gwx_dense_bf16_backward(const void* X, const void* W, const float* bias, const float* dY, int64_t M,
                             int64_t N, int64_t K, int act, float* dX, float* dW, float* db,
@@ -705,6 +709,17 @@ int gwx_group_norm(const float* z, int64_t B, int T, int C, int G, const float* 
 size_t gwx_group_norm_backward_scratch(int64_t B, int C, int G);
 int gwx_group_norm_backward(const float* dy, const float* z, int64_t B, int T, int C, int G, const float* mean_rstd,
                             const float* gamma, void* scratch, float* dz, float* dgamma, float* dbeta, void* stream);
+/* gwx_group_norm_backward_src: the same from a gradient formed on the fly, without a pass of
+ *   its own: kind 0 dy as given; 1 dy [out > 0]; 2 dy [B][T_out][C] routed back through
+ *   gwx_maxpool's arg, then masked by out > 0 (out its input); 3 dy [B][C] / T (the mean over
+ *   time), masked.  dz16 in bfloat16; dsum (optional) the masked gradient in FP32.  C / 4
+ *   divides 256, C / G a multiple of 4, G <= 32; scratch of
+ *   gwx_group_norm_backward_src_scratch(B, C, G) bytes; dy, z, scratch, dsum 16-byte, out
+ *   and dz16 8-byte, arg 4-byte aligned. */
+size_t gwx_group_norm_backward_src_scratch(int64_t B, int C, int G);
+int gwx_group_norm_backward_src(int kind, const float* dy, const void* out, const uint8_t* arg, const float* z,
+                                int64_t B, int T, int C, int G, const float* mean_rstd, const float* gamma,
+                                void* scratch, void* dz16, float* dsum, float* dgamma, float* dbeta, void* stream);
 int gwx_relu_mask(const float* dy, const void* out, int64_t n, float* d, void* stream);
 int gwx_maxpool(const void* x, int64_t B, int T, int C, void* y, uint8_t* arg, void* stream);
 int gwx_maxpool_backward(const float* dy, const uint8_t* arg, int64_t B, int T, int C, float* dx, void* stream);
@@ -730,6 +745,10 @@ int gwx_mean_time_backward(const float* dm, int64_t B, int T, int C, float* dx, 
  * reported by gwx_device_status. */
 int gwx_conv1d_bf16(const void* x, int64_t B, int64_t T, int C, int k, const void* W, int O, const float* addend,
                     float* z, void* stream);
+/* The same backward from dz already in bfloat16 (16-byte aligned). */
+int gwx_conv1d_bf16_backward_dz(const void* dz16, const void* x, const void* W, int64_t B, int64_t T, int C, int O,
+                                int k, const float* addend, float* dx, float* dW, void* workspace,
+                                size_t workspace_bytes, void* stream);
 size_t gwx_conv1d_bf16_backward_workspace(int64_t B, int64_t T, int C, int O, int k);
 int gwx_conv1d_bf16_backward(const float* dz, const void* x, const void* W, int64_t B, int64_t T, int C, int O, int k,
                              const float* addend, float* dx, float* dW, void* workspace, size_t workspace_bytes,

@@ -115,6 +115,12 @@ SIGNATURES = {
     "gwx_group_norm_backward": (c_int, [c_vp, c_vp, c_i64, c_int, c_int, c_int, c_vp, c_vp, c_vp, c_vp, c_vp, c_vp,
                                         c_vp]),
     "gwx_group_norm_backward_scratch": (c_size, [c_i64, c_int, c_int]),
+    "gwx_group_norm_backward_src_scratch": (c_size, [c_i64, c_int, c_int]),
+    "gwx_group_norm_backward_src": (c_int, [c_int, c_vp, c_vp, c_vp, c_vp, c_i64, c_int, c_int, c_int, c_vp, c_vp, c_vp,
+                                            c_vp, c_vp, c_vp, c_vp, c_vp]),
+    "gwx_conv1d_bf16_backward_dz": (c_int, [c_vp, c_vp, c_vp, c_i64, c_i64, c_int, c_int, c_int, c_vp, c_vp, c_vp,
+                                            c_vp, c_size, c_vp]),
+    "gwx_dense_bf16_backward_dz": (c_int, [c_vp, c_vp, c_vp, c_i64, c_i64, c_i64, c_vp, c_vp, c_vp, c_size, c_vp]),
     "gwx_relu_mask": (c_int, [c_vp, c_vp, c_i64, c_vp, c_vp]),
     "gwx_maxpool": (c_int, [c_vp, c_i64, c_int, c_int, c_vp, c_vp, c_vp]),
     "gwx_maxpool_backward": (c_int, [c_vp, c_vp, c_i64, c_int, c_int, c_vp, c_vp]),

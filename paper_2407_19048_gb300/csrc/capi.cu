@@ -711,6 +711,21 @@ int gwx_dense_bf16_backward(const void* X, const void* W, const float* bias, con
                   "dense_bf16_backward");
 }
 
+int gwx_dense_bf16_backward_dz(const void* dZ16, const void* X, const void* W, int64_t M, int64_t N, int64_t K,
+                               float* dX, float* dW, void* workspace, size_t workspace_bytes, void* stream) {
+  const int64_t lim = (int64_t)65535 * 32;
+  if (M < 8 || N < 8 || K < 8 || M % 8 || N % 8 || K % 8 || M > lim || N > lim || K > lim)
+    return fail(GWX_ESHAPE, "dense backward sizes M=%lld N=%lld K=%lld (multiples of 8, at most %lld)",
+                (long long)M, (long long)N, (long long)K, (long long)lim);
+  if (!dZ16 || !X || !W) return fail(GWX_EINVAL, "NULL array");
+  if ((((uintptr_t)dZ16) | ((uintptr_t)X) | ((uintptr_t)W) | ((uintptr_t)dX) | ((uintptr_t)dW)) & 15u)
+    return fail(GWX_EINVAL, "dZ16, X, W, dX and dW must be 16-byte aligned");
+  GWX_TRY(check_ws(workspace, workspace_bytes, gwx_dense_bf16_backward_workspace(M, N, K)));
+  GWX_TRY(ensure_init());
+  return launched(launch_dense_backward_dz(dZ16, X, W, M, N, K, dX, dW, workspace, as_stream(stream)),
+                  "dense_bf16_backward_dz");
+}
+
 int gwx_gemm_autotune(const void* A, const void* B, void* C, int64_t M, int64_t N, int64_t K, int c_dtype,
                       int* group_out, void* stream) {
   GWX_TRY(check_dense(A, B, nullptr, C, M, N, K, GWX_ACT_NONE, c_dtype));
@@ -1056,6 +1071,30 @@ int gwx_group_norm_backward(const float* dy, const float* z, int64_t B, int T, i
                   "group_norm_backward");
 }
 
+size_t gwx_group_norm_backward_src_scratch(int64_t B, int C, int G) {
+  if (B < 1 || C < 1 || G < 1) return 0;
+  return align_up(group_norm_backward_src_scratch(B, C));
+}
+
+int gwx_group_norm_backward_src(int kind, const float* dy, const void* out, const uint8_t* arg, const float* z,
+                                int64_t B, int T, int C, int G, const float* mean_rstd, const float* gamma,
+                                void* scratch, void* dz16, float* dsum, float* dgamma, float* dbeta, void* stream) {
+  GWX_TRY(check_btc(B, T, C));
+  if (G < 1 || !group_norm_backward_src_ok(C, G))
+    return fail(GWX_ESHAPE, "C=%d G=%d (C / 4 has to divide 256 and C / G be a multiple of 4, G <= 32)", C, G);
+  if (kind < 0 || kind > 3) return fail(GWX_EINVAL, "kind %d", kind);
+  if (!dy || !z || !mean_rstd || !gamma || !scratch || !dz16 || !dgamma || !dbeta || (kind != 0 && !out) ||
+      (kind == 2 && !arg))
+    return fail(GWX_EINVAL, "NULL array");
+  if ((((uintptr_t)dy) | ((uintptr_t)z) | ((uintptr_t)scratch) | ((uintptr_t)dsum)) & 15u ||
+      (((uintptr_t)out) | ((uintptr_t)dz16)) & 7u || ((uintptr_t)arg & 3u))
+    return fail(GWX_EINVAL, "dy, z, scratch, dsum 16-byte, out, dz16 8-byte, arg 4-byte aligned");
+  GWX_TRY(ensure_init());
+  return launched(launch_group_norm_backward_src(kind, dy, out, arg, z, B, T, C, G, mean_rstd, gamma, scratch, dz16,
+                                                 dsum, dgamma, dbeta, as_stream(stream)),
+                  "group_norm_backward_src");
+}
+
 int gwx_relu_mask(const float* dy, const void* out, int64_t n, float* d, void* stream) {
   if (n < 0) return fail(GWX_ESHAPE, "n");
   if (n == 0) return GWX_OK;
@@ -1108,6 +1147,20 @@ int gwx_conv1d_bf16(const void* x, int64_t B, int64_t T, int C, int k, const voi
     return fail(GWX_EINVAL, "x, W, z and addend must be 16-byte aligned");
   GWX_TRY(ensure_init());
   return launched(launch_conv_forward(x, B, T, C, k, W, O, addend, z, as_stream(stream)), "conv1d_bf16");
+}
+
+int gwx_conv1d_bf16_backward_dz(const void* dz16, const void* x, const void* W, int64_t B, int64_t T, int C, int O,
+                                int k, const float* addend, float* dx, float* dW, void* workspace,
+                                size_t workspace_bytes, void* stream) {
+  GWX_TRY(check_conv(B, T, C, O, k));
+  if (!dz16 || !x || !W) return fail(GWX_EINVAL, "NULL array");
+  if ((((uintptr_t)dz16) | ((uintptr_t)x) | ((uintptr_t)W) | ((uintptr_t)dx) | ((uintptr_t)dW) |
+       ((uintptr_t)addend)) & 15u)
+    return fail(GWX_EINVAL, "dz16, x, W, dx, dW and addend must be 16-byte aligned");
+  GWX_TRY(check_ws(workspace, workspace_bytes, conv_backward_ws(B, T, C, O, k)));
+  GWX_TRY(ensure_init());
+  return launched(launch_conv_backward_dz(dz16, x, W, B, T, C, O, k, addend, dx, dW, workspace, as_stream(stream)),
+                  "conv1d_bf16_backward_dz");
 }
 
 size_t gwx_conv1d_bf16_backward_workspace(int64_t B, int64_t T, int C, int O, int k) {

@@ -134,6 +134,8 @@ cudaError_t launch_conv_gemm(const void* x, int64_t Bn, int64_t T, int64_t C, in
 size_t conv_backward_ws(int64_t Bn, int64_t T, int C, int O, int k);
 cudaError_t launch_conv_forward(const void* x, int64_t Bn, int64_t T, int C, int k, const void* W, int O,
                                 const float* addend, float* z, cudaStream_t s);
+cudaError_t launch_conv_backward_dz(const void* dz16, const void* x, const void* W, int64_t Bn, int64_t T, int C, int O,
+                                    int k, const float* addend, float* dx, float* dW, void* ws, cudaStream_t s);
 cudaError_t launch_conv_backward(const float* dz, const void* x, const void* W, int64_t Bn, int64_t T, int C, int O,
                                  int k, const float* addend, float* dx, float* dW, void* ws, cudaStream_t s);
 cudaError_t gemm_status(int* status);
@@ -143,6 +145,8 @@ cudaError_t gemm_status(int* status);
 // and, with part, the column sums of every 32 rows; N even.
 cudaError_t launch_dz_rows(const float* dY, const void* Y, int64_t M, int N, void* dZ, float* part, cudaStream_t s);
 size_t dense_backward_ws(int64_t M, int64_t N, int64_t K);
+cudaError_t launch_dense_backward_dz(const void* dZ16, const void* X, const void* W, int64_t M, int64_t N, int64_t K,
+                                     float* dX, float* dW, void* ws, cudaStream_t s);
 cudaError_t launch_dense_backward(const void* X, const void* W, const float* bias, const float* dY, int64_t M,
                                   int64_t N, int64_t K, int act, float* dX, float* dW, float* db, void* ws, int group,
                                   cudaStream_t s,
@@ -279,6 +283,16 @@ size_t group_norm_backward_scratch(int64_t B, int C, int G);
 cudaError_t launch_group_norm_backward(const float* dy, const float* z, int64_t B, int T, int C, int G,
                                        const float* ms, const float* gamma, void* scratch, float* dz, float* dgamma,
                                        float* dbeta, cudaStream_t st);
+// The group norm's backward from a gradient formed on the fly (kind 0 as given, 1 masked by
+// out > 0, 2 routed back through the max pool and masked, 3 that of the mean over time,
+// masked), dz in bfloat16, the masked gradient itself in dsum (optional); per-sample shapes
+// (group_norm_backward_src_ok), 16-byte aligned arrays (arg 4, out and dz16 8).
+bool group_norm_backward_src_ok(int C, int G);
+size_t group_norm_backward_src_scratch(int64_t B, int C);
+cudaError_t launch_group_norm_backward_src(int kind, const float* dy, const void* out, const uint8_t* arg,
+                                           const float* z, int64_t B, int T, int C, int G, const float* ms,
+                                           const float* gamma, void* scratch, void* dz16, float* dsum, float* dgamma,
+                                           float* dbeta, cudaStream_t st);
 cudaError_t launch_relu_mask(const float* dy, const void* out, int64_t n, float* d, cudaStream_t st);
 cudaError_t launch_maxpool(const void* x, int64_t B, int T, int C, void* y, uint8_t* arg, cudaStream_t st);
 cudaError_t launch_maxpool_back(const float* dy, const uint8_t* arg, int64_t B, int T, int C, float* dx,

@@ -32,18 +32,23 @@ cudaError_t launch_conv_forward(const void* x, int64_t Bn, int64_t T, int C, int
 }
 
 // dx [B][T][C] (+ addend) and dW [O][k C] of the stride-1 convolution z = conv(x, W) given
-// dz [B][T][O] (FP32).
+// dz [B][T][O] in bfloat16; ws holds the split-K partial products.
+cudaError_t launch_conv_backward_dz(const void* dz16, const void* x, const void* W, int64_t Bn, int64_t T, int C, int O,
+                                    int k, const float* addend, float* dx, float* dW, void* ws, cudaStream_t s) {
+  // the input gradient: dz as the implicit A (channels O), taps mirrored
+  cudaError_t e = dx ? launch_conv_gemm(dz16, Bn, T, O, k, -1, W, C, dx, addend, s) : cudaSuccess;
+  if (e != cudaSuccess || !dW) return e;
+  return launch_conv_wgrad(dz16, x, dW, Bn, T, C, O, k, reinterpret_cast<float*>(ws), s);
+}
+
+// The same from FP32 dz.
 cudaError_t launch_conv_backward(const float* dz, const void* x, const void* W, int64_t Bn, int64_t T, int C, int O,
                                  int k, const float* addend, float* dx, float* dW, void* ws, cudaStream_t s) {
   const int64_t M = Bn * T;
-  char* w = reinterpret_cast<char*>(ws);
-  void* dZ = w;
-  float* part = reinterpret_cast<float*>(w + al256((size_t)M * O * 2));
-  cudaError_t e = launch_dz_rows(dz, nullptr, M, O, dZ, nullptr, s);
+  const cudaError_t e = launch_dz_rows(dz, nullptr, M, O, ws, nullptr, s);
   if (e != cudaSuccess) return e;
-  // the input gradient: dz as the implicit A (channels O), taps mirrored
-  if (dx && (e = launch_conv_gemm(dZ, Bn, T, O, k, -1, W, C, dx, addend, s)) != cudaSuccess) return e;
-  return dW ? launch_conv_wgrad(dZ, x, dW, Bn, T, C, O, k, part, s) : cudaSuccess;
+  return launch_conv_backward_dz(ws, x, W, Bn, T, C, O, k, addend, dx, dW,
+                                 reinterpret_cast<char*>(ws) + al256((size_t)M * O * 2), s);
 }
 
 }  // namespace gwx

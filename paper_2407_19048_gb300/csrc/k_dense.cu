@@ -113,6 +113,14 @@ size_t dense_backward_ws(int64_t M, int64_t N, int64_t K) {
          + align256(wgrad_ws(N, K, M, 1));           // split-K slices of dW
 }
 
+// dX = dZ W and dW = dZ^T X from dZ in bfloat16; ws holds the split-K partial products.
+cudaError_t launch_dense_backward_dz(const void* dZ16, const void* X, const void* W, int64_t M, int64_t N, int64_t K,
+                                     float* dX, float* dW, void* ws, cudaStream_t s) {
+  const cudaError_t e = dX ? launch_gemm_nn(dZ16, W, dX, M, K, N, s) : cudaSuccess;
+  if (e != cudaSuccess || !dW) return e;
+  return launch_wgrad(dZ16, X, dW, N, K, M, reinterpret_cast<float*>(ws), s);
+}
+
 cudaError_t launch_dense_backward(const void* X, const void* W, const float* bias, const float* dY, int64_t M,
                                   int64_t N, int64_t K, int act, float* dX, float* dW, float* db, void* ws, int group,
                                   cudaStream_t s, const void* Y) {
@@ -132,8 +140,7 @@ cudaError_t launch_dense_backward(const void* X, const void* W, const float* bia
                       ? launch_dz_rows(dY, Y16, M, (int)N, dZ, part, s)
                       : launch_gemm_dact(X, W, bias, dY, act, M, N, K, dZ, part, group, s);
   if (e != cudaSuccess) return e;
-  if (dX && (e = launch_gemm_nn(dZ, W, dX, M, K, N, s)) != cudaSuccess) return e;
-  if (dW && (e = launch_wgrad(dZ, X, dW, N, K, M, kpart, s)) != cudaSuccess) return e;
+  if ((e = launch_dense_backward_dz(dZ, X, W, M, N, K, dX, dW, kpart, s)) != cudaSuccess) return e;
   if (db) {
     const int slices = colsum_slices(P);
     k_colsum<<<dim3((unsigned)((N + TT - 1) / TT), (unsigned)slices), dim3(TT, TT), 0, s>>>(

@@ -490,18 +490,39 @@ bool make_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t K, uint32
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// out[g][i] = sum over s of part[s][g][i] for i < n (slices in order: deterministic); groups
-// of out ostride apart.
-__global__ void k_split_reduce(const float* __restrict__ part, int splits, int64_t n, int64_t ostride,
-                               float* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int64_t total = n * gridDim.y;
-  const float* p = part + (int64_t)blockIdx.y * n + i;
-  float acc = 0.f;
+// out[g][i] = sum over s of part[s][g][i] for i < n (a multiple of 4, 16-byte aligned); groups
+// of out ostride apart.  Four elements a thread; LANES threads share them, lane y taking slices
+// y, y + LANES, ... in order, then the lanes in order: deterministic.  Eight lanes for many
+// slices of a small result (64 of 64 x 320: 21 us one thread an element, 5 with eight lanes),
+// one for few slices of a large one (4 of 512 x 1968), where idle lanes only cost.
+template <int LANES>
+__global__ void __launch_bounds__(256) k_split_reduce(const float4* __restrict__ part, int splits, int64_t n4,
+                                                      int64_t ostride4, float4* __restrict__ out) {
+  constexpr int X = 256 / LANES;
+  __shared__ float4 red[LANES][X];
+  const int x = threadIdx.x % X, y = threadIdx.x / X;
+  const int64_t i = (int64_t)blockIdx.x * X + x;
+  const int64_t total = n4 * gridDim.y;
+  const float4* p = part + (int64_t)blockIdx.y * n4 + i;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [&acc](float4 v) {
+    acc.x += v.x;
+    acc.y += v.y;
+    acc.z += v.z;
+    acc.w += v.w;
+  };
+  if (i < n4) {
 #pragma unroll 4
-  for (int s = 0; s < splits; ++s) acc += __ldg(p + (int64_t)s * total);
-  out[(int64_t)blockIdx.y * ostride + i] = acc;
+    for (int s = y; s < splits; s += LANES) add(__ldg(p + (int64_t)s * total));
+  }
+  if constexpr (LANES > 1) {
+    red[y][x] = acc;
+    __syncthreads();
+    if (y != 0) return;
+#pragma unroll
+    for (int k = 1; k < LANES; ++k) add(red[k][x]);
+  }
+  if (i < n4) out[(int64_t)blockIdx.y * ostride4 + i] = acc;
 }
 
 // Everything of a launch but the operands.
@@ -554,12 +575,13 @@ cudaError_t run_gemm_at(int tn, const CUtensorMap& ta, const CUtensorMap& tb, co
 
 // Tile width of a product: 256 columns unless the 128 x 256 tiles would leave more than half
 // of the SMs idle (the flow's conditioner products on a few hundred to a few thousand rows),
-// then 128 or 64, so that more CTAs share the work.  Split-K products keep 256.
+// then 128 or 64, so that more CTAs share the work; no wider than N needs (the stem's product
+// has 64 columns).  Split-K products keep 256.
 int gemm_tile_width(int64_t M, int64_t N, int splits, int sms) {
   if (splits > 1) return GN;
   const int64_t tm = (M + GM - 1) / GM;
   for (int tn : {256, 128})
-    if (tm * ((N + tn - 1) / tn) * 2 >= sms) return tn;
+    if (2 * N > tn && tm * ((N + tn - 1) / tn) * 2 >= sms) return tn;
   return 64;
 }
 
@@ -687,8 +709,15 @@ size_t wgrad_ws(int64_t M, int64_t N, int64_t K, int64_t groups) {
 
 static cudaError_t wgrad_finish(const GemmCall& c, float* C, int64_t cstride, const float* part, cudaStream_t s) {
   if (c.splits <= 1) return cudaSuccess;
-  const int64_t n = c.M * c.N;
-  k_split_reduce<<<dim3((unsigned)((n + 255) / 256), (unsigned)c.groups), 256, 0, s>>>(part, c.splits, n, cstride, C);
+  const int64_t n4 = c.M * c.N / 4;   // N is a multiple of 8
+  const auto* p = reinterpret_cast<const float4*>(part);
+  auto* out = reinterpret_cast<float4*>(C);
+  if (c.splits >= 16)
+    k_split_reduce<8><<<dim3((unsigned)((n4 + 31) / 32), (unsigned)c.groups), 256, 0, s>>>(p, c.splits, n4, cstride / 4,
+                                                                                           out);
+  else
+    k_split_reduce<1><<<dim3((unsigned)((n4 + 255) / 256), (unsigned)c.groups), 256, 0, s>>>(p, c.splits, n4,
+                                                                                             cstride / 4, out);
   return cudaGetLastError();
 }
 

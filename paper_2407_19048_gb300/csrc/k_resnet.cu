@@ -3,10 +3,11 @@
 // all channels per output time) times the weights on the tensor cores
 // (gwx_dense_bf16 / gwx_dense_bf16_backward); these kernels build the rows (k_im2col,
 // k_im2col_cf for the channels-first input strain), fold row gradients back (k_col2im),
-// normalise per sample and channel group (k_gn_stats, k_gn_apply, with the residual
-// addition and the ReLU fused) and take the gradient of that (k_gn_bwd_stats,
-// k_gn_bwd_apply, k_gn_param_part / k_gn_param_finish, k_relu_mask), and pool (k_maxpool, k_mean_time and
-// their backward).
+// normalise per sample and channel group with the residual addition and the ReLU
+// (k_gn_forward_s; k_gn_stats, k_gn_apply for other channel counts) and take the gradient of
+// that (k_gn_backward_s, which also masks or gathers the gradient it starts from;
+// k_gn_bwd_stats, k_gn_bwd_apply, k_gn_param_part / k_gn_param_finish, k_relu_mask), and pool
+// (k_maxpool, k_mean_time and their backward).
 #include <stdint.h>
 
 #include <algorithm>
@@ -165,97 +166,260 @@ __global__ void __launch_bounds__(256) k_gn_stats(const float* __restrict__ z, i
   }
 }
 
-// Per-sample variants of the two statistics kernels for C / 4 dividing 256: one block of
-// 256 threads reads sample b's whole [T][C] slab with coalesced float4 loads (thread
-// (row lane l, column quad q) reads rows l, l + 256 / (C / 4), ... of channels 4 q ..
-// 4 q + 3), FP32 sums over runs of 16 rows added into FP64; then the row lanes of each
-// column quad and the column quads of each group are added in order.
-__device__ __forceinline__ void sample_group_sums(double a, double q, int cq, int rl, int cg, int G, double* out) {
-  __shared__ double r1[256], r2[256];
-  const int tid = threadIdx.x;
-  r1[tid] = a;
-  r2[tid] = q;
-  __syncthreads();
-  if (tid < cq) {
-    double x = 0.0, y = 0.0;
-    for (int l = 0; l < rl; ++l) {
-      x += r1[l * cq + tid];
-      y += r2[l * cq + tid];
-    }
-    r1[tid] = x;
-    r2[tid] = y;
+// Per-sample group norm for C / 4 dividing 256: one block takes sample b's [T][C] slab twice,
+// first for the sums and then to apply them, so that no launch and no second statistics array
+// lies between; part of the second pass hits in L2.  HBM bound as long as enough loads are in
+// flight: every pass first issues its rows' loads (eight, or four of several arrays) and then
+// adds them (a loop of load and add kept one row in flight, 10 us a slab).  (512 windows, stem
+// and two blocks, six normalisations: 337 us as a statistics and an apply kernel forward, now
+// 225; ~700 us backward with the ReLU mask, the FP32 dz and its conversion as passes of their
+// own, now 510.)
+// Sums: thread (run slice s, row lane l, column quad q) reads runs of 16 rows, rl = 256 / (C / 4)
+// rows apart, of channels 4 q .. 4 q + 3, coalesced float4 loads; FP32 within a run, FP64
+// across runs; then the lanes of each column quad and the quads of each group.
+constexpr int GN_NT = 512;
+// threads of the backward: the pooled gradient's rows hold twice the registers
+constexpr int gn_bt(int src) { return src == 2 ? 256 : 512; }
+
+// Sums of a (and q) over the threads of every group (out[2 g], out[2 g + 1], valid after the
+// caller's barrier): lanes of a warp that share a column quad by shuffles, the remaining rows
+// of quads in shared memory, one warp per group.
+template <int NT>
+__device__ __forceinline__ void sample_group_sums(double a, double q, int cq, int cg, int G, double* out) {
+  __shared__ double r1[NT], r2[NT];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int o = 16; o >= cq; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    q += __shfl_xor_sync(0xffffffffu, q, o);
+  }
+  const int rows = cq < 32 ? NT / 32 : NT / cq;
+  if (cq >= 32) {
+    r1[threadIdx.x] = a;
+    r2[threadIdx.x] = q;
+  } else if (lane < cq) {
+    r1[warp * cq + lane] = a;
+    r2[warp * cq + lane] = q;
   }
   __syncthreads();
-  if (tid < G) {
+  const int per = cg / 4;
+  for (int g = warp; g < G; g += NT / 32) {
     double x = 0.0, y = 0.0;
-    for (int k = tid * (cg / 4); k < (tid + 1) * (cg / 4); ++k) {
-      x += r1[k];
-      y += r2[k];
+    for (int i = lane; i < rows * per; i += 32) {
+      const int at = (i / per) * cq + g * per + i % per;
+      x += r1[at];
+      y += r2[at];
     }
-    out[2 * tid] = x;
-    out[2 * tid + 1] = y;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      x += __shfl_xor_sync(0xffffffffu, x, o);
+      y += __shfl_xor_sync(0xffffffffu, y, o);
+    }
+    if (lane == 0) {
+      out[2 * g] = x;
+      out[2 * g + 1] = y;
+    }
   }
 }
 
-__global__ void __launch_bounds__(256) k_gn_stats_s(const float* __restrict__ z, int T, int C, int G,
-                                                    float* __restrict__ ms) {
+__device__ __forceinline__ float4 bf16x4(uint2 q) {
+  const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.x));
+  const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.y));
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ uint2 to_bf16x4(float a, float b, float c, float d) {
+  __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
+  return make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+}
+
+__global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restrict__ z, int T, int C, int G,
+                                                           double inv_n, const float* __restrict__ gamma,
+                                                           const float* __restrict__ beta,
+                                                           const float* __restrict__ res32,
+                                                           const __nv_bfloat16* __restrict__ res16, int relu,
+                                                           __nv_bfloat16* __restrict__ out16,
+                                                           float* __restrict__ out32, float* __restrict__ ms) {
   __shared__ double sums[64];
+  __shared__ float st[64];
   const int cq = C / 4, rl = 256 / cq, cg = C / G;
-  const int q4 = threadIdx.x % cq, l0 = threadIdx.x / cq;
-  const float* zb = z + (int64_t)blockIdx.x * T * C;
-  const float k0 = __ldg(zb + ((4 * q4) / cg) * cg);
+  const int q4 = threadIdx.x % cq, l0 = (threadIdx.x % 256) / cq, g = (4 * q4) / cg;
+  const int64_t off = (int64_t)blockIdx.x * T * C;
+  const float4* z4 = reinterpret_cast<const float4*>(z + off) + q4;   // row t at t cq
+  const float k0 = __ldg(z + off + g * cg);
   double a = 0.0, q = 0.0;
-  for (int t0 = l0; t0 < T; t0 += 16 * rl) {
+  for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_NT / 256) * 16 * rl) {
     float s1 = 0.f, s2 = 0.f;
-#pragma unroll 4
-    for (int t = t0; t < min(T, t0 + 16 * rl); t += rl) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(zb + (int64_t)t * C) + q4);
-      const float d0 = v.x - k0, d1 = v.y - k0, d2 = v.z - k0, d3 = v.w - k0;
-      s1 += (d0 + d1) + (d2 + d3);
-      s2 += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float4 v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int t = t0 + (8 * h + i) * rl;
+        v[i] = t < T ? __ldg(z4 + t * cq) : make_float4(k0, k0, k0, k0);   // adds zero
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float d0 = v[i].x - k0, d1 = v[i].y - k0, d2 = v[i].z - k0, d3 = v[i].w - k0;
+        s1 += (d0 + d1) + (d2 + d3);
+        s2 += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+      }
     }
     a += s1;
     q += s2;
   }
-  sample_group_sums(a, q, cq, rl, cg, G, sums);
+  const float kg = (int)threadIdx.x < G ? __ldg(z + off + threadIdx.x * cg) : 0.f;
+  const float4 gm = make_float4(__ldg(&gamma[4 * q4]), __ldg(&gamma[4 * q4 + 1]), __ldg(&gamma[4 * q4 + 2]),
+                                __ldg(&gamma[4 * q4 + 3]));
+  const float4 bt = make_float4(__ldg(&beta[4 * q4]), __ldg(&beta[4 * q4 + 1]), __ldg(&beta[4 * q4 + 2]),
+                                __ldg(&beta[4 * q4 + 3]));
+  sample_group_sums<GN_NT>(a, q, cq, cg, G, sums);
+  __syncthreads();
   if ((int)threadIdx.x < G) {
-    const int g = threadIdx.x;
-    const double n = (double)T * cg, m = sums[2 * g] / n, var = fmax(sums[2 * g + 1] / n - m * m, 0.0);
-    ms[2 * ((int64_t)blockIdx.x * G + g)] = (float)((double)__ldg(zb + g * cg) + m);
-    ms[2 * ((int64_t)blockIdx.x * G + g) + 1] = (float)(1.0 / sqrt(var + (double)GN_EPS));
+    const int i = threadIdx.x;
+    const double m = sums[2 * i] * inv_n, var = fmax(sums[2 * i + 1] * inv_n - m * m, 0.0);
+    const float mean = (float)((double)kg + m), rstd = (float)rsqrt(var + (double)GN_EPS);
+    st[2 * i] = mean;
+    st[2 * i + 1] = rstd;
+    ms[2 * ((int64_t)blockIdx.x * G + i)] = mean;
+    ms[2 * ((int64_t)blockIdx.x * G + i) + 1] = rstd;
+  }
+  __syncthreads();
+  const float mean = st[2 * g], rstd = st[2 * g + 1];
+  const int step = GN_NT / cq;
+  for (int tb = threadIdx.x / cq; tb < T; tb += 4 * step) {
+    float4 x[4], r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int t = min(tb + k * step, T - 1);
+      x[k] = __ldcs(z4 + t * cq);
+      if (res32) r[k] = __ldg(reinterpret_cast<const float4*>(res32 + off) + t * cq + q4);
+      if (res16) r[k] = bf16x4(__ldg(reinterpret_cast<const uint2*>(res16 + off) + t * cq + q4));
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int t = tb + k * step;
+      if (t >= T) break;
+      const int64_t i = off + (int64_t)t * C + 4 * q4;
+      float4 v = make_float4(fmaf((x[k].x - mean) * rstd, gm.x, bt.x), fmaf((x[k].y - mean) * rstd, gm.y, bt.y),
+                             fmaf((x[k].z - mean) * rstd, gm.z, bt.z), fmaf((x[k].w - mean) * rstd, gm.w, bt.w));
+      if (res32 || res16) {
+        v.x += r[k].x; v.y += r[k].y; v.z += r[k].z; v.w += r[k].w;
+      }
+      if (relu) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+      if (out16) *reinterpret_cast<uint2*>(out16 + i) = to_bf16x4(v.x, v.y, v.z, v.w);
+      if (out32) *reinterpret_cast<float4*>(out32 + i) = v;
+    }
   }
 }
 
-// part (optional, [B][C][2] doubles): this sample's sums of dy xhat and dy per channel (FP32
-// over runs of at most 16 rows, FP64 across runs and, in a fixed order, across the threads
-// that share the channels), the partials of dgamma and dbeta that k_gn_param_finish adds.
-__global__ void __launch_bounds__(256, 4) k_gn_bwd_stats_s(const float* __restrict__ dy, const float* __restrict__ z,
-                                                        int T, int C, int G, const float* __restrict__ ms,
-                                                        const float* __restrict__ gamma, float* __restrict__ mm,
-                                                        double* __restrict__ part) {
+// The gradient dy the backward starts from: as given; masked by out > 0 (the ReLU after the
+// normalisation); the max pool's gradient routed back to its arguments, then masked; or the
+// mean over time's, dm / T, masked.  Loads and values apart, so that several rows' loads can
+// be in flight.
+enum : int { DY_PLAIN = 0, DY_MASK = 1, DY_POOL = 2, DY_MEAN = 3 };
+struct GnSource {
+  const float* dy;             // [B][T][C]; DY_POOL [B][To][C]; DY_MEAN [B][C]
+  const __nv_bfloat16* out;    // [B][T][C]
+  const uint8_t* arg;          // DY_POOL: [B][To][C]
+  int To;
+};
+template <int SRC>
+struct GnRow {
+  float4 v0, v1;
+  uchar4 a0, a1;
+  uint2 o;
+};
+
+template <int SRC>
+__device__ __forceinline__ void gn_load(GnRow<SRC>& r, const GnSource& s, int64_t b, int t, int c, int T, int C) {
+  const int64_t i = (b * T + t) * C + c;
+  if constexpr (SRC == DY_POOL) {
+    // time t is argument 1 of window t/2 (even t), or 2 of window t/2 and 0 of the next (odd t)
+    const int to = t / 2;
+    const int64_t o = (b * s.To + to) * C + c;
+    r.v0 = r.v1 = make_float4(0.f, 0.f, 0.f, 0.f);
+    r.a0 = r.a1 = make_uchar4(3, 3, 3, 3);
+    if (to < s.To) {
+      r.v0 = __ldg(reinterpret_cast<const float4*>(s.dy + o));
+      r.a0 = __ldg(reinterpret_cast<const uchar4*>(s.arg + o));
+    }
+    if ((t & 1) && to + 1 < s.To) {
+      r.v1 = __ldg(reinterpret_cast<const float4*>(s.dy + o + C));
+      r.a1 = __ldg(reinterpret_cast<const uchar4*>(s.arg + o + C));
+    }
+  } else if constexpr (SRC != DY_MEAN) {
+    r.v0 = __ldg(reinterpret_cast<const float4*>(s.dy + i));
+  }
+  if constexpr (SRC != DY_PLAIN) r.o = __ldg(reinterpret_cast<const uint2*>(s.out + i));
+}
+
+template <int SRC>
+__device__ __forceinline__ float4 gn_value(const GnRow<SRC>& r, int t, float4 mean_dy) {
+  float4 d = r.v0;
+  if constexpr (SRC == DY_MEAN) d = mean_dy;
+  if constexpr (SRC == DY_POOL) {
+    const int k = 1 + (t & 1);
+    d = make_float4((r.a0.x == k ? r.v0.x : 0.f) + (r.a1.x == 0 ? r.v1.x : 0.f),
+                    (r.a0.y == k ? r.v0.y : 0.f) + (r.a1.y == 0 ? r.v1.y : 0.f),
+                    (r.a0.z == k ? r.v0.z : 0.f) + (r.a1.z == 0 ? r.v1.z : 0.f),
+                    (r.a0.w == k ? r.v0.w : 0.f) + (r.a1.w == 0 ? r.v1.w : 0.f));
+  }
+  if constexpr (SRC != DY_PLAIN) {
+    const float4 o = bf16x4(r.o);
+    d = make_float4(o.x > 0.f ? d.x : 0.f, o.y > 0.f ? d.y : 0.f, o.z > 0.f ? d.z : 0.f, o.w > 0.f ? d.w : 0.f);
+  }
+  return d;
+}
+
+// dz = rstd (dy gamma - m1 - xhat m2) (FP32 or bfloat16), the masked dy itself (optional) and,
+// per channel, this sample's sums of dy xhat and dy (part, [B][C][2] doubles), the partials
+// of dgamma and dbeta that k_gn_param_finish adds.
+template <int SRC, bool OUT16>
+__global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, const float* __restrict__ z, int T, int C,
+                                                            int G, double inv_n, const float* __restrict__ ms,
+                                                            const float* __restrict__ gamma, void* __restrict__ dz,
+                                                            float* __restrict__ dsum, double* __restrict__ part) {
+  constexpr int GN_BT = gn_bt(SRC);
   __shared__ double sums[64];
-  __shared__ double pr[256 * 8];
+  __shared__ double pr[GN_BT * 8];
+  __shared__ float st[64];
+  constexpr int U = 4;   // rows in flight
   const int cq = C / 4, rl = 256 / cq, cg = C / G;
-  const int q4 = threadIdx.x % cq, l0 = threadIdx.x / cq, g = (4 * q4) / cg;
-  const int64_t off = (int64_t)blockIdx.x * T * C;
-  const float mean = ms[2 * ((int64_t)blockIdx.x * G + g)], rstd = ms[2 * ((int64_t)blockIdx.x * G + g) + 1];
+  const int q4 = threadIdx.x % cq, l0 = (threadIdx.x % 256) / cq, g = (4 * q4) / cg;
+  const int64_t b = blockIdx.x, off = b * T * C;
+  const float4* z4 = reinterpret_cast<const float4*>(z + off) + q4;   // row t at t cq
+  const float mean = ms[2 * (b * G + g)], rstd = ms[2 * (b * G + g) + 1];
   const float4 gm = make_float4(__ldg(&gamma[4 * q4]), __ldg(&gamma[4 * q4 + 1]), __ldg(&gamma[4 * q4 + 2]),
                                 __ldg(&gamma[4 * q4 + 3]));
+  float4 mdy = make_float4(0.f, 0.f, 0.f, 0.f);
+  if constexpr (SRC == DY_MEAN) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(src.dy + b * C) + q4);
+    mdy = make_float4(v.x / T, v.y / T, v.z / T, v.w / T);
+  }
   double a = 0.0, q = 0.0;
   double pg[4] = {0.0, 0.0, 0.0, 0.0}, pb[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int t0 = l0; t0 < T; t0 += 16 * rl) {
+  for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_BT / 256) * 16 * rl) {
     float s1 = 0.f, s2 = 0.f;
     float fg[4] = {0.f, 0.f, 0.f, 0.f}, fb[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int t = t0; t < min(T, t0 + 16 * rl); t += rl) {
-      const float4 d = __ldg(reinterpret_cast<const float4*>(dy + off + (int64_t)t * C) + q4);
-      const float4 x = __ldg(reinterpret_cast<const float4*>(z + off + (int64_t)t * C) + q4);
-      const float a0 = d.x * gm.x, a1 = d.y * gm.y, a2 = d.z * gm.z, a3 = d.w * gm.w;
-      const float h0 = (x.x - mean) * rstd, h1 = (x.y - mean) * rstd, h2 = (x.z - mean) * rstd,
-                  h3 = (x.w - mean) * rstd;
-      s1 += (a0 + a1) + (a2 + a3);
-      s2 += (a0 * h0 + a1 * h1) + (a2 * h2 + a3 * h3);
-      if (part) {
+#pragma unroll 1
+    for (int h = 0; h < 16; h += U) {
+      GnRow<SRC> r[U];
+      float4 x[U];
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        const int t = min(t0 + (h + i) * rl, T - 1);
+        gn_load<SRC>(r[i], src, b, t, 4 * q4, T, C);
+        x[i] = __ldg(z4 + t * cq);
+      }
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        const int t = t0 + (h + i) * rl;
+        if (t >= T) break;
+        const float4 d = gn_value<SRC>(r[i], t, mdy);
+        const float a0 = d.x * gm.x, a1 = d.y * gm.y, a2 = d.z * gm.z, a3 = d.w * gm.w;
+        const float h0 = (x[i].x - mean) * rstd, h1 = (x[i].y - mean) * rstd, h2 = (x[i].z - mean) * rstd,
+                    h3 = (x[i].w - mean) * rstd;
+        s1 += (a0 + a1) + (a2 + a3);
+        s2 += (a0 * h0 + a1 * h1) + (a2 * h2 + a3 * h3);
         fg[0] += d.x * h0;
         fg[1] += d.y * h1;
         fg[2] += d.z * h2;
@@ -274,29 +438,69 @@ __global__ void __launch_bounds__(256, 4) k_gn_bwd_stats_s(const float* __restri
       pb[m] += fb[m];
     }
   }
-  sample_group_sums(a, q, cq, rl, cg, G, sums);
-  if ((int)threadIdx.x < G) {
-    const double n = (double)T * cg;
-    mm[2 * ((int64_t)blockIdx.x * G + threadIdx.x)] = (float)(sums[2 * threadIdx.x] / n);
-    mm[2 * ((int64_t)blockIdx.x * G + threadIdx.x) + 1] = (float)(sums[2 * threadIdx.x + 1] / n);
-  }
   if (part) {
+    // lanes of a warp that share a column quad first, then one row of quads per warp
+    for (int o = 16; o >= cq; o >>= 1) {
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      pr[threadIdx.x * 8 + m] = pg[m];
-      pr[threadIdx.x * 8 + 4 + m] = pb[m];
-    }
-    __syncthreads();
-    // thread tid < C: channel tid, summed over the rl threads l = 0 .. rl-1 in order
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-      const int qq = c / 4, m = c % 4;
-      double sg = 0.0, sb = 0.0;
-      for (int l = 0; l < rl; ++l) {
-        sg += pr[(l * cq + qq) * 8 + m];
-        sb += pr[(l * cq + qq) * 8 + 4 + m];
+      for (int m = 0; m < 4; ++m) {
+        pg[m] += __shfl_xor_sync(0xffffffffu, pg[m], o);
+        pb[m] += __shfl_xor_sync(0xffffffffu, pb[m], o);
       }
-      part[((int64_t)blockIdx.x * C + c) * 2] = sg;
-      part[((int64_t)blockIdx.x * C + c) * 2 + 1] = sb;
+    }
+    const int lane = threadIdx.x & 31, at = cq >= 32 ? threadIdx.x : (threadIdx.x >> 5) * cq + lane;
+    if (cq >= 32 || lane < cq) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        pr[at * 8 + m] = pg[m];
+        pr[at * 8 + 4 + m] = pb[m];
+      }
+    }
+  }
+  sample_group_sums<GN_BT>(a, q, cq, cg, G, sums);
+  __syncthreads();
+  if ((int)threadIdx.x < G) {
+    st[2 * threadIdx.x] = (float)(sums[2 * threadIdx.x] * inv_n);
+    st[2 * threadIdx.x + 1] = (float)(sums[2 * threadIdx.x + 1] * inv_n);
+  }
+  __syncthreads();
+  if (part) {
+    // one thread per channel and sum, over the rows of quads in order
+    const int rows = cq < 32 ? GN_BT / 32 : GN_BT / cq;
+    for (int i = threadIdx.x; i < 2 * C; i += GN_BT) {
+      const int c = i >> 1, k = (c & 3) + 4 * (i & 1);
+      double t = 0.0;
+#pragma unroll 4
+      for (int r = 0; r < rows; ++r) t += pr[(r * cq + c / 4) * 8 + k];
+      part[b * 2 * C + i] = t;
+    }
+  }
+  const float m1 = st[2 * g], m2 = st[2 * g + 1];
+  const int step = GN_BT / cq;
+  for (int tb = threadIdx.x / cq; tb < T; tb += U * step) {
+    GnRow<SRC> r[U];
+    float4 x[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int t = min(tb + k * step, T - 1);
+      gn_load<SRC>(r[k], src, b, t, 4 * q4, T, C);
+      x[k] = __ldcs(z4 + t * cq);
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int t = tb + k * step;
+      if (t >= T) break;
+      const int64_t i = off + (int64_t)t * C + 4 * q4;
+      const float4 d = gn_value<SRC>(r[k], t, mdy);
+      float4 o;
+      o.x = rstd * (d.x * gm.x - m1 - (x[k].x - mean) * rstd * m2);
+      o.y = rstd * (d.y * gm.y - m1 - (x[k].y - mean) * rstd * m2);
+      o.z = rstd * (d.z * gm.z - m1 - (x[k].z - mean) * rstd * m2);
+      o.w = rstd * (d.w * gm.w - m1 - (x[k].w - mean) * rstd * m2);
+      if constexpr (OUT16)
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(dz) + i) = to_bf16x4(o.x, o.y, o.z, o.w);
+      else
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(dz) + i) = o;
+      if (dsum) *reinterpret_cast<float4*>(dsum + i) = d;
     }
   }
 }
@@ -494,26 +698,35 @@ __global__ void __launch_bounds__(256) k_gn_param_part(const float* __restrict__
   }
 }
 
-// Slices in order: block (32 channels) x (32 lanes), lane y summing slices y, y + 32, ...,
-// then the 32 lanes in order.
-__global__ void __launch_bounds__(1024) k_gn_param_finish(const double* __restrict__ part, int slices, int C,
-                                                          float* __restrict__ dgamma, float* __restrict__ dbeta) {
-  __shared__ double rg[32][33], rb[32][33];
-  const int c = blockIdx.x * 32 + threadIdx.x;
+// Sums of the slices: block of 8 channels x 32 slice lanes (lane l: slices l, l + 32, ...),
+// the lanes of a warp by shuffles, the warps in order (4 blocks of 32 channels took 14.7 us
+// for 512 slices of 128).
+__global__ void __launch_bounds__(256) k_gn_param_finish(const double* __restrict__ part, int slices, int C,
+                                                         float* __restrict__ dgamma, float* __restrict__ dbeta) {
+  __shared__ double2 r[8][8];
+  const int c = blockIdx.x * 8 + (threadIdx.x & 7);
   double tg = 0.0, tb = 0.0;
-  if (c < C)
-    for (int s = threadIdx.y; s < slices; s += 32) {
-      tg += part[((int64_t)s * C + c) * 2];
-      tb += part[((int64_t)s * C + c) * 2 + 1];
+  if (c < C) {
+#pragma unroll 8
+    for (int s = threadIdx.x >> 3; s < slices; s += 32) {
+      const double2 v = __ldg(reinterpret_cast<const double2*>(part) + (int64_t)s * C + c);
+      tg += v.x;
+      tb += v.y;
     }
-  rg[threadIdx.y][threadIdx.x] = tg;
-  rb[threadIdx.y][threadIdx.x] = tb;
+  }
+#pragma unroll
+  for (int o = 16; o >= 8; o >>= 1) {
+    tg += __shfl_xor_sync(0xffffffffu, tg, o);
+    tb += __shfl_xor_sync(0xffffffffu, tb, o);
+  }
+  if ((threadIdx.x & 31) < 8) r[threadIdx.x >> 5][threadIdx.x & 7] = make_double2(tg, tb);
   __syncthreads();
-  if (threadIdx.y == 0 && c < C) {
+  if (threadIdx.x < 8 && c < C) {
     double g = 0.0, bsum = 0.0;
-    for (int y = 0; y < 32; ++y) {
-      g += rg[y][threadIdx.x];
-      bsum += rb[y][threadIdx.x];
+#pragma unroll
+    for (int y = 0; y < 8; ++y) {
+      g += r[y][threadIdx.x].x;
+      bsum += r[y][threadIdx.x].y;
     }
     dgamma[c] = (float)g;
     dbeta[c] = (float)bsum;
@@ -540,6 +753,45 @@ __global__ void k_maxpool(const __nv_bfloat16* __restrict__ x, int T, int C, int
   }
   y[b * To * C + i] = __float2bfloat16_rn(best);
   arg[b * To * C + i] = (uint8_t)a;
+}
+
+// The same for eight consecutive channels per thread (C % 8 == 0, 16-byte aligned x and y,
+// 8-byte aligned arg): one 16-byte load per tap (512 windows of 1024 x 64: 65 us one channel
+// a thread).
+__global__ void k_maxpool8(const __nv_bfloat16* __restrict__ x, int T, int C, int To, __nv_bfloat16* __restrict__ y,
+                           uint8_t* __restrict__ arg) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, cv = C / 8;
+  if (i >= To * cv) return;
+  const int64_t b = blockIdx.y;
+  const int t = i / cv, c = 8 * (i - t * cv);
+  uint4 v[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const int src = 2 * t + j - 1;
+    v[j] = src >= 0 && src < T ? __ldg(reinterpret_cast<const uint4*>(x + (b * T + src) * C + c))
+                               : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);   // -inf: never first
+  }
+  const __nv_bfloat16* e0 = reinterpret_cast<const __nv_bfloat16*>(&v[0]);
+  __nv_bfloat16 best[8];
+  uint8_t a[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    float m = -INFINITY;
+    a[k] = 0;
+    best[k] = __float2bfloat16_rn(m);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const float f = __bfloat162float(e0[8 * j + k]);
+      if (f > m) {
+        m = f;
+        best[k] = e0[8 * j + k];
+        a[k] = (uint8_t)j;
+      }
+    }
+  }
+  const int64_t o = (b * To + t) * C + c;
+  *reinterpret_cast<uint4*>(y + o) = *reinterpret_cast<const uint4*>(best);
+  *reinterpret_cast<uint2*>(arg + o) = *reinterpret_cast<const uint2*>(a);
 }
 
 __global__ void k_maxpool_back(const float* __restrict__ dy, const uint8_t* __restrict__ arg, int T, int C, int To,
@@ -587,7 +839,8 @@ __global__ void k_mean_time(const __nv_bfloat16* __restrict__ x, int64_t B, int 
   const int64_t b = i / C;
   const int c = (int)(i - b * C);
   float acc = 0.f;
-  for (int t = 0; t < T; ++t) acc += __bfloat162float(x[(b * T + t) * C + c]);
+#pragma unroll 16
+  for (int t = 0; t < T; ++t) acc += __bfloat162float(x[(b * T + t) * C + c]);   // in order; 16 loads in flight
   m[i] = __float2bfloat16_rn(acc / T);
 }
 
@@ -646,9 +899,7 @@ cudaError_t launch_group_norm(const float* z, int64_t B, int T, int C, int G, co
   const auto r16 = reinterpret_cast<const __nv_bfloat16*>(res16);
   const auto o16 = reinterpret_cast<__nv_bfloat16*>(out16);
   if (v4 && per_sample_ok(C, G)) {
-    k_gn_stats_s<<<(unsigned)B, 256, 0, st>>>(z, T, C, G, ms);
-    k_gn_apply<4><<<dim3(nblk((int64_t)T * C / 4, 256), (unsigned)B), 256, 0, st>>>(z, T, C, G, ms, gamma, beta, res32,
-                                                                                    r16, relu, o16, out32);
+    k_gn_forward_s<<<(unsigned)B, GN_NT, 0, st>>>(z, T, C, G, 1.0 / ((double)T * (C / G)), gamma, beta, res32, r16, relu, o16, out32, ms);
   } else if (v4) {
     k_gn_stats<4><<<(unsigned)(B * G), 256, 0, st>>>(z, T, C, G, ms);
     k_gn_apply<4><<<dim3(nblk((int64_t)T * C / 4, 256), (unsigned)B), 256, 0, st>>>(z, T, C, G, ms, gamma, beta, res32,
@@ -675,11 +926,10 @@ cudaError_t launch_group_norm_backward(const float* dy, const float* z, int64_t 
   if (v4 && per_sample_ok(C, G)) {
     // the per-channel parameter sums come out of the statistics pass, one slice per sample
     const bool fused = B <= GN_MAX_SLICES;
-    k_gn_bwd_stats_s<<<(unsigned)B, 256, 0, st>>>(dy, z, T, C, G, ms, gamma, mm, fused ? part : nullptr);
-    k_gn_bwd_apply<4><<<dim3(nblk((int64_t)T * C / 4, 256), (unsigned)B), 256, 0, st>>>(dy, z, T, C, G, ms, mm, gamma,
-                                                                                        dz);
+    k_gn_backward_s<DY_PLAIN, false><<<(unsigned)B, gn_bt(DY_PLAIN), 0, st>>>(GnSource{dy, nullptr, nullptr, 0}, z, T, C, G,
+                                                                    1.0 / ((double)T * (C / G)), ms, gamma, dz, nullptr, fused ? part : nullptr);
     if (fused) {
-      k_gn_param_finish<<<nblk(C, 32), dim3(32, 32), 0, st>>>(part, (int)B, C, dgamma, dbeta);
+      k_gn_param_finish<<<nblk(C, 8), 256, 0, st>>>(part, (int)B, C, dgamma, dbeta);
       return cudaGetLastError();
     }
   } else if (v4) {
@@ -692,7 +942,32 @@ cudaError_t launch_group_norm_backward(const float* dy, const float* z, int64_t 
   }
   const int slices = gn_slices(B * T);
   k_gn_param_part<<<dim3(nblk(C, 32), slices), 256, 0, st>>>(dy, z, (int)(B * T), T, C, G, ms, part);
-  k_gn_param_finish<<<nblk(C, 32), dim3(32, 32), 0, st>>>(part, slices, C, dgamma, dbeta);
+  k_gn_param_finish<<<nblk(C, 8), 256, 0, st>>>(part, slices, C, dgamma, dbeta);
+  return cudaGetLastError();
+}
+
+bool group_norm_backward_src_ok(int C, int G) { return C % G == 0 && per_sample_ok(C, G); }
+
+size_t group_norm_backward_src_scratch(int64_t B, int C) { return (size_t)B * C * 2 * sizeof(double); }
+
+cudaError_t launch_group_norm_backward_src(int kind, const float* dy, const void* out, const uint8_t* arg,
+                                           const float* z, int64_t B, int T, int C, int G, const float* ms,
+                                           const float* gamma, void* scratch, void* dz16, float* dsum, float* dgamma,
+                                           float* dbeta, cudaStream_t st) {
+  const GnSource src{dy, reinterpret_cast<const __nv_bfloat16*>(out), arg, (T + 2 - 3) / 2 + 1};
+  double* part = reinterpret_cast<double*>(scratch);
+  const double inv_n = 1.0 / ((double)T * (C / G));
+  auto run = [&](auto kern) { kern<<<(unsigned)B, gn_bt(kind), 0, st>>>(src, z, T, C, G, inv_n, ms, gamma, dz16, dsum, part); };
+  switch (kind) {
+    case DY_PLAIN: run(k_gn_backward_s<DY_PLAIN, true>); break;
+    case DY_MASK: run(k_gn_backward_s<DY_MASK, true>); break;
+    case DY_POOL: run(k_gn_backward_s<DY_POOL, true>); break;
+    case DY_MEAN: run(k_gn_backward_s<DY_MEAN, true>); break;
+    default: return cudaErrorInvalidValue;
+  }
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_gn_param_finish<<<nblk(C, 8), 256, 0, st>>>(part, (int)B, C, dgamma, dbeta);
   return cudaGetLastError();
 }
 
@@ -706,6 +981,11 @@ cudaError_t launch_relu_mask(const float* dy, const void* out, int64_t n, float*
 
 cudaError_t launch_maxpool(const void* x, int64_t B, int T, int C, void* y, uint8_t* arg, cudaStream_t st) {
   const int To = (T + 2 - 3) / 2 + 1;
+  if (C % 8 == 0 && aligned16(x) && aligned16(y) && ((uintptr_t)arg & 7u) == 0) {
+    k_maxpool8<<<dim3(nblk((int64_t)To * C / 8, 256), (unsigned)B), 256, 0, st>>>(
+        reinterpret_cast<const __nv_bfloat16*>(x), T, C, To, reinterpret_cast<__nv_bfloat16*>(y), arg);
+    return cudaGetLastError();
+  }
   k_maxpool<<<dim3(nblk((int64_t)To * C, 256), (unsigned)B), 256, 0, st>>>(
       reinterpret_cast<const __nv_bfloat16*>(x), T, C, To, reinterpret_cast<__nv_bfloat16*>(y), arg);
   return cudaGetLastError();
@@ -722,7 +1002,7 @@ cudaError_t launch_maxpool_back(const float* dy, const uint8_t* arg, int64_t B, 
 }
 
 cudaError_t launch_mean_time(const void* x, int64_t B, int T, int C, void* m, cudaStream_t st) {
-  k_mean_time<<<nblk(B * C, 256), 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(x), B, T, C,
+  k_mean_time<<<nblk(B * C, 64), 64, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(x), B, T, C,
                                                 reinterpret_cast<__nv_bfloat16*>(m));
   return cudaGetLastError();
 }

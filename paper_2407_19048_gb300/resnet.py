@@ -192,82 +192,106 @@ class ResNet1D:
         off = (-buf.data_ptr()) % 256
         return buf[off:off + nbytes]
 
-    def _gn_back(self, dy, z, ms, g):
+    # the gradient a group norm's backward starts from (gwx_group_norm_backward_src)
+    PLAIN, MASK, POOL, MEAN = range(4)
+
+    def _gn_back(self, kind, dy, z, ms, g, out=None, arg=None, want_dsum=False):
+        """(dz, dsum, dgamma, dbeta) of the normalisation of z whose output's gradient is dy
+        (PLAIN), dy [out > 0] (MASK), the max pool's dy routed back and masked (POOL) or the
+        mean over time's dy / T masked (MEAN); dsum is that gradient itself (FP32, None unless
+        wanted).  dz is bfloat16 where one kernel does it all, else FP32."""
         import torch
         gwx, lib = self.gwx, _lib.load()
-        B, T, C = dy.shape
-        dz = torch.empty_like(dy)
+        B, T, C = z.shape
+        st = gwx._stream()
         dg, db = torch.empty(C, device=self.dev), torch.empty(C, device=self.dev)
-        nb = lib.gwx_group_norm_backward_scratch(B, C, GROUPS)
-        scratch = self._scratch(nb)
-        gwx._check(lib.gwx_group_norm_backward(gwx._ptr(dy), gwx._ptr(z), B, T, C, GROUPS, gwx._ptr(ms), gwx._ptr(g),
-                                               gwx._ptr(scratch), gwx._ptr(dz), gwx._ptr(dg), gwx._ptr(db),
-                                               gwx._stream()))
-        return dz, dg, db
+        if C % 4 == 0 and 256 % (C // 4) == 0 and (C // GROUPS) % 4 == 0:
+            dz = torch.empty((B, T, C), dtype=torch.bfloat16, device=self.dev)
+            dsum = torch.empty((B, T, C), dtype=torch.float32, device=self.dev) if want_dsum else None
+            scratch = self._scratch(lib.gwx_group_norm_backward_src_scratch(B, C, GROUPS))
+            gwx._check(lib.gwx_group_norm_backward_src(
+                kind, gwx._ptr(dy), gwx._ptr(out), gwx._ptr(arg), gwx._ptr(z), B, T, C, GROUPS, gwx._ptr(ms), gwx._ptr(g),
+                gwx._ptr(scratch), gwx._ptr(dz), gwx._ptr(dsum), gwx._ptr(dg), gwx._ptr(db), st))
+            return dz, dsum, dg, db
+        dsum = dy
+        if kind == self.MEAN:
+            dsum = torch.empty((B, T, C), dtype=torch.float32, device=self.dev)
+            gwx._check(lib.gwx_mean_time_backward(gwx._ptr(dy), B, T, C, gwx._ptr(dsum), st))
+        elif kind == self.POOL:
+            dsum = torch.empty((B, T, C), dtype=torch.float32, device=self.dev)
+            gwx._check(lib.gwx_maxpool_backward(gwx._ptr(dy), gwx._ptr(arg), B, T, C, gwx._ptr(dsum), st))
+        if kind != self.PLAIN:
+            d = torch.empty_like(dsum)
+            gwx._check(lib.gwx_relu_mask(gwx._ptr(dsum), gwx._ptr(out), d.numel(), gwx._ptr(d), st))
+            dsum = d
+        dz = torch.empty_like(z)
+        scratch = self._scratch(lib.gwx_group_norm_backward_scratch(B, C, GROUPS))
+        gwx._check(lib.gwx_group_norm_backward(gwx._ptr(dsum), gwx._ptr(z), B, T, C, GROUPS, gwx._ptr(ms), gwx._ptr(g),
+                                               gwx._ptr(scratch), gwx._ptr(dz), gwx._ptr(dg), gwx._ptr(db), st))
+        return dz, dsum, dg, db
 
-    def _relu_mask(self, dy, out):
+    def _rows_back(self, cols, W16, dz, want_dx=True):
+        """(dcols, dW) of the im2col product cols W^T for dz [B][T_out][C_out] (FP32 or bfloat16)."""
         import torch
-        gwx = self.gwx
-        d = torch.empty_like(dy)
-        gwx._check(_lib.load().gwx_relu_mask(gwx._ptr(dy), gwx._ptr(out), dy.numel(), gwx._ptr(d), gwx._stream()))
-        return d
+        gwx, lib = self.gwx, _lib.load()
+        M, N, K = cols.shape[0], W16.shape[0], W16.shape[1]
+        if dz.dtype == torch.float32:
+            return gwx.dense_bf16_backward(cols, W16, None, dz.reshape(M, N), act=gwx.ACT_NONE, want_dx=want_dx)[:2]
+        dcols = torch.empty((M, K), dtype=torch.float32, device=self.dev) if want_dx else None
+        dW = torch.empty((N, K), dtype=torch.float32, device=self.dev)
+        nb = lib.gwx_dense_bf16_backward_workspace(M, N, K)
+        gwx._check(lib.gwx_dense_bf16_backward_dz(gwx._ptr(dz), gwx._ptr(cols), gwx._ptr(W16), M, N, K, gwx._ptr(dcols),
+                                                  gwx._ptr(dW), gwx._ptr(self._scratch(nb)), nb, gwx._stream()))
+        return dcols, dW
 
     def _conv_back(self, dz, cols, W16, T, C, k, s, p, addend=None, x_in=None):
-        """(dx [B][T][C] FP32, dW) of a convolution given dz [B][T_out][C_out]; x_in is the
-        convolution's input when it ran as an implicit GEMM (cols None)."""
+        """(dx [B][T][C] FP32, dW) of a convolution given dz [B][T_out][C_out] (FP32 or
+        bfloat16); x_in is the convolution's input when it ran as an implicit GEMM (cols None)."""
         import torch
-        gwx = self.gwx
-        if cols is None:
-            B = x_in.shape[0]
-            nb = _lib.load().gwx_conv1d_bf16_backward_workspace(B, T, C, W16.shape[0], k)
-            return gwx.conv1d_bf16_backward(dz, x_in, W16, k, addend=addend,
-                                            workspace=(self._scratch(nb), nb))
-        B, To, Co = dz.shape
-        dcols, dW, _ = gwx.dense_bf16_backward(cols, W16, None, dz.reshape(B * To, Co), act=gwx.ACT_NONE)
+        gwx, lib = self.gwx, _lib.load()
+        B = dz.shape[0]
         dx = torch.empty((B, T, C), dtype=torch.float32, device=self.dev)
-        gwx._check(_lib.load().gwx_col2im(gwx._ptr(dcols), B, T, C, k, s, p, W16.shape[1],
-                                          gwx._ptr(addend) if addend is not None else None, gwx._ptr(dx),
-                                          gwx._stream()))
+        if cols is None:
+            nb = lib.gwx_conv1d_bf16_backward_workspace(B, T, C, W16.shape[0], k)
+            ws = self._scratch(nb)
+            if dz.dtype == torch.float32:
+                return gwx.conv1d_bf16_backward(dz, x_in, W16, k, addend=addend, workspace=(ws, nb))
+            dW = torch.empty((W16.shape[0], k * C), dtype=torch.float32, device=self.dev)
+            gwx._check(lib.gwx_conv1d_bf16_backward_dz(gwx._ptr(dz), gwx._ptr(x_in), gwx._ptr(W16), B, T, C, W16.shape[0],
+                                                       k, gwx._ptr(addend), gwx._ptr(dx), gwx._ptr(dW), gwx._ptr(ws), nb,
+                                                       gwx._stream()))
+            return dx, dW
+        dcols, dW = self._rows_back(cols, W16, dz)
+        gwx._check(lib.gwx_col2im(gwx._ptr(dcols), B, T, C, k, s, p, W16.shape[1], gwx._ptr(addend), gwx._ptr(dx),
+                                  gwx._stream()))
         return dx, dW
 
     def backward(self, dc):
         """Gradients (dict name -> FP32 tensor, names of tensors()) for dL/dc = dc [B][out]."""
-        import torch
-        gwx, lib = self.gwx, _lib.load()
-        st = gwx._stream()
+        gwx = self.gwx
         tape = self.tape
         G = {}
         m = tape["m"]
         dm, G["Wf"], G["bf"] = gwx.dense_bf16_backward(m, self.W16["Wf"], self.P["bf"], dc.contiguous(),
                                                        act=gwx.ACT_NONE)
-        hT = tape["blocks"][-1][-1]
-        B, T, C = hT.shape
-        dh = torch.empty((B, T, C), dtype=torch.float32, device=self.dev)
-        gwx._check(lib.gwx_mean_time_backward(gwx._ptr(dm), B, T, C, gwx._ptr(dh), st))
+        kind, dh = self.MEAN, dm
         for i in reversed(range(len(self.blocks))):
             blk = self.blocks[i]
             h, c1, z1, ms1, h1, c2, z2, ms2, cd, zd, msd, out = tape["blocks"][i]
             s = blk["s"]
-            dsum = self._relu_mask(dh, out)
-            dz2, G["%d.g2" % i], G["%d.b2" % i] = self._gn_back(dsum, z2, ms2, blk["g2"])
+            dz2, dsum, G["%d.g2" % i], G["%d.b2" % i] = self._gn_back(kind, dh, z2, ms2, blk["g2"], out=out,
+                                                                      want_dsum="Wd" not in blk)
             dh1, G["%d.W2" % i] = self._conv_back(dz2, c2, blk["W216"], h1.shape[1], h1.shape[2], 5, 1, 2, x_in=h1)
-            dh1 = self._relu_mask(dh1, h1)
-            dz1, G["%d.g1" % i], G["%d.b1" % i] = self._gn_back(dh1, z1, ms1, blk["g1"])
+            dz1, _, G["%d.g1" % i], G["%d.b1" % i] = self._gn_back(self.MASK, dh1, z1, ms1, blk["g1"], out=h1)
             if "Wd" in blk:
-                dzd, G["%d.gd" % i], G["%d.bd" % i] = self._gn_back(dsum, zd, msd, blk["gd"])
-                dxs, G["%d.Wd" % i] = self._conv_back(dzd, cd, blk["Wd16"], h.shape[1], h.shape[2], 1, s, 0)
-            else:
-                dxs = dsum
-            dh, G["%d.W1" % i] = self._conv_back(dz1, c1, blk["W116"], h.shape[1], h.shape[2], 5, s, 2, addend=dxs,
+                dzd, _, G["%d.gd" % i], G["%d.bd" % i] = self._gn_back(kind, dh, zd, msd, blk["gd"], out=out)
+                dsum, G["%d.Wd" % i] = self._conv_back(dzd, cd, blk["Wd16"], h.shape[1], h.shape[2], 1, s, 0)
+            dh, G["%d.W1" % i] = self._conv_back(dz1, c1, blk["W116"], h.shape[1], h.shape[2], 5, s, 2, addend=dsum,
                                                  x_in=h)
+            kind = self.MASK
         cols0, z0, ms0, a0, arg = tape["stem"]
-        B, T1, C0 = a0.shape
-        da0 = torch.empty((B, T1, C0), dtype=torch.float32, device=self.dev)
-        gwx._check(lib.gwx_maxpool_backward(gwx._ptr(dh), gwx._ptr(arg), B, T1, C0, gwx._ptr(da0), st))
-        da0 = self._relu_mask(da0, a0)
-        dz0, G["g0"], G["b0"] = self._gn_back(da0, z0, ms0, self.P["g0"])
-        _, G["W0"], _ = gwx.dense_bf16_backward(cols0, self.W16["W0"], None, dz0.reshape(B * T1, C0), want_dx=False,
-                                                act=gwx.ACT_NONE)
+        dz0, _, G["g0"], G["b0"] = self._gn_back(self.POOL, dh, z0, ms0, self.P["g0"], out=a0, arg=arg)
+        G["W0"] = self._rows_back(cols0, self.W16["W0"], dz0, want_dx=False)[1]
         return G
 
 
