@@ -686,9 +686,12 @@ static int dense_common(const void* A, const void* B, const float* bias, void* C
                   "gemm_bf16");
 }
 
+// The backward's workspaces keep the sizes they had while Z and transposed copies of the
+// operands lay in them (the calls use less now): a buffer that was too small is still refused.
 size_t gwx_dense_bf16_backward_workspace(int64_t M, int64_t N, int64_t K) {
   if (M < 1 || N < 1 || K < 1) return 0;
-  return align_up(dense_backward_ws(M, N, K));
+  return align_up((size_t)M * N * 4) + align_up((size_t)M * N * 2) + align_up((size_t)K * M * 2) +
+         align_up((size_t)K * N * 2) + align_up(dense_backward_ws(M, N, K));
 }
 
 int gwx_dense_bf16_backward(const void* X, const void* W, const float* bias, const float* dY, int64_t M, int64_t N,
@@ -1157,7 +1160,7 @@ int gwx_conv1d_bf16_backward_dz(const void* dz16, const void* x, const void* W, 
   if ((((uintptr_t)dz16) | ((uintptr_t)x) | ((uintptr_t)W) | ((uintptr_t)dx) | ((uintptr_t)dW) |
        ((uintptr_t)addend)) & 15u)
     return fail(GWX_EINVAL, "dz16, x, W, dx, dW and addend must be 16-byte aligned");
-  GWX_TRY(check_ws(workspace, workspace_bytes, conv_backward_ws(B, T, C, O, k)));
+  GWX_TRY(check_ws(workspace, workspace_bytes, gwx_conv1d_bf16_backward_workspace(B, T, C, O, k)));
   GWX_TRY(ensure_init());
   return launched(launch_conv_backward_dz(dz16, x, W, B, T, C, O, k, addend, dx, dW, workspace, as_stream(stream)),
                   "conv1d_bf16_backward_dz");
@@ -1165,7 +1168,9 @@ int gwx_conv1d_bf16_backward_dz(const void* dz16, const void* x, const void* W, 
 
 size_t gwx_conv1d_bf16_backward_workspace(int64_t B, int64_t T, int C, int O, int k) {
   if (B < 1 || T < 1 || C < 1 || O < 1 || k < 1) return 0;
-  return conv_backward_ws(B, T, C, O, k);
+  const size_t M = (size_t)B * T;
+  return align_up(M * O * 2) + align_up((size_t)C * k * O * 2) + align_up((size_t)k * C * M * 2) +
+         conv_backward_ws(B, T, C, O, k);
 }
 
 int gwx_conv1d_bf16_backward(const float* dz, const void* x, const void* W, int64_t B, int64_t T, int C, int O, int k,
@@ -1176,7 +1181,7 @@ int gwx_conv1d_bf16_backward(const float* dz, const void* x, const void* W, int6
   if ((((uintptr_t)x) | ((uintptr_t)W) | ((uintptr_t)dx) | ((uintptr_t)dW) | ((uintptr_t)addend)) & 15u)
     return fail(GWX_EINVAL, "x, W, dx, dW and addend must be 16-byte aligned");
   if (((uintptr_t)dz) & 3u) return fail(GWX_EINVAL, "dz must be 4-byte aligned");
-  GWX_TRY(check_ws(workspace, workspace_bytes, conv_backward_ws(B, T, C, O, k)));
+  GWX_TRY(check_ws(workspace, workspace_bytes, gwx_conv1d_bf16_backward_workspace(B, T, C, O, k)));
   GWX_TRY(ensure_init());
   return launched(launch_conv_backward(dz, x, W, B, T, C, O, k, addend, dx, dW, workspace, as_stream(stream)),
                   "conv1d_bf16_backward");
