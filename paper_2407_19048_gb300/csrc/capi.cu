@@ -409,9 +409,11 @@ size_t gwx_simulate_batch_workspace(int D, int64_t B, int64_t N) {
   return whiten_ws_bytes(D, N) + coef_bytes(B);
 }
 
-int gwx_prepare_batch(const gwx_prior* prior, uint64_t seed, uint32_t step, int64_t L, int64_t N, double fs,
-                      double f_lo, const int32_t* det_ids, int D, double gmst, int64_t B, double* theta,
-                      int64_t* offsets, void* workspace, size_t workspace_bytes, void* stream) {
+// gwx_prepare_batch, with the whitening filter of psd in the same launch when it is given.
+static int prepare_common(const gwx_prior* prior, uint64_t seed, uint32_t step, int64_t L, int64_t N, double fs,
+                          double f_lo, const int32_t* det_ids, int D, double gmst, int64_t B, double* theta,
+                          int64_t* offsets, const double* psd, int64_t seg_len, void* workspace,
+                          size_t workspace_bytes, void* stream) {
   if (!prior) return fail(GWX_EINVAL, "prior is NULL");
   DetParams dp;
   GWX_TRY(make_detparams(det_ids, D, dp));
@@ -422,12 +424,19 @@ int gwx_prepare_batch(const gwx_prior* prior, uint64_t seed, uint32_t step, int6
   if (!theta || !offsets) return fail(GWX_EINVAL, "NULL array");
   GWX_ALIGN8(theta);
   GWX_ALIGN8(offsets);
+  if (psd) GWX_ALIGN8(psd);
   GWX_TRY(check_ws(workspace, workspace_bytes, gwx_simulate_batch_workspace(D, B, N)));
   GWX_TRY(ensure_init());
-  cudaStream_t s = as_stream(stream);
-  GWX_TRY(launched(launch_sample_prior(*prior, seed, step, B, L, N, theta, offsets, s), "sample_prior"));
-  return launched(launch_draw_setup(theta, B, k_lo, fs / (double)N, fs, N / 2 + 1, dp, gmst, sim_coef(workspace, D, N), s),
-                  "draw set-up");
+  return launched(launch_prepare(*prior, seed, step, B, L, N, fs, dp, gmst, theta, offsets, sim_coef(workspace, D, N),
+                                 psd, seg_len, k_lo, reinterpret_cast<float*>(workspace), as_stream(stream)),
+                  "prepare");
+}
+
+int gwx_prepare_batch(const gwx_prior* prior, uint64_t seed, uint32_t step, int64_t L, int64_t N, double fs,
+                      double f_lo, const int32_t* det_ids, int D, double gmst, int64_t B, double* theta,
+                      int64_t* offsets, void* workspace, size_t workspace_bytes, void* stream) {
+  return prepare_common(prior, seed, step, L, N, fs, f_lo, det_ids, D, gmst, B, theta, offsets, nullptr, 0, workspace,
+                        workspace_bytes, stream);
 }
 
 int gwx_prepare_theta(const double* theta, int64_t L, int64_t N, double fs, double f_lo, const int32_t* det_ids,
@@ -539,10 +548,11 @@ int gwx_simulate_batch(const gwx_prior* prior, uint64_t seed, uint32_t step, con
                        size_t workspace_bytes, void* stream) {
   GWX_TRY(check_psd_args(seg_len, N));
   if (B > 0 && (!noise || !psd || !y)) return fail(GWX_EINVAL, "NULL array");
-  GWX_TRY(gwx_prepare_batch(prior, seed, step, L, N, fs, f_lo, det_ids, D, gmst, B, theta, offsets, workspace,
-                            workspace_bytes, stream));
-  return gwx_simulate_prepared(noise, L, psd, seg_len, fs, f_lo, D, B, N, offsets, y, 0, workspace, workspace_bytes,
-                               stream);
+  if (B > 0) GWX_ALIGN8(y);
+  GWX_TRY(prepare_common(prior, seed, step, L, N, fs, f_lo, det_ids, D, gmst, B, theta, offsets, psd, seg_len, workspace,
+                         workspace_bytes, stream));
+  return gwx_simulate_prepared(noise, L, psd, seg_len, fs, f_lo, D, B, N, offsets, y, GWX_SIM_FILTERS_READY, workspace,
+                               workspace_bytes, stream);
 }
 
 size_t gwx_log_likelihood_workspace(int64_t E, int D, int64_t N, int64_t S) {

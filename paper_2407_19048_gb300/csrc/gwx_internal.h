@@ -45,6 +45,10 @@ cudaError_t launch_project(const float2* hp, const float2* hc, const double* the
                            cudaStream_t s);
 cudaError_t launch_draw_setup(const double* theta, int64_t B, int k_lo, double df, double fs, int64_t F,
                               const DetParams& dp, double gmst, DrawCoef* coef, cudaStream_t s);
+// Prior draws, set-up and (psd non-NULL) the whitening filter of a batch in one launch.
+cudaError_t launch_prepare(const gwx_prior& p, uint64_t seed, uint32_t step, int64_t B, int64_t L, int64_t N, double fs,
+                           const DetParams& dp, double gmst, double* theta, int64_t* offsets, DrawCoef* coef,
+                           const double* psd, int64_t M, int k_lo, float* W, cudaStream_t s);
 cudaError_t launch_colored_noise(uint64_t seed, uint32_t step, int D, int64_t L, double fs, double f_lo,
                                  float* noise, void* ws, cudaStream_t s);
 size_t colored_noise_ws(int D, int64_t L);

@@ -220,11 +220,13 @@ __device__ __forceinline__ CropCopy crop_copy(const int64_t* offsets, int64_t b,
 // crop and the next detector's filter arrive in shared staging buffers by bulk asynchronous
 // copies issued one window ahead, so no pass waits on a global load; same arithmetic again.
 // Wcap: floats of the filter allocation W (the staged copies may read up to it).
+// nd: detectors of a draw that a block takes in turn: D, or 1 when windows rather than draws
+// are dealt out (sim_split).
 template <int LOGN, bool VEC, bool PP, bool ST>
 __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
     k_simulate(const DrawCoef* __restrict__ coef, const float* __restrict__ noise, int64_t L,
                const int64_t* __restrict__ offsets, const float* __restrict__ W, int64_t Wcap, int k_lo, int D,
-               int64_t B, float* __restrict__ y) {
+               int64_t B, int nd, float* __restrict__ y) {
   static_assert(!(ST && PP), "staging uses the in-place passes");
   using PL = SimPlan<LOGN>;
   constexpr bool R16 = PL::R16;
@@ -244,6 +246,8 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
   const uint32_t x = smem_addr(sm), x2 = x + 8u * (uint32_t)n;
   const float inv_n = 1.0f / (float)n;
   const int64_t DL = (int64_t)D * L;
+  const int per = D / nd;                       // units of a draw: 1, or D single windows
+  const int64_t units = B * per;
   const uint32_t bar_c = smem_addr(&bars[0]), bar_w = smem_addr(&bars[1]);
   uint32_t ph_c = 0, ph_w = 0;   // parity of the staging barriers' next phase
 
@@ -256,13 +260,15 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
       tc::mbar_init(bar_c, 1);
       tc::mbar_init(bar_w, 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      if (blockIdx.x < B) {
-        const CropCopy cc = crop_copy(offsets, blockIdx.x, 0, L, N, DL);
+      if (blockIdx.x < units) {
+        const int64_t b = blockIdx.x / per;
+        const int d = (int)(blockIdx.x - b * per);
+        const CropCopy cc = crop_copy(offsets, b, d, L, N, DL);
         s_o[0] = cc.o;
         tc::mbar_expect_tx(bar_c, cc.bytes);
         bulk_g2s(smem_addr(crop_s), noise + cc.src, cc.bytes, bar_c);
-        const int64_t wsrc = 0;
-        s_o[1] = 0;
+        const int64_t wsrc = ((int64_t)d * F) & ~(int64_t)3;
+        s_o[1] = (int)((int64_t)d * F - wsrc);
         const uint32_t wb = (uint32_t)(4 * ((int64_t)n + 4 < Wcap - wsrc ? (int64_t)n + 4 : Wcap - wsrc));
         tc::mbar_expect_tx(bar_w, wb);
         bulk_g2s(smem_addr(w_s), W + wsrc, wb, bar_w);
@@ -271,7 +277,9 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
     __syncthreads();
   }
 
-  for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
+  for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+    const int64_t b = u / per;
+    const int d_first = (int)(u - b * per);
     for (int i = t; i < (int)(sizeof(DrawCoef) / 16); i += T)
       reinterpret_cast<int4*>(&sc)[i] = __ldg(reinterpret_cast<const int4*>(coef + b) + i);
     int64_t off = 0;
@@ -301,11 +309,12 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
       }
     }
 
-    for (int d = 0; d < D; ++d) {
-      // the window after this one: (b, d + 1), else the block's next draw
-      const bool more = d + 1 < D || b + gridDim.x < B;
-      const int64_t b_next = d + 1 < D ? b : b + gridDim.x;
-      const int d_next = d + 1 < D ? d + 1 : 0;
+    for (int d = d_first; d < d_first + nd; ++d) {
+      // the window after this one: (b, d + 1), else the block's next unit
+      const bool same = d + 1 < d_first + nd;
+      const bool more = same || u + gridDim.x < units;
+      const int64_t b_next = same ? b : (u + gridDim.x) / per;
+      const int d_next = same ? d + 1 : (int)(u + gridDim.x - b_next * per);
 
       // first forward pass (Ns = 1), input straight from the background crop
       bool ok = true;
@@ -601,6 +610,16 @@ bool sim_can_stage(const float* noise, int64_t L, const float* W, int64_t N) {
   return (uintptr_t)noise % 16 == 0 && L % 4 == 0 && (uintptr_t)W % 16 == 0 && smem <= (size_t)227 * 1024;
 }
 
+// Whether to deal out single windows instead of draws with their D windows: a block then
+// evaluates the waveform for one window instead of D (about a quarter of a window's time), but
+// a batch of fewer draws than block slots, or whose last wave of draws is short, spreads over
+// more SMs.  64 draws of two 2048-sample windows (64 blocks of 1216 slots): see k_prepare's
+// figures; 2048 draws of three windows stay with draws (6.7 waves against 20.2 / 3).
+static bool sim_split(int64_t B, int D, int64_t slots) {
+  const int64_t by_draw = (B + slots - 1) / slots * D, by_window = (B * D + slots - 1) / slots;
+  return 5 * by_window < 4 * by_draw;
+}
+
 template <int LG, bool VEC, bool PP, bool ST>
 static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, int64_t L, const int64_t* offsets,
                                       const float* W, int64_t Wcap, int k_lo, int D, int64_t B, float* y,
@@ -621,9 +640,10 @@ static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, 
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   if (per_sm_want > 0 && per_sm_want < per_sm) per_sm = per_sm_want;
-  int64_t grid = (int64_t)sms * per_sm;
-  if (grid > B) grid = B;
-  kern<<<(unsigned)grid, NT, smem, s>>>(coef, noise, L, offsets, W, Wcap, k_lo, D, B, y);
+  const int64_t slots = (int64_t)sms * per_sm;
+  const int nd = sim_split(B, D, slots) ? 1 : D;
+  const int64_t units = B * (D / nd), grid = units < slots ? units : slots;
+  kern<<<(unsigned)grid, NT, smem, s>>>(coef, noise, L, offsets, W, Wcap, k_lo, D, B, nd, y);
   return cudaGetLastError();
 }
 

@@ -1,51 +1,30 @@
 // k_random.cu -- prior draws (A1) and the coloured Gaussian background (A4).
-#include "common.cuh"
+#include "prior.cuh"
 
 namespace gwx {
 
 cudaError_t init_tables_random() { return fill_tables_for_this_tu(); }
 
 // ----------------------------------------------------------------- A1
-// One thread per draw.  Linear maps use the non-contracting intrinsics so the
-// doubles equal a plain lo + (hi - lo) u evaluated with two roundings.
-__device__ __forceinline__ double lin_map(double lo, double hi, double u) {
-  return __dadd_rn(lo, __dmul_rn(__dsub_rn(hi, lo), u));
-}
-
-__global__ void k_sample_prior(gwx_prior p, uint32_t k0, uint32_t k1, uint32_t step, int64_t B, uint32_t span,
-                               double* __restrict__ theta, int64_t* __restrict__ offsets) {
+// One thread per draw.
+__global__ void k_sample_prior(PriorStream ps, int64_t B, uint32_t span, double* __restrict__ theta,
+                               int64_t* __restrict__ offsets) {
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
-  double u[11];
-  uint32_t woff = 0;
-#pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    const u32x4 r = philox4x32_10((uint32_t)b, (uint32_t)j, TAG_PRIOR, step, k0, k1);
-    u[2 * j] = uniform52(r.x, r.y);
-    if (j < 5) u[2 * j + 1] = uniform52(r.z, r.w);
-    else woff = r.z;
-  }
-  const double two_pi = 6.283185307179586476925286766559;
-  theta[GWX_M1 * B + b] = lin_map(p.m_lo, p.m_hi, u[0]);
-  theta[GWX_M2 * B + b] = lin_map(p.m_lo, p.m_hi, u[1]);
-  theta[GWX_CHI1 * B + b] = lin_map(p.chi_lo, p.chi_hi, u[2]);
-  theta[GWX_CHI2 * B + b] = lin_map(p.chi_lo, p.chi_hi, u[3]);
-  theta[GWX_DIST * B + b] = lin_map(p.d_lo, p.d_hi, u[4]);
-  theta[GWX_TC * B + b] = lin_map(p.tc_lo, p.tc_hi, u[5]);
-  theta[GWX_PHIC * B + b] = lin_map(p.phi_lo, p.phi_hi, u[6]);
-  theta[GWX_THETAJN * B + b] = acos(__dsub_rn(1.0, __dmul_rn(2.0, u[7])));
-  theta[GWX_PSI * B + b] = lin_map(p.psi_lo, p.psi_hi, u[8]);
-  theta[GWX_RA * B + b] = __dmul_rn(two_pi, u[9]);
-  theta[GWX_DEC * B + b] = asin(__dsub_rn(__dmul_rn(2.0, u[10]), 1.0));
-  offsets[b] = (int64_t)(((uint64_t)woff * (uint64_t)span) >> 32);
+  ps.masses(b, theta[GWX_M1 * B + b], theta[GWX_M2 * B + b]);
+  ps.spins(b, theta[GWX_CHI1 * B + b], theta[GWX_CHI2 * B + b]);
+  ps.dist_tc(b, theta[GWX_DIST * B + b], theta[GWX_TC * B + b]);
+  ps.phic_iota(b, theta[GWX_PHIC * B + b], theta[GWX_THETAJN * B + b]);
+  ps.psi_ra(b, theta[GWX_PSI * B + b], theta[GWX_RA * B + b]);
+  ps.dec_offset(b, span, theta[GWX_DEC * B + b], offsets[b]);
 }
 
 cudaError_t launch_sample_prior(const gwx_prior& p, uint64_t seed, uint32_t step, int64_t B, int64_t L, int64_t N,
                                 double* theta, int64_t* offsets, cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
   const int T = 32;   // FP64 acos/asin: spread the draws over many SMs
-  k_sample_prior<<<(unsigned)((B + T - 1) / T), T, 0, s>>>(p, (uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32),
-                                                           step, B, (uint32_t)(L - N + 1), theta, offsets);
+  const PriorStream ps{p, (uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32), step};
+  k_sample_prior<<<(unsigned)((B + T - 1) / T), T, 0, s>>>(ps, B, (uint32_t)(L - N + 1), theta, offsets);
   return cudaGetLastError();
 }
 

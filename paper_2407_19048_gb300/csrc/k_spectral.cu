@@ -3,7 +3,7 @@
 // Stockham FFT of n = N/2 complex points (the real window packed as
 // z_m = x_2m + i x_2m+1) run by n/8 threads per row; several rows share a block
 // when n/8 < 256.
-#include "common.cuh"
+#include "prior.cuh"
 
 namespace gwx {
 
@@ -125,29 +125,10 @@ cudaError_t launch_welch(const float* x, int D, int64_t L, double fs, int64_t M,
 }
 
 // ----------------------------------------------------------------- whitening filter
-// W[d][k] = M_k / sqrt(S~_k fs / 2), S~ the PSD linearly interpolated from the grid
-// fs/M to fs/N at the exact rational position k M / N.
-// W_k = M_k / sqrt(S~_k fs/2) (whitening), or M_k sqrt(S~_k fs/2) with `inverse` (the
-// unwhitening filter: its inverse on the band).
 __global__ void k_whiten_filter(const double* __restrict__ psd, int D, int64_t M, double fs, int k_lo, int64_t N,
                                 bool inverse, float* __restrict__ W) {
-  const int64_t F = N / 2 + 1;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)D * F) return;
-  const int d = (int)(i / F);
-  const int64_t k = i % F;
-  float w = 0.f;
-  if (k >= k_lo && k < N / 2) {
-    const int64_t nb = M / 2 + 1;
-    const int64_t num = k * M;
-    const int64_t j0 = num / N;
-    const int64_t j1 = j0 + 1 < nb ? j0 + 1 : nb - 1;
-    const double frac = (double)(num % N) / (double)N;
-    const double* p = psd + (int64_t)d * nb;
-    const double S = p[j0] + (p[j1] - p[j0]) * frac;
-    w = inverse ? (float)sqrt(S * fs * 0.5) : (float)(1.0 / sqrt(S * fs * 0.5));
-  }
-  W[i] = w;
+  if (i < (int64_t)D * (N / 2 + 1)) W[i] = whiten_filter_at(psd, i, M, fs, k_lo, N, inverse);
 }
 
 cudaError_t launch_whiten_filter(const double* psd, int D, int64_t M, double fs, int k_lo, int64_t N, float* W,

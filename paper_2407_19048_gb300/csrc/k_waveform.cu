@@ -1,6 +1,7 @@
 // k_waveform.cu -- per-draw set-up, TaylorF2 waveforms (A2), projection (A3) and
 // the whitened log-likelihood (A8).
 #include "fft16r.cuh"
+#include "prior.cuh"
 #include "waveform.cuh"
 
 namespace gwx {
@@ -32,6 +33,113 @@ cudaError_t launch_draw_setup(const double* theta, int64_t B, int /*k_lo*/, doub
   if (B <= 0) return cudaSuccess;
   const int T = 32;
   k_draw_setup<<<(unsigned)((B + T - 1) / T), T, 0, s>>>(theta, B, make_setup_consts(df), fs, F, dp, gmst, coef);
+  return cudaGetLastError();
+}
+
+// The whole preparation of a batch in one launch: prior draws, set-up and, in the blocks after
+// the draws', the whitening filter.  Bound by FP64 latency (a dependent operation takes ~54
+// cycles; 650 operations a draw were 17.4 us for one thread, and 64 or 8192 draws took the
+// same), so the four warps of a block share 32 draws: warp 0 the waveform's coefficients (one
+// logarithm, one exponential, a root and four divisions in a chain), warp 1 the angles and
+// theta, warps 2 and 3 two detectors each; the strain factors are combined after a barrier.
+// As three launches (prior 7.4 us, set-up 17.4, filter 4.5) 64 draws took 45 us with the pass.
+struct FilterArgs {
+  const double* psd;   // NULL: no filter
+  int64_t entries, M, N;
+  double fs;
+  int k_lo;
+  float* W;
+};
+
+__global__ void __launch_bounds__(128) k_prepare(PriorStream ps, int64_t B, uint32_t span, SetupConsts kc, double fs,
+                                                 int64_t F, DetParams dp, double gmst, unsigned draw_blocks,
+                                                 FilterArgs fa, double* __restrict__ theta,
+                                                 int64_t* __restrict__ offsets, DrawCoef* __restrict__ coef) {
+  if (blockIdx.x >= draw_blocks) {
+    const int64_t i = (int64_t)(blockIdx.x - draw_blocks) * 128 + threadIdx.x;
+    if (i < fa.entries) fa.W[i] = whiten_filter_at(fa.psd, i, fa.M, fa.fs, fa.k_lo, fa.N, false);
+    return;
+  }
+  __shared__ double s_amp[32], s_ci[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t b0 = (int64_t)blockIdx.x * 32 + lane, b = b0 < B ? b0 : B - 1;   // the last draw again past the end
+  DrawCoef c;
+  double fp[2] = {0.0, 0.0}, fc[2] = {0.0, 0.0};
+  unsigned long long nu[2] = {0ull, 0ull};
+  if (warp == 0) {
+    WaveIn in;
+    double tc, amp = 0.0;
+    ps.masses(b, in.m1, in.m2);
+    ps.spins(b, in.chi1, in.chi2);
+    ps.dist_tc(b, in.dist, tc);
+    const u32x4 r = ps.words(b, 3);
+    in.phic = lin_map(ps.p.phi_lo, ps.p.phi_hi, uniform52(r.x, r.y));
+    waveform_coef(in, kc, F, c, &amp);
+    s_amp[lane] = amp;
+  } else if (warp == 1) {
+    double v[11];
+    int64_t off;
+    ps.phic_iota(b, v[GWX_PHIC], v[GWX_THETAJN]);
+    s_ci[lane] = cos(v[GWX_THETAJN]);
+    ps.masses(b, v[GWX_M1], v[GWX_M2]);
+    ps.spins(b, v[GWX_CHI1], v[GWX_CHI2]);
+    ps.dist_tc(b, v[GWX_DIST], v[GWX_TC]);
+    ps.psi_ra(b, v[GWX_PSI], v[GWX_RA]);
+    ps.dec_offset(b, span, v[GWX_DEC], off);
+    if (b0 < B) {
+#pragma unroll
+      for (int i = 0; i < 11; ++i) theta[i * B + b] = v[i];
+      offsets[b] = off;
+    }
+  } else {
+    double psi, ra, dec, dist, tc;
+    int64_t off;
+    ps.psi_ra(b, psi, ra);
+    ps.dec_offset(b, span, dec, off);
+    ps.dist_tc(b, dist, tc);
+    const SkyFrame s = sky_frame(psi, ra, dec, gmst);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      // slots warp - 2 and warp, as constants so that DetParams stays in the parameter bank
+      if (warp == 2) {
+        if (2 * i < dp.D) antenna(dp, 2 * i, s, kc.df, tc, fp[i], fc[i], nu[i]);
+      } else {
+        if (2 * i + 1 < dp.D) antenna(dp, 2 * i + 1, s, kc.df, tc, fp[i], fc[i], nu[i]);
+      }
+    }
+  }
+  __syncthreads();
+  if (b0 >= B) return;
+  if (warp == 0) {
+    set_inclination(s_ci[lane], c);
+    float4* o = reinterpret_cast<float4*>(coef + b);
+    o[0] = make_float4(c.c0.x, c.c0.y, c.c2.x, c.c2.y);
+    o[1] = make_float4(c.c3.x, c.c3.y, c.d5.x, c.d5.y);
+    o[2] = make_float4(c.c4, c.c6, c.d6, c.c7);
+    o[3] = make_float4(c.cph, c.amp, c.qp, c.qc_im);
+    reinterpret_cast<int4*>(o)[4] = make_int4(c.kcut, 0, 0, 0);
+  } else if (warp >= 2) {
+    set_inclination(s_ci[lane], c);
+    const double scale = fs * s_amp[lane];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int d = 2 * i + warp - 2;
+      coef[b].g[d] = d < dp.D ? strain_factor(scale, fp[i], fc[i], c.qp, c.qc_im) : make_float4(0.f, 0.f, 0.f, 0.f);
+      coef[b].nu[d] = nu[i];
+    }
+  }
+}
+
+cudaError_t launch_prepare(const gwx_prior& p, uint64_t seed, uint32_t step, int64_t B, int64_t L, int64_t N, double fs,
+                           const DetParams& dp, double gmst, double* theta, int64_t* offsets, DrawCoef* coef,
+                           const double* psd, int64_t M, int k_lo, float* W, cudaStream_t s) {
+  static_assert(GWX_MAX_DET == 4, "two detector slots per warp");
+  if (B <= 0) return cudaSuccess;
+  const PriorStream ps{p, (uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32), step};
+  const FilterArgs fa{psd, psd ? dp.D * (N / 2 + 1) : 0, M, N, fs, k_lo, W};
+  const unsigned nb = (unsigned)((B + 31) / 32), nf = (unsigned)((fa.entries + 127) / 128);
+  k_prepare<<<nb + nf, 128, 0, s>>>(ps, B, (uint32_t)(L - N + 1), make_setup_consts(fs / (double)N), fs, N / 2 + 1, dp,
+                                    gmst, nb, fa, theta, offsets, coef);
   return cudaGetLastError();
 }
 

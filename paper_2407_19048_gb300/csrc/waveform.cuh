@@ -50,16 +50,23 @@ static inline SetupConsts make_setup_consts(double df) {
           INV_6P15_PI / (MTSUN_S * df)};
 }
 
-// Waveform part of the set-up: PN phase coefficients in turns, amplitude and cut-off.
+// Waveform part of the set-up: PN phase coefficients in turns, amplitude and cut-off, for
+// ci = cos(theta_JN).
 // Written for the GPU's scarce FP64 throughput: constant ratios are folded at compile
 // time, one logarithm serves both ln V and M^(5/6), and the remaining divisions are
 // the few reciprocals that depend on the draw.
-__device__ inline void draw_waveform_coef(const double* th, int64_t B, int64_t b, const SetupConsts& k, int64_t F,
-                                          DrawCoef& c, double* amp64 = nullptr) {
-  const double m1 = th_at(th, B, b, GWX_M1), m2 = th_at(th, B, b, GWX_M2);
-  const double chi1 = th_at(th, B, b, GWX_CHI1), chi2 = th_at(th, B, b, GWX_CHI2);
-  const double phic = th_at(th, B, b, GWX_PHIC);
-  const double iota = th_at(th, B, b, GWX_THETAJN);
+struct WaveIn {
+  double m1, m2, chi1, chi2, phic, dist;
+};
+
+__device__ __forceinline__ void set_inclination(double ci, DrawCoef& c) {
+  c.qp = (float)(0.5 * (1.0 + ci * ci));
+  c.qc_im = (float)ci;
+}
+
+__device__ __forceinline__ void waveform_coef(const WaveIn& in, const SetupConsts& k, int64_t F, DrawCoef& c,
+                                              double* amp64) {
+  const double m1 = in.m1, m2 = in.m2, chi1 = in.chi1, chi2 = in.chi2, phic = in.phic;
   const double mt = m1 + m2;
   const double inv_mt = 1.0 / mt;
   const double M = mt * MTSUN_S;
@@ -97,37 +104,78 @@ __device__ inline void draw_waveform_coef(const double* th, int64_t B, int64_t b
   c.cph = (float)cph;
   // A(df) = sqrt(5/24) pi^{-2/3} Mc^{5/6} df^{-7/6} / D with Mc^{5/6} = M^{5/6} eta^{1/2}
   // = V^2 (V eta)^{1/2} (pi df)^{-5/6}; k.amp_k folds the constants and df^{-7/6}.
-  const double amp = k.amp_k * (V * V) * sqrt(V * eta) / th_at(th, B, b, GWX_DIST);
+  const double amp = k.amp_k * (V * V) * sqrt(V * eta) / in.dist;
   if (amp64) *amp64 = amp;
   c.amp = (float)amp;
   const double kc = floor(k.isco_bins * inv_mt);
   c.kcut = kc > (double)(F - 1) ? (int)(F - 1) : (int)kc;
-  const double ci = cos(iota);
-  c.qp = (float)(0.5 * (1.0 + ci * ci));
-  c.qc_im = (float)ci;
   c.pad0 = c.pad1 = c.pad2 = 0;
+}
+
+__device__ inline void draw_waveform_coef(const double* th, int64_t B, int64_t b, const SetupConsts& k, int64_t F,
+                                          DrawCoef& c, double* amp64 = nullptr) {
+  const WaveIn in{th_at(th, B, b, GWX_M1),   th_at(th, B, b, GWX_M2),   th_at(th, B, b, GWX_CHI1),
+                  th_at(th, B, b, GWX_CHI2), th_at(th, B, b, GWX_PHIC), th_at(th, B, b, GWX_DIST)};
+  const double iota = th_at(th, B, b, GWX_THETAJN);
+  waveform_coef(in, k, F, c, amp64);
+  set_inclination(cos(iota), c);
 }
 
 // Projection part: scale * (F+ qp - i Fx qc) per detector as a complex double-float,
 // and the per-detector linear phase (tc + dt_d) df modulo one as a 2^-64 fixed point,
 // for a given merger time tc (the sky position and polarisation from theta).
-__device__ inline void draw_detector_coef_at(const double* th, int64_t B, int64_t b, double df, const DetParams& dp,
-                                             double gmst, double qp, double qc, double scale, double tc, DrawCoef& c) {
-  const double psi = th_at(th, B, b, GWX_PSI);
-  const double ra = th_at(th, B, b, GWX_RA), dec = th_at(th, B, b, GWX_DEC);
+struct SkyFrame {   // unit vector to the source and the polarisation basis
+  double n[3], X[3], Y[3];
+};
+
+__device__ __forceinline__ SkyFrame sky_frame(double psi, double ra, double dec, double gmst) {
   double sd, cd, sp, cp, spsi, cpsi;
   sincos(dec, &sd, &cd);
   sincos(ra - gmst, &sp, &cp);
   sincos(psi, &spsi, &cpsi);
-  const double n[3] = {cd * cp, cd * sp, sd};
+  SkyFrame s;
+  s.n[0] = cd * cp;
+  s.n[1] = cd * sp;
+  s.n[2] = sd;
   const double eth[3] = {sd * cp, sd * sp, -cd};
   const double eph[3] = {-sp, cp, 0.0};
-  double X[3], Y[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    X[i] = cpsi * eth[i] + spsi * eph[i];
-    Y[i] = spsi * eth[i] - cpsi * eph[i];
+    s.X[i] = cpsi * eth[i] + spsi * eph[i];
+    s.Y[i] = spsi * eth[i] - cpsi * eph[i];
   }
+  return s;
+}
+
+// F+, Fx and (tc + dt) df modulo one as a 2^-64 fixed point, of detector slot d.
+__device__ __forceinline__ void antenna(const DetParams& dp, int d, const SkyFrame& s, double df, double tc, double& fp,
+                                        double& fc, unsigned long long& nu) {
+  const double* T = dp.tensor[d];
+  double DX[3], DY[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    DX[i] = T[3 * i] * s.X[0] + T[3 * i + 1] * s.X[1] + T[3 * i + 2] * s.X[2];
+    DY[i] = T[3 * i] * s.Y[0] + T[3 * i + 1] * s.Y[1] + T[3 * i + 2] * s.Y[2];
+  }
+  fp = s.X[0] * DX[0] + s.X[1] * DX[1] + s.X[2] * DX[2] - (s.Y[0] * DY[0] + s.Y[1] * DY[1] + s.Y[2] * DY[2]);
+  fc = s.X[0] * DY[0] + s.X[1] * DY[1] + s.X[2] * DY[2] + (s.Y[0] * DX[0] + s.Y[1] * DX[1] + s.Y[2] * DX[2]);
+  const double dt = -(dp.pos[d][0] * s.n[0] + dp.pos[d][1] * s.n[1] + dp.pos[d][2] * s.n[2]) * INV_C;
+  double x = (tc + dt) * df;
+  x -= floor(x);
+  const double fx = ldexp(x, 64);
+  nu = fx >= 18446744073709551615.0 ? 0ull : (unsigned long long)fx;
+}
+
+// scale (F+ qp + Fx (-i qc))
+__device__ __forceinline__ float4 strain_factor(double scale, double fp, double fc, double qp, double qc) {
+  const float2 re = split_df(scale * fp * qp), im = split_df(-scale * fc * qc);
+  return make_float4(re.x, re.y, im.x, im.y);
+}
+
+__device__ inline void draw_detector_coef_at(const double* th, int64_t B, int64_t b, double df, const DetParams& dp,
+                                             double gmst, double qp, double qc, double scale, double tc, DrawCoef& c) {
+  const SkyFrame s =
+      sky_frame(th_at(th, B, b, GWX_PSI), th_at(th, B, b, GWX_RA), th_at(th, B, b, GWX_DEC), gmst);
   // unrolled over the detector slots so that DetParams stays in the parameter bank
 #pragma unroll
   for (int d = 0; d < GWX_MAX_DET; ++d) {
@@ -136,23 +184,9 @@ __device__ inline void draw_detector_coef_at(const double* th, int64_t B, int64_
       c.nu[d] = 0ull;
       continue;
     }
-    const double* T = dp.tensor[d];
-    double DX[3], DY[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      DX[i] = T[3 * i] * X[0] + T[3 * i + 1] * X[1] + T[3 * i + 2] * X[2];
-      DY[i] = T[3 * i] * Y[0] + T[3 * i + 1] * Y[1] + T[3 * i + 2] * Y[2];
-    }
-    const double fp = X[0] * DX[0] + X[1] * DX[1] + X[2] * DX[2] - (Y[0] * DY[0] + Y[1] * DY[1] + Y[2] * DY[2]);
-    const double fc = X[0] * DY[0] + X[1] * DY[1] + X[2] * DY[2] + (Y[0] * DX[0] + Y[1] * DX[1] + Y[2] * DX[2]);
-    const double dt = -(dp.pos[d][0] * n[0] + dp.pos[d][1] * n[1] + dp.pos[d][2] * n[2]) * INV_C;
-    // scale (F+ qp + Fx (-i qc))
-    const float2 re = split_df(scale * fp * qp), im = split_df(-scale * fc * qc);
-    c.g[d] = make_float4(re.x, re.y, im.x, im.y);
-    double x = (tc + dt) * df;
-    x -= floor(x);
-    double fx = ldexp(x, 64);
-    c.nu[d] = fx >= 18446744073709551615.0 ? 0ull : (unsigned long long)fx;
+    double fp, fc;
+    antenna(dp, d, s, df, tc, fp, fc, c.nu[d]);
+    c.g[d] = strain_factor(scale, fp, fc, qp, qc);
   }
 }
 

@@ -29,9 +29,9 @@ from . import DETECTORS, NPARAM, _det_ids, _prior, _ptr, _stream, _workspace, _c
 
 
 class Simulator:
-    # kernels per call: prepare 2, colored noise 2, Welch 2, simulate_prepared 2 (1 when the
-    # whitening filter of its workspace is still current)
-    LAUNCHES = {"prepare": 2, "colored_noise": 2, "welch": 2, "simulate": 2, "simulate_reuse": 1}
+    # kernels per call: prepare 1, colored noise 2, Welch 2, simulate_prepared 2 (1 when the
+    # whitening filter of its workspace is still current, or came with the preparation)
+    LAUNCHES = {"prepare": 1, "colored_noise": 2, "welch": 2, "simulate": 2, "simulate_reuse": 1}
 
     def __init__(self, workload, device=None, noise_on_device=True, pipeline=False, background_every=1):
         import torch
@@ -139,7 +139,7 @@ class Simulator:
                                            self.ids, self.D, self.gmst, self.B, self.N, _ptr(self.y),
                                            _ptr(self.theta), _ptr(self.offsets), _ptr(ws), nb, _stream()))
         self._filter_version[self._slot] = self._psd_version
-        self.launches += self.LAUNCHES["prepare"] + self.LAUNCHES["simulate"]
+        self.launches += self.LAUNCHES["prepare"] + self.LAUNCHES["simulate_reuse"]
 
     def autotune(self, step=0):
         """Time the fused pass's launch shapes (bit-identical outputs) on a batch of this
