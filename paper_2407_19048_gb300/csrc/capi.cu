@@ -391,7 +391,7 @@ static int whiten_common(bool inverse, const float* d, const double* psd, int64_
   float* W = reinterpret_cast<float*>(workspace);
   cudaStream_t s = as_stream(stream);
   GWX_TRY(launched(launch_whiten_filter(psd, D, seg_len, fs, k_lo, N, W, s, inverse), "whiten filter"));
-  return launched(launch_whiten_rows(d, W, B * D, D, N, y, s), "whiten");
+  return launched(launch_whiten_windows(d, W, sim_filter_floats(D, N), B, D, N, y, s), "whiten");
 }
 
 int gwx_whiten(const float* d, const double* psd, int64_t seg_len, double fs, double f_lo, int64_t B, int D,

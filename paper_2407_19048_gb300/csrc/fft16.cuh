@@ -82,8 +82,9 @@ __device__ __forceinline__ void store_pass(uint32_t x, int j, const float2* v) {
   }
 }
 
-// One shared-memory-to-shared-memory pass; thread t owns butterflies t + i n/16.
-template <int LOGN, int R, int Ns, bool INV>
+// One shared-memory-to-shared-memory pass; thread t owns butterflies t + i n/16.  EXACT: the
+// radix-8 sqrt(1/2) products rounded once (see dft8).
+template <int LOGN, int R, int Ns, bool INV, bool EXACT = false>
 __device__ __forceinline__ void pass16(uint32_t x, int t) {
   constexpr int n = 1 << LOGN;
   constexpr int NBT = 16 / R;
@@ -99,7 +100,7 @@ __device__ __forceinline__ void pass16(uint32_t x, int t) {
 #pragma unroll
       for (int r = 1; r < R; ++r) v[i][r] = cmul(v[i][r], w[r]);
     }
-    dftR<R, INV, false>(v[i]);
+    dftR<R, INV, EXACT>(v[i]);
   }
   __syncthreads();
 #pragma unroll
@@ -159,23 +160,23 @@ struct InvMiddlePP {
 };
 
 // Middle passes of the forward transform: radix 8 with Ns = 8^p, p = 1 .. P-2.
-template <int LOGN, int p, int PMAX>
+template <int LOGN, int p, int PMAX, bool EXACT = false>
 struct FwdMiddle {
   static __device__ __forceinline__ void run(uint32_t x, int t) {
     if constexpr (p <= PMAX) {
-      pass16<LOGN, 8, (1 << (3 * p)), false>(x, t);
-      FwdMiddle<LOGN, p + 1, PMAX>::run(x, t);
+      pass16<LOGN, 8, (1 << (3 * p)), false, EXACT>(x, t);
+      FwdMiddle<LOGN, p + 1, PMAX, EXACT>::run(x, t);
     }
   }
 };
 
 // Middle passes of the inverse transform: radix 8 with Ns = RL 8^(p-1), p = 1 .. P-2.
-template <int LOGN, int p, int PMAX, int RL>
+template <int LOGN, int p, int PMAX, int RL, bool EXACT = false>
 struct InvMiddle {
   static __device__ __forceinline__ void run(uint32_t x, int t) {
     if constexpr (p <= PMAX) {
-      pass16<LOGN, 8, RL * (1 << (3 * (p - 1))), true>(x, t);
-      InvMiddle<LOGN, p + 1, PMAX, RL>::run(x, t);
+      pass16<LOGN, 8, RL * (1 << (3 * (p - 1))), true, EXACT>(x, t);
+      InvMiddle<LOGN, p + 1, PMAX, RL, EXACT>::run(x, t);
     }
   }
 };

@@ -57,9 +57,10 @@ cudaError_t launch_welch(const float* x, int D, int64_t L, double fs, int64_t M,
 size_t welch_ws(int D, int64_t L, int64_t M, int64_t stride);
 cudaError_t launch_whiten_filter(const double* psd, int D, int64_t M, double fs, int k_lo, int64_t N, float* W,
                                  cudaStream_t s, bool inverse = false);
-// Packed-domain whitening coefficients (alpha, beta) [D][N/2] from W [D][N/2+1].
-cudaError_t launch_whiten_rows(const float* d, const float* W, int64_t rows, int D, int64_t N, float* y,
-                               cudaStream_t s);
+// Whitening of the windows d [B][D][N] (8-byte aligned) with the filter W [D][N/2+1] (Wcap
+// floats allocated, a multiple of 4); y may be d.
+cudaError_t launch_whiten_windows(const float* d, const float* W, int64_t Wcap, int64_t B, int D, int64_t N, float* y,
+                                  cudaStream_t s);
 cudaError_t launch_inject_rows(const float* noise, int D, int64_t L, const int64_t* offsets, const float2* hdet,
                                int64_t B, int64_t N, double fs, float* d, cudaStream_t s);
 cudaError_t launch_inject_padded(const float* noise, int D, int64_t L, const int64_t* offsets, const float* htd,

@@ -129,9 +129,10 @@ __device__ __forceinline__ float2 rot_turns8(float2 x, int e) {
 // R16: radix-16 passes (one butterfly per thread, swizzle sw16) when log2 n is not a
 // multiple of 4, else radix-8 passes (two butterflies per thread, swizzle sw).  Either
 // way the forward transform ends with the short radix RL and the inverse starts with it.
-template <int LOGN>
+// (WAVE false, whitening alone, always takes radix-8 passes: half the rounding error.)
+template <int LOGN, bool WAVE = true>
 struct SimPlan {
-  static constexpr bool R16 = (LOGN % 4) != 0;
+  static constexpr bool R16 = WAVE && (LOGN % 4) != 0;
   static constexpr int n = 1 << LOGN;
   static constexpr int T = n / 16;
   static constexpr int RL = R16 ? (1 << (LOGN % 4)) : Plan16<LOGN>::RL;
@@ -208,6 +209,14 @@ __device__ __forceinline__ CropCopy crop_copy(const int64_t* offsets, int64_t b,
   return c;
 }
 
+// The same of a row of single windows (WAVE false): whole rows, each aligned.
+template <bool WAVE>
+__device__ __forceinline__ CropCopy window_copy(const int64_t* offsets, int64_t b, int d, int64_t L, int64_t N,
+                                                int64_t DL, int D) {
+  if constexpr (WAVE) return crop_copy(offsets, b, d, L, N, DL);
+  return CropCopy{(b * D + d) * N, (uint32_t)(4 * N), 0};
+}
+
 // One block per draw (persistent over draws), n/16 threads.  The D windows go
 // through the shared window buffer in turn; the waveform values of the bins a
 // thread owns are computed once per draw and shared by the detectors.
@@ -220,15 +229,23 @@ __device__ __forceinline__ CropCopy crop_copy(const int64_t* offsets, int64_t b,
 // crop and the next detector's filter arrive in shared staging buffers by bulk asynchronous
 // copies issued one window ahead, so no pass waits on a global load; same arithmetic again.
 // Wcap: floats of the filter allocation W (the staged copies may read up to it).
+// WAVE false: whitening alone.  The windows are the rows of `noise` [B][D][N] themselves
+// (16-byte aligned when staged), there is no waveform and no table of its values, and the
+// radix-8 butterflies take the exactly rounded sqrt(1/2) products.  (One block a row with
+// eight values a thread, the spectrum unpacked, scaled and repacked through shared memory,
+// took 34.6 ns a window of 8192 samples; this form 24.3, or 26.4 from unstaged rows, 32 when
+// those run three blocks an SM in fewer registers.)
 // nd: detectors of a draw that a block takes in turn: D, or 1 when windows rather than draws
 // are dealt out (sim_split).
-template <int LOGN, bool VEC, bool PP, bool ST>
+template <int LOGN, bool VEC, bool PP, bool ST, bool WAVE>
 __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
     k_simulate(const DrawCoef* __restrict__ coef, const float* __restrict__ noise, int64_t L,
                const int64_t* __restrict__ offsets, const float* __restrict__ W, int64_t Wcap, int k_lo, int D,
                int64_t B, int nd, float* __restrict__ y) {
   static_assert(!(ST && PP), "staging uses the in-place passes");
-  using PL = SimPlan<LOGN>;
+  static_assert(WAVE || !PP, "whitening alone uses the in-place passes");
+  using PL = SimPlan<LOGN, WAVE>;
+  constexpr bool EXACT = !WAVE;
   constexpr bool R16 = PL::R16;
   constexpr int n = PL::n, T = PL::T, RL = PL::RL, NB = PL::NB, SLOTS = PL::SLOTS, MID = PL::MID;
   constexpr int64_t N = 2 * n;
@@ -238,14 +255,14 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
   __shared__ __align__(8) uint64_t bars[2];   // staging barriers: crop, filter
   __shared__ int s_o[2];                      // offsets within the staged crop and filter
   float2 (*wv)[T] = reinterpret_cast<float2 (*)[T]>(sm + (PP ? 2 : 1) * n);   // 16 x T waveform values
-  float* crop_s = reinterpret_cast<float*>(sm + 2 * n);                        // ST: N + 4 floats
+  float* crop_s = reinterpret_cast<float*>(sm + (WAVE ? 2 : 1) * n);           // ST: N + 4 floats
   float* w_s = crop_s + N + 4;                                                  // ST: n + 4 floats
 #define WIDX(s, h, r) (((s) * 2 + (h)) * RL + (r))
   const int t = threadIdx.x;
   const int lane = t & 31;
   const uint32_t x = smem_addr(sm), x2 = x + 8u * (uint32_t)n;
   const float inv_n = 1.0f / (float)n;
-  const int64_t DL = (int64_t)D * L;
+  const int64_t DL = WAVE ? (int64_t)D * L : B * D * N;
   const int per = D / nd;                       // units of a draw: 1, or D single windows
   const int64_t units = B * per;
   const uint32_t bar_c = smem_addr(&bars[0]), bar_w = smem_addr(&bars[1]);
@@ -263,7 +280,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
       if (blockIdx.x < units) {
         const int64_t b = blockIdx.x / per;
         const int d = (int)(blockIdx.x - b * per);
-        const CropCopy cc = crop_copy(offsets, b, d, L, N, DL);
+        const CropCopy cc = window_copy<WAVE>(offsets, b, d, L, N, DL, D);
         s_o[0] = cc.o;
         tc::mbar_expect_tx(bar_c, cc.bytes);
         bulk_g2s(smem_addr(crop_s), noise + cc.src, cc.bytes, bar_c);
@@ -280,23 +297,24 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
   for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
     const int64_t b = u / per;
     const int d_first = (int)(u - b * per);
-    for (int i = t; i < (int)(sizeof(DrawCoef) / 16); i += T)
-      reinterpret_cast<int4*>(&sc)[i] = __ldg(reinterpret_cast<const int4*>(coef + b) + i);
+    if constexpr (WAVE)
+      for (int i = t; i < (int)(sizeof(DrawCoef) / 16); i += T)
+        reinterpret_cast<int4*>(&sc)[i] = __ldg(reinterpret_cast<const int4*>(coef + b) + i);
     int64_t off = 0;
-    if constexpr (!ST) {
+    if constexpr (WAVE && !ST) {
       off = __ldg(&offsets[b]);
       off = off < 0 ? 0 : (off > L - N ? L - N : off);   // keep a bad offset inside the stretch
     }
     const int64_t a0 = off & ~(int64_t)1;
     const bool odd = (off & 1) != 0;
-    __syncthreads();
+    if constexpr (WAVE) __syncthreads();
     const DrawCoef& c = sc;
 
     // waveform values (turns, amplitude factor) of the 16 bins this thread owns in the
     // short-radix pass, kept in shared memory as wv[v][t] for the D detectors (a rolled
     // loop: the evaluation is long, and 32 inlined copies crowd the instruction cache)
 #pragma unroll 1
-    for (int s = 0; s < SLOTS; ++s) {
+    for (int s = 0; WAVE && s < SLOTS; ++s) {
       const int p = t + s * T;
       const int jA = p, jB = p ? NB - p : NB / 2;
 #pragma unroll 1
@@ -349,13 +367,13 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
             float2 v[8];
 #pragma unroll
             for (int r = 0; r < 8; ++r) v[r] = staged(j + r * (n / 8));
-            dft8<false, false>(v);
+            dft8<false, EXACT>(v);
             store_pass<8, 1>(x, j, v);
           }
         }
       } else {
-        const float* row = noise + (int64_t)d * L + a0;
-        const int64_t at0 = (int64_t)d * L + a0;
+        const int64_t at0 = WAVE ? (int64_t)d * L + a0 : (b * D + d) * N;
+        const float* row = noise + at0;
         if constexpr (R16) {
           float2 v[16];
 #pragma unroll
@@ -375,7 +393,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
               const int m = j + r * (n / 8);
               v[r] = crop_point<VEC, T>(row, m, odd, lane, at0 + 2 * m, DL);
             }
-            dft8<false, false>(v);
+            dft8<false, EXACT>(v);
             store_pass<8, 1>(x, j, v);
           }
         }
@@ -392,7 +410,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
         }
         // every read of the staged crop is done: fetch the next window's
         if (t == 0 && more) {
-          const CropCopy cc = crop_copy(offsets, b_next, d_next, L, N, DL);
+          const CropCopy cc = window_copy<WAVE>(offsets, b_next, d_next, L, N, DL, D);
           s_o[0] = cc.o;
           proxy_fence_async();
           tc::mbar_expect_tx(bar_c, cc.bytes);
@@ -407,14 +425,22 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
       } else if constexpr (PP) {
         xf = FwdMiddlePP<LOGN, 1, MID>::run(x, x2, t);
       } else {
-        FwdMiddle<LOGN, 1, MID>::run(x, t);
+        FwdMiddle<LOGN, 1, MID, EXACT>::run(x, t);
       }
       const uint32_t xi = PP ? (xf == x ? x2 : x) : x;
 
       // last forward pass (radix RL, Ns = NB) on butterfly pairs, frequency-domain
       // step and first inverse pass, all in registers
-      const float2 gd = make_float2(c.g[d].x, c.g[d].z);
-      const unsigned long long nu = c.nu[d];
+      float2 gd = make_float2(0.f, 0.f);
+      unsigned long long nu = 0ull;
+      if constexpr (WAVE) {
+        gd = make_float2(c.g[d].x, c.g[d].z);
+        nu = c.nu[d];
+      }
+      auto wave = [&](int i) -> float2 {   // waveform value i of this thread's bins
+        if constexpr (WAVE) return wv[i][t];
+        return make_float2(0.f, 0.f);
+      };
       const float* Wd = W + (int64_t)d * F;
       int ow = 0;
       if constexpr (ST) {
@@ -468,13 +494,13 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
             }
           }
         }
-        dftR<RL, false, false>(vA[s]);
-        dftR<RL, false, false>(vB[s]);
+        dftR<RL, false, EXACT>(vA[s]);
+        dftR<RL, false, EXACT>(vB[s]);
         // now vA[s][r] = Z[jA + NB r], vB[s][r] = Z[jB + NB r]
         if (p != 0) {
 #pragma unroll
           for (int r = 0; r < RL; ++r) {
-            const float2 ea = wv[WIDX(s, 0, r)][t], eb = wv[WIDX(s, 1, RL - 1 - r)][t];
+            const float2 ea = wave(WIDX(s, 0, r)), eb = wave(WIDX(s, 1, RL - 1 - r));
             const int k = jA + NB * r;
             const float2 e = rot_pi16(u, r * (16 / RL));   // e^{i pi k/n}
             fd_pair<LOGN>(vA[s][r], vB[s][RL - 1 - r], k, ea.x, ea.y, eb.x, eb.y, gd, nu, s_of(k), s_of(n - k), e.x,
@@ -482,26 +508,26 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
           }
         } else {
           fd_dc(vA[s][0], s_of(0), s_of(n));
-          const float2 eh = wv[WIDX(s, 0, RL / 2)][t];
+          const float2 eh = wave(WIDX(s, 0, RL / 2));
           fd_half<LOGN>(vA[s][RL / 2], eh.x, eh.y, gd, nu, s_of(n / 2));
 #pragma unroll
           for (int r = 1; r < RL / 2; ++r) {
-            const float2 ea = wv[WIDX(s, 0, r)][t], eb = wv[WIDX(s, 0, RL - r)][t];
+            const float2 ea = wave(WIDX(s, 0, r)), eb = wave(WIDX(s, 0, RL - r));
             const int k = NB * r;
             const float2 e = eipi16(r * (16 / RL));
             fd_pair<LOGN>(vA[s][r], vA[s][RL - r], k, ea.x, ea.y, eb.x, eb.y, gd, nu, s_of(k), s_of(n - k), e.x, e.y);
           }
 #pragma unroll
           for (int r = 0; r < RL / 2; ++r) {
-            const float2 ea = wv[WIDX(s, 1, r)][t], eb = wv[WIDX(s, 1, RL - 1 - r)][t];
+            const float2 ea = wave(WIDX(s, 1, r)), eb = wave(WIDX(s, 1, RL - 1 - r));
             const int k = NB / 2 + NB * r;
             const float2 e = eipi16(8 / RL + r * (16 / RL));
             fd_pair<LOGN>(vB[s][r], vB[s][RL - 1 - r], k, ea.x, ea.y, eb.x, eb.y, gd, nu, s_of(k), s_of(n - k), e.x,
                           e.y);
           }
         }
-        dftR<RL, true, false>(vA[s]);
-        dftR<RL, true, false>(vB[s]);
+        dftR<RL, true, EXACT>(vA[s]);
+        dftR<RL, true, EXACT>(vB[s]);
       }
       // in place, every read of the last forward pass must precede the writes below; with
       // two buffers the first inverse pass writes the other one
@@ -540,7 +566,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
       } else if constexpr (PP) {
         xl = InvMiddlePP<LOGN, 1, MID, RL>::run(xi, xf, t);
       } else {
-        InvMiddle<LOGN, 1, MID, RL>::run(x, t);
+        InvMiddle<LOGN, 1, MID, RL, EXACT>::run(x, t);
       }
 
       // last inverse pass (Ns = n/R), output straight to the whitened batch
@@ -567,7 +593,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
           pass_twiddles<8, n / 8, true>(j, w);
 #pragma unroll
           for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], w[r]);
-          dft8<true, false>(v);
+          dft8<true, EXACT>(v);
 #pragma unroll
           for (int r = 0; r < 8; ++r)
             if (GWX_IDX_OK((b * D + d) * N + 2 * (j + r * (n / 8)) + 1, B * D * N, 0x104))
@@ -620,7 +646,7 @@ static bool sim_split(int64_t B, int D, int64_t slots) {
   return 5 * by_window < 4 * by_draw;
 }
 
-template <int LG, bool VEC, bool PP, bool ST>
+template <int LG, bool VEC, bool PP, bool ST, bool WAVE = true>
 static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, int64_t L, const int64_t* offsets,
                                       const float* W, int64_t Wcap, int k_lo, int D, int64_t B, float* y,
                                       int per_sm_want, cudaStream_t s) {
@@ -628,9 +654,9 @@ static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, 
   constexpr size_t n = (size_t)1 << LG;
   // one (or two, PP) window buffers plus 16 waveform values per thread; staged: the crop
   // (N + 4 floats) and the filter (n + 4 floats) after them
-  const size_t smem = (PP ? 2 : 1) * n * sizeof(float2) + (size_t)16 * NT * sizeof(float2) +
+  const size_t smem = (PP ? 2 : 1) * n * sizeof(float2) + (WAVE ? (size_t)16 * NT * sizeof(float2) : 0) +
                       (ST ? (2 * n + 4 + n + 4) * sizeof(float) : 0);
-  auto kern = k_simulate<LG, VEC, PP, ST>;
+  auto kern = k_simulate<LG, VEC, PP, ST, WAVE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
@@ -641,10 +667,23 @@ static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, 
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   if (per_sm_want > 0 && per_sm_want < per_sm) per_sm = per_sm_want;
   const int64_t slots = (int64_t)sms * per_sm;
-  const int nd = sim_split(B, D, slots) ? 1 : D;
+  const int nd = !WAVE || sim_split(B, D, slots) ? 1 : D;
   const int64_t units = B * (D / nd), grid = units < slots ? units : slots;
   kern<<<(unsigned)grid, NT, smem, s>>>(coef, noise, L, offsets, W, Wcap, k_lo, D, B, nd, y);
   return cudaGetLastError();
+}
+
+// Whitening of the windows d [B][D][N] with the filter W (Wcap floats allocated): staged
+// wherever the rows may be copied in bulk, else read in pairs (a base 8-byte aligned only).
+cudaError_t launch_whiten_windows(const float* d, const float* W, int64_t Wcap, int64_t B, int D, int64_t N, float* y,
+                                  cudaStream_t s) {
+  if (B <= 0) return cudaSuccess;
+  const bool st = (uintptr_t)d % 16 == 0 && (uintptr_t)W % 16 == 0;
+  return dispatch_log<7, 13>(ilog2_exact(N / 2), [&](auto cst) {
+    constexpr int LG = decltype(cst)::value;
+    return st ? launch_simulate_lg<LG, true, false, true, false>(nullptr, d, N, nullptr, W, Wcap, 0, D, B, y, 0, s)
+              : launch_simulate_lg<LG, true, false, false, false>(nullptr, d, N, nullptr, W, Wcap, 0, D, B, y, 0, s);
+  });
 }
 
 cudaError_t launch_simulate_fused(const DrawCoef* coef, const float* noise, int64_t L, const int64_t* offsets,

@@ -71,7 +71,7 @@ int gwx_whiten_static(const float* d, const double* psd, int64_t seg_len, double
   // every filter entry the rows read is written first, so no clearing is needed
   st = launch_status(launch_whiten_filter(psd, D, seg_len, fs, k_lo, N, W, s), "gwx_whiten_static: whiten filter");
   if (st != GWX_OK) return st;
-  return launch_status(launch_whiten_rows(d, W, B * D, D, N, y, s), "gwx_whiten_static: whiten");
+  return launch_status(launch_whiten_windows(d, W, (int64_t)kStaticFilterFloats, B, D, N, y, s), "gwx_whiten_static: whiten");
 }
 
 }  // extern "C"

@@ -1,4 +1,4 @@
-// k_spectral.cu -- Welch PSD (A5), whitening filter and whitening (A7), crop and
+// k_spectral.cu -- Welch PSD (A5), whitening filter (A7; the windows in k_fused.cu), crop and
 // injection (A6), and row-wise real FFTs.  Every transform is a shared-memory
 // Stockham FFT of n = N/2 complex points (the real window packed as
 // z_m = x_2m + i x_2m+1) run by n/8 threads per row; several rows share a block
@@ -160,64 +160,6 @@ __device__ __forceinline__ void store_real_row(const float2* z, float* row, int 
     const int m = t + i * (n / 8);
     __stcs(&r2[m], z[sw(m)]);
   }
-}
-
-// ----------------------------------------------------------------- A7 whiten rows
-template <int LOGN>
-__global__ void __launch_bounds__(RowGeom<LOGN>::THREADS) k_whiten_rows(const float* __restrict__ din,
-                                                                         const float* __restrict__ W, int64_t rows,
-                                                                         int D, float* __restrict__ yout) {
-  using Gm = RowGeom<LOGN>;
-  constexpr int n = Gm::n;
-  constexpr int64_t N = 2 * n;
-  constexpr int64_t F = n + 1;
-  extern __shared__ float2 sm[];
-  const int g = threadIdx.x / Gm::TPR, t = threadIdx.x % Gm::TPR;
-  const int64_t r = (int64_t)blockIdx.x * Gm::G + g;
-  const bool live = r < rows;
-  float2* z = sm + g * n;
-  load_real_row<LOGN>(z, din + r * N, t, live);
-  __syncthreads();
-  fft_smem<LOGN, false>(z, t);
-  const float* Wd = W + (int64_t)(live ? (int)(r % D) : 0) * F;
-  const float inv_n = 1.0f / (float)n;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int k = t + i * (n / 8);
-    if (k == 0) {
-      const float2 z0 = z[0];
-      const float y0 = (z0.x + z0.y) * __ldg(&Wd[0]) * inv_n, yn = (z0.x - z0.y) * __ldg(&Wd[n]) * inv_n;
-      z[0] = make_float2(0.5f * (y0 + yn), 0.5f * (y0 - yn));
-      continue;
-    }
-    const float2 wk = pack_twiddle(k, LOGN + 1);
-    float2 xk, xnk, zk, znk;
-    unpack_pair(z[sw(k)], z[sw(n - k)], wk, xk, xnk);
-    pack_pair(cscale(xk, __ldg(&Wd[k]) * inv_n), cscale(xnk, __ldg(&Wd[n - k]) * inv_n), wk, zk, znk);
-    z[sw(k)] = zk;
-    z[sw(n - k)] = znk;
-  }
-  if (t == 0) {   // k = n/2 pairs with itself
-    const int h = n / 2;
-    const float2 wk = pack_twiddle(h, LOGN + 1);
-    float2 xk, xnk, zk, znk;
-    unpack_pair(z[sw(h)], z[sw(h)], wk, xk, xnk);
-    const float s_ = __ldg(&Wd[h]) * inv_n;
-    pack_pair(cscale(xk, s_), cscale(xk, s_), wk, zk, znk);
-    z[sw(h)] = zk;
-  }
-  __syncthreads();
-  fft_smem<LOGN, true>(z, t);
-  store_real_row<LOGN>(z, yout + r * N, t, live);
-}
-
-cudaError_t launch_whiten_rows(const float* d, const float* W, int64_t rows, int D, int64_t N, float* y,
-                               cudaStream_t s) {
-  return dispatch_log<4, 13>(ilog2_exact(N / 2), [&](auto c) {
-    constexpr int LG = decltype(c)::value;
-    using Gm = RowGeom<LG>;
-    return launch_rows(k_whiten_rows<LG>, rows, Gm::G, Gm::THREADS, Gm::SMEM, s, d, W, rows, D, y);
-  });
 }
 
 // ----------------------------------------------------------------- A6 inject rows
