@@ -43,6 +43,13 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// The same of max(a, 0), max(b, 0): the maximum is taken on the rounded pair in one instruction
+// (rounding is monotonic and keeps zero, so the values are the same; a NaN gives 0 as fmaxf does).
+__device__ __forceinline__ uint32_t pack2_relu(float a, float b) {
+  __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(a, b), __floats2bfloat162_rn(0.f, 0.f));
+  return *reinterpret_cast<uint32_t*>(&h);
+}
+
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }

@@ -206,24 +206,26 @@ __global__ void k_flow_input_backward(int l, const float* __restrict__ dX, int C
   }
 }
 
-__global__ void k_flow_base(uint32_t k0, uint32_t k1, uint32_t counter, int64_t row0, int64_t n,
-                            float* __restrict__ z) {
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// The kernels of one FP64 chain a row (targets, base normals, proposal) are bound by the FP64
+// pipe, a warp instruction 16 cycles of it: what counts is that every SM gets the same number
+// of warps.  One warp a block: 20,000 draws are at most 5 warps on an SM where blocks of 128
+// were 8 (157 blocks on 152 SMs); base normals one (row, pair) a thread, 16.1 -> 10.3 us,
+// proposal 23.7 -> 16.9 us.
+constexpr int ROW_NT = 32;
+
+__global__ void __launch_bounds__(ROW_NT) k_flow_base(uint32_t k0, uint32_t k1, uint32_t counter, int64_t row0,
+                                                      int64_t n, float* __restrict__ z) {
+  const int64_t at = (int64_t)blockIdx.x * ROW_NT + threadIdx.x;
+  const int64_t r = at >> 2;
   if (r >= n) return;
-  const uint32_t s = (uint32_t)(row0 + r);
-  float v[8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const u32x4 w = philox4x32_10(s, (uint32_t)i, TAG_FLOW, counter, k0, k1);
-    const double u0 = uniform52(w.x, w.y), u1 = uniform52(w.z, w.w);
-    // radius in FP64 (the logarithm near u0 -> 0 sets the tail), angle in FP32
-    const float rad = (float)sqrt(-2.0 * log(u0));
-    float sn, cs;
-    sincospif((float)(2.0 * u1), &sn, &cs);
-    v[2 * i] = rad * cs;
-    v[2 * i + 1] = rad * sn;
-  }
-  store8(z + r * 8, v);
+  const int i = (int)(at & 3);
+  const u32x4 w = philox4x32_10((uint32_t)(row0 + r), (uint32_t)i, TAG_FLOW, counter, k0, k1);
+  const double u0 = uniform52(w.x, w.y), u1 = uniform52(w.z, w.w);
+  // radius in FP64 (the logarithm near u0 -> 0 sets the tail), angle in FP32
+  const float rad = (float)sqrt(-2.0 * log(u0));
+  float sn, cs;
+  sincospif((float)(2.0 * u1), &sn, &cs);
+  reinterpret_cast<float2*>(z)[at] = make_float2(rad * cs, rad * sn);
 }
 
 __global__ void k_flow_proposal(const float* __restrict__ x, const float* __restrict__ z,
@@ -369,7 +371,7 @@ int64_t flow_layout(const gwx_flow_shape& sh, int64_t* off) {
 // ---- stage launchers ----
 cudaError_t launch_flow_targets(const double* theta, int64_t B, const double* mean8, const double* scale8, float* x,
                                 cudaStream_t s) {
-  k_flow_targets<<<blocks(B, 32), 32, 0, s>>>(theta, B, make_std(mean8, scale8), x);
+  k_flow_targets<<<blocks(B, ROW_NT), ROW_NT, 0, s>>>(theta, B, make_std(mean8, scale8), x);
   return cudaGetLastError();
 }
 
@@ -405,8 +407,8 @@ cudaError_t launch_flow_input_backward(int l, const float* dX, int C, int64_t B,
 }
 
 cudaError_t launch_flow_base(uint64_t seed, uint32_t counter, int64_t row0, int64_t n, float* z, cudaStream_t s) {
-  k_flow_base<<<blocks(n, 128), 128, 0, s>>>((uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32), counter, row0, n,
-                                             z);
+  k_flow_base<<<blocks(4 * n, ROW_NT), ROW_NT, 0, s>>>((uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32), counter,
+                                                       row0, n, z);
   return cudaGetLastError();
 }
 
@@ -418,9 +420,9 @@ cudaError_t launch_flow_proposal(const float* x, const float* z, const float* su
   Std8 st = make_std(mean8, scale8);
   st.ln_prior0 = log(2.0) - 2.0 * log(pr.m_hi - pr.m_lo) - log(pr.d_hi - pr.d_lo) - log(8.0 * PI_F) -
                  log(pr.psi_hi - pr.psi_lo) - log(pr.phi_hi - pr.phi_lo);
-  k_flow_proposal<<<blocks(n, 128), 128, 0, s>>>(x, z, sum_s, n, row0, S, st, pr,
-                                                 (uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32), counter,
-                                                 theta, log_q, log_ratio);
+  k_flow_proposal<<<blocks(n, ROW_NT), ROW_NT, 0, s>>>(x, z, sum_s, n, row0, S, st, pr,
+                                                       (uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32), counter,
+                                                       theta, log_q, log_ratio);
   return cudaGetLastError();
 }
 

@@ -2,23 +2,29 @@
 // kernel (the draw step of Sec. 5's posterior estimator).  Each CTA takes 128 draws at a
 // time through all K coupling layers without leaving the SM:
 //   - warp 0 streams each layer's conditioner weights from L2 with 3-D TMA boxes into a
-//     two-slot ring (part 0: V1; parts 1..H/128: pairs of V2's 64-column K-blocks; last
-//     part: V3 padded to 16 rows by the box's zero fill);
+//     two-slot ring (part 0: V1; parts 1..H/128: pairs of V2's 64-column K-blocks) and a
+//     buffer for V3 (padded to 16 rows by the box's zero fill), and its biases;
 //   - warp 1 issues tcgen05.mma: acc1 = X V1^T, acc2 = g1 V2^T, acc3 = g2 V3^T (FP32 in
-//     tensor memory, columns 0 and 256; acc3 reuses acc1's columns).  The products are cut
-//     into 128-column parts (N) and 128-column rounds of their input (K) so that the
-//     row warps and the tensor core overlap: the rows drain acc1's first part while the
-//     second is computed, acc2's first K round runs while the rows write the second
-//     quarter-pair of g1, and so on;
-//   - warps 2-9 own one draw (row) per thread, two warps per tensor-memory lane quarter:
-//     the first keeps the draw's eight coordinates and its log-scale sum in registers,
-//     writes the conditioning half of the conditioner input X once per layer and applies
-//     the coupling step from acc3; both write the context into X once per tile and half
-//     of the hidden activations g1, g2 (bias, ReLU, bfloat16) each, into shared memory in
-//     the 128-byte-swizzle layout the MMA reads.
-// The activations never go to global memory: per draw and layer only the weights (shared
-// by all draws, L2-resident) move.  Every mbarrier wait is bounded; on expiry the CTA
-// records a status, stops and frees its tensor memory.
+//     tensor memory), acc2 and acc3 in rounds of 128 columns of their input, so that the
+//     first round runs while the rows write the second's;
+//   - warps 2-17 own one draw (row) per thread, four warps per tensor-memory lane quarter:
+//     each writes a share of the context into the conditioner input X once per tile and
+//     of the hidden activations g1, g2 (bias, ReLU, bfloat16), and applies the coupling step
+//     to one of the four transformed coordinates; the first writes the conditioning half
+//     of X once per layer.
+// The activations stay in tensor memory: 32 accumulator columns are read, and 16 columns of
+// bfloat16 pairs written over the first of them, from where the next product takes its A
+// operand (columns 0..255 acc1, then g1; 256..511 acc2, then g2; acc3 in 16..31, which g1
+// leaves free).  Per draw and layer only the weights (shared by all draws, L2-resident) move.
+//
+// Bound by one tile's chain MMA -> drain -> MMA -> drain -> MMA -> coupling: of ~6900 cycles a
+// layer at H = 256 the products take 640 + 2048 + 256 and each hand-over ~300 more.  As
+// 128-column MMAs (which cost nearly what 256 columns do) from g in shared memory, eight row
+// warps and biases by every thread from L2, a layer took 9200: 20,000 draws of 16 layers
+// 163 us, now 122 (157 tiles on 152 SMs, two rounds; A from tensor memory 147, biases staged
+// 134, four warps a quarter and 256-column MMAs with the fragment-shaped drain 122).
+// Every mbarrier wait is bounded; on expiry the CTA records a status, stops and frees its
+// tensor memory.
 #include "flow_tile.cuh"
 
 namespace gwx {
@@ -27,7 +33,11 @@ namespace {
 
 using namespace flowt;
 
-constexpr size_t FUSED_SMEM = (size_t)X_BYTES + G_BYTES + 2 * SLOT_BYTES + 1024;
+constexpr uint32_t V3_BYTES = 16 * 256 * 2;
+constexpr size_t FUSED_SMEM = (size_t)X_BYTES + 2 * SLOT_BYTES + V3_BYTES + 1024;
+constexpr int ROW_WARPS = 16;                // four warps a tensor-memory lane quarter
+constexpr int S_THREADS = 64 + 32 * ROW_WARPS;
+constexpr uint32_t ACC2 = 256, ACC3 = 16;   // tensor-memory columns of the second and third products
 
 __device__ int g_flow_status;
 
@@ -45,46 +55,49 @@ struct FusedArgs {
   float* ss_out;                  // [n]
 };
 
-// v_b <- v_b e^s + mu with mu_j = o_j + b3_j, s_j = 3 tanh((o_{4+j} + b3_{4+j}) / 3);
-// b3: the layer's eight output biases, in registers
+// Coordinate j of the transformed half, and v[Bc(P, j)] = x[j] for all of them.
 template <int P>
-__device__ __forceinline__ void couple(float* v, const float* o, const float* b3, float& ss) {
+__device__ __forceinline__ float half_at(const float* v, int j) {
+  return j == 0 ? v[Bc(P, 0)] : j == 1 ? v[Bc(P, 1)] : j == 2 ? v[Bc(P, 2)] : v[Bc(P, 3)];
+}
+template <int P>
+__device__ __forceinline__ void set_half(float* v, const float* x) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float s = S_MAX * tanhf((o[4 + j] + b3[4 + j]) / S_MAX);
-    v[Bc(P, j)] = fmaf(v[Bc(P, j)], expf(s), o[j] + b3[j]);
-    ss += s;
-  }
+  for (int j = 0; j < 4; ++j) v[Bc(P, j)] = x[j];
 }
 
-__global__ void __launch_bounds__(F_THREADS, 1)
+__global__ void __launch_bounds__(S_THREADS, 1)
     k_flow_sample_fused(const __grid_constant__ CUtensorMap mv1, const __grid_constant__ CUtensorMap mv2,
                         const __grid_constant__ CUtensorMap mv3, FusedArgs a) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full[2], empty[2], xready, gready[2], acc1f[2], acc2f[2], acc3f;
+  __shared__ __align__(8) uint64_t full[3], empty[3], xready, gready[2], acc1f, acc2f, acc3f, biasf[2], cplf[4];
+  __shared__ __align__(16) float sb[2][2 * 256 + 8];       // biases of a layer: first, second, third product
+  __shared__ float s_new[4][FM], s_log[4][FM];              // the rows' transformed coordinates and log scales
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t base = (su32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t sx = base, sg = base + X_BYTES, sw = base + X_BYTES + G_BYTES;
+  const uint32_t sx = base, sw = base + X_BYTES, sv3 = sw + 2 * SLOT_BYTES;
   const int H = a.H, K = a.K, C = a.C;
   const int NP = 2 + H / 128;                              // weight parts per layer
   const int NR = H / 128;                                  // 128-column parts and rounds
   const int tiles = (int)((a.n + FM - 1) / FM);
-  const uint32_t id_128 = idesc_bf16(FM, 128), id_16 = idesc_bf16(FM, 16);
+  const uint32_t id_h = idesc_bf16(FM, (uint32_t)H), id_16 = idesc_bf16(FM, 16);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < 3; ++s) {
       mbar_init(su32(&full[s]), 1);
       mbar_init(su32(&empty[s]), 1);
     }
-    mbar_init(su32(&xready), 8);
+    mbar_init(su32(&xready), ROW_WARPS);
     for (int r = 0; r < 2; ++r) {
-      mbar_init(su32(&gready[r]), 8);
-      mbar_init(su32(&acc1f[r]), 1);
-      mbar_init(su32(&acc2f[r]), 1);
+      mbar_init(su32(&gready[r]), ROW_WARPS);
+      mbar_init(su32(&biasf[r]), 1);
     }
+    mbar_init(su32(&acc1f), 1);
+    mbar_init(su32(&acc2f), 1);
     mbar_init(su32(&acc3f), 1);
+    for (int q = 0; q < 4; ++q) mbar_init(su32(&cplf[q]), 4);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -100,20 +113,30 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   const uint32_t tmem = tmem_slot;
 
   if (warp == 0) {
-    uint32_t it = 0;
+    uint32_t it = 0, li = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
-      for (int l = 0; l < K && ok; ++l)
-        for (int p = 0; p < NP; ++p, ++it) {
-          const uint32_t s = it & 1u;
-          if (!mbar_wait_warp(su32(&empty[s]), ((it >> 1) & 1u) ^ 1u, F_WAIT) ||
+      for (int l = 0; l < K && ok; ++l, ++li)
+        for (int p = 0; p < NP; ++p) {
+          const bool last = p == NP - 1;
+          const uint32_t s = last ? 2u : it & 1u;
+          if (!mbar_wait_warp(su32(&empty[s]), ((last ? li : it >> 1) & 1u) ^ 1u, F_WAIT) ||
               __any_sync(0xffffffffu, *(volatile int*)&abort_flag)) {
             ok = false;
             break;
           }
           const uint32_t dst = sw + s * SLOT_BYTES, bar = su32(&full[s]);
           if (elect_one()) {
-            if (p == NP - 1) {
+            if (p == 0) {
+              // the slot just freed was filled in the layer before (two parts back), so the rows
+              // are through the one before that, whose biases these replace
+              const uint32_t bb = su32(&biasf[li & 1u]), d = su32(sb[li & 1u]);
+              mbar_expect_tx(bb, (uint32_t)H * 8u + 32u);
+              bulk_load(d, a.e1 + l * a.lstride, (uint32_t)H * 4u, bb);
+              bulk_load(d + 1024u, a.e2 + l * a.lstride, (uint32_t)H * 4u, bb);
+              bulk_load(d + 2048u, a.e3 + l * a.lstride, 32u, bb);
+            }
+            if (last) {
               mbar_expect_tx(bar, (uint32_t)H * 32u);
               for (int kb = 0; kb < H / 64; ++kb) tma_load_3d(dst + 2048u * kb, &mv3, 64 * kb, 0, l, bar);
             } else {
@@ -125,11 +148,13 @@ __global__ void __launch_bounds__(F_THREADS, 1)
             }
           }
           __syncwarp();
+          it += !last;
         }
     if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else if (warp == 1) {
     uint32_t it = 0, li = 0;
     bool ok = true;
+    const int xk = (8 + C + 15) / 16;                        // K steps of X that hold values
     auto wait_on = [&](uint64_t* bar, uint32_t parity) -> bool {
       const bool got = mbar_wait_warp(su32(bar), parity, F_WAIT);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -137,17 +162,17 @@ __global__ void __launch_bounds__(F_THREADS, 1)
     };
     for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
       for (int l = 0; l < K && ok; ++l, ++li) {
-        // acc1 = X V1^T, one 128-column part at a time
+        // acc1 = X V1^T
         uint32_t slot = it & 1u, wb = sw + slot * SLOT_BYTES;
         if (!(ok = wait_on(&full[slot], (it >> 1) & 1u) && wait_on(&xready, li & 1u))) break;
         if (elect_one()) {
-          for (int np = 0; np < NR; ++np) {
+          const uint64_t da = sw128_desc(sx), db = sw128_desc(wb);
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk)
-              mma_bf16(tmem + 128u * np, sw128_desc(sx + KB_BYTES * (kk >> 2) + 32u * (kk & 3)),
-                       sw128_desc(wb + (uint32_t)H * 128u * (kk >> 2) + 16384u * np + 32u * (kk & 3)), id_128, kk != 0);
-            mma_commit(su32(&acc1f[np]));
-          }
+          for (int kk = 0; kk < 8; ++kk)
+            if (kk < xk)
+              mma_bf16(tmem, da + (KB_BYTES * (kk >> 2) + 32u * (kk & 3)) / 16,
+                       db + ((uint32_t)H * 128u * (kk >> 2) + 32u * (kk & 3)) / 16, id_h, kk != 0);
+          mma_commit(su32(&acc1f));
           mma_commit(su32(&empty[slot]));
         }
         __syncwarp();
@@ -157,14 +182,12 @@ __global__ void __launch_bounds__(F_THREADS, 1)
           slot = it & 1u, wb = sw + slot * SLOT_BYTES;
           if (!(ok = wait_on(&full[slot], (it >> 1) & 1u) && wait_on(&gready[pr], 0u))) break;
           if (elect_one()) {
-            for (int np = 0; np < NR; ++np) {
+            const uint64_t db = sw128_desc(wb);
 #pragma unroll
-              for (int kk = 0; kk < 8; ++kk)
-                mma_bf16(tmem + 256u + 128u * np, sw128_desc(sg + KB_BYTES * (2 * pr + (kk >> 2)) + 32u * (kk & 3)),
-                         sw128_desc(wb + (uint32_t)H * 128u * (kk >> 2) + 16384u * np + 32u * (kk & 3)), id_128,
-                         (pr | kk) != 0);
-              if (pr == NR - 1) mma_commit(su32(&acc2f[np]));
-            }
+            for (int kk = 0; kk < 8; ++kk)
+              mma_bf16_ts(tmem + ACC2, tmem + 128u * pr + 32u * (kk >> 1) + 8u * (kk & 1),
+                          db + ((uint32_t)H * 128u * (kk >> 2) + 32u * (kk & 3)) / 16, id_h, (pr | kk) != 0);
+            if (pr == NR - 1) mma_commit(su32(&acc2f));
             mma_commit(su32(&empty[slot]));
           }
           __syncwarp();
@@ -172,36 +195,32 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         }
         if (!ok) break;
         // acc3 = g2 V3^T (16 rows, 8 of them the conditioner's outputs)
-        slot = it & 1u, wb = sw + slot * SLOT_BYTES;
-        if (!(ok = wait_on(&full[slot], (it >> 1) & 1u))) break;
+        if (!(ok = wait_on(&full[2], li & 1u))) break;
         for (int r = 0; r < NR; ++r) {
           if (!(ok = wait_on(&gready[r], 1u))) break;
           if (elect_one()) {
+            const uint64_t db = sw128_desc(sv3 + 4096u * r);
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-              const int kb = 2 * r + (kk >> 2);
-              mma_bf16(tmem, sw128_desc(sg + KB_BYTES * kb + 32u * (kk & 3)), sw128_desc(wb + 2048u * kb + 32u * (kk & 3)),
-                       id_16, (r | kk) != 0);
-            }
+            for (int kk = 0; kk < 8; ++kk)
+              mma_bf16_ts(tmem + ACC3, tmem + ACC2 + 128u * r + 32u * (kk >> 1) + 8u * (kk & 1),
+                          db + (2048u * (kk >> 2) + 32u * (kk & 3)) / 16, id_16, (r | kk) != 0);
             if (r == NR - 1) {
               mma_commit(su32(&acc3f));
-              mma_commit(su32(&empty[slot]));
+              mma_commit(su32(&empty[2]));
             }
           }
           __syncwarp();
         }
-        ++it;
       }
     if (!ok && lane == 0) atomicExch(&abort_flag, 1);
   } else {
     const int q = warp & 3;
-    const int h = (warp - 2) >> 2;                             // which half of the columns
+    const int h = (warp - 2) >> 2;                             // which 32 of every 128 columns
     const int r = 32 * q + lane;                               // row of the tile = tensor-memory lane
     const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16);
     uint32_t li = 0;
     bool ok = true;
     auto arrive = [&](uint64_t* bar) {
-      proxy_fence();
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(su32(bar));
@@ -209,46 +228,37 @@ __global__ void __launch_bounds__(F_THREADS, 1)
     auto wait_on = [&](uint64_t* bar, uint32_t parity) -> bool {
       const bool got = mbar_wait(su32(bar), parity, F_WAIT);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      return __all_sync(0xffffffffu, got) && !*(volatile int*)&abort_flag;
+      return __all_sync(0xffffffffu, got);
     };
-    // bias + ReLU of 64 accumulator columns (chunk c: two loads, one wait) into K-block c
-    // of the activation tile g; round rd of a hidden layer is chunk 2 rd + h.  The chunk's
-    // biases bb (loaded by load_bias before the wait for its accumulator, so that their
-    // latency overlaps the products) are read from registers.
-    auto load_bias = [&](const float* bias, int c, float4* bb) {
-      const float4* b4 = reinterpret_cast<const float4*>(bias + 64 * c);
+    // bias + ReLU of 32 accumulator columns (chunk c), written over the chunk's own first 16 as
+    // bfloat16 pairs; round rd of a hidden layer is chunk 4 rd + h.  In the fragment shape a
+    // thread holds 8 columns of 4 rows and reads 8 biases (32 columns of one row would be 32
+    // biases: 512 cycles of shared-memory reads a round, of 540)
+    auto hidden = [&](uint32_t col0, const float* bias, int c) {
+      const uint32_t at = lane_addr + col0 + 32u * c;
+      uint32_t raw[2][16], w[2][8];
+      tmem_ld_frag_async(at, raw[0]);
+      tmem_ld_frag_async(at + (16u << 16), raw[1]);
+      float2 b[4];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) bb[i] = __ldg(b4 + i);
-    };
-    auto hidden = [&](uint32_t col0, const float4* bb, int c) {
-      uint32_t raw[2][32];
-      tmem_ld32_async(lane_addr + col0 + 64u * c, raw[0]);
-      tmem_ld32_async(lane_addr + col0 + 64u * c + 32u, raw[1]);
+      for (int i = 0; i < 4; ++i) b[i] = *reinterpret_cast<const float2*>(bias + 32 * c + 8 * i + 2 * (lane & 3));
       tmem_wait_ld();
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        uint32_t w[16];
+      for (int k = 0; k < 2; ++k) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const float4 b = bb[8 * hh + i];
-          w[2 * i] = pack2(fmaxf(__uint_as_float(raw[hh][4 * i]) + b.x, 0.f),
-                           fmaxf(__uint_as_float(raw[hh][4 * i + 1]) + b.y, 0.f));
-          w[2 * i + 1] = pack2(fmaxf(__uint_as_float(raw[hh][4 * i + 2]) + b.z, 0.f),
-                               fmaxf(__uint_as_float(raw[hh][4 * i + 3]) + b.w, 0.f));
+          const float2 s = add2(make_float2(__uint_as_float(raw[k][2 * i]), __uint_as_float(raw[k][2 * i + 1])), b[i / 2]);
+          w[k][i] = pack2_relu(s.x, s.y);
         }
-#pragma unroll
-        for (int t4 = 0; t4 < 4; ++t4) {
-          const int col = 64 * c + 32 * hh + 8 * t4;
-          sts128(sg + KB_BYTES * (col >> 6) + swz(r, (col & 63) >> 3), w[4 * t4], w[4 * t4 + 1], w[4 * t4 + 2],
-                 w[4 * t4 + 3]);
-        }
+        tmem_st_frag(at + ((uint32_t)(16 * k) << 16), w[k]);
       }
+      tmem_wait_st();
     };
     for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
       const int64_t row = (int64_t)t * FM + r;
       const bool valid = row < a.n;
       float v[8], ss = 0.f;
-      if (valid && h == 0) {
+      if (valid) {
         const float4 z0 = reinterpret_cast<const float4*>(a.z + row * 8)[0];
         const float4 z1 = reinterpret_cast<const float4*>(a.z + row * 8)[1];
         v[0] = z0.x; v[1] = z0.y; v[2] = z0.z; v[3] = z0.w; v[4] = z1.x; v[5] = z1.y; v[6] = z1.z; v[7] = z1.w;
@@ -267,7 +277,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         e = lo;
       }
       const uint4* crow = reinterpret_cast<const uint4*>(a.ctx + e * C);
-      for (int g = h == 0 ? 1 : 8; g < (h == 0 ? 8 : 16); ++g) {
+      for (int g = h == 0 ? 1 : 4 * h; g < 4 * h + 4; ++g) {
         uint4 d = make_uint4(0u, 0u, 0u, 0u);
         if (valid && g <= C / 8) d = __ldg(crow + (g - 1));
         sts128(sx + KB_BYTES * (g >> 3) + swz(r, g & 7), d.x, d.y, d.z, d.w);
@@ -284,38 +294,49 @@ __global__ void __launch_bounds__(F_THREADS, 1)
           }
           sts128(sx + swz(r, 0), w0, w1, 0u, 0u);
         }
+        proxy_fence();
         arrive(&xready);
-        for (int rd = 0; rd < NR && ok; ++rd) {
-          float4 bb[16];
-          load_bias(a.e1 + l * a.lstride, 2 * rd + h, bb);
-          if (!(ok = wait_on(&acc1f[rd], li & 1u))) break;
-          hidden(0u, bb, 2 * rd + h);
+        const float* bl = sb[li & 1u];
+        if (!(ok = wait_on(&biasf[li & 1u], (li >> 1) & 1u) && !*(volatile int*)&abort_flag)) break;
+        if (!(ok = wait_on(&acc1f, li & 1u))) break;
+        for (int rd = 0; rd < NR; ++rd) {
+          hidden(0u, bl, 4 * rd + h);
           arrive(&gready[rd]);
         }
-        for (int rd = 0; rd < NR && ok; ++rd) {
-          float4 bb[16];
-          load_bias(a.e2 + l * a.lstride, 2 * rd + h, bb);
-          if (!(ok = wait_on(&acc2f[rd], li & 1u))) break;
-          hidden(256u, bb, 2 * rd + h);
+        if (!(ok = wait_on(&acc2f, li & 1u))) break;
+        for (int rd = 0; rd < NR; ++rd) {
+          hidden(ACC2, bl + 256, 4 * rd + h);
           arrive(&gready[rd]);
         }
-        if (!ok) break;
-        if (h != 0) continue;                                  // the coupling step is the first warp's
-        float b3[8];
-        {
-          const float4* b4 = reinterpret_cast<const float4*>(a.e3 + l * a.lstride);
-          const float4 lo4 = __ldg(b4), hi4 = __ldg(b4 + 1);
-          b3[0] = lo4.x; b3[1] = lo4.y; b3[2] = lo4.z; b3[3] = lo4.w;
-          b3[4] = hi4.x; b3[5] = hi4.y; b3[6] = hi4.z; b3[7] = hi4.w;
-        }
+        // v_b <- v_b e^s + mu with mu_j = o_j + b3_j, s_j = 3 tanh((o_{4+j} + b3_{4+j}) / 3):
+        // coordinate j by warp h = j of the quarter, handed to the others in shared memory
         if (!(ok = wait_on(&acc3f, li & 1u))) break;
-        float o[16];
-        tmem_ld16(lane_addr, o);
+        const uint32_t om = tmem_ld1_async(lane_addr + ACC3 + h), os = tmem_ld1_async(lane_addr + ACC3 + 4u + h);
+        tmem_wait_ld();
+        float vb;
         switch (p) {
-          case 0: couple<0>(v, o, b3, ss); break;
-          case 1: couple<1>(v, o, b3, ss); break;
-          case 2: couple<2>(v, o, b3, ss); break;
-          default: couple<3>(v, o, b3, ss); break;
+          case 0: vb = half_at<0>(v, h); break;
+          case 1: vb = half_at<1>(v, h); break;
+          case 2: vb = half_at<2>(v, h); break;
+          default: vb = half_at<3>(v, h); break;
+        }
+        const float s = S_MAX * tanhf((__uint_as_float(os) + bl[512 + 4 + h]) / S_MAX);
+        s_new[h][r] = fmaf(vb, expf(s), __uint_as_float(om) + bl[512 + h]);
+        s_log[h][r] = s;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(su32(&cplf[q]));
+        if (!(ok = wait_on(&cplf[q], li & 1u))) break;
+        float x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          x[j] = s_new[j][r];
+          ss += s_log[j][r];
+        }
+        switch (p) {
+          case 0: set_half<0>(v, x); break;
+          case 1: set_half<1>(v, x); break;
+          case 2: set_half<2>(v, x); break;
+          default: set_half<3>(v, x); break;
         }
       }
       if (!ok) break;
@@ -377,7 +398,7 @@ cudaError_t launch_flow_sample_fused(const void* params_bf16, const float* param
   const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
   e = cudaFuncSetAttribute(k_flow_sample_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM);
   if (e != cudaSuccess) return e;
-  k_flow_sample_fused<<<grid, F_THREADS, FUSED_SMEM, s>>>(m1, m2, m3, a);
+  k_flow_sample_fused<<<grid, S_THREADS, FUSED_SMEM, s>>>(m1, m2, m3, a);
   return cudaGetLastError();
 }
 
