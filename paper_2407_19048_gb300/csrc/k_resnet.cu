@@ -21,6 +21,7 @@ namespace gwx {
 namespace {
 
 constexpr float GN_EPS = 1e-5f;
+constexpr float GN_SCALE = 1.f / (1 << 24);   // of the sums of squares, against overflow of their total
 
 inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(256) k_gn_stats(const float* __restrict__ z, i
       const float4 v = __ldg(reinterpret_cast<const float4*>(zb + (int64_t)t * C + c));
       const float d0 = v.x - k0, d1 = v.y - k0, d2 = v.z - k0, d3 = v.w - k0;
       s1 += (d0 + d1) + (d2 + d3);
-      s2 += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+      s2 += fmaf(d0, d0, __fmul_rn(d1, d1)) + fmaf(d2, d2, __fmul_rn(d3, d3));
     } else {
       const float d = __ldg(zb + (int64_t)t * C + c) - k0;
       s1 += d;
@@ -172,53 +173,87 @@ __global__ void __launch_bounds__(256) k_gn_stats(const float* __restrict__ z, i
 // flight: every pass first issues its rows' loads (eight, or four of several arrays) and then
 // adds them (a loop of load and add kept one row in flight, 10 us a slab).  (512 windows, stem
 // and two blocks, six normalisations: 337 us as a statistics and an apply kernel forward, now
-// 225; ~700 us backward with the ReLU mask, the FP32 dz and its conversion as passes of their
-// own, now 510.)
+// 203; ~700 us backward with the ReLU mask, the FP32 dz and its conversion as passes of their
+// own, now 467.  Slabs staged in shared memory by asynchronous copies, columns split over
+// blocks, read every array once but left too few threads for the runs: 194 and 504.)
 // Sums: thread (run slice s, row lane l, column quad q) reads runs of 16 rows, rl = 256 / (C / 4)
-// rows apart, of channels 4 q .. 4 q + 3, coalesced float4 loads; FP32 within a run, FP64
+// rows apart, of channels 4 q .. 4 q + 3, coalesced float4 loads; FP32 within a run (the
+// contractions spelled out: the compiler's choice changes with the code around), two-float sums
 // across runs; then the lanes of each column quad and the quads of each group.
 constexpr int GN_NT = 512;
 // threads of the backward: the pooled gradient's rows hold twice the registers
 constexpr int gn_bt(int src) { return src == 2 ? 256 : 512; }
 
+// Sums across runs, lanes and warps: a value and the rounding errors of its additions (Knuth's
+// two-sum), about 48 bits.  Six FP32 additions a term; an FP64 addition holds the SM's FP64
+// pipe for 16 cycles a warp (forward 227 -> 203 us, backward 510 -> 467 for the above).
+struct Sum2 {
+  float h = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = __fadd_rn(h, x), z = __fsub_rn(t, h);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(t, z)), __fsub_rn(x, z)));
+    h = t;
+  }
+  __device__ __forceinline__ void add(const Sum2& o) {
+    add(o.h);
+    l = __fadd_rn(l, o.l);
+  }
+  __device__ __forceinline__ void add_lanes(int o) {
+    Sum2 x;
+    x.h = __shfl_xor_sync(0xffffffffu, h, o);
+    x.l = __shfl_xor_sync(0xffffffffu, l, o);
+    add(x);
+  }
+  // (an infinite sum's error is not a number)
+  __device__ __forceinline__ double value() const { return isfinite(h) ? (double)h + (double)l : (double)h; }
+};
+
 // Sums of a (and q) over the threads of every group (out[2 g], out[2 g + 1], valid after the
 // caller's barrier): lanes of a warp that share a column quad by shuffles, the remaining rows
 // of quads in shared memory, one warp per group.
 template <int NT>
-__device__ __forceinline__ void sample_group_sums(double a, double q, int cq, int cg, int G, double* out) {
-  __shared__ double r1[NT], r2[NT];
+__device__ __forceinline__ void sample_group_sums(Sum2 a, Sum2 q, int cq, int cg, int G, double* out) {
+  __shared__ float4 r[NT];   // (a, q) of a quad
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int o = 16; o >= cq; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    q += __shfl_xor_sync(0xffffffffu, q, o);
+    a.add_lanes(o);
+    q.add_lanes(o);
   }
   const int rows = cq < 32 ? NT / 32 : NT / cq;
   if (cq >= 32) {
-    r1[threadIdx.x] = a;
-    r2[threadIdx.x] = q;
+    r[threadIdx.x] = make_float4(a.h, a.l, q.h, q.l);
   } else if (lane < cq) {
-    r1[warp * cq + lane] = a;
-    r2[warp * cq + lane] = q;
+    r[warp * cq + lane] = make_float4(a.h, a.l, q.h, q.l);
   }
   __syncthreads();
   const int per = cg / 4;
   for (int g = warp; g < G; g += NT / 32) {
-    double x = 0.0, y = 0.0;
+    Sum2 x, y;
     for (int i = lane; i < rows * per; i += 32) {
-      const int at = (i / per) * cq + g * per + i % per;
-      x += r1[at];
-      y += r2[at];
+      const float4 v = r[(i / per) * cq + g * per + i % per];
+      x.add(v.x);
+      x.l += v.y;
+      y.add(v.z);
+      y.l += v.w;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      x += __shfl_xor_sync(0xffffffffu, x, o);
-      y += __shfl_xor_sync(0xffffffffu, y, o);
+      x.add_lanes(o);
+      y.add_lanes(o);
     }
     if (lane == 0) {
-      out[2 * g] = x;
-      out[2 * g + 1] = y;
+      out[2 * g] = x.value();
+      out[2 * g + 1] = y.value();
     }
   }
+}
+
+// 1 / sqrt(v) in FP64 from the single-precision value and one Newton step (error below 1e-13; the
+// library's FP64 call is a chain of some 2000 cycles here)
+__device__ __forceinline__ double inv_sqrt(double v) {
+  if (!(v < 1e30)) return rsqrt(v);
+  const double y = (double)rsqrtf((float)v);
+  return y * (1.5 - 0.5 * v * y * y);
 }
 
 __device__ __forceinline__ float4 bf16x4(uint2 q) {
@@ -245,7 +280,7 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
   const int64_t off = (int64_t)blockIdx.x * T * C;
   const float4* z4 = reinterpret_cast<const float4*>(z + off) + q4;   // row t at t cq
   const float k0 = __ldg(z + off + g * cg);
-  double a = 0.0, q = 0.0;
+  Sum2 a, q;
   for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_NT / 256) * 16 * rl) {
     float s1 = 0.f, s2 = 0.f;
 #pragma unroll
@@ -260,11 +295,11 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
       for (int i = 0; i < 8; ++i) {
         const float d0 = v[i].x - k0, d1 = v[i].y - k0, d2 = v[i].z - k0, d3 = v[i].w - k0;
         s1 += (d0 + d1) + (d2 + d3);
-        s2 += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+        s2 += fmaf(d0, d0, __fmul_rn(d1, d1)) + fmaf(d2, d2, __fmul_rn(d3, d3));
       }
     }
-    a += s1;
-    q += s2;
+    a.add(s1);
+    q.add(__fmul_rn(s2, GN_SCALE));
   }
   const float kg = (int)threadIdx.x < G ? __ldg(z + off + threadIdx.x * cg) : 0.f;
   const float4 gm = make_float4(__ldg(&gamma[4 * q4]), __ldg(&gamma[4 * q4 + 1]), __ldg(&gamma[4 * q4 + 2]),
@@ -275,8 +310,8 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
   __syncthreads();
   if ((int)threadIdx.x < G) {
     const int i = threadIdx.x;
-    const double m = sums[2 * i] * inv_n, var = fmax(sums[2 * i + 1] * inv_n - m * m, 0.0);
-    const float mean = (float)((double)kg + m), rstd = (float)rsqrt(var + (double)GN_EPS);
+    const double m = sums[2 * i] * inv_n, var = fmax(sums[2 * i + 1] * (inv_n / GN_SCALE) - m * m, 0.0);
+    const float mean = (float)((double)kg + m), rstd = (float)inv_sqrt(var + (double)GN_EPS);
     st[2 * i] = mean;
     st[2 * i + 1] = rstd;
     ms[2 * ((int64_t)blockIdx.x * G + i)] = mean;
@@ -334,6 +369,7 @@ __device__ __forceinline__ void gn_load(GnRow<SRC>& r, const GnSource& s, int64_
   const int64_t i = (b * T + t) * C + c;
   if constexpr (SRC == DY_POOL) {
     // time t is argument 1 of window t/2 (even t), or 2 of window t/2 and 0 of the next (odd t)
+    // (both loads always, without branches: 193 us where this takes 167)
     const int to = t / 2;
     const int64_t o = (b * s.To + to) * C + c;
     r.v0 = r.v1 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -380,7 +416,7 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
                                                             float* __restrict__ dsum, double* __restrict__ part) {
   constexpr int GN_BT = gn_bt(SRC);
   __shared__ double sums[64];
-  __shared__ double pr[GN_BT * 8];
+  __shared__ float2 pr[GN_BT * 8];
   __shared__ float st[64];
   constexpr int U = 4;   // rows in flight
   const int cq = C / 4, rl = 256 / cq, cg = C / G;
@@ -395,8 +431,7 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
     const float4 v = __ldg(reinterpret_cast<const float4*>(src.dy + b * C) + q4);
     mdy = make_float4(v.x / T, v.y / T, v.z / T, v.w / T);
   }
-  double a = 0.0, q = 0.0;
-  double pg[4] = {0.0, 0.0, 0.0, 0.0}, pb[4] = {0.0, 0.0, 0.0, 0.0};
+  Sum2 a, q, pg[4], pb[4];
   for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_BT / 256) * 16 * rl) {
     float s1 = 0.f, s2 = 0.f;
     float fg[4] = {0.f, 0.f, 0.f, 0.f}, fb[4] = {0.f, 0.f, 0.f, 0.f};
@@ -430,12 +465,12 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
         fb[3] += d.w;
       }
     }
-    a += s1;
-    q += s2;
+    a.add(s1);
+    q.add(s2);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      pg[m] += fg[m];
-      pb[m] += fb[m];
+      pg[m].add(fg[m]);
+      pb[m].add(fb[m]);
     }
   }
   if (part) {
@@ -443,16 +478,16 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
     for (int o = 16; o >= cq; o >>= 1) {
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        pg[m] += __shfl_xor_sync(0xffffffffu, pg[m], o);
-        pb[m] += __shfl_xor_sync(0xffffffffu, pb[m], o);
+        pg[m].add_lanes(o);
+        pb[m].add_lanes(o);
       }
     }
     const int lane = threadIdx.x & 31, at = cq >= 32 ? threadIdx.x : (threadIdx.x >> 5) * cq + lane;
     if (cq >= 32 || lane < cq) {
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        pr[at * 8 + m] = pg[m];
-        pr[at * 8 + 4 + m] = pb[m];
+        pr[at * 8 + m] = make_float2(pg[m].h, pg[m].l);
+        pr[at * 8 + 4 + m] = make_float2(pb[m].h, pb[m].l);
       }
     }
   }
@@ -468,10 +503,14 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
     const int rows = cq < 32 ? GN_BT / 32 : GN_BT / cq;
     for (int i = threadIdx.x; i < 2 * C; i += GN_BT) {
       const int c = i >> 1, k = (c & 3) + 4 * (i & 1);
-      double t = 0.0;
+      Sum2 t;
 #pragma unroll 4
-      for (int r = 0; r < rows; ++r) t += pr[(r * cq + c / 4) * 8 + k];
-      part[b * 2 * C + i] = t;
+      for (int r = 0; r < rows; ++r) {
+        const float2 v = pr[(r * cq + c / 4) * 8 + k];
+        t.add(v.x);
+        t.l += v.y;
+      }
+      part[b * 2 * C + i] = t.value();
     }
   }
   const float m1 = st[2 * g], m2 = st[2 * g + 1];
@@ -698,33 +737,35 @@ __global__ void __launch_bounds__(256) k_gn_param_part(const float* __restrict__
   }
 }
 
-// Sums of the slices: block of 8 channels x 32 slice lanes (lane l: slices l, l + 32, ...),
-// the lanes of a warp by shuffles, the warps in order (4 blocks of 32 channels took 14.7 us
-// for 512 slices of 128).
-__global__ void __launch_bounds__(256) k_gn_param_finish(const double* __restrict__ part, int slices, int C,
-                                                         float* __restrict__ dgamma, float* __restrict__ dbeta) {
-  __shared__ double2 r[8][8];
-  const int c = blockIdx.x * 8 + (threadIdx.x & 7);
+// Sums of the slices: block of 2 channels x 128 slice lanes (lane l: slices l, l + 128, ...),
+// the lanes of a warp by shuffles, the warps in order.  Two channels a block, so that the FP64
+// additions are spread over many SMs (512 slices of 128 channels: 4 blocks of 32 took 14.7 us,
+// 16 of 8 8.0, these 5.0).
+constexpr int PF_C = 2, PF_NT = 256;
+__global__ void __launch_bounds__(PF_NT) k_gn_param_finish(const double* __restrict__ part, int slices, int C,
+                                                           float* __restrict__ dgamma, float* __restrict__ dbeta) {
+  __shared__ double2 r[PF_NT / 32][PF_C];
+  const int c = blockIdx.x * PF_C + (threadIdx.x & (PF_C - 1));
   double tg = 0.0, tb = 0.0;
   if (c < C) {
-#pragma unroll 8
-    for (int s = threadIdx.x >> 3; s < slices; s += 32) {
+#pragma unroll 4
+    for (int s = threadIdx.x / PF_C; s < slices; s += PF_NT / PF_C) {
       const double2 v = __ldg(reinterpret_cast<const double2*>(part) + (int64_t)s * C + c);
       tg += v.x;
       tb += v.y;
     }
   }
 #pragma unroll
-  for (int o = 16; o >= 8; o >>= 1) {
+  for (int o = 16; o >= PF_C; o >>= 1) {
     tg += __shfl_xor_sync(0xffffffffu, tg, o);
     tb += __shfl_xor_sync(0xffffffffu, tb, o);
   }
-  if ((threadIdx.x & 31) < 8) r[threadIdx.x >> 5][threadIdx.x & 7] = make_double2(tg, tb);
+  if ((threadIdx.x & 31) < PF_C) r[threadIdx.x >> 5][threadIdx.x & (PF_C - 1)] = make_double2(tg, tb);
   __syncthreads();
-  if (threadIdx.x < 8 && c < C) {
+  if (threadIdx.x < PF_C && c < C) {
     double g = 0.0, bsum = 0.0;
 #pragma unroll
-    for (int y = 0; y < 8; ++y) {
+    for (int y = 0; y < PF_NT / 32; ++y) {
       g += r[y][threadIdx.x].x;
       bsum += r[y][threadIdx.x].y;
     }
@@ -912,6 +953,15 @@ cudaError_t launch_group_norm(const float* z, int64_t B, int T, int C, int G, co
   return cudaGetLastError();
 }
 
+template <int SRC, bool OUT16>
+static cudaError_t launch_gn_backward(const GnSource& src, const float* z, int64_t B, int T, int C, int G,
+                                      const float* ms, const float* gamma, void* dz, float* dsum, double* part,
+                                      cudaStream_t st) {
+  const double inv_n = 1.0 / ((double)T * (C / G));
+  k_gn_backward_s<SRC, OUT16><<<(unsigned)B, gn_bt(SRC), 0, st>>>(src, z, T, C, G, inv_n, ms, gamma, dz, dsum, part);
+  return cudaGetLastError();
+}
+
 size_t group_norm_backward_scratch(int64_t B, int C, int G) {
   return (size_t)B * G * 2 * sizeof(float) + 256 + (size_t)GN_MAX_SLICES * C * 2 * sizeof(double);
 }
@@ -926,10 +976,11 @@ cudaError_t launch_group_norm_backward(const float* dy, const float* z, int64_t 
   if (v4 && per_sample_ok(C, G)) {
     // the per-channel parameter sums come out of the statistics pass, one slice per sample
     const bool fused = B <= GN_MAX_SLICES;
-    k_gn_backward_s<DY_PLAIN, false><<<(unsigned)B, gn_bt(DY_PLAIN), 0, st>>>(GnSource{dy, nullptr, nullptr, 0}, z, T, C, G,
-                                                                    1.0 / ((double)T * (C / G)), ms, gamma, dz, nullptr, fused ? part : nullptr);
+    const cudaError_t e = launch_gn_backward<DY_PLAIN, false>(GnSource{dy, nullptr, nullptr, 0}, z, B, T, C, G, ms, gamma,
+                                                              dz, nullptr, fused ? part : nullptr, st);
+    if (e != cudaSuccess) return e;
     if (fused) {
-      k_gn_param_finish<<<nblk(C, 8), 256, 0, st>>>(part, (int)B, C, dgamma, dbeta);
+      k_gn_param_finish<<<nblk(C, PF_C), PF_NT, 0, st>>>(part, (int)B, C, dgamma, dbeta);
       return cudaGetLastError();
     }
   } else if (v4) {
@@ -942,7 +993,7 @@ cudaError_t launch_group_norm_backward(const float* dy, const float* z, int64_t 
   }
   const int slices = gn_slices(B * T);
   k_gn_param_part<<<dim3(nblk(C, 32), slices), 256, 0, st>>>(dy, z, (int)(B * T), T, C, G, ms, part);
-  k_gn_param_finish<<<nblk(C, 8), 256, 0, st>>>(part, slices, C, dgamma, dbeta);
+  k_gn_param_finish<<<nblk(C, PF_C), PF_NT, 0, st>>>(part, slices, C, dgamma, dbeta);
   return cudaGetLastError();
 }
 
@@ -956,18 +1007,16 @@ cudaError_t launch_group_norm_backward_src(int kind, const float* dy, const void
                                            float* dbeta, cudaStream_t st) {
   const GnSource src{dy, reinterpret_cast<const __nv_bfloat16*>(out), arg, (T + 2 - 3) / 2 + 1};
   double* part = reinterpret_cast<double*>(scratch);
-  const double inv_n = 1.0 / ((double)T * (C / G));
-  auto run = [&](auto kern) { kern<<<(unsigned)B, gn_bt(kind), 0, st>>>(src, z, T, C, G, inv_n, ms, gamma, dz16, dsum, part); };
+  cudaError_t e = cudaErrorInvalidValue;
   switch (kind) {
-    case DY_PLAIN: run(k_gn_backward_s<DY_PLAIN, true>); break;
-    case DY_MASK: run(k_gn_backward_s<DY_MASK, true>); break;
-    case DY_POOL: run(k_gn_backward_s<DY_POOL, true>); break;
-    case DY_MEAN: run(k_gn_backward_s<DY_MEAN, true>); break;
-    default: return cudaErrorInvalidValue;
+    case DY_PLAIN: e = launch_gn_backward<DY_PLAIN, true>(src, z, B, T, C, G, ms, gamma, dz16, dsum, part, st); break;
+    case DY_MASK: e = launch_gn_backward<DY_MASK, true>(src, z, B, T, C, G, ms, gamma, dz16, dsum, part, st); break;
+    case DY_POOL: e = launch_gn_backward<DY_POOL, true>(src, z, B, T, C, G, ms, gamma, dz16, dsum, part, st); break;
+    case DY_MEAN: e = launch_gn_backward<DY_MEAN, true>(src, z, B, T, C, G, ms, gamma, dz16, dsum, part, st); break;
+    default: break;
   }
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_gn_param_finish<<<nblk(C, 8), 256, 0, st>>>(part, (int)B, C, dgamma, dbeta);
+  k_gn_param_finish<<<nblk(C, PF_C), PF_NT, 0, st>>>(part, (int)B, C, dgamma, dbeta);
   return cudaGetLastError();
 }
 
