@@ -236,18 +236,18 @@ __global__ void __launch_bounds__(S_THREADS, 1)
     // biases: 512 cycles of shared-memory reads a round, of 540)
     auto hidden = [&](uint32_t col0, const float* bias, int c) {
       const uint32_t at = lane_addr + col0 + 32u * c;
-      uint32_t raw[2][16], w[2][8];
-      tmem_ld_frag_async(at, raw[0]);
-      tmem_ld_frag_async(at + (16u << 16), raw[1]);
+      uint32_t raw[32], w[2][8];
+      tmem_ld_frag_async(at, raw);
+      tmem_ld_frag_async(at + (16u << 16), raw + 16);
       float2 b[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) b[i] = *reinterpret_cast<const float2*>(bias + 32 * c + 8 * i + 2 * (lane & 3));
-      tmem_wait_ld();
+      tmem_wait_ld32(raw);
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const float2 s = add2(make_float2(__uint_as_float(raw[k][2 * i]), __uint_as_float(raw[k][2 * i + 1])), b[i / 2]);
+          const float2 s = add2(make_float2(__uint_as_float(raw[16 * k + 2 * i]), __uint_as_float(raw[16 * k + 2 * i + 1])), b[i / 2]);
           w[k][i] = pack2_relu(s.x, s.y);
         }
         tmem_st_frag(at + ((uint32_t)(16 * k) << 16), w[k]);
@@ -311,8 +311,8 @@ __global__ void __launch_bounds__(S_THREADS, 1)
         // v_b <- v_b e^s + mu with mu_j = o_j + b3_j, s_j = 3 tanh((o_{4+j} + b3_{4+j}) / 3):
         // coordinate j by warp h = j of the quarter, handed to the others in shared memory
         if (!(ok = wait_on(&acc3f, li & 1u))) break;
-        const uint32_t om = tmem_ld1_async(lane_addr + ACC3 + h), os = tmem_ld1_async(lane_addr + ACC3 + 4u + h);
-        tmem_wait_ld();
+        uint32_t om = tmem_ld1_async(lane_addr + ACC3 + h), os = tmem_ld1_async(lane_addr + ACC3 + 4u + h);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(om), "+r"(os)::"memory");
         float vb;
         switch (p) {
           case 0: vb = half_at<0>(v, h); break;

@@ -115,20 +115,16 @@ __device__ __forceinline__ float act_grad(float z, int act) {
 
 __device__ int g_gemm_status;
 
-// Fused epilogue of a dense layer on 32 accumulator columns starting at col0:
-// z = acc + bias[col], then the activation (0 identity, 1 ReLU, 2 GELU z Phi(z)).
-__device__ __forceinline__ void epilogue_ops(float* v, const float* __restrict__ bias, int act, int col0, int N) {
-  if (bias) {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] += (col0 + i < N) ? __ldg(&bias[col0 + i]) : 0.f;
-  }
-  if (act == 1) {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i], 0.f);
-  } else if (act == 2) {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = 0.5f * v[i] * erfcf(-0.70710678118654752f * v[i]);
-  }
+// Four consecutive floats from p (n of them exist; vec: p is 16-byte aligned and n >= 4).
+__device__ __forceinline__ float4 load4(const float* __restrict__ p, int n, bool vec) {
+  if (vec) return __ldg(reinterpret_cast<const float4*>(p));
+  return make_float4(__ldg(p), n > 1 ? __ldg(p + 1) : 0.f, n > 2 ? __ldg(p + 2) : 0.f, n > 3 ? __ldg(p + 3) : 0.f);
+}
+
+__device__ __forceinline__ float act_of(float z, int act) {
+  if (act == 1) return fmaxf(z, 0.f);
+  if (act == 2) return 0.5f * z * erfcf(-0.70710678118654752f * z);
+  return z;
 }
 
 // Tile t of a persistent CTA -> (tm, tn): bands of `group` tile-rows, columns fastest
@@ -162,7 +158,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   static_assert(MW == 1 || OPS == OP_KK, "wide tiles are for plain products");
   constexpr bool A_MN = op_a_mn(OPS), B_MN = op_b_mn(OPS);
   constexpr uint32_t CHUNK = 64 * GK * 2;   // one 64-column box of an MN-major operand
-  const float* addend = OUT == OUT_DACT ? nullptr : extra;
   constexpr int GN = TN_;
   using TL = Tile<TN_, MW>;
   constexpr int GMT = TL::ROWS;
@@ -340,8 +335,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     const int hsel = (warp - 2) >> 2;
     const int c_lo = MW == 1 ? hsel * (GN / 64) : 0, c_hi = MW == 1 ? c_lo + GN / 64 : GN / 32;
     const int msel = MW == 1 ? 0 : hsel;
-    float* ebuf = reinterpret_cast<float*>(smem_raw + (base - su32(smem_raw)) + STAGES * STAGE_BYTES +
-                                           (warp - 2) * EPI_BUF_BYTES);
+    const uint32_t ebuf = base + STAGES * STAGE_BYTES + (uint32_t)(warp - 2) * EPI_BUF_BYTES;
     uint32_t tl = 0;
     for (int w = blockIdx.x; w < work; w += gridDim.x, ++tl) {
       int tm, tn;
@@ -355,84 +349,115 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         if (lane == 0) atomicExch(&abort_flag, 1);
         break;
       }
-      // Each warp stages its 32 rows x 32 columns through a swizzled shared tile (word j of
-      // row r at r * 32 + (j ^ r): conflict-free both ways), then stores whole row segments:
-      // FP32 one 128-byte row per instruction, bfloat16 two 64-byte rows per instruction.
+      // Each warp turns 32 rows x 32 columns around in a shared tile (16-byte chunk j of row r at
+      // chunk j ^ (r mod 8): conflict-free both ways), after which a lane holds four consecutive
+      // columns of rows 4 k + lane / 8: bias, addend and dY are read, and C written, four values
+      // at a time and four whole row segments an instruction.  (One value at a time, with the
+      // bias read by every row, the epilogue of one tile took 8000 cycles at 128 columns of
+      // bfloat16, 25000 with dY, 16000 at 256 columns of FP32: as long as the products.)
       const int row0 = tm * GMT + GM * msel + 32 * q;
+      const int c_end = row0 < M ? min(c_hi, (N - tn * GN + 31) / 32) : c_lo;
+      const uint32_t tcol = tmem + ((uint32_t)(32 * q) << 16) + (acc + (uint32_t)msel) * TMEM_COLS;
+      constexpr int ESZ = OUT == OUT_F32 ? 4 : 2;
+      uint8_t* out = reinterpret_cast<uint8_t*>(C) + slice * ESZ;
+      const bool vec = N % 4 == 0 && (uintptr_t)out % (4 * ESZ) == 0;
+      const bool vec_b = (uintptr_t)bias % 16 == 0, vec_x = N % 4 == 0 && (uintptr_t)extra % 16 == 0;
+      const int rl = lane >> 3, jc = lane & 7;
+      uint32_t raw[32];
+      if (c_lo < c_end) tmem_ld32_async(tcol + 32u * c_lo, raw);
 #pragma unroll 1
-      for (int c = c_lo; c < c_hi; ++c) {
-        float v[32];
-        const int col0 = tn * GN + 32 * c;
-        // addend row segment of this lane's row (columns col0 .. col0 + 31; N % 32 == 0 and a
-        // 16-byte aligned addend when one is given), fetched before the accumulator so that
-        // its latency overlaps the tensor-memory load
-        float4 ad[8];
-        if (addend != nullptr) {
-          const bool in = row0 + lane < M && col0 < N;
-          const float4* ap = reinterpret_cast<const float4*>(addend + (int64_t)(row0 + lane) * N + col0);
+      for (int c = c_lo; c < c_end; ++c) {
+        const int col = tn * GN + 32 * c + 4 * jc, left = N - col;   // this lane's columns
+        // the rows' addend or dY, and the bias, before the accumulator, so that their latency
+        // overlaps the tensor-memory load
+        float4 x[8], b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (extra != nullptr) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) ad[j] = in ? __ldg(ap + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        // dY of this lane's column (OUT_DACT), fetched early for the same reason
-        float dy[32];
-        if constexpr (OUT == OUT_DACT) {
-          const float* yp = extra + (int64_t)row0 * N + col0 + lane;
-#pragma unroll
-          for (int r = 0; r < 32; ++r)
-            dy[r] = row0 + r < M && col0 + lane < N ? __ldg(yp + (int64_t)r * N) : 0.f;
-        }
-        tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (acc + (uint32_t)msel) * TMEM_COLS + (uint32_t)(32 * c), v);
-        if (row0 >= M || col0 >= N) continue;   // warp-uniform
-        if (addend != nullptr) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            v[4 * j] += ad[j].x;
-            v[4 * j + 1] += ad[j].y;
-            v[4 * j + 2] += ad[j].z;
-            v[4 * j + 3] += ad[j].w;
+          for (int k = 0; k < 8; ++k) {
+            const int r = row0 + 4 * k + rl;
+            x[k] = r < M && left > 0 ? load4(extra + (int64_t)r * N + col, left, vec_x) : make_float4(0.f, 0.f, 0.f, 0.f);
           }
         }
-        epilogue_ops(v, bias, OUT == OUT_DACT ? 0 : act, col0, N);
+        if (bias != nullptr && left > 0) b4 = load4(bias + col, left, vec_b && left >= 4);
+        tmem_wait_ld32(raw);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) ebuf[lane * 32 + (j ^ lane)] = v[j];
+        for (int j = 0; j < 8; ++j)
+          sts128(ebuf + 128u * lane + (uint32_t)((j ^ (lane & 7)) << 4), raw[4 * j], raw[4 * j + 1], raw[4 * j + 2],
+                 raw[4 * j + 3]);
         __syncwarp();
-        if constexpr (OUT == OUT_DACT) {
-          __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(C);
-          const int col = col0 + lane;
-          float sum = 0.f;
+        if (c + 1 < c_end) tmem_ld32_async(tcol + 32u * (c + 1), raw);
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-          for (int r = 0; r < 32; ++r) {
-            float a = dy[r];
-            if (act != 0) a *= act_grad(ebuf[r * 32 + (lane ^ r)], act);
-            sum += a;
-            if (row0 + r < M && col < N) out[(int64_t)(row0 + r) * N + col] = __float2bfloat16_rn(a);
+        for (int k = 0; k < 8; ++k) {
+          const int r = 4 * k + rl, grow = row0 + r;
+          float4 v = lds128(ebuf + 128u * r + (uint32_t)((jc ^ (r & 7)) << 4));
+          if (OUT != OUT_DACT && extra != nullptr) {
+            v.x += x[k].x;
+            v.y += x[k].y;
+            v.z += x[k].z;
+            v.w += x[k].w;
           }
-          if (col < N) colsum[(int64_t)(row0 / 32) * N + col] = sum;
-        } else if constexpr (OUT == OUT_BF16) {
-          __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(C) + slice;
-          const int w = lane & 15, col = col0 + 2 * w;
-#pragma unroll 4
-          for (int r2 = 0; r2 < 16; ++r2) {
-            const int r = 2 * r2 + (lane >> 4);
-            const int grow = row0 + r;
-            const float a = ebuf[r * 32 + ((2 * w) ^ r)], b = ebuf[r * 32 + ((2 * w + 1) ^ r)];
-            if (grow < M) {
-              __nv_bfloat16* o = out + (int64_t)grow * N + col;
-              if (col + 1 < N && (N % 2) == 0) {
-                *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(a, b);
-              } else {
-                if (col < N) o[0] = __float2bfloat16_rn(a);
-                if (col + 1 < N) o[1] = __float2bfloat16_rn(b);
-              }
+          if (bias != nullptr) {
+            v.x += b4.x;
+            v.y += b4.y;
+            v.z += b4.z;
+            v.w += b4.w;
+          }
+          if constexpr (OUT == OUT_DACT) {
+            float4 a = x[k];
+            if (act != 0) {
+              a.x *= act_grad(v.x, act);
+              a.y *= act_grad(v.y, act);
+              a.z *= act_grad(v.z, act);
+              a.w *= act_grad(v.w, act);
+            }
+            v = a;
+            sum.x += a.x;
+            sum.y += a.y;
+            sum.z += a.z;
+            sum.w += a.w;
+          } else if (act != 0) {
+            v = make_float4(act_of(v.x, act), act_of(v.y, act), act_of(v.z, act), act_of(v.w, act));
+          }
+          if (grow >= M || left <= 0) continue;
+          if constexpr (OUT == OUT_F32) {
+            float* o = reinterpret_cast<float*>(out) + (int64_t)grow * N + col;
+            if (vec) {
+              *reinterpret_cast<float4*>(o) = v;
+            } else {
+              o[0] = v.x;
+              if (left > 1) o[1] = v.y;
+              if (left > 2) o[2] = v.z;
+              if (left > 3) o[3] = v.w;
+            }
+          } else {
+            __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(out) + (int64_t)grow * N + col;
+            if (vec) {
+              const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+              *reinterpret_cast<uint2*>(o) =
+                  make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            } else {
+              o[0] = __float2bfloat16_rn(v.x);
+              if (left > 1) o[1] = __float2bfloat16_rn(v.y);
+              if (left > 2) o[2] = __float2bfloat16_rn(v.z);
+              if (left > 3) o[3] = __float2bfloat16_rn(v.w);
             }
           }
-        } else {
-          float* out = reinterpret_cast<float*>(C) + slice;
-          const int col = col0 + lane;
-#pragma unroll 4
-          for (int r = 0; r < 32; ++r) {
-            const float a = ebuf[r * 32 + (lane ^ r)];
-            if (row0 + r < M && col < N) out[(int64_t)(row0 + r) * N + col] = a;
+        }
+        if constexpr (OUT == OUT_DACT) {
+#pragma unroll
+          for (int o = 16; o >= 8; o >>= 1) {
+            sum.x += __shfl_xor_sync(0xffffffffu, sum.x, o);
+            sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o);
+            sum.z += __shfl_xor_sync(0xffffffffu, sum.z, o);
+            sum.w += __shfl_xor_sync(0xffffffffu, sum.w, o);
+          }
+          if (rl == 0 && left > 0) {
+            float* o = colsum + (int64_t)(row0 / 32) * N + col;
+            o[0] = sum.x;
+            if (left > 1) o[1] = sum.y;
+            if (left > 2) o[2] = sum.z;
+            if (left > 3) o[3] = sum.w;
           }
         }
         __syncwarp();
