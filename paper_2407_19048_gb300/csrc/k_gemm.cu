@@ -127,15 +127,49 @@ __device__ __forceinline__ float act_of(float z, int act) {
   return z;
 }
 
-// Tile t of a persistent CTA -> (tm, tn): bands of `group` tile-rows, columns fastest
-// within a band, so the CTAs working at the same time share a few A and B panels in L2.
+// Division by a number known at launch: q = floor(n m / 2^32) with m = floor(2^32 / d) + 1 is
+// the quotient or one more for every 32-bit n (m d - 2^32 <= d).
+struct Div {
+  uint32_t d, m;   // m = 0: d = 1
+};
+inline Div make_div(int64_t d) { return d <= 1 ? Div{1u, 0u} : Div{(uint32_t)d, 0xffffffffu / (uint32_t)d + 1u}; }
+__device__ __forceinline__ int divide(const Div& v, int n, int& rem) {
+  uint32_t q = v.m ? __umulhi((uint32_t)n, v.m) : (uint32_t)n;
+  int r = n - (int)(q * v.d);
+  if (r < 0) {
+    --q;
+    r += (int)v.d;
+  }
+  rem = r;
+  return (int)q;
+}
+
+// Work item w of a persistent CTA -> K slice, group z and tile (tm, tn), tile fastest; the tiles
+// in bands of `group` tile-rows, columns fastest within a band, so that the CTAs working at
+// the same time share a few A and B panels in L2.  (Plain divisions cost every role of the
+// kernel 640 cycles a tile, as much as four K blocks.)
 constexpr int DEFAULT_GROUP = 16;
-__device__ __forceinline__ void tile_coords(int t, int TM, int TN, int group, int& tm, int& tn) {
-  const int band = t / (group * TN);
-  const int r = t - band * group * TN;
-  const int rows = min(group, TM - band * group);
-  tm = band * group + r % rows;
-  tn = r / rows;
+struct WorkMap {
+  Div per, tiles, band, group, last;   // last: the rows of the last band
+  int TM;
+};
+inline WorkMap make_work_map(int64_t TM, int64_t TN, int group, int groups) {
+  const int64_t rest = TM % group;
+  return WorkMap{make_div(TM * TN * groups), make_div(TM * TN), make_div(group * TN), make_div(group),
+                 make_div(rest ? rest : group), (int)TM};
+}
+struct WorkItem {
+  int tm, tn, z, slice;
+};
+__device__ __forceinline__ WorkItem work_item(const WorkMap& m, int w) {
+  WorkItem i;
+  int r, t;
+  i.slice = divide(m.per, w, r);
+  i.z = divide(m.tiles, r, t);
+  const int first = divide(m.band, t, r) * (int)m.group.d;
+  i.tn = divide(first + (int)m.group.d <= m.TM ? m.group : m.last, r, i.tm);
+  i.tm += first;
+  return i;
 }
 
 // Persistent, warp-specialised: warp 0 lane 0 produces (TMA), warp 1 allocates tensor
@@ -152,7 +186,7 @@ __device__ __forceinline__ void tile_coords(int t, int TM, int TN, int group, in
 template <int OUT, int TN_, int OPS, int MW = 1>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     k_gemm_bf16(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, void* __restrict__ C,
-                const float* __restrict__ bias, int act, int group, int M, int N, int K, int kbs, int splits,
+                const float* __restrict__ bias, int act, const WorkMap map, int M, int N, int K, int kbs, int splits,
                 const float* __restrict__ extra, float* __restrict__ colsum, int groups, int64_t cstride,
                 ConvGeo geo) {
   static_assert(MW == 1 || OPS == OP_KK, "wide tiles are for plain products");
@@ -175,10 +209,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t base = (su32(smem_raw) + 1023u) & ~1023u;   // 1024-byte aligned stages
   const int KB = (K + GK - 1) / GK;
-  const int TM = (M + GMT - 1) / GMT, TN = (N + GN - 1) / GN;
-  const int tiles = TM * TN;
-  const int per = tiles * groups;
-  const int work = per * splits;   // (tile, group, K slice) triples, tile fastest
+  const int work = (int)map.per.d * splits;   // (tile, group, K slice) triples, tile fastest
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -207,10 +238,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     uint32_t s = 0, ph = 1;   // stage and the parity of its "empty" phase (the first round finds them free)
     bool ok = true, ready = true;
     for (int w = blockIdx.x; w < work && ok; w += gridDim.x) {
-      int tm, tn;
-      tile_coords(w % tiles, TM, TN, group, tm, tn);
-      const int z = (w % per) / tiles;
-      const int kb0 = (w / per) * kbs, kb1 = min(KB, kb0 + kbs);
+      const WorkItem item = work_item(map, w);
+      const int tm = item.tm, tn = item.tn, z = item.z;
+      const int kb0 = item.slice * kbs, kb1 = min(KB, kb0 + kbs);
       for (int k0 = kb0; k0 < kb1; k0 += KPS) {
         if (!__all_sync(0xffffffffu, ready) && !mbar_wait_warp(su32(&empty[s]), ph, WAIT_POLLS)) {
           ok = false;
@@ -280,7 +310,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     bool ok = true;
     for (int w = blockIdx.x; w < work && ok; w += gridDim.x, ++tl) {
       const uint32_t acc = tl % NACC;
-      const int kb0 = (w / per) * kbs, kb1 = min(KB, kb0 + kbs);
+      int unused;
+      const int kb0 = divide(map.per, w, unused) * kbs, kb1 = min(KB, kb0 + kbs);
       if (tl >= NACC && !mbar_wait_warp(su32(&tempty[acc]), ((tl / NACC) - 1) & 1u, WAIT_POLLS)) {
         ok = false;
         break;
@@ -338,10 +369,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     const uint32_t ebuf = base + STAGES * STAGE_BYTES + (uint32_t)(warp - 2) * EPI_BUF_BYTES;
     uint32_t tl = 0;
     for (int w = blockIdx.x; w < work; w += gridDim.x, ++tl) {
-      int tm, tn;
-      tile_coords(w % tiles, TM, TN, group, tm, tn);
-      const size_t slice = splits > 1 ? (size_t)(w / tiles) * (size_t)M * (size_t)N
-                                      : (size_t)((w % per) / tiles) * (size_t)cstride;
+      const WorkItem item = work_item(map, w);
+      const int tm = item.tm, tn = item.tn;
+      const size_t slice = splits > 1 ? (size_t)(item.slice * groups + item.z) * (size_t)M * (size_t)N
+                                      : (size_t)item.z * (size_t)cstride;
       const uint32_t acc = tl % NACC;
       const bool have = mbar_wait(su32(&tfull[acc]), (tl / NACC) & 1u, WAIT_POLLS);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -386,11 +417,16 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                  raw[4 * j + 3]);
         __syncwarp();
         if (c + 1 < c_end) tmem_ld32_async(tcol + 32u * (c + 1), raw);
-        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f), vk[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const int r = 4 * k + rl, grow = row0 + r;
-          float4 v = lds128(ebuf + 128u * r + (uint32_t)((jc ^ (r & 7)) << 4));
+          const int r = 4 * k + rl;
+          vk[k] = lds128(ebuf + 128u * r + (uint32_t)((jc ^ (r & 7)) << 4));
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int grow = row0 + 4 * k + rl;
+          float4 v = vk[k];
           if (OUT != OUT_DACT && extra != nullptr) {
             v.x += x[k].x;
             v.y += x[k].y;
@@ -577,14 +613,14 @@ cudaError_t run_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmCal
   const int KB = (int)((c.K + GK - 1) / GK);
   const int kbs = (KB + c.splits - 1) / c.splits;   // every slice has at least one K block
   const int splits = (KB + kbs - 1) / kbs;
-  const int64_t work = ((c.M + Tile<TN_, MW>::ROWS - 1) / Tile<TN_, MW>::ROWS) * ((c.N + TN_ - 1) / TN_) * splits *
-                       c.groups;
+  const int64_t TM = (c.M + Tile<TN_, MW>::ROWS - 1) / Tile<TN_, MW>::ROWS, TN = (c.N + TN_ - 1) / TN_;
+  const int64_t work = TM * TN * splits * c.groups;
   const unsigned grid = (unsigned)(work < sms ? work : sms);   // persistent: one CTA per SM
   constexpr size_t smem = Tile<TN_, MW>::SMEM;
   auto kern = k_gemm_bf16<OUT, TN_, OPS, MW>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, GEMM_THREADS, smem, s>>>(ta, tb, c.C, c.bias, c.act, c.group, (int)c.M, (int)c.N, (int)c.K, kbs, splits,
+  kern<<<grid, GEMM_THREADS, smem, s>>>(ta, tb, c.C, c.bias, c.act, make_work_map(TM, TN, c.group, c.groups), (int)c.M, (int)c.N, (int)c.K, kbs, splits,
                                         c.extra, c.colsum, c.groups, c.cstride, c.geo);
   return cudaGetLastError();
 }
