@@ -64,26 +64,44 @@ __device__ __forceinline__ int64_t event_of(const int64_t* __restrict__ off, int
   return lo;
 }
 
-// FP64 latency (two powers, a sine, a cosine): one-warp blocks spread the rows over the SMs
-// (4096 rows: 16 us in 32 blocks of 128 threads).
-__global__ void k_flow_targets(const double* __restrict__ theta, int64_t B, Std8 st, float* __restrict__ x) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  const double m1 = theta[b], m2 = theta[B + b];
-  const double big = fmax(m1, m2), small = fmin(m1, m2);
-  double r[8];
-  r[0] = pow(m1 * m2, 0.6) / pow(m1 + m2, 0.2);
-  r[1] = small / big;
-  r[2] = theta[4 * B + b];
-  r[3] = cos(theta[7 * B + b]);
-  r[4] = theta[9 * B + b];
-  r[5] = sin(theta[10 * B + b]);
-  r[6] = theta[8 * B + b];
-  r[7] = theta[6 * B + b];
-  float v[8];
-#pragma unroll
-  for (int p = 0; p < 8; ++p) v[p] = (float)((r[p] - st.mean[p]) / st.scale[p]);
-  store8(x + b * 8, v);
+// Four warps a block of 32 rows, one transcendental function of each row a warp: the FP64 chain of
+// a row is latency (4096 rows: 16 us with one thread a row in 32 blocks, 14.5 in 128, 7.0 now).
+constexpr int TGT_ROWS = 32;
+__global__ void __launch_bounds__(4 * TGT_ROWS) k_flow_targets(const double* __restrict__ theta, int64_t B, Std8 st,
+                                                               float* __restrict__ x) {
+  __shared__ double f[4][TGT_ROWS];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t b = (int64_t)blockIdx.x * TGT_ROWS + lane;
+  const bool in = b < B;
+  const double m1 = in ? theta[b] : 1.0, m2 = in ? theta[B + b] : 1.0;
+  if (in) {
+    double v;
+    if (w == 0) v = pow(m1 * m2, 0.6);
+    else if (w == 1) v = pow(m1 + m2, 0.2);
+    else if (w == 2) v = cos(theta[7 * B + b]);
+    else v = sin(theta[10 * B + b]);
+    f[w][lane] = v;
+  }
+  __syncthreads();
+  if (!in) return;
+  // warp w standardises coordinates 2 w and 2 w + 1
+  double r0, r1;
+  if (w == 0) {
+    r0 = f[0][lane] / f[1][lane];
+    r1 = fmin(m1, m2) / fmax(m1, m2);
+  } else if (w == 1) {
+    r0 = theta[4 * B + b];
+    r1 = f[2][lane];
+  } else if (w == 2) {
+    r0 = theta[9 * B + b];
+    r1 = f[3][lane];
+  } else {
+    r0 = theta[8 * B + b];
+    r1 = theta[6 * B + b];
+  }
+  const int p = 2 * w;
+  reinterpret_cast<float2*>(x + b * 8)[w] =
+      make_float2((float)((r0 - st.mean[p]) / st.scale[p]), (float)((r1 - st.mean[p + 1]) / st.scale[p + 1]));
 }
 
 // One thread per (row, 16-byte chunk of the row): chunk 0 holds bf16(v_a) and four
@@ -206,7 +224,7 @@ __global__ void k_flow_input_backward(int l, const float* __restrict__ dX, int C
   }
 }
 
-// The kernels of one FP64 chain a row (targets, base normals, proposal) are bound by the FP64
+// The kernels of one FP64 chain a row (base normals, proposal) are bound by the FP64
 // pipe, a warp instruction 16 cycles of it: what counts is that every SM gets the same number
 // of warps.  One warp a block: 20,000 draws are at most 5 warps on an SM where blocks of 128
 // were 8 (157 blocks on 152 SMs); base normals one (row, pair) a thread, 16.1 -> 10.3 us,
@@ -371,7 +389,7 @@ int64_t flow_layout(const gwx_flow_shape& sh, int64_t* off) {
 // ---- stage launchers ----
 cudaError_t launch_flow_targets(const double* theta, int64_t B, const double* mean8, const double* scale8, float* x,
                                 cudaStream_t s) {
-  k_flow_targets<<<blocks(B, ROW_NT), ROW_NT, 0, s>>>(theta, B, make_std(mean8, scale8), x);
+  k_flow_targets<<<blocks(B, TGT_ROWS), 4 * TGT_ROWS, 0, s>>>(theta, B, make_std(mean8, scale8), x);
   return cudaGetLastError();
 }
 
