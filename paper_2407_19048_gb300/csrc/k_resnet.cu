@@ -15,6 +15,7 @@
 #include <cuda_bf16.h>
 
 #include "gwx_internal.h"
+#include "sum2.cuh"
 
 namespace gwx {
 
@@ -59,6 +60,29 @@ __global__ void k_im2col_cf(const float* __restrict__ y, int D, int N, int k, in
     if (src >= 0 && src < N) v = y[(b * D + c) * N + src];
   }
   cols[(b * To + t) * K + col] = __float2bfloat16_rn(v);
+}
+
+// The same, 8 columns (16 bytes) a thread (one column: 34 us for 512 windows of 2 x 2048 samples,
+// 7 taps; now 11).
+__global__ void k_im2col_cf8(const float* __restrict__ y, int D, int N, int k, int s, int p, int To, int K,
+                             __nv_bfloat16* __restrict__ cols) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int ch = K / 8;
+  if (i >= To * ch) return;
+  const int64_t b = blockIdx.y;
+  const int t = i / ch, q = i - t * ch;
+  int j = 8 * q / D, c = 8 * q - j * D;
+  float v[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const int src = s * t + j - p;
+    v[e] = j < k && src >= 0 && src < N ? __ldg(y + (b * D + c) * N + src) : 0.f;
+    if (++c == D) c = 0, ++j;
+  }
+  __align__(16) __nv_bfloat162 h[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) h[e] = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
+  reinterpret_cast<uint4*>(cols + (b * To + t) * K)[q] = *reinterpret_cast<const uint4*>(h);
 }
 
 // dx[b][t][c] = (addend) + sum over taps j with s t_out = t + p - j of dcols[b, t_out][j C + c]
@@ -179,34 +203,10 @@ __global__ void __launch_bounds__(256) k_gn_stats(const float* __restrict__ z, i
 // Sums: thread (run slice s, row lane l, column quad q) reads runs of 16 rows, rl = 256 / (C / 4)
 // rows apart, of channels 4 q .. 4 q + 3, coalesced float4 loads; FP32 within a run (the
 // contractions spelled out: the compiler's choice changes with the code around), two-float sums
-// across runs; then the lanes of each column quad and the quads of each group.
+// across runs (sum2.cuh; in FP64 forward 227 us, backward 510); then the lanes of each column quad and the quads of each group.
 constexpr int GN_NT = 512;
 // threads of the backward: the pooled gradient's rows hold twice the registers
 constexpr int gn_bt(int src) { return src == 2 ? 256 : 512; }
-
-// Sums across runs, lanes and warps: a value and the rounding errors of its additions (Knuth's
-// two-sum), about 48 bits.  Six FP32 additions a term; an FP64 addition holds the SM's FP64
-// pipe for 16 cycles a warp (forward 227 -> 203 us, backward 510 -> 467 for the above).
-struct Sum2 {
-  float h = 0.f, l = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float t = __fadd_rn(h, x), z = __fsub_rn(t, h);
-    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(t, z)), __fsub_rn(x, z)));
-    h = t;
-  }
-  __device__ __forceinline__ void add(const Sum2& o) {
-    add(o.h);
-    l = __fadd_rn(l, o.l);
-  }
-  __device__ __forceinline__ void add_lanes(int o) {
-    Sum2 x;
-    x.h = __shfl_xor_sync(0xffffffffu, h, o);
-    x.l = __shfl_xor_sync(0xffffffffu, l, o);
-    add(x);
-  }
-  // (an infinite sum's error is not a number)
-  __device__ __forceinline__ double value() const { return isfinite(h) ? (double)h + (double)l : (double)h; }
-};
 
 // Sums of a (and q) over the threads of every group (out[2 g], out[2 g + 1], valid after the
 // caller's barrier): lanes of a warp that share a column quad by shuffles, the remaining rows
@@ -885,6 +885,32 @@ __global__ void k_mean_time(const __nv_bfloat16* __restrict__ x, int64_t B, int 
   m[i] = __float2bfloat16_rn(acc / T);
 }
 
+// The same, two channels a thread and 32 loads in flight (512 windows of 256 x 128: 25.4 us with one
+// channel and 16 loads, now 12.7).
+__global__ void k_mean_time2(const __nv_bfloat16* __restrict__ x, int64_t B, int T, int C,
+                             __nv_bfloat16* __restrict__ m) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int h = C / 2;
+  if (i >= B * h) return;
+  const int64_t b = i / h;
+  const uint32_t* p = reinterpret_cast<const uint32_t*>(x) + b * T * h + (i - b * h);
+  float a0 = 0.f, a1 = 0.f;
+  auto add = [&](uint32_t v) {   // a bfloat16 is the upper half of its float
+    a0 += __uint_as_float(v << 16);
+    a1 += __uint_as_float(v & 0xffff0000u);
+  };
+  int t = 0;
+  for (; t + 32 <= T; t += 32) {
+    uint32_t v[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) v[k] = __ldg(p + (t + k) * h);
+#pragma unroll
+    for (int k = 0; k < 32; ++k) add(v[k]);
+  }
+  for (; t < T; ++t) add(__ldg(p + t * h));
+  reinterpret_cast<__nv_bfloat162*>(m)[i] = __floats2bfloat162_rn(a0 / T, a1 / T);
+}
+
 __global__ void k_mean_time_back(const float* __restrict__ dm, int T, int C, float* __restrict__ dx) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= T * C) return;
@@ -910,8 +936,12 @@ cudaError_t launch_im2col(const void* x, int64_t B, int T, int C, int k, int s, 
 cudaError_t launch_im2col_cf(const float* y, int64_t B, int D, int N, int k, int s, int p, int K, void* cols,
                              cudaStream_t st) {
   const int To = (N + 2 * p - k) / s + 1;
-  k_im2col_cf<<<dim3(nblk((int64_t)To * K, 256), (unsigned)B), 256, 0, st>>>(y, D, N, k, s, p, To, K,
-                                                                             reinterpret_cast<__nv_bfloat16*>(cols));
+  if (K % 8 == 0 && aligned16(cols))
+    k_im2col_cf8<<<dim3(nblk((int64_t)To * (K / 8), 256), (unsigned)B), 256, 0, st>>>(
+        y, D, N, k, s, p, To, K, reinterpret_cast<__nv_bfloat16*>(cols));
+  else
+    k_im2col_cf<<<dim3(nblk((int64_t)To * K, 256), (unsigned)B), 256, 0, st>>>(y, D, N, k, s, p, To, K,
+                                                                               reinterpret_cast<__nv_bfloat16*>(cols));
   return cudaGetLastError();
 }
 
@@ -1051,8 +1081,12 @@ cudaError_t launch_maxpool_back(const float* dy, const uint8_t* arg, int64_t B, 
 }
 
 cudaError_t launch_mean_time(const void* x, int64_t B, int T, int C, void* m, cudaStream_t st) {
-  k_mean_time<<<nblk(B * C, 64), 64, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(x), B, T, C,
-                                                reinterpret_cast<__nv_bfloat16*>(m));
+  const auto x16 = reinterpret_cast<const __nv_bfloat16*>(x);
+  const auto m16 = reinterpret_cast<__nv_bfloat16*>(m);
+  if (C % 2 == 0 && ((uintptr_t)x & 3u) == 0 && ((uintptr_t)m & 3u) == 0)
+    k_mean_time2<<<nblk(B * C / 2, 64), 64, 0, st>>>(x16, B, T, C, m16);
+  else
+    k_mean_time<<<nblk(B * C, 64), 64, 0, st>>>(x16, B, T, C, m16);
   return cudaGetLastError();
 }
 
