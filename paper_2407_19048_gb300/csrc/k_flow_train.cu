@@ -1,14 +1,14 @@
 // k_flow_train.cu -- the coupling flow's density direction and its backward as one persistent
 // tensor-core kernel each (the training step of Sec. 5): a CTA takes 128 rows through all K
-// coupling layers without leaving the SM, with the roles and the shared-memory and
-// tensor-memory layout of the sampling kernel (k_flow_fused.cu).
+// coupling layers without leaving the SM.
 //
-// k_flow_density applies the layers K-1 .. 0 to x.  For training it also stores what the
-// backward needs: each layer's output and conditioner output o (FP32), the conditioner's
-// input X and hidden activations g1, g2 (bfloat16, row-major, straight from the shared tiles
-// by TMA stores of 32 rows x 64 columns a warp), and the signs of g1, g2 as bits.
+// k_flow_density applies the layers K-1 .. 0 to x, with the roles of the sampling kernel
+// (flow_tile.cuh, k_flow_fused.cu).  For training it also stores what the backward needs: each
+// layer's output and conditioner output o (FP32), the conditioner's input X and hidden
+// activations g1, g2 (bfloat16, row-major, by TMA stores), and the signs of g1, g2 as bits.
 //
-// k_flow_backward undoes layer 0 first.  Per layer the rows form dL/do in registers, and
+// k_flow_backward undoes layer 0 first, eight row warps, operands in shared memory.  Per layer
+// the rows form dL/do in registers, and
 // three products run as in the forward pass, each weight matrix read as it lies (K is its
 // row index: MN-major descriptors), the ReLU masks and the FP32 column sums of every 32 rows
 // (the bias gradients' partials) in the drain between them:
@@ -19,9 +19,10 @@
 //
 // Every value is rounded where, and summed in the order that, the layer-by-layer kernels
 // do, so the results are theirs bit for bit (weight gradients: to the order of the batch
-// sum).  Latency bound: one tile's chain MMA -> drain -> MMA, ~5 us a layer; a batch of 4096
-// fills 32 SMs.  As ~370 launches of 3 to 13 us (each layer: input rows, three products,
-// coupling step; backward 17 kernels) the step took 3.04 ms.
+// sum).  Latency bound: one tile's chain MMA -> drain -> MMA, 6.4 us a layer of 256 in the
+// density with what it keeps (3.8 without; 6.9 with the operands in shared memory), 7.9 in the
+// backward; a batch of 4096 fills 32 SMs.  As ~370 launches of 3 to 13 us (each layer: input
+// rows, three products, coupling step; backward 17 kernels) the step took 3.04 ms, now 0.55.
 #include "flow_tile.cuh"
 #include "sum2.cuh"
 
@@ -31,26 +32,15 @@ namespace {
 
 using namespace flowt;
 
-constexpr size_t DENSITY_SMEM = (size_t)X_BYTES + G_BYTES + 2 * SLOT_BYTES + 1024;
+constexpr uint32_t STAGE_BYTES = 32 * 64;                // a row warp's 32 rows x 32 columns on their way out
+constexpr size_t DENSITY_SMEM = (size_t)FWD_BYTES + ROW_WARPS * STAGE_BYTES + 1024;
 constexpr size_t BACKWARD_SMEM = (size_t)KB_BYTES + G_BYTES + 2 * SLOT_BYTES + 1024;
 constexpr double LN_2PI = 1.8378770664093454835606594728112353;
 
 __device__ int g_train_status;
 
-// v_b <- (v_b - mu) e^-s with mu_j = o_j, s_j = 3 tanh(o_{4+j} / 3); returns sum_j s_j.
-template <int P>
-__device__ __forceinline__ float uncouple(float* v, const float* o) {
-  float acc = 0.f;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float s = S_MAX * tanhf(o[4 + j] / S_MAX);
-    v[Bc(P, j)] = (v[Bc(P, j)] - o[j]) * expf(-s);
-    acc += s;
-  }
-  return acc;
-}
-
-// Backward of that step with output w, given g = dL/dw and the weight of sum_s in the loss:
+// Backward of the step w_b = (v_b - mu) e^-s, mu_j = o_j, s_j = 3 tanh(o_{4+j} / 3), given
+// g = dL/dw and the weight of sum_s in the loss:
 // d = dL/do, and g becomes dL/dv_in (without the conditioner's share).
 template <int P>
 __device__ __forceinline__ void uncouple_back(const float* w, const float* o, float* g, float row_weight, float* d) {
@@ -80,15 +70,27 @@ __device__ __forceinline__ void store8(float* p, const float* v) {
   reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
 }
 
-// Signs of 32 non-negative bfloat16 values packed in 16 words (values 2 i, 2 i + 1 in word i):
-// bit i for value 2 i, bit 16 + i for value 2 i + 1, set when the value is not zero.  Adding
-// 0x7fff to a half-word in [0, 0x7fff] sets its top bit exactly when it is not zero, without
-// a carry into the other half.
-__device__ __forceinline__ uint32_t sign_bits(const uint32_t* w) {
-  uint32_t m = 0;
+// Signs of 32 columns (pairs of non-negative bfloat16 values in the fragment shape of
+// fwd_hidden) of row 16 (j / 2) + 8 (j % 2) + lane / 4, j = lane % 4: bit i for column 2 i,
+// bit 16 + i for column 2 i + 1, set when the value is not zero.  Adding 0x7fff to a half-word
+// in [0, 0x7fff] sets its top bit exactly when it is not zero, without a carry into the other.
+__device__ __forceinline__ uint32_t sign_bits(const uint32_t w[2][8]) {
+  const int j = threadIdx.x & 3;
+  uint32_t own = 0;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) m = (m >> 1) | (((w[i] & 0x7fff7fffu) + 0x7fff7fffu) & 0x80008000u);
-  return m;
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      uint32_t m = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        m |= ((((w[k][2 * i + e] & 0x7fff7fffu) + 0x7fff7fffu) & 0x80008000u) >> 15) << (4 * i);
+      m <<= j;
+      m |= __shfl_xor_sync(0xffffffffu, m, 1);
+      m |= __shfl_xor_sync(0xffffffffu, m, 2);
+      if (j == 2 * k + e) own = m;
+    }
+  return own;
 }
 __device__ __forceinline__ bool sign_of(uint32_t m, int col) { return (m >> ((col >> 1) + 16 * (col & 1))) & 1u; }
 
@@ -121,14 +123,19 @@ struct DensityArgs {
   float* z_out;                   // [n][8] (density only; may be x)
   float* ss_out;                  // [n]    (density only)
   // training (save): layer l's output at xs + l n 8, conditioner output at o + l n 8, sign
-  // bits of g1, g2 [K][n][H / 64], FP64 sums of the loss over every 32 rows
+  // bits of g1, g2 (mask_at), FP64 sums of the loss over every 32 rows
   int save;
   float* xs;
   float* o;
-  uint2* m1;
-  uint2* m2;
+  uint32_t* m1;
+  uint32_t* m2;
   double* loss_part;
 };
+
+// Word of rows 32 p .. (one a row) and columns 32 c .. of layer l among the sign bits, [K][P][H / 32][32].
+__device__ __forceinline__ int64_t mask_at(int l, int64_t p, int64_t P, int chunks, int c) {
+  return ((l * P + p) * chunks + c) * 32;
+}
 
 // Barriers, tensor memory and the weight ring of both kernels.
 struct Ring {
@@ -169,172 +176,44 @@ __device__ __forceinline__ void arrive_rows(uint64_t* bar) {
   if ((threadIdx.x & 31) == 0) mbar_arrive(su32(bar));
 }
 
-// The three products of the forward conditioner of one layer (as in k_flow_fused.cu).
-__global__ void __launch_bounds__(F_THREADS, 1)
+// As the sampling kernel with the layers the other way round and the coupling step undone; for
+// training also what the backward needs goes out: the hidden activations by way of 2 KiB a row
+// warp (the next product reads them from tensor memory, so that the stores are off its path).
+__global__ void __launch_bounds__(FWD_THREADS, 1)
     k_flow_density(const __grid_constant__ CUtensorMap mv1, const __grid_constant__ CUtensorMap mv2,
                    const __grid_constant__ CUtensorMap mv3, const __grid_constant__ CUtensorMap sx_map,
                    const __grid_constant__ CUtensorMap s1_map, const __grid_constant__ CUtensorMap s2_map,
                    DensityArgs a) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) Ring rg;
-  __shared__ uint32_t tmem_slot;
-  __shared__ int abort_flag;
+  __shared__ __align__(16) FwdRing rg;
+  __shared__ float s_o[8][FM];                                 // the rows' conditioner outputs
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t base = (su32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t sx = base, sg = base + X_BYTES, sw = base + X_BYTES + G_BYTES;
-  const int H = a.H, K = a.K, C = a.C;
-  const int NR = H / 128, NP = 2 + NR;                     // 128-column parts and rounds; weight parts per layer
+  const uint32_t sx = base, sw = base + X_BYTES;
+  const int K = a.K, C = a.C, H = a.H, NR = H / 128;           // 128-column rounds of the hidden layers
   const int tiles = (int)((a.n + FM - 1) / FM);
-  const uint32_t id_128 = idesc_bf16(FM, 128), id_16 = idesc_bf16(FM, 16);
-
-  if (threadIdx.x == 0) ring_init(&rg, &abort_flag);
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_slot)),
-                 "r"(512)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_slot;
+  const FwdWeights wt{&mv1, &mv2, &mv3, a.e1, a.e2, a.e3, a.lstride, C, H, K, tiles, true};
+  const uint32_t tmem = fwd_begin(rg);
 
   if (warp == 0) {
-    uint32_t it = 0;
-    bool ok = true;
-    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
-      for (int l = K - 1; l >= 0 && ok; --l)
-        for (int p = 0; p < NP; ++p, ++it) {
-          const uint32_t s = it & 1u;
-          if (!mbar_wait_warp(su32(&rg.empty[s]), ((it >> 1) & 1u) ^ 1u, F_WAIT) ||
-              __any_sync(0xffffffffu, *(volatile int*)&abort_flag)) {
-            ok = false;
-            break;
-          }
-          const uint32_t dst = sw + s * SLOT_BYTES, bar = su32(&rg.full[s]);
-          if (elect_one()) {
-            if (p == NP - 1) {
-              mbar_expect_tx(bar, (uint32_t)H * 32u);
-              for (int kb = 0; kb < H / 64; ++kb) tma_load_3d(dst + 2048u * kb, &mv3, 64 * kb, 0, l, bar);
-            } else {
-              const CUtensorMap* m = p == 0 ? &mv1 : &mv2;
-              const int kb0 = p == 0 ? 0 : 2 * (p - 1);
-              mbar_expect_tx(bar, (uint32_t)H * 256u);
-              tma_load_3d(dst, m, 64 * kb0, 0, l, bar);
-              tma_load_3d(dst + (uint32_t)H * 128u, m, 64 * (kb0 + 1), 0, l, bar);
-            }
-          }
-          __syncwarp();
-        }
-    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
+    fwd_produce(rg, wt, sw);
   } else if (warp == 1) {
-    uint32_t it = 0, li = 0;
-    bool ok = true;
-    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x)
-      for (int l = K - 1; l >= 0 && ok; --l, ++li) {
-        // acc1 = X V1^T, one 128-column part at a time
-        uint32_t slot = it & 1u, wb = sw + slot * SLOT_BYTES;
-        if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u) && wait_mma(&rg.in_ready, li & 1u))) break;
-        if (elect_one()) {
-          for (int np = 0; np < NR; ++np) {
-#pragma unroll
-            for (int kk = 0; kk < 8; ++kk)
-              mma_bf16(tmem + 128u * np, sw128_desc(sx + KB_BYTES * (kk >> 2) + 32u * (kk & 3)),
-                       sw128_desc(wb + (uint32_t)H * 128u * (kk >> 2) + 16384u * np + 32u * (kk & 3)), id_128, kk != 0);
-            mma_commit(su32(&rg.acc1f[np]));
-          }
-          mma_commit(su32(&rg.empty[slot]));
-        }
-        __syncwarp();
-        ++it;
-        // acc2 = g1 V2^T: K round pr (g1 columns 128 pr ..) once the rows have written it
-        for (int pr = 0; pr < NR; ++pr) {
-          slot = it & 1u, wb = sw + slot * SLOT_BYTES;
-          if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u) && wait_mma(&rg.gready[pr], 0u))) break;
-          if (elect_one()) {
-            for (int np = 0; np < NR; ++np) {
-#pragma unroll
-              for (int kk = 0; kk < 8; ++kk)
-                mma_bf16(tmem + 256u + 128u * np, sw128_desc(sg + KB_BYTES * (2 * pr + (kk >> 2)) + 32u * (kk & 3)),
-                         sw128_desc(wb + (uint32_t)H * 128u * (kk >> 2) + 16384u * np + 32u * (kk & 3)), id_128,
-                         (pr | kk) != 0);
-              if (pr == NR - 1) mma_commit(su32(&rg.acc2f[np]));
-            }
-            mma_commit(su32(&rg.empty[slot]));
-          }
-          __syncwarp();
-          ++it;
-        }
-        if (!ok) break;
-        // acc3 = g2 V3^T (16 rows, 8 of them the conditioner's outputs)
-        slot = it & 1u, wb = sw + slot * SLOT_BYTES;
-        if (!(ok = wait_mma(&rg.full[slot], (it >> 1) & 1u))) break;
-        for (int r = 0; r < NR; ++r) {
-          if (!(ok = wait_mma(&rg.gready[r], 1u))) break;
-          if (elect_one()) {
-#pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-              const int kb = 2 * r + (kk >> 2);
-              mma_bf16(tmem, sw128_desc(sg + KB_BYTES * kb + 32u * (kk & 3)), sw128_desc(wb + 2048u * kb + 32u * (kk & 3)),
-                       id_16, (r | kk) != 0);
-            }
-            if (r == NR - 1) {
-              mma_commit(su32(&rg.acc3f));
-              mma_commit(su32(&rg.empty[slot]));
-            }
-          }
-          __syncwarp();
-        }
-        ++it;
-      }
-    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
+    fwd_multiply(rg, wt, tmem, sx, sw);
   } else {
     const int q = warp & 3;
-    const int h = (warp - 2) >> 2;                             // which half of the columns
+    const int h = (warp - 2) >> 2;                             // which 32 of every 128 columns
     const int r = 32 * q + lane;                               // row of the tile = tensor-memory lane
     const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16);
+    const uint32_t stage = base + FWD_BYTES + (uint32_t)(warp - 2) * STAGE_BYTES;
     uint32_t li = 0;
     bool ok = true;
-    auto load_bias = [&](const float* bias, int c, float4* bb) {
-      const float4* b4 = reinterpret_cast<const float4*>(bias + 64 * c);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) bb[i] = __ldg(b4 + i);
-    };
-    // bias + ReLU of 64 accumulator columns (chunk c) into K-block c; returns their sign bits
-    auto hidden = [&](uint32_t col0, const float4* bb, int c) -> uint2 {
-      uint32_t raw[2][32];
-      uint32_t bits[2];
-      tmem_ld32_async(lane_addr + col0 + 64u * c, raw[0]);
-      tmem_ld32_async(lane_addr + col0 + 64u * c + 32u, raw[1]);
-      tmem_wait_ld();
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        uint32_t w[16];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float4 b = bb[8 * hh + i];
-          w[2 * i] = pack2(fmaxf(__uint_as_float(raw[hh][4 * i]) + b.x, 0.f),
-                           fmaxf(__uint_as_float(raw[hh][4 * i + 1]) + b.y, 0.f));
-          w[2 * i + 1] = pack2(fmaxf(__uint_as_float(raw[hh][4 * i + 2]) + b.z, 0.f),
-                               fmaxf(__uint_as_float(raw[hh][4 * i + 3]) + b.w, 0.f));
-        }
-#pragma unroll
-        for (int t4 = 0; t4 < 4; ++t4) {
-          const int col = 64 * c + 32 * hh + 8 * t4;
-          sts128(sg + KB_BYTES * (col >> 6) + swz(r, (col & 63) >> 3), w[4 * t4], w[4 * t4 + 1], w[4 * t4 + 2],
-                 w[4 * t4 + 3]);
-        }
-        bits[hh] = sign_bits(w);
-      }
-      return make_uint2(bits[0], bits[1]);
-    };
     for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
       const int64_t row = (int64_t)t * FM + r;
       const int wrow = t * FM + 32 * q;                        // first row of this warp
       const bool valid = row < a.n;
       const bool save = a.save != 0 && wrow < a.n;             // uniform over the warp
       float v[8], ss = 0.f;
-      if (valid && h == 0) {
+      if (valid) {
         load8(a.x + row * 8, v);
       } else {
 #pragma unroll
@@ -350,84 +229,107 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         }
         e = lo;
       }
-      if (a.save != 0) {                                       // the last tile's stores have read the input rows
+      const uint4* crow = reinterpret_cast<const uint4*>(a.ctx + e * C);
+      for (int g = h == 0 ? 1 : 4 * h; g < 4 * h + 4; ++g) {
+        uint4 x = make_uint4(0u, 0u, 0u, 0u);
+        if (valid && g <= C / 8) x = __ldg(crow + (g - 1));
+        sts128(sx + KB_BYTES * (g >> 3) + swz(r, g & 7), x.x, x.y, x.z, x.w);
+      }
+      // chunk c (32 columns) of a hidden layer: signs and activations out, when the chunk before has
+      // left this warp's buffer (4096 rows, 16 layers: 102 us; 125 with plain 16-byte stores, 109
+      // with signs and rows by bulk copies as well; 61 of it the chain, the rest what is kept).
+      auto keep = [&](const uint32_t w[2][8], int c, int l, const CUtensorMap* map, uint32_t* masks) {
+        const uint32_t bits = sign_bits(w);
         if (lane == 0) tma_store_wait_read();
         __syncwarp();
-      }
-      const uint4* crow = reinterpret_cast<const uint4*>(a.ctx + e * C);
-      for (int g = h == 0 ? 1 : 8; g < (h == 0 ? 8 : 16); ++g) {
-        uint4 d = make_uint4(0u, 0u, 0u, 0u);
-        if (valid && g <= C / 8) d = __ldg(crow + (g - 1));
-        sts128(sx + KB_BYTES * (g >> 3) + swz(r, g & 7), d.x, d.y, d.z, d.w);
-      }
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int rr = 16 * k + 8 * (i & 1) + (lane >> 2);
+            sts32(stage + 64u * rr + (uint32_t)((((i >> 1) ^ (rr >> 1)) & 3) << 4) + 4u * (lane & 3), w[k][i]);
+          }
+        proxy_fence();
+        __syncwarp();
+        if (lane == 0) tma_store_3d(map, stage, 32 * c, wrow, l);
+        const int rj = 16 * ((lane & 3) >> 1) + 8 * (lane & 1) + (lane >> 2);
+        masks[mask_at(l, wrow / 32, (a.n + 31) / 32, H / 32, c) + rj] = bits;
+      };
+      uint32_t w[2][2][8];                                     // this warp's chunks of a hidden layer
       for (int l = K - 1; l >= 0; --l, ++li) {
         const int p = l & 3;
-        if (save && lane == 0) tma_store_wait_read();
-        __syncwarp();
         if (h == 0) {
           uint32_t w0, w1;
-          switch (p) {
-            case 0: pack_half<0>(v, w0, w1); break;
-            case 1: pack_half<1>(v, w0, w1); break;
-            case 2: pack_half<2>(v, w0, w1); break;
-            default: pack_half<3>(v, w0, w1); break;
-          }
+          pack_half(p, v, w0, w1);
           sts128(sx + swz(r, 0), w0, w1, 0u, 0u);
         }
-        arrive_rows(&rg.in_ready);
-        if (save && lane == 0 && (h == 0 || 8 + C > 64))
-          tma_store_3d(&sx_map, sx + KB_BYTES * h + 4096u * q, 64 * h, wrow, l);
-        for (int rd = 0; rd < NR && ok; ++rd) {
-          float4 bb[16];
-          load_bias(a.e1 + l * a.lstride, 2 * rd + h, bb);
-          if (!(ok = wait_rows(&rg.acc1f[rd], li & 1u, &abort_flag))) break;
-          const int c = 2 * rd + h;
-          const uint2 m = hidden(0u, bb, c);
-          arrive_rows(&rg.gready[rd]);
-          if (save) {
-            if (lane == 0) tma_store_3d(&s1_map, sg + KB_BYTES * c + 4096u * q, 64 * c, wrow, l);
-            if (valid) a.m1[((int64_t)l * a.n + row) * (H / 64) + c] = m;
-          }
-        }
-        for (int rd = 0; rd < NR && ok; ++rd) {
-          float4 bb[16];
-          load_bias(a.e2 + l * a.lstride, 2 * rd + h, bb);
-          if (!(ok = wait_rows(&rg.acc2f[rd], li & 1u, &abort_flag))) break;
-          const int c = 2 * rd + h;
-          if (save) {                                          // g1's stores have read the tile
-            if (lane == 0) tma_store_wait_read();
-            __syncwarp();
-          }
-          const uint2 m = hidden(256u, bb, c);
-          arrive_rows(&rg.gready[rd]);
-          if (save) {
-            if (lane == 0) tma_store_3d(&s2_map, sg + KB_BYTES * c + 4096u * q, 64 * c, wrow, l);
-            if (valid) a.m2[((int64_t)l * a.n + row) * (H / 64) + c] = m;
-          }
-        }
-        if (!ok) break;
-        if (h != 0) continue;                                  // the coupling step is the first warp's
-        float b3[8];
-        load8(a.e3 + l * a.lstride, b3);
-        if (!(ok = wait_rows(&rg.acc3f, li & 1u, &abort_flag))) break;
-        float o[16];
-        tmem_ld16(lane_addr, o);
+        proxy_fence();
+        row_arrive(&rg.xready);
+        // what goes out does so while the tensor core works, a chunk at a time with a pause for the
+        // buffer: the second chunk of the last layer's g2 here, g1 and the first of g2 below
+        if (save && l < K - 1 && NR > 1) keep(w[1], 4 + h, l + 1, &s2_map, a.m2);
+        const float* bl = rg.sb[li & 1u];
+        if (!(ok = row_wait(&rg.biasf[li & 1u], (li >> 1) & 1u) && !*(volatile int*)&rg.abort_flag)) break;
+        if (!(ok = row_wait(&rg.acc1f, li & 1u))) break;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) o[j] += b3[j];
-        float sl;
-        switch (p) {
-          case 0: sl = uncouple<0>(v, o); break;
-          case 1: sl = uncouple<1>(v, o); break;
-          case 2: sl = uncouple<2>(v, o); break;
-          default: sl = uncouple<3>(v, o); break;
+        for (int rd = 0; rd < 2; ++rd) {
+          if (rd >= NR) break;
+          const int c = 4 * rd + h;
+          fwd_hidden(lane_addr + 32u * c, bl + 32 * c, w[rd]);
+          row_arrive(&rg.gready[rd]);
         }
+        if (save) {
+          keep(w[0], h, l, &s1_map, a.m1);
+          if (NR > 1) keep(w[1], 4 + h, l, &s1_map, a.m1);
+        }
+        // the input rows (all four warps' columns: acc1 followed their arrivals)
+        if (save && lane == 0 && (h == 0 || (h == 1 && 8 + C > 64)))
+          tma_store_3d(&sx_map, sx + KB_BYTES * h + 4096u * q, 64 * h, wrow, l);
+        if (!(ok = row_wait(&rg.acc2f, li & 1u))) break;
+#pragma unroll
+        for (int rd = 0; rd < 2; ++rd) {
+          if (rd >= NR) break;
+          const int c = 4 * rd + h;
+          fwd_hidden(lane_addr + ACC2 + 32u * c, bl + 256 + 32 * c, w[rd]);
+          row_arrive(&rg.gready[rd]);
+        }
+        if (save) keep(w[0], h, l, &s2_map, a.m2);
+        // v_b <- (v_b - mu) e^-s with mu_j = o_j, s_j = 3 tanh(o_{4+j} / 3): coordinate j by warp
+        // h = j of the quarter, handed to the others in shared memory
+        if (!(ok = row_wait(&rg.acc3f, li & 1u))) break;
+        uint32_t om = tmem_ld1_async(lane_addr + ACC3 + h), os = tmem_ld1_async(lane_addr + ACC3 + 4u + h);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(om), "+r"(os)::"memory");
+        const float mu = __uint_as_float(om) + bl[512 + h], ol = __uint_as_float(os) + bl[512 + 4 + h];
+        const float s = S_MAX * tanhf(ol / S_MAX);
+        rg.s_new[h][r] = (half_at(p, v, h) - mu) * expf(-s);
+        rg.s_log[h][r] = s;
+        if (save) {
+          s_o[h][r] = mu;
+          s_o[4 + h][r] = ol;
+          // the input rows have been read before the quarter may write new ones
+          if (lane == 0) tma_store_wait_read();
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(su32(&rg.cplf[q]));
+        if (!(ok = row_wait(&rg.cplf[q], li & 1u))) break;
+        float x[4], sl = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          x[j] = rg.s_new[j][r];
+          sl += rg.s_log[j][r];
+        }
+        set_half(p, v, x);
         ss = l == K - 1 ? sl : ss + sl;
-        if (save && valid) {
+        if (save && valid && h == 0) store8(a.xs + ((int64_t)l * a.n + row) * 8, v);
+        if (save && valid && h == 1) {
+          float o[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) o[j] = s_o[j][r];
           store8(a.o + ((int64_t)l * a.n + row) * 8, o);
-          store8(a.xs + ((int64_t)l * a.n + row) * 8, v);
         }
       }
       if (!ok) break;
+      if (save && NR > 1) keep(w[1], 4 + h, 0, &s2_map, a.m2);
       if (h != 0) continue;
       if (a.save == 0) {
         if (valid) {
@@ -449,21 +351,16 @@ __global__ void __launch_bounds__(F_THREADS, 1)
       }
     }
     if (a.save != 0 && lane == 0) tma_store_wait();            // before the shared tiles go away
-    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
+    if (!ok && lane == 0) atomicExch(&rg.abort_flag, 1);
   }
-  __syncwarp();
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (threadIdx.x == 0 && *(volatile int*)&abort_flag) atomicExch(&g_train_status, 1);
-  if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  fwd_end(rg, tmem, &g_train_status);
 }
 
 struct BackwardArgs {
   const float* xs;                // [K][n][8] layer outputs (xs[0] = z)
   const float* o;                 // [K][n][8]
-  const uint2* m1;                // [K][n][H / 64] sign bits of g1, g2
-  const uint2* m2;
+  const uint32_t* m1;             // sign bits of g1, g2 (mask_at)
+  const uint32_t* m2;
   int64_t n;
   int C, H, K;
   float inv_n;
@@ -655,8 +552,9 @@ __global__ void __launch_bounds__(F_THREADS, 1)
 #pragma unroll
         for (int rd = 0; rd < 2; ++rd) {
           const bool have = valid && rd < NR;
-          k2[rd] = have ? __ldg(&a.m2[at * (H / 64) + 2 * rd + h]) : make_uint2(0u, 0u);
-          k1[rd] = have ? __ldg(&a.m1[at * (H / 64) + 2 * rd + h]) : make_uint2(0u, 0u);
+          const int64_t m = mask_at(l, wrow / 32, a.P, H / 32, 2 * (2 * rd + h)) + lane;
+          k2[rd] = have ? make_uint2(__ldg(&a.m2[m]), __ldg(&a.m2[m + 32])) : make_uint2(0u, 0u);
+          k1[rd] = have ? make_uint2(__ldg(&a.m1[m]), __ldg(&a.m1[m + 32])) : make_uint2(0u, 0u);
         }
         if (h == 0) {
           float d[8];
@@ -827,8 +725,8 @@ cudaError_t run_density(const void* params_bf16, const float* params, const int6
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_flow_density, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSITY_SMEM);
   if (e != cudaSuccess) return e;
-  k_flow_density<<<grid, F_THREADS, DENSITY_SMEM, s>>>(m1, m2, m3, stores ? stores[0] : m1, stores ? stores[1] : m1,
-                                                       stores ? stores[2] : m1, a);
+  k_flow_density<<<grid, FWD_THREADS, DENSITY_SMEM, s>>>(m1, m2, m3, stores ? stores[0] : m1, stores ? stores[1] : m1,
+                                                         stores ? stores[2] : m1, a);
   return cudaGetLastError();
 }
 
@@ -873,8 +771,8 @@ FlowTrainBufs flow_train_bufs(int64_t n, int C, int H, int K, void* base, size_t
   f.dz1 = take(Kn * H * 2);
   f.dz2 = take(Kn * H * 2);
   f.dO = take(Kn * 8 * 2);
-  f.m1 = take(Kn * (H / 64) * 8);
-  f.m2 = take(Kn * (H / 64) * 8);
+  f.m1 = take(K * P * H * 4);
+  f.m2 = take(K * P * H * 4);
   f.o = reinterpret_cast<float*>(take(Kn * 8 * 4));
   f.p1 = reinterpret_cast<float*>(take(K * P * H * 4));
   f.p2 = reinterpret_cast<float*>(take(K * P * H * 4));
@@ -895,8 +793,8 @@ cudaError_t launch_flow_train_fused(const void* params_bf16, const float* params
   const int64_t lstride = K > 1 ? off_t[12] - off_t[6] : 64;
   // forward, with what the backward needs
   CUtensorMap st[3], b1, b2, w1, w2, w3;
-  if (!layer_map(&st[0], f.X, 8 + C, n, K, n * (8 + C), 32u) || !layer_map(&st[1], f.g1, H, n, K, n * H, 32u) ||
-      !layer_map(&st[2], f.g2, H, n, K, n * H, 32u) || !layer_map(&b1, f.dz1, H, n, K, n * H, 32u) ||
+  if (!layer_map(&st[0], f.X, 8 + C, n, K, n * (8 + C), 32u) || !layer_map(&st[1], f.g1, H, n, K, n * H, 32u, 32u) ||
+      !layer_map(&st[2], f.g2, H, n, K, n * H, 32u, 32u) || !layer_map(&b1, f.dz1, H, n, K, n * H, 32u) ||
       !layer_map(&b2, f.dz2, H, n, K, n * H, 32u) ||
       !layer_map(&w1, p16 + off_t[6], 8 + C, H, K, lstride, (uint32_t)H) ||
       !layer_map(&w2, p16 + off_t[8], H, H, K, lstride, 128u) || !layer_map(&w3, p16 + off_t[10], H, 8, K, lstride, 16u))
@@ -911,8 +809,8 @@ cudaError_t launch_flow_train_fused(const void* params_bf16, const float* params
   a.save = 1;
   a.xs = xs;
   a.o = f.o;
-  a.m1 = reinterpret_cast<uint2*>(f.m1);
-  a.m2 = reinterpret_cast<uint2*>(f.m2);
+  a.m1 = reinterpret_cast<uint32_t*>(f.m1);
+  a.m2 = reinterpret_cast<uint32_t*>(f.m2);
   a.loss_part = f.loss_part;
   cudaError_t e = run_density(params_bf16, params, off_t, a, st, s);
   if (e != cudaSuccess) return e;
