@@ -162,6 +162,8 @@ cudaError_t launch_features(const float* y, int64_t B, int D, int64_t N, int k_l
                             void* out, cudaStream_t s);
 // Cross-spectral columns (k_cross_features) from a spectrum Y complex [B][D][N/2+1] that
 // launch_features left in its workspace, or from y (rfft into ws first).
+cudaError_t launch_spectral_columns(const float* y, int64_t B, int D, int64_t N, int k_lo, int G, int F_pad, bool cross,
+                                    bool lag, void* ws, void* out, cudaStream_t s);
 cudaError_t launch_cross_from_spectrum(const void* Y, int64_t B, int D, int64_t N, int k_lo, int G, int F_pad,
                                        int col0, void* out, cudaStream_t s);
 cudaError_t launch_cross_features(const float* y, int64_t B, int D, int64_t N, int k_lo, int G, int F_pad, int col0,

@@ -468,14 +468,8 @@ Params make_params(const gwx_flow_shape& sh, const float* p, const void* p16) {
 cudaError_t embed_forward(const FlowDims& d, const Params& P, const float* y, int64_t R, int D, int64_t N, int k_lo,
                           void* fws, __nv_bfloat16* feat, __nv_bfloat16* h1, __nv_bfloat16* h2, __nv_bfloat16* ctx,
                           cudaStream_t s) {
-  FL_TRY(launch_features(y, R, D, N, k_lo, (int)d.G, (int)d.F, fws, feat, s));
-  const int ng = (int)((N / 2 - k_lo) / d.G);
-  int col = D * ng;
-  if (d.extra & GWX_FLOW_CROSS) {
-    FL_TRY(launch_cross_from_spectrum(fws, R, D, N, k_lo, (int)d.G, (int)d.F, col, feat, s));
-    col += D * (D - 1) * ng;
-  }
-  if (d.extra & GWX_FLOW_LAG) FL_TRY(launch_lag_from_spectrum(fws, R, D, N, k_lo, (int)d.G, (int)d.F, col, feat, s));
+  FL_TRY(launch_spectral_columns(y, R, D, N, k_lo, (int)d.G, (int)d.F, (d.extra & GWX_FLOW_CROSS) != 0,
+                                 (d.extra & GWX_FLOW_LAG) != 0, fws, feat, s));
   FL_TRY(launch_gemm_bf16(feat, P.W(0), h1, R, d.He, d.F, true, P.b(1), GWX_ACT_RELU, 0, s));
   FL_TRY(launch_gemm_bf16(h1, P.W(2), h2, R, d.He, d.He, true, P.b(3), GWX_ACT_RELU, 0, s));
   return launch_gemm_bf16(h2, P.W(4), ctx, R, d.C, d.He, true, P.b(5), GWX_ACT_NONE, 0, s);

@@ -98,6 +98,81 @@ __global__ void k_lag_features(const float2* __restrict__ Y, int D, int64_t F, i
   row[(2 * d + 1) * ng + g] = __float2bfloat16_rn(im * inv);
 }
 
+// All columns of a row in one pass over its spectra: log powers, then the cross spectra of every
+// pair (cross), then the lag-one products (lag), zeros up to F_pad; the sums and columns of the
+// three kernels above (whose norms are this one's powers).  HBM bound: a thread takes one
+// group of every detector; block (b, chunk of 128 groups).  (4096 windows of 2 x 2048 samples: 56
+// us as three kernels, each reading the spectra, 16 now; one window 8.7 us, 3.5 now.)
+constexpr int SC_NT = 128;
+template <int D>
+__global__ void __launch_bounds__(SC_NT) k_spectral_columns(const float2* __restrict__ Y, int64_t F, int N, int k_lo,
+                                                            int G, int ng, int chunks, int F_pad, bool cross, bool lag,
+                                                            __nv_bfloat16* __restrict__ out) {
+  constexpr int P = D * (D - 1) / 2;
+  const int64_t b = blockIdx.x / chunks;
+  const int chunk = (int)(blockIdx.x - b * chunks);
+  const int g = chunk * SC_NT + threadIdx.x;
+  __nv_bfloat16* row = out + b * F_pad;
+  const int col_c = D * ng, col_l = col_c + (cross ? 2 * P * ng : 0), end = col_l + (lag ? 2 * D * ng : 0);
+  if (chunk == 0)
+    for (int c = end + threadIdx.x; c < F_pad; c += SC_NT) row[c] = __float2bfloat16_rn(0.f);
+  if (g >= ng) return;
+  const float2* y = Y + b * D * F + k_lo + (int64_t)g * G;
+  float pw[D], nb[D], lre[D], lim[D], cre[P > 0 ? P : 1], cim[P > 0 ? P : 1];
+  float2 u[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    pw[d] = nb[d] = lre[d] = lim[d] = 0.f;
+    u[d] = __ldg(y + d * F);
+  }
+#pragma unroll
+  for (int p = 0; p < P; ++p) cre[p] = cim[p] = 0.f;
+#pragma unroll 4
+  for (int k = 0; k < G; ++k) {
+    float2 v[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) v[d] = lag || k + 1 < G ? __ldg(y + d * F + k + 1) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      pw[d] = fmaf(u[d].x, u[d].x, fmaf(u[d].y, u[d].y, pw[d]));
+      lre[d] = fmaf(u[d].x, v[d].x, fmaf(u[d].y, v[d].y, lre[d]));
+      lim[d] = fmaf(u[d].y, v[d].x, fmaf(-u[d].x, v[d].y, lim[d]));
+      nb[d] = fmaf(v[d].x, v[d].x, fmaf(v[d].y, v[d].y, nb[d]));
+    }
+    int p = 0;
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+#pragma unroll
+      for (int c = a + 1; c < D; ++c, ++p) {
+        cre[p] = fmaf(u[a].x, u[c].x, fmaf(u[a].y, u[c].y, cre[p]));
+        cim[p] = fmaf(u[a].y, u[c].x, fmaf(-u[a].x, u[c].y, cim[p]));
+      }
+#pragma unroll
+    for (int d = 0; d < D; ++d) u[d] = v[d];
+  }
+#pragma unroll
+  for (int d = 0; d < D; ++d) row[d * ng + g] = __float2bfloat16_rn(logf(pw[d] / ((float)N * (float)G)));
+  if (cross) {
+    int p = 0;
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+#pragma unroll
+      for (int c = a + 1; c < D; ++c, ++p) {
+        const float inv = rsqrtf(pw[a] * pw[c]);
+        row[col_c + 2 * p * ng + g] = __float2bfloat16_rn(cre[p] * inv);
+        row[col_c + (2 * p + 1) * ng + g] = __float2bfloat16_rn(cim[p] * inv);
+      }
+  }
+  if (lag) {
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const float inv = rsqrtf(pw[d] * nb[d]);
+      row[col_l + 2 * d * ng + g] = __float2bfloat16_rn(lre[d] * inv);
+      row[col_l + (2 * d + 1) * ng + g] = __float2bfloat16_rn(lim[d] * inv);
+    }
+  }
+}
+
 struct Std3 {
   double mean[3], scale[3];
 };
@@ -364,6 +439,36 @@ cudaError_t launch_lag_from_spectrum(const void* Y, int64_t B, int D, int64_t N,
                                                                  k_lo, G, ng, F_pad, col0, B,
                                                                  reinterpret_cast<__nv_bfloat16*>(out));
   return cudaGetLastError();
+}
+
+// Spectra of y into ws, then every column of the flow's feature rows.
+cudaError_t launch_spectral_columns(const float* y, int64_t B, int D, int64_t N, int k_lo, int G, int F_pad, bool cross,
+                                    bool lag, void* ws, void* out, cudaStream_t s) {
+  const int ng = (int)((N / 2 - k_lo) / G), chunks = ng > 0 ? (ng + SC_NT - 1) / SC_NT : 1;
+  if (D > 4) {   // more detectors than a thread holds: a kernel a kind of column
+    cudaError_t e = launch_features(y, B, D, N, k_lo, G, F_pad, ws, out, s);
+    int col = D * ng;
+    if (e == cudaSuccess && cross) {
+      e = launch_cross_from_spectrum(ws, B, D, N, k_lo, G, F_pad, col, out, s);
+      col += D * (D - 1) * ng;
+    }
+    return e == cudaSuccess && lag ? launch_lag_from_spectrum(ws, B, D, N, k_lo, G, F_pad, col, out, s) : e;
+  }
+  float2* Y = reinterpret_cast<float2*>(ws);
+  const cudaError_t e = launch_rfft_rows(y, B * D, N, Y, s);
+  if (e != cudaSuccess || B <= 0) return e;
+  auto run = [&](auto kern) {
+    kern<<<(unsigned)(B * chunks), SC_NT, 0, s>>>(Y, N / 2 + 1, (int)N, k_lo, G, ng, chunks, F_pad, cross, lag,
+                                                  reinterpret_cast<__nv_bfloat16*>(out));
+    return cudaGetLastError();
+  };
+  switch (D) {
+    case 1: return run(k_spectral_columns<1>);
+    case 2: return run(k_spectral_columns<2>);
+    case 3: return run(k_spectral_columns<3>);
+    case 4: return run(k_spectral_columns<4>);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t launch_lag_features(const float* y, int64_t B, int D, int64_t N, int k_lo, int G, int F_pad, int col0,
