@@ -127,6 +127,7 @@ cudaError_t launch_welch(const float* x, int D, int64_t L, double fs, int64_t M,
 // ----------------------------------------------------------------- whitening filter
 __global__ void k_whiten_filter(const double* __restrict__ psd, int D, int64_t M, double fs, int k_lo, int64_t N,
                                 bool inverse, float* __restrict__ W) {
+  asm volatile("griddepcontrol.launch_dependents;");   // as in k_prepare
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < (int64_t)D * (N / 2 + 1)) W[i] = whiten_filter_at(psd, i, M, fs, k_lo, N, inverse);
 }

@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(128) k_prepare(PriorStream ps, int64_t B, uint
                                                  int64_t F, DetParams dp, double gmst, unsigned draw_blocks,
                                                  FilterArgs fa, double* __restrict__ theta,
                                                  int64_t* __restrict__ offsets, DrawCoef* __restrict__ coef) {
+  asm volatile("griddepcontrol.launch_dependents;");   // the fused pass may set itself up (it waits for this kernel's end)
   if (blockIdx.x >= draw_blocks) {
     const int64_t i = (int64_t)(blockIdx.x - draw_blocks) * 128 + threadIdx.x;
     if (i < fa.entries) fa.W[i] = whiten_filter_at(fa.psd, i, fa.M, fa.fs, fa.k_lo, fa.N, false);
