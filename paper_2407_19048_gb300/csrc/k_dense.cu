@@ -12,6 +12,7 @@
 #include <algorithm>
 
 #include "gwx_internal.h"
+#include "pdl.cuh"
 #include "sum2.cuh"
 
 namespace gwx {
@@ -27,6 +28,7 @@ constexpr int TT = 32;   // rows of a column-sum partial; columns of a k_colsum 
 __global__ void __launch_bounds__(256) k_dz_rows(const float* __restrict__ dY, const __nv_bfloat16* __restrict__ Y,
                                                  int64_t M, int N, __nv_bfloat16* __restrict__ dZ,
                                                  float* __restrict__ part) {
+  pdl_enter();
   const int units = (N + 63) / 64;
   const int64_t u = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int64_t p = u / units;
@@ -42,7 +44,7 @@ __global__ void __launch_bounds__(256) k_dz_rows(const float* __restrict__ dY, c
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const int64_t at = (m0 + min(r0 + i, rows - 1)) * N + col;
-      v[i] = pairs ? __ldg(reinterpret_cast<const float2*>(dY + at)) : make_float2(__ldg(dY + at), __ldg(dY + at + 1));
+      v[i] = pairs ? __ldca(reinterpret_cast<const float2*>(dY + at)) : make_float2(__ldca(dY + at), __ldca(dY + at + 1));
       if (Y != nullptr) y[i] = *reinterpret_cast<const __nv_bfloat162*>(Y + at);
     }
 #pragma unroll
@@ -72,13 +74,14 @@ int colsum_slices(int64_t P) { return (int)std::min<int64_t>(CS_MAX_SLICES, std:
 
 __global__ void __launch_bounds__(1024) k_colsum(const float* __restrict__ part, int P, int N,
                                                  double* __restrict__ part2, float* __restrict__ db) {
+  pdl_enter();
   __shared__ float2 red[TT][TT + 1];
   const int n = blockIdx.x * TT + threadIdx.x;
   const int per = (P + gridDim.y - 1) / gridDim.y, p0 = blockIdx.y * per, p1 = min(P, p0 + per);
   Sum2 s;
   if (n < N)
 #pragma unroll 4
-    for (int p = p0 + threadIdx.y; p < p1; p += TT) s.add(__ldg(&part[(int64_t)p * N + n]));
+    for (int p = p0 + threadIdx.y; p < p1; p += TT) s.add(__ldca(&part[(int64_t)p * N + n]));
   red[threadIdx.y][threadIdx.x] = make_float2(s.h, s.l);
   __syncthreads();
   const float2 v = red[threadIdx.x][threadIdx.y];
@@ -94,6 +97,7 @@ __global__ void __launch_bounds__(1024) k_colsum(const float* __restrict__ part,
 }
 
 __global__ void k_colsum_finish(const double* __restrict__ part2, int slices, int N, float* __restrict__ db) {
+  pdl_enter();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
   double t = 0.0;
@@ -107,8 +111,7 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 cudaError_t launch_dz_rows(const float* dY, const void* Y, int64_t M, int N, void* dZ, float* part, cudaStream_t s) {
   const int64_t units = (M + TT - 1) / TT * ((N + 63) / 64);
-  k_dz_rows<<<(unsigned)((units + 7) / 8), 256, 0, s>>>(dY, reinterpret_cast<const __nv_bfloat16*>(Y), M, N,
-                                                        reinterpret_cast<__nv_bfloat16*>(dZ), part);
+  pdl_launch(k_dz_rows, dim3((unsigned)((units + 7) / 8)), dim3(256), 0, s, dY, reinterpret_cast<const __nv_bfloat16*>(Y), M, N, reinterpret_cast<__nv_bfloat16*>(dZ), part);
   return cudaGetLastError();
 }
 
@@ -150,9 +153,8 @@ cudaError_t launch_dense_backward(const void* X, const void* W, const float* bia
   if ((e = launch_dense_backward_dz(dZ, X, W, M, N, K, dX, dW, kpart, s)) != cudaSuccess) return e;
   if (db) {
     const int slices = colsum_slices(P);
-    k_colsum<<<dim3((unsigned)((N + TT - 1) / TT), (unsigned)slices), dim3(TT, TT), 0, s>>>(
-        part, (int)P, (int)N, part2, slices == 1 ? db : nullptr);
-    if (slices > 1) k_colsum_finish<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(part2, slices, (int)N, db);
+    pdl_launch(k_colsum, dim3(dim3((unsigned)((N + TT - 1) / TT), (unsigned)slices)), dim3(dim3(TT, TT)), 0, s, part, (int)P, (int)N, part2, slices == 1 ? db : nullptr);
+    if (slices > 1) pdl_launch(k_colsum_finish, dim3((unsigned)((N + 127) / 128)), dim3(128), 0, s, part2, slices, (int)N, db);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -26,6 +26,7 @@
 // Every mbarrier wait is bounded; on expiry the CTA records a status, stops and frees its
 // tensor memory.
 #include "flow_tile.cuh"
+#include "pdl.cuh"
 
 namespace gwx {
 
@@ -63,6 +64,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
   const int tiles = (int)((a.n + FM - 1) / FM);
   const FwdWeights wt{&mv1, &mv2, &mv3, a.e1, a.e2, a.e3, a.lstride, C, a.H, K, tiles, false};
   const uint32_t tmem = fwd_begin(rg);
+  pdl_enter();
 
   if (warp == 0) {
     fwd_produce(rg, wt, sw);
@@ -93,14 +95,14 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
         int64_t lo = 0, hi = a.E, s = a.row0 + row;
         while (hi - lo > 1) {
           const int64_t mid = (lo + hi) >> 1;
-          if (__ldg(&a.off[mid]) <= s) lo = mid; else hi = mid;
+          if (__ldca(&a.off[mid]) <= s) lo = mid; else hi = mid;
         }
         e = lo;
       }
       const uint4* crow = reinterpret_cast<const uint4*>(a.ctx + e * C);
       for (int g = h == 0 ? 1 : 4 * h; g < 4 * h + 4; ++g) {
         uint4 d = make_uint4(0u, 0u, 0u, 0u);
-        if (valid && g <= C / 8) d = __ldg(crow + (g - 1));
+        if (valid && g <= C / 8) d = __ldca(crow + (g - 1));
         sts128(sx + KB_BYTES * (g >> 3) + swz(r, g & 7), d.x, d.y, d.z, d.w);
       }
       for (int l = 0; l < K; ++l, ++li) {
@@ -200,7 +202,7 @@ cudaError_t launch_flow_sample_fused(const void* params_bf16, const float* param
   const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
   e = cudaFuncSetAttribute(k_flow_sample_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM);
   if (e != cudaSuccess) return e;
-  k_flow_sample_fused<<<grid, FWD_THREADS, FUSED_SMEM, s>>>(m1, m2, m3, a);
+  pdl_launch(k_flow_sample_fused, dim3(grid), dim3(FWD_THREADS), FUSED_SMEM, s, m1, m2, m3, a);
   return cudaGetLastError();
 }
 

@@ -24,6 +24,7 @@
 // backward; a batch of 4096 fills 32 SMs.  As ~370 launches of 3 to 13 us (each layer: input
 // rows, three products, coupling step; backward 17 kernels) the step took 3.04 ms, now 0.55.
 #include "flow_tile.cuh"
+#include "pdl.cuh"
 #include "sum2.cuh"
 
 namespace gwx {
@@ -194,6 +195,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
   const int tiles = (int)((a.n + FM - 1) / FM);
   const FwdWeights wt{&mv1, &mv2, &mv3, a.e1, a.e2, a.e3, a.lstride, C, H, K, tiles, true};
   const uint32_t tmem = fwd_begin(rg);
+  pdl_enter();
 
   if (warp == 0) {
     fwd_produce(rg, wt, sw);
@@ -225,14 +227,14 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
         int64_t lo = 0, hi = a.E, s = a.row0 + row;
         while (hi - lo > 1) {
           const int64_t mid = (lo + hi) >> 1;
-          if (__ldg(&a.off[mid]) <= s) lo = mid; else hi = mid;
+          if (__ldca(&a.off[mid]) <= s) lo = mid; else hi = mid;
         }
         e = lo;
       }
       const uint4* crow = reinterpret_cast<const uint4*>(a.ctx + e * C);
       for (int g = h == 0 ? 1 : 4 * h; g < 4 * h + 4; ++g) {
         uint4 x = make_uint4(0u, 0u, 0u, 0u);
-        if (valid && g <= C / 8) x = __ldg(crow + (g - 1));
+        if (valid && g <= C / 8) x = __ldca(crow + (g - 1));
         sts128(sx + KB_BYTES * (g >> 3) + swz(r, g & 7), x.x, x.y, x.z, x.w);
       }
       // chunk c (32 columns) of a hidden layer: signs and activations out, when the chunk before has
@@ -400,6 +402,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
+  pdl_enter();
 
   if (warp == 0) {
     uint32_t it = 0;
@@ -553,8 +556,8 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         for (int rd = 0; rd < 2; ++rd) {
           const bool have = valid && rd < NR;
           const int64_t m = mask_at(l, wrow / 32, a.P, H / 32, 2 * (2 * rd + h)) + lane;
-          k2[rd] = have ? make_uint2(__ldg(&a.m2[m]), __ldg(&a.m2[m + 32])) : make_uint2(0u, 0u);
-          k1[rd] = have ? make_uint2(__ldg(&a.m1[m]), __ldg(&a.m1[m + 32])) : make_uint2(0u, 0u);
+          k2[rd] = have ? make_uint2(__ldca(&a.m2[m]), __ldca(&a.m2[m + 32])) : make_uint2(0u, 0u);
+          k1[rd] = have ? make_uint2(__ldca(&a.m1[m]), __ldca(&a.m1[m + 32])) : make_uint2(0u, 0u);
         }
         if (h == 0) {
           float d[8];
@@ -663,6 +666,7 @@ __global__ void __launch_bounds__(1024) k_flow_bias_grads(const float* __restric
                                                           float* __restrict__ g3, int64_t lstride,
                                                           const double* __restrict__ loss_part, double n,
                                                           double* __restrict__ loss) {
+  pdl_enter();
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, l = blockIdx.y;
   if (l == K) {
     __shared__ double red[32][33];
@@ -686,7 +690,7 @@ __global__ void __launch_bounds__(1024) k_flow_bias_grads(const float* __restric
   Sum2 s;
   if (col0 + tx < cols)
 #pragma unroll 4
-    for (int64_t i = ty; i < P; i += 32) s.add(__ldg(&p[i * cols + col0 + tx]));
+    for (int64_t i = ty; i < P; i += 32) s.add(__ldca(&p[i * cols + col0 + tx]));
   red[ty][tx] = make_float2(s.h, s.l);
   __syncthreads();
   const float2 v = red[tx][ty];
@@ -725,8 +729,7 @@ cudaError_t run_density(const void* params_bf16, const float* params, const int6
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_flow_density, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSITY_SMEM);
   if (e != cudaSuccess) return e;
-  k_flow_density<<<grid, FWD_THREADS, DENSITY_SMEM, s>>>(m1, m2, m3, stores ? stores[0] : m1, stores ? stores[1] : m1,
-                                                         stores ? stores[2] : m1, a);
+  pdl_launch(k_flow_density, dim3(grid), dim3(FWD_THREADS), DENSITY_SMEM, s, m1, m2, m3, stores ? stores[0] : m1, stores ? stores[1] : m1, stores ? stores[2] : m1, a);
   return cudaGetLastError();
 }
 
@@ -836,7 +839,7 @@ cudaError_t launch_flow_train_fused(const void* params_bf16, const float* params
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_flow_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BACKWARD_SMEM);
   if (e != cudaSuccess) return e;
-  k_flow_backward<<<grid, F_THREADS, BACKWARD_SMEM, s>>>(w1, w2, w3, b1, b2, b);
+  pdl_launch(k_flow_backward, dim3(grid), dim3(F_THREADS), BACKWARD_SMEM, s, w1, w2, w3, b1, b2, b);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // weight gradients of all layers, one grouped product per kind; bias gradients and the loss
   if ((e = launch_wgrad(f.dO, f.g2, grads + off_t[10], 8, H, n, f.kpart, s, K, n * 8, n * H, lstride)) != cudaSuccess ||
@@ -845,9 +848,7 @@ cudaError_t launch_flow_train_fused(const void* params_bf16, const float* params
       (e = launch_wgrad(f.dz1, f.X, grads + off_t[6], H, 8 + C, n, f.kpart, s, K, n * H, n * (8 + C), lstride)) !=
           cudaSuccess)
     return e;
-  k_flow_bias_grads<<<dim3((unsigned)(2 * (H / 32) + 1), (unsigned)(K + 1)), 1024, 0, s>>>(
-      f.p1, f.p2, f.p3, b.P, H, K, grads + off_t[7], grads + off_t[9], grads + off_t[11], lstride, f.loss_part,
-      (double)n, loss_mean);
+  pdl_launch(k_flow_bias_grads, dim3(dim3((unsigned)(2 * (H / 32) + 1), (unsigned)(K + 1))), dim3(1024), 0, s, f.p1, f.p2, f.p3, b.P, H, K, grads + off_t[7], grads + off_t[9], grads + off_t[11], lstride, f.loss_part, (double)n, loss_mean);
   return cudaGetLastError();
 }
 

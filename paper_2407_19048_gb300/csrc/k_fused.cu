@@ -6,6 +6,8 @@
 // complex points each; the waveform of a bin is evaluated once and projected onto
 // all D detectors, so the frequency-domain stage costs one phase/amplitude
 // evaluation per bin plus one complex exponential per detector.
+#include <atomic>
+
 #include <map>
 #include <mutex>
 #include <utility>
@@ -666,7 +668,14 @@ static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, 
   int dev = 0, sms = 0, per_sm = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
+  // blocks of this kernel that fit an SM of device dev, asked once (the query costs the host 3 us,
+  // much of a small call)
+  static std::atomic<int> fit[16];
+  if (e == cudaSuccess && dev < 16) per_sm = fit[dev].load(std::memory_order_relaxed);
+  if (e == cudaSuccess && per_sm == 0) {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
+    if (e == cudaSuccess && dev < 16) fit[dev].store(per_sm, std::memory_order_relaxed);
+  }
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   if (per_sm_want > 0 && per_sm_want < per_sm) per_sm = per_sm_want;

@@ -41,6 +41,7 @@
 #include <cuda_bf16.h>
 
 #include "gwx_internal.h"
+#include "pdl.cuh"
 #include "tc05.cuh"
 
 namespace gwx {
@@ -117,8 +118,8 @@ __device__ int g_gemm_status;
 
 // Four consecutive floats from p (n of them exist; vec: p is 16-byte aligned and n >= 4).
 __device__ __forceinline__ float4 load4(const float* __restrict__ p, int n, bool vec) {
-  if (vec) return __ldg(reinterpret_cast<const float4*>(p));
-  return make_float4(__ldg(p), n > 1 ? __ldg(p + 1) : 0.f, n > 2 ? __ldg(p + 2) : 0.f, n > 3 ? __ldg(p + 3) : 0.f);
+  if (vec) return __ldca(reinterpret_cast<const float4*>(p));
+  return make_float4(__ldca(p), n > 1 ? __ldca(p + 1) : 0.f, n > 2 ? __ldca(p + 2) : 0.f, n > 3 ? __ldca(p + 3) : 0.f);
 }
 
 __device__ __forceinline__ float act_of(float z, int act) {
@@ -233,6 +234,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
+  pdl_enter();
 
   if (warp == 0) {
     uint32_t s = 0, ph = 1;   // stage and the parity of its "empty" phase (the first round finds them free)
@@ -559,6 +561,7 @@ bool make_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t K, uint32
 template <int LANES>
 __global__ void __launch_bounds__(256) k_split_reduce(const float4* __restrict__ part, int splits, int64_t n4,
                                                       int64_t ostride4, float4* __restrict__ out) {
+  pdl_enter();
   constexpr int X = 256 / LANES;
   __shared__ float4 red[LANES][X];
   const int x = threadIdx.x % X, y = threadIdx.x / X;
@@ -574,7 +577,7 @@ __global__ void __launch_bounds__(256) k_split_reduce(const float4* __restrict__
   };
   if (i < n4) {
 #pragma unroll 4
-    for (int s = y; s < splits; s += LANES) add(__ldg(p + (int64_t)s * total));
+    for (int s = y; s < splits; s += LANES) add(__ldca(p + (int64_t)s * total));
   }
   if constexpr (LANES > 1) {
     red[y][x] = acc;
@@ -620,8 +623,7 @@ cudaError_t run_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmCal
   auto kern = k_gemm_bf16<OUT, TN_, OPS, MW>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, GEMM_THREADS, smem, s>>>(ta, tb, c.C, c.bias, c.act, make_work_map(TM, TN, c.group, c.groups), (int)c.M, (int)c.N, (int)c.K, kbs, splits,
-                                        c.extra, c.colsum, c.groups, c.cstride, c.geo);
+  pdl_launch(kern, dim3(grid), dim3(GEMM_THREADS), smem, s, ta, tb, c.C, c.bias, c.act, make_work_map(TM, TN, c.group, c.groups), (int)c.M, (int)c.N, (int)c.K, kbs, splits, c.extra, c.colsum, c.groups, c.cstride, c.geo);
   return cudaGetLastError();
 }
 
@@ -774,11 +776,9 @@ static cudaError_t wgrad_finish(const GemmCall& c, float* C, int64_t cstride, co
   const auto* p = reinterpret_cast<const float4*>(part);
   auto* out = reinterpret_cast<float4*>(C);
   if (c.splits >= 16)
-    k_split_reduce<8><<<dim3((unsigned)((n4 + 31) / 32), (unsigned)c.groups), 256, 0, s>>>(p, c.splits, n4, cstride / 4,
-                                                                                           out);
+    pdl_launch(k_split_reduce<8>, dim3(dim3((unsigned)((n4 + 31) / 32), (unsigned)c.groups)), dim3(256), 0, s, p, c.splits, n4, cstride / 4, out);
   else
-    k_split_reduce<1><<<dim3((unsigned)((n4 + 255) / 256), (unsigned)c.groups), 256, 0, s>>>(p, c.splits, n4,
-                                                                                             cstride / 4, out);
+    pdl_launch(k_split_reduce<1>, dim3(dim3((unsigned)((n4 + 255) / 256), (unsigned)c.groups)), dim3(256), 0, s, p, c.splits, n4, cstride / 4, out);
   return cudaGetLastError();
 }
 

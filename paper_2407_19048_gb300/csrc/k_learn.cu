@@ -13,6 +13,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "pdl.cuh"
 
 namespace gwx {
 
@@ -108,6 +109,7 @@ template <int D>
 __global__ void __launch_bounds__(SC_NT) k_spectral_columns(const float2* __restrict__ Y, int64_t F, int N, int k_lo,
                                                             int G, int ng, int chunks, int F_pad, bool cross, bool lag,
                                                             __nv_bfloat16* __restrict__ out) {
+  pdl_enter();
   constexpr int P = D * (D - 1) / 2;
   const int64_t b = blockIdx.x / chunks;
   const int chunk = (int)(blockIdx.x - b * chunks);
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(SC_NT) k_spectral_columns(const float2* __rest
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     pw[d] = nb[d] = lre[d] = lim[d] = 0.f;
-    u[d] = __ldg(y + d * F);
+    u[d] = __ldca(y + d * F);
   }
 #pragma unroll
   for (int p = 0; p < P; ++p) cre[p] = cim[p] = 0.f;
@@ -131,7 +133,7 @@ __global__ void __launch_bounds__(SC_NT) k_spectral_columns(const float2* __rest
   for (int k = 0; k < G; ++k) {
     float2 v[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) v[d] = lag || k + 1 < G ? __ldg(y + d * F + k + 1) : make_float2(0.f, 0.f);
+    for (int d = 0; d < D; ++d) v[d] = lag || k + 1 < G ? __ldca(y + d * F + k + 1) : make_float2(0.f, 0.f);
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       pw[d] = fmaf(u[d].x, u[d].x, fmaf(u[d].y, u[d].y, pw[d]));
@@ -458,8 +460,7 @@ cudaError_t launch_spectral_columns(const float* y, int64_t B, int D, int64_t N,
   const cudaError_t e = launch_rfft_rows(y, B * D, N, Y, s);
   if (e != cudaSuccess || B <= 0) return e;
   auto run = [&](auto kern) {
-    kern<<<(unsigned)(B * chunks), SC_NT, 0, s>>>(Y, N / 2 + 1, (int)N, k_lo, G, ng, chunks, F_pad, cross, lag,
-                                                  reinterpret_cast<__nv_bfloat16*>(out));
+    pdl_launch(kern, dim3((unsigned)(B * chunks)), dim3(SC_NT), 0, s, Y, N / 2 + 1, (int)N, k_lo, G, ng, chunks, F_pad, cross, lag, reinterpret_cast<__nv_bfloat16*>(out));
     return cudaGetLastError();
   };
   switch (D) {

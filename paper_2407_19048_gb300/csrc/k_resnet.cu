@@ -15,6 +15,7 @@
 #include <cuda_bf16.h>
 
 #include "gwx_internal.h"
+#include "pdl.cuh"
 #include "sum2.cuh"
 
 namespace gwx {
@@ -35,6 +36,7 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 // columns >= k C); one thread per 8 columns (C % 8 == 0, so a chunk stays in one tap).
 __global__ void k_im2col(const __nv_bfloat16* __restrict__ x, int T, int C, int k, int s, int p, int To, int K,
                          __nv_bfloat16* __restrict__ cols) {
+  pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int ch = K / 8;
   if (i >= To * ch) return;
@@ -66,6 +68,7 @@ __global__ void k_im2col_cf(const float* __restrict__ y, int D, int N, int k, in
 // 7 taps; now 11).
 __global__ void k_im2col_cf8(const float* __restrict__ y, int D, int N, int k, int s, int p, int To, int K,
                              __nv_bfloat16* __restrict__ cols) {
+  pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int ch = K / 8;
   if (i >= To * ch) return;
@@ -76,7 +79,7 @@ __global__ void k_im2col_cf8(const float* __restrict__ y, int D, int N, int k, i
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
     const int src = s * t + j - p;
-    v[e] = j < k && src >= 0 && src < N ? __ldg(y + (b * D + c) * N + src) : 0.f;
+    v[e] = j < k && src >= 0 && src < N ? __ldca(y + (b * D + c) * N + src) : 0.f;
     if (++c == D) c = 0, ++j;
   }
   __align__(16) __nv_bfloat162 h[4];
@@ -108,6 +111,7 @@ __global__ void k_col2im(const float* __restrict__ dcols, int T, int C, int k, i
 template <int KT>
 __global__ void k_col2im4(const float* __restrict__ dcols, int T, int C, int s, int p, int To, int K,
                           const float* __restrict__ addend, float* __restrict__ dx) {
+  pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= T * C / 4) return;
   const int64_t b = blockIdx.y;
@@ -118,7 +122,7 @@ __global__ void k_col2im4(const float* __restrict__ dcols, int T, int C, int s, 
     const int num = t + p - j;
     const int to = num / s;
     v[j] = (num >= 0 && num - to * s == 0 && to < To)
-               ? __ldg(reinterpret_cast<const float4*>(dcols + (b * To + to) * K + j * C + c))
+               ? __ldca(reinterpret_cast<const float4*>(dcols + (b * To + to) * K + j * C + c))
                : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   const int64_t o = b * T * C + 4 * (int64_t)i;
@@ -166,18 +170,18 @@ __global__ void __launch_bounds__(256) k_gn_stats(const float* __restrict__ z, i
                                                   float* __restrict__ ms) {
   const int b = blockIdx.x / G, g = blockIdx.x - (blockIdx.x / G) * G, cg = C / G, cv = cg / VEC;
   const float* zb = z + (int64_t)b * T * C + g * cg;
-  const float k0 = __ldg(zb);
+  const float k0 = __ldca(zb);
   float s1 = 0.f, s2 = 0.f;
 #pragma unroll 4
   for (int e = threadIdx.x; e < T * cv; e += blockDim.x) {
     const int t = e / cv, c = (e - t * cv) * VEC;
     if constexpr (VEC == 4) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(zb + (int64_t)t * C + c));
+      const float4 v = __ldca(reinterpret_cast<const float4*>(zb + (int64_t)t * C + c));
       const float d0 = v.x - k0, d1 = v.y - k0, d2 = v.z - k0, d3 = v.w - k0;
       s1 += (d0 + d1) + (d2 + d3);
       s2 += fmaf(d0, d0, __fmul_rn(d1, d1)) + fmaf(d2, d2, __fmul_rn(d3, d3));
     } else {
-      const float d = __ldg(zb + (int64_t)t * C + c) - k0;
+      const float d = __ldca(zb + (int64_t)t * C + c) - k0;
       s1 += d;
       s2 += d * d;
     }
@@ -273,13 +277,14 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
                                                            const __nv_bfloat16* __restrict__ res16, int relu,
                                                            __nv_bfloat16* __restrict__ out16,
                                                            float* __restrict__ out32, float* __restrict__ ms) {
+  pdl_enter();
   __shared__ double sums[64];
   __shared__ float st[64];
   const int cq = C / 4, rl = 256 / cq, cg = C / G;
   const int q4 = threadIdx.x % cq, l0 = (threadIdx.x % 256) / cq, g = (4 * q4) / cg;
   const int64_t off = (int64_t)blockIdx.x * T * C;
   const float4* z4 = reinterpret_cast<const float4*>(z + off) + q4;   // row t at t cq
-  const float k0 = __ldg(z + off + g * cg);
+  const float k0 = __ldca(z + off + g * cg);
   Sum2 a, q;
   for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_NT / 256) * 16 * rl) {
     float s1 = 0.f, s2 = 0.f;
@@ -289,7 +294,7 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int t = t0 + (8 * h + i) * rl;
-        v[i] = t < T ? __ldg(z4 + t * cq) : make_float4(k0, k0, k0, k0);   // adds zero
+        v[i] = t < T ? __ldca(z4 + t * cq) : make_float4(k0, k0, k0, k0);   // adds zero
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -301,11 +306,11 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
     a.add(s1);
     q.add(__fmul_rn(s2, GN_SCALE));
   }
-  const float kg = (int)threadIdx.x < G ? __ldg(z + off + threadIdx.x * cg) : 0.f;
-  const float4 gm = make_float4(__ldg(&gamma[4 * q4]), __ldg(&gamma[4 * q4 + 1]), __ldg(&gamma[4 * q4 + 2]),
-                                __ldg(&gamma[4 * q4 + 3]));
-  const float4 bt = make_float4(__ldg(&beta[4 * q4]), __ldg(&beta[4 * q4 + 1]), __ldg(&beta[4 * q4 + 2]),
-                                __ldg(&beta[4 * q4 + 3]));
+  const float kg = (int)threadIdx.x < G ? __ldca(z + off + threadIdx.x * cg) : 0.f;
+  const float4 gm = make_float4(__ldca(&gamma[4 * q4]), __ldca(&gamma[4 * q4 + 1]), __ldca(&gamma[4 * q4 + 2]),
+                                __ldca(&gamma[4 * q4 + 3]));
+  const float4 bt = make_float4(__ldca(&beta[4 * q4]), __ldca(&beta[4 * q4 + 1]), __ldca(&beta[4 * q4 + 2]),
+                                __ldca(&beta[4 * q4 + 3]));
   sample_group_sums<GN_NT>(a, q, cq, cg, G, sums);
   __syncthreads();
   if ((int)threadIdx.x < G) {
@@ -326,8 +331,8 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
     for (int k = 0; k < 4; ++k) {
       const int t = min(tb + k * step, T - 1);
       x[k] = __ldcs(z4 + t * cq);
-      if (res32) r[k] = __ldg(reinterpret_cast<const float4*>(res32 + off) + t * cq + q4);
-      if (res16) r[k] = bf16x4(__ldg(reinterpret_cast<const uint2*>(res16 + off) + t * cq + q4));
+      if (res32) r[k] = __ldca(reinterpret_cast<const float4*>(res32 + off) + t * cq + q4);
+      if (res16) r[k] = bf16x4(__ldca(reinterpret_cast<const uint2*>(res16 + off) + t * cq + q4));
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -375,17 +380,17 @@ __device__ __forceinline__ void gn_load(GnRow<SRC>& r, const GnSource& s, int64_
     r.v0 = r.v1 = make_float4(0.f, 0.f, 0.f, 0.f);
     r.a0 = r.a1 = make_uchar4(3, 3, 3, 3);
     if (to < s.To) {
-      r.v0 = __ldg(reinterpret_cast<const float4*>(s.dy + o));
-      r.a0 = __ldg(reinterpret_cast<const uchar4*>(s.arg + o));
+      r.v0 = __ldca(reinterpret_cast<const float4*>(s.dy + o));
+      r.a0 = __ldca(reinterpret_cast<const uchar4*>(s.arg + o));
     }
     if ((t & 1) && to + 1 < s.To) {
-      r.v1 = __ldg(reinterpret_cast<const float4*>(s.dy + o + C));
-      r.a1 = __ldg(reinterpret_cast<const uchar4*>(s.arg + o + C));
+      r.v1 = __ldca(reinterpret_cast<const float4*>(s.dy + o + C));
+      r.a1 = __ldca(reinterpret_cast<const uchar4*>(s.arg + o + C));
     }
   } else if constexpr (SRC != DY_MEAN) {
-    r.v0 = __ldg(reinterpret_cast<const float4*>(s.dy + i));
+    r.v0 = __ldca(reinterpret_cast<const float4*>(s.dy + i));
   }
-  if constexpr (SRC != DY_PLAIN) r.o = __ldg(reinterpret_cast<const uint2*>(s.out + i));
+  if constexpr (SRC != DY_PLAIN) r.o = __ldca(reinterpret_cast<const uint2*>(s.out + i));
 }
 
 template <int SRC>
@@ -414,6 +419,7 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
                                                             int G, double inv_n, const float* __restrict__ ms,
                                                             const float* __restrict__ gamma, void* __restrict__ dz,
                                                             float* __restrict__ dsum, double* __restrict__ part) {
+  pdl_enter();
   constexpr int GN_BT = gn_bt(SRC);
   __shared__ double sums[64];
   __shared__ float2 pr[GN_BT * 8];
@@ -424,11 +430,11 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
   const int64_t b = blockIdx.x, off = b * T * C;
   const float4* z4 = reinterpret_cast<const float4*>(z + off) + q4;   // row t at t cq
   const float mean = ms[2 * (b * G + g)], rstd = ms[2 * (b * G + g) + 1];
-  const float4 gm = make_float4(__ldg(&gamma[4 * q4]), __ldg(&gamma[4 * q4 + 1]), __ldg(&gamma[4 * q4 + 2]),
-                                __ldg(&gamma[4 * q4 + 3]));
+  const float4 gm = make_float4(__ldca(&gamma[4 * q4]), __ldca(&gamma[4 * q4 + 1]), __ldca(&gamma[4 * q4 + 2]),
+                                __ldca(&gamma[4 * q4 + 3]));
   float4 mdy = make_float4(0.f, 0.f, 0.f, 0.f);
   if constexpr (SRC == DY_MEAN) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(src.dy + b * C) + q4);
+    const float4 v = __ldca(reinterpret_cast<const float4*>(src.dy + b * C) + q4);
     mdy = make_float4(v.x / T, v.y / T, v.z / T, v.w / T);
   }
   Sum2 a, q, pg[4], pb[4];
@@ -443,7 +449,7 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
       for (int i = 0; i < U; ++i) {
         const int t = min(t0 + (h + i) * rl, T - 1);
         gn_load<SRC>(r[i], src, b, t, 4 * q4, T, C);
-        x[i] = __ldg(z4 + t * cq);
+        x[i] = __ldca(z4 + t * cq);
       }
 #pragma unroll
       for (int i = 0; i < U; ++i) {
@@ -565,7 +571,7 @@ __global__ void k_gn_apply(const float* __restrict__ z, int T, int C, int G, con
     v[0] = z[i];
   }
 #pragma unroll
-  for (int u = 0; u < VEC; ++u) v[u] = fmaf((v[u] - mean) * rstd, __ldg(&gamma[c + u]), __ldg(&beta[c + u]));
+  for (int u = 0; u < VEC; ++u) v[u] = fmaf((v[u] - mean) * rstd, __ldca(&gamma[c + u]), __ldca(&beta[c + u]));
   if (res32) {
     if constexpr (VEC == 4) {
       const float4 q = *reinterpret_cast<const float4*>(res32 + i);
@@ -615,8 +621,8 @@ __global__ void k_relu_mask4(const float* __restrict__ dy, const __nv_bfloat16* 
                              float* __restrict__ d) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n4) return;
-  const float4 g = __ldg(reinterpret_cast<const float4*>(dy) + i);
-  const uint2 q = __ldg(reinterpret_cast<const uint2*>(out) + i);
+  const float4 g = __ldca(reinterpret_cast<const float4*>(dy) + i);
+  const uint2 q = __ldca(reinterpret_cast<const uint2*>(out) + i);
   const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.x));
   const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.y));
   reinterpret_cast<float4*>(d)[i] = make_float4(lo.x > 0.f ? g.x : 0.f, lo.y > 0.f ? g.y : 0.f,
@@ -637,18 +643,18 @@ __global__ void __launch_bounds__(256) k_gn_bwd_stats(const float* __restrict__ 
     const int t = e / cv, c = (e - t * cv) * VEC;
     const int64_t i = base + (int64_t)t * C + c;
     if constexpr (VEC == 4) {
-      const float4 d = __ldg(reinterpret_cast<const float4*>(dy + i));
-      const float4 x = __ldg(reinterpret_cast<const float4*>(z + i));
-      const float4 gm = make_float4(__ldg(&gamma[g * cg + c]), __ldg(&gamma[g * cg + c + 1]),
-                                    __ldg(&gamma[g * cg + c + 2]), __ldg(&gamma[g * cg + c + 3]));
+      const float4 d = __ldca(reinterpret_cast<const float4*>(dy + i));
+      const float4 x = __ldca(reinterpret_cast<const float4*>(z + i));
+      const float4 gm = make_float4(__ldca(&gamma[g * cg + c]), __ldca(&gamma[g * cg + c + 1]),
+                                    __ldca(&gamma[g * cg + c + 2]), __ldca(&gamma[g * cg + c + 3]));
       const float a0 = d.x * gm.x, a1 = d.y * gm.y, a2 = d.z * gm.z, a3 = d.w * gm.w;
       s1 += (a0 + a1) + (a2 + a3);
       s2 += (a0 * ((x.x - mean) * rstd) + a1 * ((x.y - mean) * rstd)) +
             (a2 * ((x.z - mean) * rstd) + a3 * ((x.w - mean) * rstd));
     } else {
-      const float a = __ldg(dy + i) * __ldg(&gamma[g * cg + c]);
+      const float a = __ldca(dy + i) * __ldca(&gamma[g * cg + c]);
       s1 += a;
-      s2 += a * ((__ldg(z + i) - mean) * rstd);
+      s2 += a * ((__ldca(z + i) - mean) * rstd);
     }
   }
   double a = s1, q = s2;
@@ -675,10 +681,10 @@ __global__ void k_gn_bwd_apply(const float* __restrict__ dy, const float* __rest
     const float4 d = *reinterpret_cast<const float4*>(dy + i);
     const float4 x = *reinterpret_cast<const float4*>(z + i);
     float4 o;
-    o.x = rstd * (d.x * __ldg(&gamma[c]) - m1 - (x.x - mean) * rstd * m2);
-    o.y = rstd * (d.y * __ldg(&gamma[c + 1]) - m1 - (x.y - mean) * rstd * m2);
-    o.z = rstd * (d.z * __ldg(&gamma[c + 2]) - m1 - (x.z - mean) * rstd * m2);
-    o.w = rstd * (d.w * __ldg(&gamma[c + 3]) - m1 - (x.w - mean) * rstd * m2);
+    o.x = rstd * (d.x * __ldca(&gamma[c]) - m1 - (x.x - mean) * rstd * m2);
+    o.y = rstd * (d.y * __ldca(&gamma[c + 1]) - m1 - (x.y - mean) * rstd * m2);
+    o.z = rstd * (d.z * __ldca(&gamma[c + 2]) - m1 - (x.z - mean) * rstd * m2);
+    o.w = rstd * (d.w * __ldca(&gamma[c + 3]) - m1 - (x.w - mean) * rstd * m2);
     *reinterpret_cast<float4*>(dz + i) = o;
   } else {
     dz[i] = rstd * (dy[i] * gamma[c] - m1 - (z[i] - mean) * rstd * m2);
@@ -709,8 +715,8 @@ __global__ void __launch_bounds__(256) k_gn_param_part(const float* __restrict__
       float fg = 0.f, fb = 0.f;
       for (int n = 0; n < 64 && r < r1; ++n) {
         const int64_t i = (int64_t)r * C + c;
-        const float d = __ldg(dy + i);
-        fg += d * ((__ldg(z + i) - ms[2 * (b * G + g)]) * ms[2 * (b * G + g) + 1]);
+        const float d = __ldca(dy + i);
+        fg += d * ((__ldca(z + i) - ms[2 * (b * G + g)]) * ms[2 * (b * G + g) + 1]);
         fb += d;
         r += 8;
         t += 8;
@@ -744,13 +750,14 @@ __global__ void __launch_bounds__(256) k_gn_param_part(const float* __restrict__
 constexpr int PF_C = 2, PF_NT = 256;
 __global__ void __launch_bounds__(PF_NT) k_gn_param_finish(const double* __restrict__ part, int slices, int C,
                                                            float* __restrict__ dgamma, float* __restrict__ dbeta) {
+  pdl_enter();
   __shared__ double2 r[PF_NT / 32][PF_C];
   const int c = blockIdx.x * PF_C + (threadIdx.x & (PF_C - 1));
   double tg = 0.0, tb = 0.0;
   if (c < C) {
 #pragma unroll 4
     for (int s = threadIdx.x / PF_C; s < slices; s += PF_NT / PF_C) {
-      const double2 v = __ldg(reinterpret_cast<const double2*>(part) + (int64_t)s * C + c);
+      const double2 v = __ldca(reinterpret_cast<const double2*>(part) + (int64_t)s * C + c);
       tg += v.x;
       tb += v.y;
     }
@@ -801,6 +808,7 @@ __global__ void k_maxpool(const __nv_bfloat16* __restrict__ x, int T, int C, int
 // a thread).
 __global__ void k_maxpool8(const __nv_bfloat16* __restrict__ x, int T, int C, int To, __nv_bfloat16* __restrict__ y,
                            uint8_t* __restrict__ arg) {
+  pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x, cv = C / 8;
   if (i >= To * cv) return;
   const int64_t b = blockIdx.y;
@@ -809,7 +817,7 @@ __global__ void k_maxpool8(const __nv_bfloat16* __restrict__ x, int T, int C, in
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     const int src = 2 * t + j - 1;
-    v[j] = src >= 0 && src < T ? __ldg(reinterpret_cast<const uint4*>(x + (b * T + src) * C + c))
+    v[j] = src >= 0 && src < T ? __ldca(reinterpret_cast<const uint4*>(x + (b * T + src) * C + c))
                                : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);   // -inf: never first
   }
   const __nv_bfloat16* e0 = reinterpret_cast<const __nv_bfloat16*>(&v[0]);
@@ -862,8 +870,8 @@ __global__ void k_maxpool_back4(const float* __restrict__ dy, const uint8_t* __r
   for (int to = t / 2; to <= (t + 1) / 2; ++to) {
     if (to >= To) continue;
     const int64_t o = (b * To + to) * C + c;
-    const float4 d = __ldg(reinterpret_cast<const float4*>(dy + o));
-    const uchar4 a = __ldg(reinterpret_cast<const uchar4*>(arg + o));
+    const float4 d = __ldca(reinterpret_cast<const float4*>(dy + o));
+    const uchar4 a = __ldca(reinterpret_cast<const uchar4*>(arg + o));
     const int base = 2 * to - 1;
     if (base + (int)a.x == t) acc.x += d.x;
     if (base + (int)a.y == t) acc.y += d.y;
@@ -889,6 +897,7 @@ __global__ void k_mean_time(const __nv_bfloat16* __restrict__ x, int64_t B, int 
 // channel and 16 loads, now 12.7).
 __global__ void k_mean_time2(const __nv_bfloat16* __restrict__ x, int64_t B, int T, int C,
                              __nv_bfloat16* __restrict__ m) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int h = C / 2;
   if (i >= B * h) return;
@@ -903,11 +912,11 @@ __global__ void k_mean_time2(const __nv_bfloat16* __restrict__ x, int64_t B, int
   for (; t + 32 <= T; t += 32) {
     uint32_t v[32];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = __ldg(p + (t + k) * h);
+    for (int k = 0; k < 32; ++k) v[k] = __ldca(p + (t + k) * h);
 #pragma unroll
     for (int k = 0; k < 32; ++k) add(v[k]);
   }
-  for (; t < T; ++t) add(__ldg(p + t * h));
+  for (; t < T; ++t) add(__ldca(p + t * h));
   reinterpret_cast<__nv_bfloat162*>(m)[i] = __floats2bfloat162_rn(a0 / T, a1 / T);
 }
 
@@ -928,8 +937,7 @@ bool aligned8(const void* p) { return ((uintptr_t)p & 7u) == 0; }
 cudaError_t launch_im2col(const void* x, int64_t B, int T, int C, int k, int s, int p, int K, void* cols,
                           cudaStream_t st) {
   const int To = (T + 2 * p - k) / s + 1;
-  k_im2col<<<dim3(nblk((int64_t)To * (K / 8), 256), (unsigned)B), 256, 0, st>>>(
-      reinterpret_cast<const __nv_bfloat16*>(x), T, C, k, s, p, To, K, reinterpret_cast<__nv_bfloat16*>(cols));
+  pdl_launch(k_im2col, dim3(dim3(nblk((int64_t)To * (K / 8), 256), (unsigned)B)), dim3(256), 0, st, reinterpret_cast<const __nv_bfloat16*>(x), T, C, k, s, p, To, K, reinterpret_cast<__nv_bfloat16*>(cols));
   return cudaGetLastError();
 }
 
@@ -937,8 +945,7 @@ cudaError_t launch_im2col_cf(const float* y, int64_t B, int D, int N, int k, int
                              cudaStream_t st) {
   const int To = (N + 2 * p - k) / s + 1;
   if (K % 8 == 0 && aligned16(cols))
-    k_im2col_cf8<<<dim3(nblk((int64_t)To * (K / 8), 256), (unsigned)B), 256, 0, st>>>(
-        y, D, N, k, s, p, To, K, reinterpret_cast<__nv_bfloat16*>(cols));
+    pdl_launch(k_im2col_cf8, dim3(dim3(nblk((int64_t)To * (K / 8), 256), (unsigned)B)), dim3(256), 0, st, y, D, N, k, s, p, To, K, reinterpret_cast<__nv_bfloat16*>(cols));
   else
     k_im2col_cf<<<dim3(nblk((int64_t)To * K, 256), (unsigned)B), 256, 0, st>>>(y, D, N, k, s, p, To, K,
                                                                                reinterpret_cast<__nv_bfloat16*>(cols));
@@ -951,9 +958,9 @@ cudaError_t launch_col2im(const float* dcols, int64_t B, int T, int C, int k, in
   const bool v4 = C % 4 == 0 && K % 4 == 0 && aligned16(dcols) && aligned16(addend) && aligned16(dx);
   const dim3 g4(nblk((int64_t)T * C / 4, 256), (unsigned)B);
   if (v4 && k == 1) {
-    k_col2im4<1><<<g4, 256, 0, st>>>(dcols, T, C, s, p, To, K, addend, dx);
+    pdl_launch(k_col2im4<1>, dim3(g4), dim3(256), 0, st, dcols, T, C, s, p, To, K, addend, dx);
   } else if (v4 && k == 5) {
-    k_col2im4<5><<<g4, 256, 0, st>>>(dcols, T, C, s, p, To, K, addend, dx);
+    pdl_launch(k_col2im4<5>, dim3(g4), dim3(256), 0, st, dcols, T, C, s, p, To, K, addend, dx);
   } else if (v4 && k == 7) {
     k_col2im4<7><<<g4, 256, 0, st>>>(dcols, T, C, s, p, To, K, addend, dx);
   } else {
@@ -970,7 +977,7 @@ cudaError_t launch_group_norm(const float* z, int64_t B, int T, int C, int G, co
   const auto r16 = reinterpret_cast<const __nv_bfloat16*>(res16);
   const auto o16 = reinterpret_cast<__nv_bfloat16*>(out16);
   if (v4 && per_sample_ok(C, G)) {
-    k_gn_forward_s<<<(unsigned)B, GN_NT, 0, st>>>(z, T, C, G, 1.0 / ((double)T * (C / G)), gamma, beta, res32, r16, relu, o16, out32, ms);
+    pdl_launch(k_gn_forward_s, dim3((unsigned)B), dim3(GN_NT), 0, st, z, T, C, G, 1.0 / ((double)T * (C / G)), gamma, beta, res32, r16, relu, o16, out32, ms);
   } else if (v4) {
     k_gn_stats<4><<<(unsigned)(B * G), 256, 0, st>>>(z, T, C, G, ms);
     k_gn_apply<4><<<dim3(nblk((int64_t)T * C / 4, 256), (unsigned)B), 256, 0, st>>>(z, T, C, G, ms, gamma, beta, res32,
@@ -988,7 +995,7 @@ static cudaError_t launch_gn_backward(const GnSource& src, const float* z, int64
                                       const float* ms, const float* gamma, void* dz, float* dsum, double* part,
                                       cudaStream_t st) {
   const double inv_n = 1.0 / ((double)T * (C / G));
-  k_gn_backward_s<SRC, OUT16><<<(unsigned)B, gn_bt(SRC), 0, st>>>(src, z, T, C, G, inv_n, ms, gamma, dz, dsum, part);
+  pdl_launch(k_gn_backward_s<SRC, OUT16>, dim3((unsigned)B), dim3(gn_bt(SRC)), 0, st, src, z, T, C, G, inv_n, ms, gamma, dz, dsum, part);
   return cudaGetLastError();
 }
 
@@ -1010,7 +1017,7 @@ cudaError_t launch_group_norm_backward(const float* dy, const float* z, int64_t 
                                                               dz, nullptr, fused ? part : nullptr, st);
     if (e != cudaSuccess) return e;
     if (fused) {
-      k_gn_param_finish<<<nblk(C, PF_C), PF_NT, 0, st>>>(part, (int)B, C, dgamma, dbeta);
+      pdl_launch(k_gn_param_finish, dim3(nblk(C, PF_C)), dim3(PF_NT), 0, st, part, (int)B, C, dgamma, dbeta);
       return cudaGetLastError();
     }
   } else if (v4) {
@@ -1023,7 +1030,7 @@ cudaError_t launch_group_norm_backward(const float* dy, const float* z, int64_t 
   }
   const int slices = gn_slices(B * T);
   k_gn_param_part<<<dim3(nblk(C, 32), slices), 256, 0, st>>>(dy, z, (int)(B * T), T, C, G, ms, part);
-  k_gn_param_finish<<<nblk(C, PF_C), PF_NT, 0, st>>>(part, slices, C, dgamma, dbeta);
+  pdl_launch(k_gn_param_finish, dim3(nblk(C, PF_C)), dim3(PF_NT), 0, st, part, slices, C, dgamma, dbeta);
   return cudaGetLastError();
 }
 
@@ -1046,7 +1053,7 @@ cudaError_t launch_group_norm_backward_src(int kind, const float* dy, const void
     default: break;
   }
   if (e != cudaSuccess) return e;
-  k_gn_param_finish<<<nblk(C, PF_C), PF_NT, 0, st>>>(part, (int)B, C, dgamma, dbeta);
+  pdl_launch(k_gn_param_finish, dim3(nblk(C, PF_C)), dim3(PF_NT), 0, st, part, (int)B, C, dgamma, dbeta);
   return cudaGetLastError();
 }
 
@@ -1061,8 +1068,7 @@ cudaError_t launch_relu_mask(const float* dy, const void* out, int64_t n, float*
 cudaError_t launch_maxpool(const void* x, int64_t B, int T, int C, void* y, uint8_t* arg, cudaStream_t st) {
   const int To = (T + 2 - 3) / 2 + 1;
   if (C % 8 == 0 && aligned16(x) && aligned16(y) && ((uintptr_t)arg & 7u) == 0) {
-    k_maxpool8<<<dim3(nblk((int64_t)To * C / 8, 256), (unsigned)B), 256, 0, st>>>(
-        reinterpret_cast<const __nv_bfloat16*>(x), T, C, To, reinterpret_cast<__nv_bfloat16*>(y), arg);
+    pdl_launch(k_maxpool8, dim3(dim3(nblk((int64_t)To * C / 8, 256), (unsigned)B)), dim3(256), 0, st, reinterpret_cast<const __nv_bfloat16*>(x), T, C, To, reinterpret_cast<__nv_bfloat16*>(y), arg);
     return cudaGetLastError();
   }
   k_maxpool<<<dim3(nblk((int64_t)To * C, 256), (unsigned)B), 256, 0, st>>>(
@@ -1084,7 +1090,7 @@ cudaError_t launch_mean_time(const void* x, int64_t B, int T, int C, void* m, cu
   const auto x16 = reinterpret_cast<const __nv_bfloat16*>(x);
   const auto m16 = reinterpret_cast<__nv_bfloat16*>(m);
   if (C % 2 == 0 && ((uintptr_t)x & 3u) == 0 && ((uintptr_t)m & 3u) == 0)
-    k_mean_time2<<<nblk(B * C / 2, 64), 64, 0, st>>>(x16, B, T, C, m16);
+    pdl_launch(k_mean_time2, dim3(nblk(B * C / 2, 64)), dim3(64), 0, st, x16, B, T, C, m16);
   else
     k_mean_time<<<nblk(B * C, 64), 64, 0, st>>>(x16, B, T, C, m16);
   return cudaGetLastError();
