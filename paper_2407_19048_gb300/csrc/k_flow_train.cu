@@ -22,7 +22,7 @@
 // sum).  Latency bound: one tile's chain MMA -> drain -> MMA, 6.4 us a layer of 256 in the
 // density with what it keeps (3.8 without; 6.9 with the operands in shared memory), 7.9 in the
 // backward; a batch of 4096 fills 32 SMs.  As ~370 launches of 3 to 13 us (each layer: input
-// rows, three products, coupling step; backward 17 kernels) the step took 3.04 ms, now 0.55.
+// rows, three products, coupling step; backward 17 kernels) the step took 3.04 ms, now 0.45.
 #include "flow_tile.cuh"
 #include "pdl.cuh"
 #include "sum2.cuh"
