@@ -7,7 +7,7 @@ the shortcut), the mean over time and a fully connected layer to the representat
 The stride-1 kernel-5 convolutions are implicit GEMMs on the tensor cores
 (`gwx_conv1d_bf16`: the A tiles come from a 3-D tensor map of the activations; backward
 `gwx_conv1d_bf16_backward`: the input gradient is the same product with mirrored taps, the
-weight gradient a split-K product over transposed rows); the stem, the strided entries and
+weight gradient a split-K product of rows read as they lie); the stem, the strided entries and
 the 1 x 1 shortcuts use im2col rows times the weights (`gwx_im2col`, `gwx_dense_bf16`;
 backward `gwx_dense_bf16_backward`, `gwx_col2im`).  Normalisation, residual addition and
 ReLU are fused (`gwx_group_norm`), and the backward pass mirrors the forward call by call.
