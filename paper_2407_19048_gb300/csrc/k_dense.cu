@@ -25,7 +25,7 @@ constexpr int TT = 32;   // rows of a column-sum partial; columns of a k_colsum 
 // since a positive float never rounds to a bfloat16 zero short of 1e-40) in bfloat16, and the
 // FP32 column sums of every 32 rows into part.  HBM bound: a warp takes 32 rows x 64 columns,
 // 256-byte row segments in (sixteen in flight), 128-byte segments out.
-__global__ void __launch_bounds__(256) k_dz_rows(const float* __restrict__ dY, const __nv_bfloat16* __restrict__ Y,
+__global__ void __launch_bounds__(256) k_dz_rows(const float* dY, const __nv_bfloat16* Y,
                                                  int64_t M, int N, __nv_bfloat16* __restrict__ dZ,
                                                  float* __restrict__ part) {
   pdl_enter();
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(256) k_dz_rows(const float* __restrict__ dY, c
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const int64_t at = (m0 + min(r0 + i, rows - 1)) * N + col;
-      v[i] = pairs ? __ldca(reinterpret_cast<const float2*>(dY + at)) : make_float2(__ldca(dY + at), __ldca(dY + at + 1));
+      v[i] = pairs ? *reinterpret_cast<const float2*>(dY + at) : make_float2(dY[at], dY[at + 1]);
       if (Y != nullptr) y[i] = *reinterpret_cast<const __nv_bfloat162*>(Y + at);
     }
 #pragma unroll
@@ -72,7 +72,7 @@ constexpr int CS_MAX_SLICES = 64;
 
 int colsum_slices(int64_t P) { return (int)std::min<int64_t>(CS_MAX_SLICES, std::max<int64_t>(1, (P + 255) / 256)); }
 
-__global__ void __launch_bounds__(1024) k_colsum(const float* __restrict__ part, int P, int N,
+__global__ void __launch_bounds__(1024) k_colsum(const float* part, int P, int N,
                                                  double* __restrict__ part2, float* __restrict__ db) {
   pdl_enter();
   __shared__ float2 red[TT][TT + 1];
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(1024) k_colsum(const float* __restrict__ part,
   Sum2 s;
   if (n < N)
 #pragma unroll 4
-    for (int p = p0 + threadIdx.y; p < p1; p += TT) s.add(__ldca(&part[(int64_t)p * N + n]));
+    for (int p = p0 + threadIdx.y; p < p1; p += TT) s.add(part[(int64_t)p * N + n]);
   red[threadIdx.y][threadIdx.x] = make_float2(s.h, s.l);
   __syncthreads();
   const float2 v = red[threadIdx.x][threadIdx.y];
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(1024) k_colsum(const float* __restrict__ part,
   }
 }
 
-__global__ void k_colsum_finish(const double* __restrict__ part2, int slices, int N, float* __restrict__ db) {
+__global__ void k_colsum_finish(const double* part2, int slices, int N, float* __restrict__ db) {
   pdl_enter();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;

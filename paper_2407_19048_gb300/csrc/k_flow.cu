@@ -68,7 +68,7 @@ __device__ __forceinline__ int64_t event_of(const int64_t* __restrict__ off, int
 // Four warps a block of 32 rows, one transcendental function of each row a warp: the FP64 chain of
 // a row is latency (4096 rows: 16 us with one thread a row in 32 blocks, 14.5 in 128, 7.0 now).
 constexpr int TGT_ROWS = 32;
-__global__ void __launch_bounds__(4 * TGT_ROWS) k_flow_targets(const double* __restrict__ theta, int64_t B, Std8 st,
+__global__ void __launch_bounds__(4 * TGT_ROWS) k_flow_targets(const double* theta, int64_t B, Std8 st,
                                                                float* __restrict__ x) {
   pdl_enter();
   __shared__ double f[4][TGT_ROWS];
@@ -249,8 +249,8 @@ __global__ void __launch_bounds__(ROW_NT) k_flow_base(uint32_t k0, uint32_t k1, 
   reinterpret_cast<float2*>(z)[at] = make_float2(rad * cs, rad * sn);
 }
 
-__global__ void k_flow_proposal(const float* __restrict__ x, const float* __restrict__ z,
-                                const float* __restrict__ sum_s, int64_t n, int64_t row0, int64_t S, Std8 st,
+__global__ void k_flow_proposal(const float* x, const float* z, const float* sum_s, int64_t n, int64_t row0,
+                                int64_t S, Std8 st,
                                 gwx_prior pr, uint32_t k0, uint32_t k1, uint32_t counter,
                                 double* __restrict__ theta, double* __restrict__ log_q,
                                 double* __restrict__ log_ratio) {

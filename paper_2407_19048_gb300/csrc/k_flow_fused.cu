@@ -95,14 +95,14 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
         int64_t lo = 0, hi = a.E, s = a.row0 + row;
         while (hi - lo > 1) {
           const int64_t mid = (lo + hi) >> 1;
-          if (__ldca(&a.off[mid]) <= s) lo = mid; else hi = mid;
+          if (a.off[mid] <= s) lo = mid; else hi = mid;
         }
         e = lo;
       }
       const uint4* crow = reinterpret_cast<const uint4*>(a.ctx + e * C);
       for (int g = h == 0 ? 1 : 4 * h; g < 4 * h + 4; ++g) {
         uint4 d = make_uint4(0u, 0u, 0u, 0u);
-        if (valid && g <= C / 8) d = __ldca(crow + (g - 1));
+        if (valid && g <= C / 8) d = crow[g - 1];
         sts128(sx + KB_BYTES * (g >> 3) + swz(r, g & 7), d.x, d.y, d.z, d.w);
       }
       for (int l = 0; l < K; ++l, ++li) {

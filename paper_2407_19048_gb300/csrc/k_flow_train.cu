@@ -227,14 +227,14 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
         int64_t lo = 0, hi = a.E, s = a.row0 + row;
         while (hi - lo > 1) {
           const int64_t mid = (lo + hi) >> 1;
-          if (__ldca(&a.off[mid]) <= s) lo = mid; else hi = mid;
+          if (a.off[mid] <= s) lo = mid; else hi = mid;
         }
         e = lo;
       }
       const uint4* crow = reinterpret_cast<const uint4*>(a.ctx + e * C);
       for (int g = h == 0 ? 1 : 4 * h; g < 4 * h + 4; ++g) {
         uint4 x = make_uint4(0u, 0u, 0u, 0u);
-        if (valid && g <= C / 8) x = __ldca(crow + (g - 1));
+        if (valid && g <= C / 8) x = crow[g - 1];
         sts128(sx + KB_BYTES * (g >> 3) + swz(r, g & 7), x.x, x.y, x.z, x.w);
       }
       // chunk c (32 columns) of a hidden layer: signs and activations out, when the chunk before has
@@ -556,8 +556,8 @@ __global__ void __launch_bounds__(F_THREADS, 1)
         for (int rd = 0; rd < 2; ++rd) {
           const bool have = valid && rd < NR;
           const int64_t m = mask_at(l, wrow / 32, a.P, H / 32, 2 * (2 * rd + h)) + lane;
-          k2[rd] = have ? make_uint2(__ldca(&a.m2[m]), __ldca(&a.m2[m + 32])) : make_uint2(0u, 0u);
-          k1[rd] = have ? make_uint2(__ldca(&a.m1[m]), __ldca(&a.m1[m + 32])) : make_uint2(0u, 0u);
+          k2[rd] = have ? make_uint2(a.m2[m], a.m2[m + 32]) : make_uint2(0u, 0u);
+          k1[rd] = have ? make_uint2(a.m1[m], a.m1[m + 32]) : make_uint2(0u, 0u);
         }
         if (h == 0) {
           float d[8];
@@ -660,11 +660,11 @@ __global__ void __launch_bounds__(F_THREADS, 1)
 // (p1, p2, p3: H, H and 8 columns) of layer l, 32 row lanes and then a warp a column, in
 // two-float arithmetic (FP64: 9.8 us for 16 layers of 256 and 128 partials, 6.2 now); the
 // extra block (0, K) sums the loss in FP64.
-__global__ void __launch_bounds__(1024) k_flow_bias_grads(const float* __restrict__ p1, const float* __restrict__ p2,
-                                                          const float* __restrict__ p3, int64_t P, int H, int K,
+__global__ void __launch_bounds__(1024) k_flow_bias_grads(const float* p1, const float* p2, const float* p3,
+                                                          int64_t P, int H, int K,
                                                           float* __restrict__ g1, float* __restrict__ g2,
                                                           float* __restrict__ g3, int64_t lstride,
-                                                          const double* __restrict__ loss_part, double n,
+                                                          const double* loss_part, double n,
                                                           double* __restrict__ loss) {
   pdl_enter();
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, l = blockIdx.y;
@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(1024) k_flow_bias_grads(const float* __restric
   Sum2 s;
   if (col0 + tx < cols)
 #pragma unroll 4
-    for (int64_t i = ty; i < P; i += 32) s.add(__ldca(&p[i * cols + col0 + tx]));
+    for (int64_t i = ty; i < P; i += 32) s.add(p[i * cols + col0 + tx]);
   red[ty][tx] = make_float2(s.h, s.l);
   __syncthreads();
   const float2 v = red[tx][ty];

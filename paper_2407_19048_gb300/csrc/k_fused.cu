@@ -160,19 +160,19 @@ template <bool VEC, int T>
 __device__ __forceinline__ float2 crop_point(const float* row, int m, bool odd, int lane, int64_t at, int64_t DL) {
   if constexpr (!VEC) {
     const int o = odd ? 1 : 0;
-    return GWX_IDX_OK(at + o + 1, DL, 0x101) ? make_float2(__ldca(&row[o + 2 * m]), __ldca(&row[o + 2 * m + 1]))
+    return GWX_IDX_OK(at + o + 1, DL, 0x101) ? make_float2(row[o + 2 * m], row[o + 2 * m + 1])
                                             : make_float2(0.f, 0.f);
   } else {
     const float2* row2 = reinterpret_cast<const float2*>(row);
-    const float2 q = GWX_IDX_OK(at + 1, DL, 0x102) ? __ldca(&row2[m]) : make_float2(0.f, 0.f);
+    const float2 q = GWX_IDX_OK(at + 1, DL, 0x102) ? row2[m] : make_float2(0.f, 0.f);
     if (!odd) return q;
     // the window starts at an odd sample: pair (own .y, next pair's .x)
     float nx;
     if constexpr (T >= 32) {
       nx = __shfl_down_sync(0xffffffffu, q.x, 1);
-      if (lane == 31) nx = GWX_IDX_OK(at + 2, DL, 0x103) ? __ldca(&row[2 * m + 2]) : 0.f;
+      if (lane == 31) nx = GWX_IDX_OK(at + 2, DL, 0x103) ? row[2 * m + 2] : 0.f;
     } else {
-      nx = GWX_IDX_OK(at + 2, DL, 0x103) ? __ldca(&row[2 * m + 2]) : 0.f;
+      nx = GWX_IDX_OK(at + 2, DL, 0x103) ? row[2 * m + 2] : 0.f;
     }
     return make_float2(q.y, nx);
   }
@@ -200,7 +200,7 @@ struct CropCopy {
 };
 __device__ __forceinline__ CropCopy crop_copy(const int64_t* offsets, int64_t b, int d, int64_t L, int64_t N,
                                               int64_t DL) {
-  int64_t off = __ldcg(&offsets[b]);
+  int64_t off = offsets[b];
   off = off < 0 ? 0 : (off > L - N ? L - N : off);   // keep a bad offset inside the stretch
   const int64_t first = (int64_t)d * L + off;
   CropCopy c;
@@ -241,9 +241,9 @@ __device__ __forceinline__ CropCopy window_copy(const int64_t* offsets, int64_t 
 // are dealt out (sim_split).
 template <int LOGN, bool VEC, bool PP, bool ST, bool WAVE>
 __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
-    k_simulate(const DrawCoef* __restrict__ coef, const float* __restrict__ noise, int64_t L,
-               const int64_t* __restrict__ offsets, const float* __restrict__ W, int64_t Wcap, int k_lo, int D,
-               int64_t B, int nd, float* __restrict__ y) {
+    k_simulate(const DrawCoef* coef, const float* noise, int64_t L,
+               const int64_t* offsets, const float* W, int64_t Wcap, int k_lo, int D,
+               int64_t B, int nd, float* y) {
   static_assert(!(ST && PP), "staging uses the in-place passes");
   static_assert(WAVE || !PP, "whitening alone uses the in-place passes");
   using PL = SimPlan<LOGN, WAVE>;
@@ -274,8 +274,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
   // follow from it by fixed rotations
   const float2 bt = cconj(__ldg(&g_tw[t << (13 - LOGN)]));
   // everything up to here overlaps the end of the kernel before this one (launch_simulate_lg);
-  // what that kernel wrote is not read-only for this one, so no load below goes by way of __ldg
-  // but those of the constant tables
+  // the reads below keep the rule of pdl.cuh (whitening also writes over its own windows)
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   if constexpr (ST) {
@@ -305,10 +304,10 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
     const int d_first = (int)(u - b * per);
     if constexpr (WAVE)
       for (int i = t; i < (int)(sizeof(DrawCoef) / 16); i += T)
-        reinterpret_cast<int4*>(&sc)[i] = __ldcg(reinterpret_cast<const int4*>(coef + b) + i);
+        reinterpret_cast<int4*>(&sc)[i] = reinterpret_cast<const int4*>(coef + b)[i];
     int64_t off = 0;
     if constexpr (WAVE && !ST) {
-      off = __ldcg(&offsets[b]);
+      off = offsets[b];
       off = off < 0 ? 0 : (off > L - N ? L - N : off);   // keep a bad offset inside the stretch
     }
     const int64_t a0 = off & ~(int64_t)1;
@@ -456,7 +455,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
       }
       // s_k = W_k / n for bin k of this detector, rounded on its own (an explicit product
       // cannot be fused into a later addition, so every launch shape rounds alike)
-      auto s_of = [&](int k) -> float { return __fmul_rn(ST ? w_s[ow + k] : __ldca(&Wd[k]), inv_n); };
+      auto s_of = [&](int k) -> float { return __fmul_rn(ST ? w_s[ow + k] : Wd[k], inv_n); };
       float2 vA[SLOTS][RL], vB[SLOTS][RL];
 #pragma unroll
       for (int s = 0; s < SLOTS; ++s) {

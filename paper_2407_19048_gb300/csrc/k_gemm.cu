@@ -117,9 +117,9 @@ __device__ __forceinline__ float act_grad(float z, int act) {
 __device__ int g_gemm_status;
 
 // Four consecutive floats from p (n of them exist; vec: p is 16-byte aligned and n >= 4).
-__device__ __forceinline__ float4 load4(const float* __restrict__ p, int n, bool vec) {
-  if (vec) return __ldca(reinterpret_cast<const float4*>(p));
-  return make_float4(__ldca(p), n > 1 ? __ldca(p + 1) : 0.f, n > 2 ? __ldca(p + 2) : 0.f, n > 3 ? __ldca(p + 3) : 0.f);
+__device__ __forceinline__ float4 load4(const float* p, int n, bool vec) {
+  if (vec) return *reinterpret_cast<const float4*>(p);
+  return make_float4(p[0], n > 1 ? p[1] : 0.f, n > 2 ? p[2] : 0.f, n > 3 ? p[3] : 0.f);
 }
 
 __device__ __forceinline__ float act_of(float z, int act) {
@@ -187,8 +187,8 @@ __device__ __forceinline__ WorkItem work_item(const WorkMap& m, int w) {
 template <int OUT, int TN_, int OPS, int MW = 1>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     k_gemm_bf16(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, void* __restrict__ C,
-                const float* __restrict__ bias, int act, const WorkMap map, int M, int N, int K, int kbs, int splits,
-                const float* __restrict__ extra, float* __restrict__ colsum, int groups, int64_t cstride,
+                const float* bias, int act, const WorkMap map, int M, int N, int K, int kbs, int splits,
+                const float* extra, float* __restrict__ colsum, int groups, int64_t cstride,
                 ConvGeo geo) {
   static_assert(MW == 1 || OPS == OP_KK, "wide tiles are for plain products");
   constexpr bool A_MN = op_a_mn(OPS), B_MN = op_b_mn(OPS);
@@ -559,7 +559,7 @@ bool make_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t K, uint32
 // slices of a small result (64 of 64 x 320: 21 us one thread an element, 5 with eight lanes),
 // one for few slices of a large one (4 of 512 x 1968), where idle lanes only cost.
 template <int LANES>
-__global__ void __launch_bounds__(256) k_split_reduce(const float4* __restrict__ part, int splits, int64_t n4,
+__global__ void __launch_bounds__(256) k_split_reduce(const float4* part, int splits, int64_t n4,
                                                       int64_t ostride4, float4* __restrict__ out) {
   pdl_enter();
   constexpr int X = 256 / LANES;
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(256) k_split_reduce(const float4* __restrict__
   };
   if (i < n4) {
 #pragma unroll 4
-    for (int s = y; s < splits; s += LANES) add(__ldca(p + (int64_t)s * total));
+    for (int s = y; s < splits; s += LANES) add(p[(int64_t)s * total]);
   }
   if constexpr (LANES > 1) {
     red[y][x] = acc;

@@ -106,7 +106,7 @@ __global__ void k_lag_features(const float2* __restrict__ Y, int D, int64_t F, i
 // us as three kernels, each reading the spectra, 16 now; one window 8.7 us, 3.5 now.)
 constexpr int SC_NT = 128;
 template <int D>
-__global__ void __launch_bounds__(SC_NT) k_spectral_columns(const float2* __restrict__ Y, int64_t F, int N, int k_lo,
+__global__ void __launch_bounds__(SC_NT) k_spectral_columns(const float2* Y, int64_t F, int N, int k_lo,
                                                             int G, int ng, int chunks, int F_pad, bool cross, bool lag,
                                                             __nv_bfloat16* __restrict__ out) {
   pdl_enter();
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(SC_NT) k_spectral_columns(const float2* __rest
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     pw[d] = nb[d] = lre[d] = lim[d] = 0.f;
-    u[d] = __ldca(y + d * F);
+    u[d] = y[d * F];
   }
 #pragma unroll
   for (int p = 0; p < P; ++p) cre[p] = cim[p] = 0.f;
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(SC_NT) k_spectral_columns(const float2* __rest
   for (int k = 0; k < G; ++k) {
     float2 v[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) v[d] = lag || k + 1 < G ? __ldca(y + d * F + k + 1) : make_float2(0.f, 0.f);
+    for (int d = 0; d < D; ++d) v[d] = lag || k + 1 < G ? y[d * F + k + 1] : make_float2(0.f, 0.f);
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       pw[d] = fmaf(u[d].x, u[d].x, fmaf(u[d].y, u[d].y, pw[d]));

@@ -34,7 +34,7 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 // cols[(b To + t) K + j C + c] = x[b][s t + j - p][c] (zero outside the series and for
 // columns >= k C); one thread per 8 columns (C % 8 == 0, so a chunk stays in one tap).
-__global__ void k_im2col(const __nv_bfloat16* __restrict__ x, int T, int C, int k, int s, int p, int To, int K,
+__global__ void k_im2col(const __nv_bfloat16* x, int T, int C, int k, int s, int p, int To, int K,
                          __nv_bfloat16* __restrict__ cols) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -66,7 +66,7 @@ __global__ void k_im2col_cf(const float* __restrict__ y, int D, int N, int k, in
 
 // The same, 8 columns (16 bytes) a thread (one column: 34 us for 512 windows of 2 x 2048 samples,
 // 7 taps; now 11).
-__global__ void k_im2col_cf8(const float* __restrict__ y, int D, int N, int k, int s, int p, int To, int K,
+__global__ void k_im2col_cf8(const float* y, int D, int N, int k, int s, int p, int To, int K,
                              __nv_bfloat16* __restrict__ cols) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -79,7 +79,7 @@ __global__ void k_im2col_cf8(const float* __restrict__ y, int D, int N, int k, i
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
     const int src = s * t + j - p;
-    v[e] = j < k && src >= 0 && src < N ? __ldca(y + (b * D + c) * N + src) : 0.f;
+    v[e] = j < k && src >= 0 && src < N ? y[(b * D + c) * N + src] : 0.f;
     if (++c == D) c = 0, ++j;
   }
   __align__(16) __nv_bfloat162 h[4];
@@ -109,8 +109,8 @@ __global__ void k_col2im(const float* __restrict__ dcols, int T, int C, int k, i
 // The same with KT taps known at compile time and four channels per thread: all taps'
 // float4 loads are issued before the sums (in tap order, as above).
 template <int KT>
-__global__ void k_col2im4(const float* __restrict__ dcols, int T, int C, int s, int p, int To, int K,
-                          const float* __restrict__ addend, float* __restrict__ dx) {
+__global__ void k_col2im4(const float* dcols, int T, int C, int s, int p, int To, int K,
+                          const float* addend, float* __restrict__ dx) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= T * C / 4) return;
@@ -122,7 +122,7 @@ __global__ void k_col2im4(const float* __restrict__ dcols, int T, int C, int s, 
     const int num = t + p - j;
     const int to = num / s;
     v[j] = (num >= 0 && num - to * s == 0 && to < To)
-               ? __ldca(reinterpret_cast<const float4*>(dcols + (b * To + to) * K + j * C + c))
+               ? *reinterpret_cast<const float4*>(dcols + (b * To + to) * K + j * C + c)
                : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   const int64_t o = b * T * C + 4 * (int64_t)i;
@@ -170,18 +170,18 @@ __global__ void __launch_bounds__(256) k_gn_stats(const float* __restrict__ z, i
                                                   float* __restrict__ ms) {
   const int b = blockIdx.x / G, g = blockIdx.x - (blockIdx.x / G) * G, cg = C / G, cv = cg / VEC;
   const float* zb = z + (int64_t)b * T * C + g * cg;
-  const float k0 = __ldca(zb);
+  const float k0 = __ldg(zb);
   float s1 = 0.f, s2 = 0.f;
 #pragma unroll 4
   for (int e = threadIdx.x; e < T * cv; e += blockDim.x) {
     const int t = e / cv, c = (e - t * cv) * VEC;
     if constexpr (VEC == 4) {
-      const float4 v = __ldca(reinterpret_cast<const float4*>(zb + (int64_t)t * C + c));
+      const float4 v = __ldg(reinterpret_cast<const float4*>(zb + (int64_t)t * C + c));
       const float d0 = v.x - k0, d1 = v.y - k0, d2 = v.z - k0, d3 = v.w - k0;
       s1 += (d0 + d1) + (d2 + d3);
       s2 += fmaf(d0, d0, __fmul_rn(d1, d1)) + fmaf(d2, d2, __fmul_rn(d3, d3));
     } else {
-      const float d = __ldca(zb + (int64_t)t * C + c) - k0;
+      const float d = __ldg(zb + (int64_t)t * C + c) - k0;
       s1 += d;
       s2 += d * d;
     }
@@ -270,11 +270,9 @@ __device__ __forceinline__ uint2 to_bf16x4(float a, float b, float c, float d) {
   return make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
 }
 
-__global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restrict__ z, int T, int C, int G,
-                                                           double inv_n, const float* __restrict__ gamma,
-                                                           const float* __restrict__ beta,
-                                                           const float* __restrict__ res32,
-                                                           const __nv_bfloat16* __restrict__ res16, int relu,
+__global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* z, int T, int C, int G,
+                                                           double inv_n, const float* gamma, const float* beta,
+                                                           const float* res32, const __nv_bfloat16* res16, int relu,
                                                            __nv_bfloat16* __restrict__ out16,
                                                            float* __restrict__ out32, float* __restrict__ ms) {
   pdl_enter();
@@ -284,7 +282,7 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
   const int q4 = threadIdx.x % cq, l0 = (threadIdx.x % 256) / cq, g = (4 * q4) / cg;
   const int64_t off = (int64_t)blockIdx.x * T * C;
   const float4* z4 = reinterpret_cast<const float4*>(z + off) + q4;   // row t at t cq
-  const float k0 = __ldca(z + off + g * cg);
+  const float k0 = z[off + g * cg];
   Sum2 a, q;
   for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_NT / 256) * 16 * rl) {
     float s1 = 0.f, s2 = 0.f;
@@ -294,7 +292,7 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int t = t0 + (8 * h + i) * rl;
-        v[i] = t < T ? __ldca(z4 + t * cq) : make_float4(k0, k0, k0, k0);   // adds zero
+        v[i] = t < T ? z4[t * cq] : make_float4(k0, k0, k0, k0);   // adds zero
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -306,11 +304,9 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
     a.add(s1);
     q.add(__fmul_rn(s2, GN_SCALE));
   }
-  const float kg = (int)threadIdx.x < G ? __ldca(z + off + threadIdx.x * cg) : 0.f;
-  const float4 gm = make_float4(__ldca(&gamma[4 * q4]), __ldca(&gamma[4 * q4 + 1]), __ldca(&gamma[4 * q4 + 2]),
-                                __ldca(&gamma[4 * q4 + 3]));
-  const float4 bt = make_float4(__ldca(&beta[4 * q4]), __ldca(&beta[4 * q4 + 1]), __ldca(&beta[4 * q4 + 2]),
-                                __ldca(&beta[4 * q4 + 3]));
+  const float kg = (int)threadIdx.x < G ? z[off + threadIdx.x * cg] : 0.f;
+  const float4 gm = make_float4(gamma[4 * q4], gamma[4 * q4 + 1], gamma[4 * q4 + 2], gamma[4 * q4 + 3]);
+  const float4 bt = make_float4(beta[4 * q4], beta[4 * q4 + 1], beta[4 * q4 + 2], beta[4 * q4 + 3]);
   sample_group_sums<GN_NT>(a, q, cq, cg, G, sums);
   __syncthreads();
   if ((int)threadIdx.x < G) {
@@ -330,9 +326,9 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* __restri
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int t = min(tb + k * step, T - 1);
-      x[k] = __ldcs(z4 + t * cq);
-      if (res32) r[k] = __ldca(reinterpret_cast<const float4*>(res32 + off) + t * cq + q4);
-      if (res16) r[k] = bf16x4(__ldca(reinterpret_cast<const uint2*>(res16 + off) + t * cq + q4));
+      x[k] = ld_stream(z4 + t * cq);
+      if (res32) r[k] = reinterpret_cast<const float4*>(res32 + off)[t * cq + q4];
+      if (res16) r[k] = bf16x4(reinterpret_cast<const uint2*>(res16 + off)[t * cq + q4]);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -380,17 +376,17 @@ __device__ __forceinline__ void gn_load(GnRow<SRC>& r, const GnSource& s, int64_
     r.v0 = r.v1 = make_float4(0.f, 0.f, 0.f, 0.f);
     r.a0 = r.a1 = make_uchar4(3, 3, 3, 3);
     if (to < s.To) {
-      r.v0 = __ldca(reinterpret_cast<const float4*>(s.dy + o));
-      r.a0 = __ldca(reinterpret_cast<const uchar4*>(s.arg + o));
+      r.v0 = *reinterpret_cast<const float4*>(s.dy + o);
+      r.a0 = *reinterpret_cast<const uchar4*>(s.arg + o);
     }
     if ((t & 1) && to + 1 < s.To) {
-      r.v1 = __ldca(reinterpret_cast<const float4*>(s.dy + o + C));
-      r.a1 = __ldca(reinterpret_cast<const uchar4*>(s.arg + o + C));
+      r.v1 = *reinterpret_cast<const float4*>(s.dy + o + C);
+      r.a1 = *reinterpret_cast<const uchar4*>(s.arg + o + C);
     }
   } else if constexpr (SRC != DY_MEAN) {
-    r.v0 = __ldca(reinterpret_cast<const float4*>(s.dy + i));
+    r.v0 = *reinterpret_cast<const float4*>(s.dy + i);
   }
-  if constexpr (SRC != DY_PLAIN) r.o = __ldca(reinterpret_cast<const uint2*>(s.out + i));
+  if constexpr (SRC != DY_PLAIN) r.o = *reinterpret_cast<const uint2*>(s.out + i);
 }
 
 template <int SRC>
@@ -415,9 +411,9 @@ __device__ __forceinline__ float4 gn_value(const GnRow<SRC>& r, int t, float4 me
 // per channel, this sample's sums of dy xhat and dy (part, [B][C][2] doubles), the partials
 // of dgamma and dbeta that k_gn_param_finish adds.
 template <int SRC, bool OUT16>
-__global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, const float* __restrict__ z, int T, int C,
-                                                            int G, double inv_n, const float* __restrict__ ms,
-                                                            const float* __restrict__ gamma, void* __restrict__ dz,
+__global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, const float* z, int T, int C,
+                                                            int G, double inv_n, const float* ms,
+                                                            const float* gamma, void* __restrict__ dz,
                                                             float* __restrict__ dsum, double* __restrict__ part) {
   pdl_enter();
   constexpr int GN_BT = gn_bt(SRC);
@@ -430,11 +426,10 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
   const int64_t b = blockIdx.x, off = b * T * C;
   const float4* z4 = reinterpret_cast<const float4*>(z + off) + q4;   // row t at t cq
   const float mean = ms[2 * (b * G + g)], rstd = ms[2 * (b * G + g) + 1];
-  const float4 gm = make_float4(__ldca(&gamma[4 * q4]), __ldca(&gamma[4 * q4 + 1]), __ldca(&gamma[4 * q4 + 2]),
-                                __ldca(&gamma[4 * q4 + 3]));
+  const float4 gm = make_float4(gamma[4 * q4], gamma[4 * q4 + 1], gamma[4 * q4 + 2], gamma[4 * q4 + 3]);
   float4 mdy = make_float4(0.f, 0.f, 0.f, 0.f);
   if constexpr (SRC == DY_MEAN) {
-    const float4 v = __ldca(reinterpret_cast<const float4*>(src.dy + b * C) + q4);
+    const float4 v = reinterpret_cast<const float4*>(src.dy + b * C)[q4];
     mdy = make_float4(v.x / T, v.y / T, v.z / T, v.w / T);
   }
   Sum2 a, q, pg[4], pb[4];
@@ -449,7 +444,7 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
       for (int i = 0; i < U; ++i) {
         const int t = min(t0 + (h + i) * rl, T - 1);
         gn_load<SRC>(r[i], src, b, t, 4 * q4, T, C);
-        x[i] = __ldca(z4 + t * cq);
+        x[i] = z4[t * cq];
       }
 #pragma unroll
       for (int i = 0; i < U; ++i) {
@@ -528,7 +523,7 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
     for (int k = 0; k < U; ++k) {
       const int t = min(tb + k * step, T - 1);
       gn_load<SRC>(r[k], src, b, t, 4 * q4, T, C);
-      x[k] = __ldcs(z4 + t * cq);
+      x[k] = ld_stream(z4 + t * cq);
     }
 #pragma unroll
     for (int k = 0; k < U; ++k) {
@@ -571,7 +566,7 @@ __global__ void k_gn_apply(const float* __restrict__ z, int T, int C, int G, con
     v[0] = z[i];
   }
 #pragma unroll
-  for (int u = 0; u < VEC; ++u) v[u] = fmaf((v[u] - mean) * rstd, __ldca(&gamma[c + u]), __ldca(&beta[c + u]));
+  for (int u = 0; u < VEC; ++u) v[u] = fmaf((v[u] - mean) * rstd, __ldg(&gamma[c + u]), __ldg(&beta[c + u]));
   if (res32) {
     if constexpr (VEC == 4) {
       const float4 q = *reinterpret_cast<const float4*>(res32 + i);
@@ -621,8 +616,8 @@ __global__ void k_relu_mask4(const float* __restrict__ dy, const __nv_bfloat16* 
                              float* __restrict__ d) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n4) return;
-  const float4 g = __ldca(reinterpret_cast<const float4*>(dy) + i);
-  const uint2 q = __ldca(reinterpret_cast<const uint2*>(out) + i);
+  const float4 g = __ldg(reinterpret_cast<const float4*>(dy) + i);
+  const uint2 q = __ldg(reinterpret_cast<const uint2*>(out) + i);
   const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.x));
   const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.y));
   reinterpret_cast<float4*>(d)[i] = make_float4(lo.x > 0.f ? g.x : 0.f, lo.y > 0.f ? g.y : 0.f,
@@ -643,18 +638,18 @@ __global__ void __launch_bounds__(256) k_gn_bwd_stats(const float* __restrict__ 
     const int t = e / cv, c = (e - t * cv) * VEC;
     const int64_t i = base + (int64_t)t * C + c;
     if constexpr (VEC == 4) {
-      const float4 d = __ldca(reinterpret_cast<const float4*>(dy + i));
-      const float4 x = __ldca(reinterpret_cast<const float4*>(z + i));
-      const float4 gm = make_float4(__ldca(&gamma[g * cg + c]), __ldca(&gamma[g * cg + c + 1]),
-                                    __ldca(&gamma[g * cg + c + 2]), __ldca(&gamma[g * cg + c + 3]));
+      const float4 d = __ldg(reinterpret_cast<const float4*>(dy + i));
+      const float4 x = __ldg(reinterpret_cast<const float4*>(z + i));
+      const float4 gm = make_float4(__ldg(&gamma[g * cg + c]), __ldg(&gamma[g * cg + c + 1]),
+                                    __ldg(&gamma[g * cg + c + 2]), __ldg(&gamma[g * cg + c + 3]));
       const float a0 = d.x * gm.x, a1 = d.y * gm.y, a2 = d.z * gm.z, a3 = d.w * gm.w;
       s1 += (a0 + a1) + (a2 + a3);
       s2 += (a0 * ((x.x - mean) * rstd) + a1 * ((x.y - mean) * rstd)) +
             (a2 * ((x.z - mean) * rstd) + a3 * ((x.w - mean) * rstd));
     } else {
-      const float a = __ldca(dy + i) * __ldca(&gamma[g * cg + c]);
+      const float a = __ldg(dy + i) * __ldg(&gamma[g * cg + c]);
       s1 += a;
-      s2 += a * ((__ldca(z + i) - mean) * rstd);
+      s2 += a * ((__ldg(z + i) - mean) * rstd);
     }
   }
   double a = s1, q = s2;
@@ -681,10 +676,10 @@ __global__ void k_gn_bwd_apply(const float* __restrict__ dy, const float* __rest
     const float4 d = *reinterpret_cast<const float4*>(dy + i);
     const float4 x = *reinterpret_cast<const float4*>(z + i);
     float4 o;
-    o.x = rstd * (d.x * __ldca(&gamma[c]) - m1 - (x.x - mean) * rstd * m2);
-    o.y = rstd * (d.y * __ldca(&gamma[c + 1]) - m1 - (x.y - mean) * rstd * m2);
-    o.z = rstd * (d.z * __ldca(&gamma[c + 2]) - m1 - (x.z - mean) * rstd * m2);
-    o.w = rstd * (d.w * __ldca(&gamma[c + 3]) - m1 - (x.w - mean) * rstd * m2);
+    o.x = rstd * (d.x * __ldg(&gamma[c]) - m1 - (x.x - mean) * rstd * m2);
+    o.y = rstd * (d.y * __ldg(&gamma[c + 1]) - m1 - (x.y - mean) * rstd * m2);
+    o.z = rstd * (d.z * __ldg(&gamma[c + 2]) - m1 - (x.z - mean) * rstd * m2);
+    o.w = rstd * (d.w * __ldg(&gamma[c + 3]) - m1 - (x.w - mean) * rstd * m2);
     *reinterpret_cast<float4*>(dz + i) = o;
   } else {
     dz[i] = rstd * (dy[i] * gamma[c] - m1 - (z[i] - mean) * rstd * m2);
@@ -715,8 +710,8 @@ __global__ void __launch_bounds__(256) k_gn_param_part(const float* __restrict__
       float fg = 0.f, fb = 0.f;
       for (int n = 0; n < 64 && r < r1; ++n) {
         const int64_t i = (int64_t)r * C + c;
-        const float d = __ldca(dy + i);
-        fg += d * ((__ldca(z + i) - ms[2 * (b * G + g)]) * ms[2 * (b * G + g) + 1]);
+        const float d = __ldg(dy + i);
+        fg += d * ((__ldg(z + i) - ms[2 * (b * G + g)]) * ms[2 * (b * G + g) + 1]);
         fb += d;
         r += 8;
         t += 8;
@@ -748,7 +743,7 @@ __global__ void __launch_bounds__(256) k_gn_param_part(const float* __restrict__
 // additions are spread over many SMs (512 slices of 128 channels: 4 blocks of 32 took 14.7 us,
 // 16 of 8 8.0, these 5.0).
 constexpr int PF_C = 2, PF_NT = 256;
-__global__ void __launch_bounds__(PF_NT) k_gn_param_finish(const double* __restrict__ part, int slices, int C,
+__global__ void __launch_bounds__(PF_NT) k_gn_param_finish(const double* part, int slices, int C,
                                                            float* __restrict__ dgamma, float* __restrict__ dbeta) {
   pdl_enter();
   __shared__ double2 r[PF_NT / 32][PF_C];
@@ -757,7 +752,7 @@ __global__ void __launch_bounds__(PF_NT) k_gn_param_finish(const double* __restr
   if (c < C) {
 #pragma unroll 4
     for (int s = threadIdx.x / PF_C; s < slices; s += PF_NT / PF_C) {
-      const double2 v = __ldca(reinterpret_cast<const double2*>(part) + (int64_t)s * C + c);
+      const double2 v = reinterpret_cast<const double2*>(part)[(int64_t)s * C + c];
       tg += v.x;
       tb += v.y;
     }
@@ -806,7 +801,7 @@ __global__ void k_maxpool(const __nv_bfloat16* __restrict__ x, int T, int C, int
 // The same for eight consecutive channels per thread (C % 8 == 0, 16-byte aligned x and y,
 // 8-byte aligned arg): one 16-byte load per tap (512 windows of 1024 x 64: 65 us one channel
 // a thread).
-__global__ void k_maxpool8(const __nv_bfloat16* __restrict__ x, int T, int C, int To, __nv_bfloat16* __restrict__ y,
+__global__ void k_maxpool8(const __nv_bfloat16* x, int T, int C, int To, __nv_bfloat16* __restrict__ y,
                            uint8_t* __restrict__ arg) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x, cv = C / 8;
@@ -817,7 +812,7 @@ __global__ void k_maxpool8(const __nv_bfloat16* __restrict__ x, int T, int C, in
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     const int src = 2 * t + j - 1;
-    v[j] = src >= 0 && src < T ? __ldca(reinterpret_cast<const uint4*>(x + (b * T + src) * C + c))
+    v[j] = src >= 0 && src < T ? *reinterpret_cast<const uint4*>(x + (b * T + src) * C + c)
                                : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);   // -inf: never first
   }
   const __nv_bfloat16* e0 = reinterpret_cast<const __nv_bfloat16*>(&v[0]);
@@ -870,8 +865,8 @@ __global__ void k_maxpool_back4(const float* __restrict__ dy, const uint8_t* __r
   for (int to = t / 2; to <= (t + 1) / 2; ++to) {
     if (to >= To) continue;
     const int64_t o = (b * To + to) * C + c;
-    const float4 d = __ldca(reinterpret_cast<const float4*>(dy + o));
-    const uchar4 a = __ldca(reinterpret_cast<const uchar4*>(arg + o));
+    const float4 d = __ldg(reinterpret_cast<const float4*>(dy + o));
+    const uchar4 a = __ldg(reinterpret_cast<const uchar4*>(arg + o));
     const int base = 2 * to - 1;
     if (base + (int)a.x == t) acc.x += d.x;
     if (base + (int)a.y == t) acc.y += d.y;
@@ -895,7 +890,7 @@ __global__ void k_mean_time(const __nv_bfloat16* __restrict__ x, int64_t B, int 
 
 // The same, two channels a thread and 32 loads in flight (512 windows of 256 x 128: 25.4 us with one
 // channel and 16 loads, now 12.7).
-__global__ void k_mean_time2(const __nv_bfloat16* __restrict__ x, int64_t B, int T, int C,
+__global__ void k_mean_time2(const __nv_bfloat16* x, int64_t B, int T, int C,
                              __nv_bfloat16* __restrict__ m) {
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -912,11 +907,11 @@ __global__ void k_mean_time2(const __nv_bfloat16* __restrict__ x, int64_t B, int
   for (; t + 32 <= T; t += 32) {
     uint32_t v[32];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = __ldca(p + (t + k) * h);
+    for (int k = 0; k < 32; ++k) v[k] = p[(t + k) * h];
 #pragma unroll
     for (int k = 0; k < 32; ++k) add(v[k]);
   }
-  for (; t < T; ++t) add(__ldca(p + t * h));
+  for (; t < T; ++t) add(p[t * h]);
   reinterpret_cast<__nv_bfloat162*>(m)[i] = __floats2bfloat162_rn(a0 / T, a1 / T);
 }
 

@@ -8,9 +8,15 @@
 // successor start.  So at most two kernels of a stream are on the GPU at once, no kernel can end
 // before its predecessors, and nothing that a block reads after entering can have been cached
 // before it was written.  Every block has to enter; a kernel launched the ordinary way may
-// enter as well (nothing to wait for).  (Flow gradients of 4096 windows, 28 launches, 510 -> 449
-// us; ResNet stem and two blocks, 54 launches, 1477 -> 1398; 4096 x 1968 x 512 dense forward and
-// backward, 6 launches, 75 -> 65; 20,000 posterior draws 185 -> 171.)
+// enter as well (nothing to wait for).
+// Reads behind the wait: plain loads by pointers without __restrict__ (or ld_stream).  A const
+// __restrict__ pointer promises that nobody writes its data while the kernel runs, which does
+// not hold here: the compiler may take the read-only path, or move the load up over the wait.  The
+// load intrinsics with a cache hint say nothing about their order either.  Constant tables may
+// go by way of __ldg.
+// (Flow gradients of 4096 windows, 28 launches, 510 -> 449 us; ResNet stem and two blocks, 54
+// launches, 1477 -> 1398; 4096 x 1968 x 512 dense forward and backward, 6 launches, 75 -> 65;
+// 20,000 posterior draws 185 -> 171.)
 #pragma once
 
 #include <utility>
@@ -22,6 +28,16 @@ namespace gwx {
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// A read that is not needed again (evicted first), in its place behind the wait.
+__device__ __forceinline__ float4 ld_stream(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p)
+               : "memory");
+  return v;
 }
 
 template <class... P, class... A>
