@@ -752,9 +752,9 @@ __global__ void __launch_bounds__(PF_NT) k_gn_param_finish(const double* part, i
   if (c < C) {
 #pragma unroll 4
     for (int s = threadIdx.x / PF_C; s < slices; s += PF_NT / PF_C) {
-      const double2 v = reinterpret_cast<const double2*>(part)[(int64_t)s * C + c];
-      tg += v.x;
-      tb += v.y;
+      const double* v = part + ((int64_t)s * C + c) * 2;   // (a caller's scratch: 8-byte aligned)
+      tg += v[0];
+      tb += v[1];
     }
   }
 #pragma unroll
