@@ -816,8 +816,8 @@ __global__ void k_maxpool8(const __nv_bfloat16* x, int T, int C, int To, __nv_bf
                                : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);   // -inf: never first
   }
   const __nv_bfloat16* e0 = reinterpret_cast<const __nv_bfloat16*>(&v[0]);
-  __nv_bfloat16 best[8];
-  uint8_t a[8];
+  __align__(16) __nv_bfloat16 best[8];   // stored whole below
+  __align__(8) uint8_t a[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     float m = -INFINITY;
