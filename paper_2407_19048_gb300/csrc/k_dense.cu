@@ -87,13 +87,11 @@ __global__ void __launch_bounds__(1024) k_colsum(const float* part, int P, int N
   const float2 v = red[threadIdx.x][threadIdx.y];
   s.h = v.x;
   s.l = v.y;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s.add_lanes(o);
   const int c = blockIdx.x * TT + threadIdx.y;
-  if (threadIdx.x == 0 && c < N) {
-    if (db) db[c] = (float)s.value();
-    else part2[(int64_t)blockIdx.y * N + c] = s.value();
-  }
+  warp_total(s, part + (int64_t)p0 * N + c, p1 - p0, N, c < N, [&](auto t) {
+    if (db) db[c] = t.rounded();
+    else part2[(int64_t)blockIdx.y * N + c] = t.value();
+  });
 }
 
 __global__ void k_colsum_finish(const double* part2, int slices, int N, float* __restrict__ db) {

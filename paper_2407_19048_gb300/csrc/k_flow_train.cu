@@ -696,10 +696,9 @@ __global__ void __launch_bounds__(1024) k_flow_bias_grads(const float* p1, const
   const float2 v = red[tx][ty];
   s.h = v.x;
   s.l = v.y;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s.add_lanes(o);
-  if (tx == 0 && col0 + ty < cols)
-    (kind == 0 ? g1 : (kind == 1 ? g2 : g3))[(int64_t)l * lstride + col0 + ty] = (float)s.value();
+  const int c = col0 + ty;
+  warp_total(s, p + c, P, cols, c < cols,
+             [&](auto t) { (kind == 0 ? g1 : (kind == 1 ? g2 : g3))[(int64_t)l * lstride + c] = t.rounded(); });
 }
 
 cudaError_t tile_grid(int64_t n, unsigned* grid) {

@@ -30,7 +30,8 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 // Index arithmetic: every kernel runs on a grid whose y coordinate is the sample b and
 // whose x threads cover one sample's elements, so the divisions below are 32-bit (the
 // C-ABI keeps T C below 2^31 and B below 65536); sums are FP32 per thread over a few
-// dozen terms and FP64 across threads (GB300's FP64 rate is a small fraction of FP32).
+// dozen terms, and FP64 or two floats across threads (GB300's FP64 rate is a small fraction of
+// FP32's).
 
 // cols[(b To + t) K + j C + c] = x[b][s t + j - p][c] (zero outside the series and for
 // columns >= k C); one thread per 8 columns (C % 8 == 0, so a chunk stays in one tap).
@@ -207,17 +208,22 @@ __global__ void __launch_bounds__(256) k_gn_stats(const float* __restrict__ z, i
 // Sums: thread (run slice s, row lane l, column quad q) reads runs of 16 rows, rl = 256 / (C / 4)
 // rows apart, of channels 4 q .. 4 q + 3, coalesced float4 loads; FP32 within a run (the
 // contractions spelled out: the compiler's choice changes with the code around), two-float sums
-// across runs (sum2.cuh; in FP64 forward 227 us, backward 510); then the lanes of each column quad and the quads of each group.
+// across runs (sum2.cuh; in FP64 forward 227 us, backward 510); then the lanes of each column
+// quad and the quads of each group.  A block whose totals leave the range of two floats takes its
+// sums again in FP64.
 constexpr int GN_NT = 512;
 // threads of the backward: the pooled gradient's rows hold twice the registers
 constexpr int gn_bt(int src) { return src == 2 ? 256 : 512; }
 
 // Sums of a (and q) over the threads of every group (out[2 g], out[2 g + 1], valid after the
 // caller's barrier): lanes of a warp that share a column quad by shuffles, the remaining rows
-// of quads in shared memory, one warp per group.
-template <int NT>
-__device__ __forceinline__ void sample_group_sums(Sum2 a, Sum2 q, int cq, int cg, int G, double* out) {
-  __shared__ float4 r[NT];   // (a, q) of a quad
+// of quads in shared memory (r, NT entries), one warp per group.  True where a sum of this thread
+// is not finite.
+struct __align__(16) QuadSums {
+  uint64_t a, q;   // as bits()
+};
+template <int NT, class S>
+__device__ __forceinline__ bool sample_group_sums(S a, S q, int cq, int cg, int G, QuadSums* r, double* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int o = 16; o >= cq; o >>= 1) {
     a.add_lanes(o);
@@ -225,20 +231,19 @@ __device__ __forceinline__ void sample_group_sums(Sum2 a, Sum2 q, int cq, int cg
   }
   const int rows = cq < 32 ? NT / 32 : NT / cq;
   if (cq >= 32) {
-    r[threadIdx.x] = make_float4(a.h, a.l, q.h, q.l);
+    r[threadIdx.x] = QuadSums{a.bits(), q.bits()};
   } else if (lane < cq) {
-    r[warp * cq + lane] = make_float4(a.h, a.l, q.h, q.l);
+    r[warp * cq + lane] = QuadSums{a.bits(), q.bits()};
   }
   __syncthreads();
   const int per = cg / 4;
+  bool over = false;
   for (int g = warp; g < G; g += NT / 32) {
-    Sum2 x, y;
+    S x, y;
     for (int i = lane; i < rows * per; i += 32) {
-      const float4 v = r[(i / per) * cq + g * per + i % per];
-      x.add(v.x);
-      x.l += v.y;
-      y.add(v.z);
-      y.l += v.w;
+      const QuadSums v = r[(i / per) * cq + g * per + i % per];
+      x.add_bits(v.a);
+      y.add_bits(v.q);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -249,7 +254,9 @@ __device__ __forceinline__ void sample_group_sums(Sum2 a, Sum2 q, int cq, int cg
       out[2 * g] = x.value();
       out[2 * g + 1] = y.value();
     }
+    over |= !x.finite() || !y.finite();
   }
+  return over;
 }
 
 // 1 / sqrt(v) in FP64 from the single-precision value and one Newton step (error below 1e-13; the
@@ -278,37 +285,43 @@ __global__ void __launch_bounds__(GN_NT, 2) k_gn_forward_s(const float* z, int T
   pdl_enter();
   __shared__ double sums[64];
   __shared__ float st[64];
+  __shared__ QuadSums quads[GN_NT];
   const int cq = C / 4, rl = 256 / cq, cg = C / G;
   const int q4 = threadIdx.x % cq, l0 = (threadIdx.x % 256) / cq, g = (4 * q4) / cg;
   const int64_t off = (int64_t)blockIdx.x * T * C;
   const float4* z4 = reinterpret_cast<const float4*>(z + off) + q4;   // row t at t cq
   const float k0 = z[off + g * cg];
-  Sum2 a, q;
-  for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_NT / 256) * 16 * rl) {
-    float s1 = 0.f, s2 = 0.f;
+  auto collect = [&](auto zero) {   // the sums, in the arithmetic of `zero`; true: out of its range
+    decltype(zero) a, q;
+    for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_NT / 256) * 16 * rl) {
+      float s1 = 0.f, s2 = 0.f;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float4 v[8];
+      for (int h = 0; h < 2; ++h) {
+        float4 v[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int t = t0 + (8 * h + i) * rl;
-        v[i] = t < T ? z4[t * cq] : make_float4(k0, k0, k0, k0);   // adds zero
+        for (int i = 0; i < 8; ++i) {
+          const int t = t0 + (8 * h + i) * rl;
+          v[i] = t < T ? z4[t * cq] : make_float4(k0, k0, k0, k0);   // adds zero
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float d0 = v[i].x - k0, d1 = v[i].y - k0, d2 = v[i].z - k0, d3 = v[i].w - k0;
+          s1 += (d0 + d1) + (d2 + d3);
+          s2 += fmaf(d0, d0, __fmul_rn(d1, d1)) + fmaf(d2, d2, __fmul_rn(d3, d3));
+        }
       }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float d0 = v[i].x - k0, d1 = v[i].y - k0, d2 = v[i].z - k0, d3 = v[i].w - k0;
-        s1 += (d0 + d1) + (d2 + d3);
-        s2 += fmaf(d0, d0, __fmul_rn(d1, d1)) + fmaf(d2, d2, __fmul_rn(d3, d3));
-      }
+      a.add(s1);
+      q.add(__fmul_rn(s2, GN_SCALE));
     }
-    a.add(s1);
-    q.add(__fmul_rn(s2, GN_SCALE));
-  }
+    return sample_group_sums<GN_NT>(a, q, cq, cg, G, quads, sums);
+  };
   const float kg = (int)threadIdx.x < G ? z[off + threadIdx.x * cg] : 0.f;
   const float4 gm = make_float4(gamma[4 * q4], gamma[4 * q4 + 1], gamma[4 * q4 + 2], gamma[4 * q4 + 3]);
   const float4 bt = make_float4(beta[4 * q4], beta[4 * q4 + 1], beta[4 * q4 + 2], beta[4 * q4 + 3]);
-  sample_group_sums<GN_NT>(a, q, cq, cg, G, sums);
-  __syncthreads();
+  if (__syncthreads_or(collect(Sum2()))) {
+    collect(Sum64());
+    __syncthreads();
+  }
   if ((int)threadIdx.x < G) {
     const int i = threadIdx.x;
     const double m = sums[2 * i] * inv_n, var = fmax(sums[2 * i + 1] * (inv_n / GN_SCALE) - m * m, 0.0);
@@ -418,8 +431,9 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
   pdl_enter();
   constexpr int GN_BT = gn_bt(SRC);
   __shared__ double sums[64];
-  __shared__ float2 pr[GN_BT * 8];
+  __shared__ uint64_t pr[GN_BT * 8];   // as bits()
   __shared__ float st[64];
+  __shared__ QuadSums quads[GN_BT];
   constexpr int U = 4;   // rows in flight
   const int cq = C / 4, rl = 256 / cq, cg = C / G;
   const int q4 = threadIdx.x % cq, l0 = (threadIdx.x % 256) / cq, g = (4 * q4) / cg;
@@ -432,88 +446,92 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
     const float4 v = reinterpret_cast<const float4*>(src.dy + b * C)[q4];
     mdy = make_float4(v.x / T, v.y / T, v.z / T, v.w / T);
   }
-  Sum2 a, q, pg[4], pb[4];
-  for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_BT / 256) * 16 * rl) {
-    float s1 = 0.f, s2 = 0.f;
-    float fg[4] = {0.f, 0.f, 0.f, 0.f}, fb[4] = {0.f, 0.f, 0.f, 0.f};
+  auto collect = [&](auto zero) {   // the sums, in the arithmetic of `zero`; true: out of its range
+    using S = decltype(zero);
+    S a, q, pg[4], pb[4];
+    for (int t0 = l0 + (threadIdx.x / 256) * 16 * rl; t0 < T; t0 += (GN_BT / 256) * 16 * rl) {
+      float s1 = 0.f, s2 = 0.f;
+      float fg[4] = {0.f, 0.f, 0.f, 0.f}, fb[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-    for (int h = 0; h < 16; h += U) {
-      GnRow<SRC> r[U];
-      float4 x[U];
+      for (int h = 0; h < 16; h += U) {
+        GnRow<SRC> r[U];
+        float4 x[U];
 #pragma unroll
-      for (int i = 0; i < U; ++i) {
-        const int t = min(t0 + (h + i) * rl, T - 1);
-        gn_load<SRC>(r[i], src, b, t, 4 * q4, T, C);
-        x[i] = z4[t * cq];
+        for (int i = 0; i < U; ++i) {
+          const int t = min(t0 + (h + i) * rl, T - 1);
+          gn_load<SRC>(r[i], src, b, t, 4 * q4, T, C);
+          x[i] = z4[t * cq];
+        }
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+          const int t = t0 + (h + i) * rl;
+          if (t >= T) break;
+          const float4 d = gn_value<SRC>(r[i], t, mdy);
+          const float a0 = d.x * gm.x, a1 = d.y * gm.y, a2 = d.z * gm.z, a3 = d.w * gm.w;
+          const float h0 = (x[i].x - mean) * rstd, h1 = (x[i].y - mean) * rstd, h2 = (x[i].z - mean) * rstd,
+                      h3 = (x[i].w - mean) * rstd;
+          s1 += (a0 + a1) + (a2 + a3);
+          s2 += (a0 * h0 + a1 * h1) + (a2 * h2 + a3 * h3);
+          fg[0] += d.x * h0;
+          fg[1] += d.y * h1;
+          fg[2] += d.z * h2;
+          fg[3] += d.w * h3;
+          fb[0] += d.x;
+          fb[1] += d.y;
+          fb[2] += d.z;
+          fb[3] += d.w;
+        }
       }
-#pragma unroll
-      for (int i = 0; i < U; ++i) {
-        const int t = t0 + (h + i) * rl;
-        if (t >= T) break;
-        const float4 d = gn_value<SRC>(r[i], t, mdy);
-        const float a0 = d.x * gm.x, a1 = d.y * gm.y, a2 = d.z * gm.z, a3 = d.w * gm.w;
-        const float h0 = (x[i].x - mean) * rstd, h1 = (x[i].y - mean) * rstd, h2 = (x[i].z - mean) * rstd,
-                    h3 = (x[i].w - mean) * rstd;
-        s1 += (a0 + a1) + (a2 + a3);
-        s2 += (a0 * h0 + a1 * h1) + (a2 * h2 + a3 * h3);
-        fg[0] += d.x * h0;
-        fg[1] += d.y * h1;
-        fg[2] += d.z * h2;
-        fg[3] += d.w * h3;
-        fb[0] += d.x;
-        fb[1] += d.y;
-        fb[2] += d.z;
-        fb[3] += d.w;
-      }
-    }
-    a.add(s1);
-    q.add(s2);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      pg[m].add(fg[m]);
-      pb[m].add(fb[m]);
-    }
-  }
-  if (part) {
-    // lanes of a warp that share a column quad first, then one row of quads per warp
-    for (int o = 16; o >= cq; o >>= 1) {
+      a.add(s1);
+      q.add(s2);
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        pg[m].add_lanes(o);
-        pb[m].add_lanes(o);
+        pg[m].add(fg[m]);
+        pb[m].add(fb[m]);
       }
     }
-    const int lane = threadIdx.x & 31, at = cq >= 32 ? threadIdx.x : (threadIdx.x >> 5) * cq + lane;
-    if (cq >= 32 || lane < cq) {
+    if (part) {
+      // lanes of a warp that share a column quad first, then one row of quads per warp
+      for (int o = 16; o >= cq; o >>= 1) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        pr[at * 8 + m] = make_float2(pg[m].h, pg[m].l);
-        pr[at * 8 + 4 + m] = make_float2(pb[m].h, pb[m].l);
+        for (int m = 0; m < 4; ++m) {
+          pg[m].add_lanes(o);
+          pb[m].add_lanes(o);
+        }
+      }
+      const int lane = threadIdx.x & 31, at = cq >= 32 ? threadIdx.x : (threadIdx.x >> 5) * cq + lane;
+      if (cq >= 32 || lane < cq) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          pr[at * 8 + m] = pg[m].bits();
+          pr[at * 8 + 4 + m] = pb[m].bits();
+        }
       }
     }
+    bool over = sample_group_sums<GN_BT>(a, q, cq, cg, G, quads, sums);
+    if (part) {
+      // one thread per channel and sum, over the rows of quads in order
+      const int rows = cq < 32 ? GN_BT / 32 : GN_BT / cq;
+      for (int i = threadIdx.x; i < 2 * C; i += GN_BT) {
+        const int c = i >> 1, k = (c & 3) + 4 * (i & 1);
+        S t;
+#pragma unroll 4
+        for (int r = 0; r < rows; ++r) t.add_bits(pr[(r * cq + c / 4) * 8 + k]);
+        part[b * 2 * C + i] = t.value();
+        over |= !t.finite();
+      }
+    }
+    return over;
+  };
+  if (__syncthreads_or(collect(Sum2()))) {
+    collect(Sum64());
+    __syncthreads();
   }
-  sample_group_sums<GN_BT>(a, q, cq, cg, G, sums);
-  __syncthreads();
   if ((int)threadIdx.x < G) {
     st[2 * threadIdx.x] = (float)(sums[2 * threadIdx.x] * inv_n);
     st[2 * threadIdx.x + 1] = (float)(sums[2 * threadIdx.x + 1] * inv_n);
   }
   __syncthreads();
-  if (part) {
-    // one thread per channel and sum, over the rows of quads in order
-    const int rows = cq < 32 ? GN_BT / 32 : GN_BT / cq;
-    for (int i = threadIdx.x; i < 2 * C; i += GN_BT) {
-      const int c = i >> 1, k = (c & 3) + 4 * (i & 1);
-      Sum2 t;
-#pragma unroll 4
-      for (int r = 0; r < rows; ++r) {
-        const float2 v = pr[(r * cq + c / 4) * 8 + k];
-        t.add(v.x);
-        t.l += v.y;
-      }
-      part[b * 2 * C + i] = t.value();
-    }
-  }
   const float m1 = st[2 * g], m2 = st[2 * g + 1];
   const int step = GN_BT / cq;
   for (int tb = threadIdx.x / cq; tb < T; tb += U * step) {
