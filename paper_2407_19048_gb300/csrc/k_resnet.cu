@@ -259,11 +259,12 @@ __device__ __forceinline__ bool sample_group_sums(S a, S q, int cq, int cg, int 
   return over;
 }
 
-// 1 / sqrt(v) in FP64 from the single-precision value and one Newton step (error below 1e-13; the
-// library's FP64 call is a chain of some 2000 cycles here)
+// 1 / sqrt(v) in FP64 from the single-precision value and two Newton steps (errors of 2^-22, 1e-13
+// and FP64's rounding; the library's FP64 call is a chain of some 2000 cycles here)
 __device__ __forceinline__ double inv_sqrt(double v) {
   if (!(v < 1e30)) return rsqrt(v);
-  const double y = (double)rsqrtf((float)v);
+  double y = (double)rsqrtf((float)v);
+  y *= 1.5 - 0.5 * v * y * y;
   return y * (1.5 - 0.5 * v * y * y);
 }
 
