@@ -239,13 +239,16 @@ __device__ __forceinline__ CropCopy window_copy(const int64_t* offsets, int64_t 
 // those run three blocks an SM in fewer registers.)
 // nd: detectors of a draw that a block takes in turn: D, or 1 when windows rather than draws
 // are dealt out (sim_split).
-template <int LOGN, bool VEC, bool PP, bool ST, bool WAVE>
-__global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
+// GW (whitening alone, not staged): windows side by side in a block of one warp, n/16 threads
+// each (launch_whiten_windows).
+template <int LOGN, bool VEC, bool PP, bool ST, bool WAVE, int GW>
+__global__ void __launch_bounds__((1 << LOGN) / 16 * GW, GW > 1 ? 16 : (LOGN >= 13 ? 1 : 2))
     k_simulate(const DrawCoef* coef, const float* noise, int64_t L,
                const int64_t* offsets, const float* W, int64_t Wcap, int k_lo, int D,
                int64_t B, int nd, float* y) {
   static_assert(!(ST && PP), "staging uses the in-place passes");
   static_assert(WAVE || !PP, "whitening alone uses the in-place passes");
+  static_assert(GW == 1 || (!WAVE && !ST), "several windows a block: whitening from unstaged rows");
   using PL = SimPlan<LOGN, WAVE>;
   constexpr bool EXACT = !WAVE;
   constexpr bool R16 = PL::R16;
@@ -260,9 +263,10 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
   float* crop_s = reinterpret_cast<float*>(sm + (WAVE ? 2 : 1) * n);           // ST: N + 4 floats
   float* w_s = crop_s + N + 4;                                                  // ST: n + 4 floats
 #define WIDX(s, h, r) (((s) * 2 + (h)) * RL + (r))
-  const int t = threadIdx.x;
+  const int grp = GW == 1 ? 0 : threadIdx.x / T;   // this thread's window of the block's
+  const int t = threadIdx.x - grp * T;
   const int lane = t & 31;
-  const uint32_t x = smem_addr(sm), x2 = x + 8u * (uint32_t)n;
+  const uint32_t x = smem_addr(sm) + 8u * (uint32_t)(grp * n), x2 = x + 8u * (uint32_t)n;
   const float inv_n = 1.0f / (float)n;
   const int64_t DL = WAVE ? (int64_t)D * L : B * D * N;
   const int per = D / nd;                       // units of a draw: 1, or D single windows
@@ -299,7 +303,10 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
     __syncthreads();
   }
 
-  for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+  for (int64_t u0 = (int64_t)blockIdx.x * GW; u0 < units; u0 += (int64_t)gridDim.x * GW) {
+    // past the last window a group computes it again and stores nothing
+    const bool live = GW == 1 || u0 + grp < units;
+    const int64_t u = live ? u0 + grp : units - 1;
     const int64_t b = u / per;
     const int d_first = (int)(u - b * per);
     if constexpr (WAVE)
@@ -601,7 +608,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, LOGN >= 13 ? 1 : 2)
           dft8<true, EXACT>(v);
 #pragma unroll
           for (int r = 0; r < 8; ++r)
-            if (GWX_IDX_OK((b * D + d) * N + 2 * (j + r * (n / 8)) + 1, B * D * N, 0x104))
+            if (live && GWX_IDX_OK((b * D + d) * N + 2 * (j + r * (n / 8)) + 1, B * D * N, 0x104))
               __stcs(&out[j + r * (n / 8)], v[r]);
         }
       }
@@ -651,17 +658,17 @@ static bool sim_split(int64_t B, int D, int64_t slots) {
   return 5 * by_window < 4 * by_draw;
 }
 
-template <int LG, bool VEC, bool PP, bool ST, bool WAVE = true>
+template <int LG, bool VEC, bool PP, bool ST, bool WAVE = true, int GW = 1>
 static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, int64_t L, const int64_t* offsets,
                                       const float* W, int64_t Wcap, int k_lo, int D, int64_t B, float* y,
                                       int per_sm_want, cudaStream_t s) {
-  constexpr int NT = Plan16<LG>::T;
+  constexpr int NT = Plan16<LG>::T * GW;
   constexpr size_t n = (size_t)1 << LG;
   // one (or two, PP) window buffers plus 16 waveform values per thread; staged: the crop
   // (N + 4 floats) and the filter (n + 4 floats) after them
-  const size_t smem = (PP ? 2 : 1) * n * sizeof(float2) + (WAVE ? (size_t)16 * NT * sizeof(float2) : 0) +
+  const size_t smem = (PP ? 2 : GW) * n * sizeof(float2) + (WAVE ? (size_t)16 * NT * sizeof(float2) : 0) +
                       (ST ? (2 * n + 4 + n + 4) * sizeof(float) : 0);
-  auto kern = k_simulate<LG, VEC, PP, ST, WAVE>;
+  auto kern = k_simulate<LG, VEC, PP, ST, WAVE, GW>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
@@ -680,7 +687,7 @@ static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, 
   if (per_sm_want > 0 && per_sm_want < per_sm) per_sm = per_sm_want;
   const int64_t slots = (int64_t)sms * per_sm;
   const int nd = !WAVE || sim_split(B, D, slots) ? 1 : D;
-  const int64_t units = B * (D / nd), grid = units < slots ? units : slots;
+  const int64_t units = (B * (D / nd) + GW - 1) / GW, grid = units < slots ? units : slots;
   // The blocks may start once every block of the kernel before has (k_prepare, k_whiten_filter say
   // so at their start) and wait for its end themselves: the launch and their set-up lie under it
   // (64 draws of two detectors 21.7 us a batch without, 20.1 with; whitening 3003 windows 79.9, 76.9).
@@ -699,12 +706,26 @@ static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, 
 
 // Whitening of the windows d [B][D][N] with the filter W (Wcap floats allocated): staged
 // wherever the rows may be copied in bulk, else read in pairs (a base 8-byte aligned only).
+// Windows of 256 and 512 samples have 8 and 16 threads: many of them share a block of one full
+// warp, four or two at a time.  (20,000 x 2 windows, one a block 86.1 and 90.8 us, four or two
+// 34.9 and 50.3, in blocks of 128 threads 34.9 and 54; 600 windows 6.05 and 6.37, 1000 6.56
+// both, 2000 9.1 and 7.0, of 256 samples: from about six windows an SM on it pays, and four is
+// where one a block is left.)
 cudaError_t launch_whiten_windows(const float* d, const float* W, int64_t Wcap, int64_t B, int D, int64_t N, float* y,
                                   cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
   const bool st = (uintptr_t)d % 16 == 0 && (uintptr_t)W % 16 == 0;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const bool many = B * D > 4 * (int64_t)sms;
   return dispatch_log<7, 13>(ilog2_exact(N / 2), [&](auto cst) {
     constexpr int LG = decltype(cst)::value;
+    if constexpr (LG <= 8)
+      if (many)
+        return launch_simulate_lg<LG, true, false, false, false, (512 >> LG)>(nullptr, d, N, nullptr, W, Wcap, 0, D, B, y,
+                                                                              0, s);
     return st ? launch_simulate_lg<LG, true, false, true, false>(nullptr, d, N, nullptr, W, Wcap, 0, D, B, y, 0, s)
               : launch_simulate_lg<LG, true, false, false, false>(nullptr, d, N, nullptr, W, Wcap, 0, D, B, y, 0, s);
   });
