@@ -173,15 +173,73 @@ __device__ __forceinline__ WorkItem work_item(const WorkMap& m, int w) {
   return i;
 }
 
-// Persistent, warp-specialised: warp 0 lane 0 produces (TMA), warp 1 allocates tensor
-// memory and its lane 0 issues the MMAs, warps 2-9 drain accumulators.  MW = 1: two
+// The epilogue of a turned 32 x 32 tile at (row0, c0) whose rows are not multiples of four values: a
+// lane keeps P values of a row, W / P lanes a row (W = 8 in a narrow product), value by value to
+// memory, bfloat16 pairs whole where N is even.  Eight values are read, finished and written at a
+// time.  (8192 x 1001 x 512: four columns a lane 30.8 us FP32 and 30.7 bfloat16, value by value 24.6
+// and 24.7, now 18.2 and 18.6; 20000 x 7 x 128 8.3, now 6.3.)
+template <int OUT, int W>
+__device__ __forceinline__ void ragged_rows(uint32_t ebuf, void* out, const float* bias, int act, int row0, int c0, int M,
+                                            int N) {
+  constexpr int P = OUT == OUT_F32 ? 1 : 2, L = W / P, RPI = 32 / L;   // lanes a row, rows an iteration
+  int lane = threadIdx.x & 31;
+  asm volatile("" : "+r"(lane));   // (what follows from it is not kept in registers across the other path's loop)
+  const int cl = P * (lane % L), col = c0 + cl, rl = lane / L;
+  const bool in0 = col < N, in1 = P == 2 && col + 1 < N, pairs = N % 2 == 0;
+  const float b0 = bias != nullptr && in0 ? bias[col] : 0.f, b1 = bias != nullptr && in1 ? bias[col + 1] : 0.f;
+  constexpr int U = L < 8 ? L : 8;
+  int64_t at = (int64_t)(row0 + rl) * N + col;
+#pragma unroll 1
+  for (int k0 = 0; k0 < L; k0 += U) {
+    float v0[U], v1[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int r = RPI * (k0 + k) + rl;
+      const uint32_t src = ebuf + 128u * r + (uint32_t)(((cl >> 2) ^ (r & 7)) << 4) + 4u * (cl & 3);
+      if constexpr (P == 1) v0[k] = lds32(src);
+      else lds64(src, v0[k], v1[k]);
+    }
+    if (bias != nullptr) {
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        v0[k] += b0;
+        if (P == 2) v1[k] += b1;
+      }
+    }
+    if (act != 0) {
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        v0[k] = act_of(v0[k], act);
+        if (P == 2) v1[k] = act_of(v1[k], act);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k, at += (int64_t)RPI * N) {
+      if (row0 + RPI * (k0 + k) + rl >= M || !in0) continue;
+      if constexpr (P == 1) {
+        reinterpret_cast<float*>(out)[at] = v0[k];
+      } else {
+        __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(out) + at;
+        if (pairs) {
+          *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(v0[k], v1[k]);
+        } else {
+          o[0] = __float2bfloat16_rn(v0[k]);
+          if (in1) o[1] = __float2bfloat16_rn(v1[k]);
+        }
+      }
+    }
+  }
+}
+
+// Persistent, warp-specialised: warp 0 produces (TMA), warp 1 allocates tensor memory and
+// issues the MMAs, one elected lane of their uniform loops each; warps 2-9 drain accumulators.  MW = 1: two
 // TN_-column accumulators alternate between tiles, so a tile's epilogue overlaps the next
 // tile's main loop; MW = 2 (256 x 256 tiles): the two accumulators are the tile's two
 // 128-row halves and the next tile waits for both to drain.  "tfull" (MMA commit) and
 // "tempty" (one arrival per epilogue warp) hand them over.
 // TN_: tile width; OPS: operand layouts.  extra: with OUT_DACT the dY of C = dY act'(Z)
-// (any N); else an optional addend (N % 32 == 0, 16-byte aligned): C = (A B^T + addend),
-// then bias and activation.  colsum (OUT_DACT): [ceil(M/32)][N].
+// (N % 8 == 0, 4-byte aligned); of a convolution an optional addend (N % 64 == 0, 16-byte
+// aligned): C = A B^T + addend.  colsum (OUT_DACT): [ceil(M/32)][N], 16-byte aligned.
 // groups: independent products (OP_TN; map coordinate z), group g's C at + g cstride; with
 // splits > 1 the slice's partial product of group g at C + (slice groups + g) M N.
 template <int OUT, int TN_, int OPS, int MW = 1>
@@ -391,9 +449,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       const int row0 = tm * GMT + GM * msel + 32 * q;
       const int c_end = row0 < M ? min(c_hi, (N - tn * GN + 31) / 32) : c_lo;
       const uint32_t tcol = tmem + ((uint32_t)(32 * q) << 16) + (acc + (uint32_t)msel) * TMEM_COLS;
+      // Rows that are not multiples of four values (plain products alone; the others' N is a
+      // multiple of 8 and their C 16-byte aligned): ragged_rows.
       constexpr int ESZ = OUT == OUT_F32 ? 4 : 2;
       uint8_t* out = reinterpret_cast<uint8_t*>(C) + slice * ESZ;
-      const bool vec = N % 4 == 0 && (uintptr_t)out % (4 * ESZ) == 0;
+      constexpr bool EXTRA = OUT == OUT_DACT || op_conv_a(OPS);
+      constexpr bool RAGGED = OPS == OP_KK && OUT != OUT_DACT;
+      const bool vec = !RAGGED || (N % 4 == 0 && (uintptr_t)out % (4 * ESZ) == 0);
       const bool vec_b = (uintptr_t)bias % 16 == 0, vec_x = N % 4 == 0 && (uintptr_t)extra % 16 == 0;
       const int rl = lane >> 3, jc = lane & 7;
       uint32_t raw[32];
@@ -404,20 +466,28 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         // the rows' addend or dY, and the bias, before the accumulator, so that their latency
         // overlaps the tensor-memory load
         float4 x[8], b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (extra != nullptr) {
+        if (EXTRA && extra != nullptr) {
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
             const int r = row0 + 4 * k + rl;
             x[k] = r < M && left > 0 ? load4(extra + (int64_t)r * N + col, left, vec_x) : make_float4(0.f, 0.f, 0.f, 0.f);
           }
         }
-        if (bias != nullptr && left > 0) b4 = load4(bias + col, left, vec_b && left >= 4);
+        if (bias != nullptr && vec && left > 0) b4 = load4(bias + col, left, vec_b && left >= 4);
         tmem_wait_ld32(raw);
 #pragma unroll
         for (int j = 0; j < 8; ++j)
           sts128(ebuf + 128u * lane + (uint32_t)((j ^ (lane & 7)) << 4), raw[4 * j], raw[4 * j + 1], raw[4 * j + 2],
                  raw[4 * j + 3]);
         __syncwarp();
+        if (RAGGED && !vec) {
+          const int c0 = tn * GN + 32 * c;
+          if (N - c0 > 8) ragged_rows<OUT, 32>(ebuf, out, bias, act, row0, c0, M, N);
+          else ragged_rows<OUT, 8>(ebuf, out, bias, act, row0, c0, M, N);
+          __syncwarp();
+          if (c + 1 < c_end) tmem_ld32_async(tcol + 32u * (c + 1), raw);
+          continue;
+        }
         if (c + 1 < c_end) tmem_ld32_async(tcol + 32u * (c + 1), raw);
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f), vk[8];
 #pragma unroll
@@ -429,7 +499,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         for (int k = 0; k < 8; ++k) {
           const int grow = row0 + 4 * k + rl;
           float4 v = vk[k];
-          if (OUT != OUT_DACT && extra != nullptr) {
+          if (EXTRA && OUT != OUT_DACT && extra != nullptr) {
             v.x += x[k].x;
             v.y += x[k].y;
             v.z += x[k].z;
@@ -459,27 +529,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           }
           if (grow >= M || left <= 0) continue;
           if constexpr (OUT == OUT_F32) {
-            float* o = reinterpret_cast<float*>(out) + (int64_t)grow * N + col;
-            if (vec) {
-              *reinterpret_cast<float4*>(o) = v;
-            } else {
-              o[0] = v.x;
-              if (left > 1) o[1] = v.y;
-              if (left > 2) o[2] = v.z;
-              if (left > 3) o[3] = v.w;
-            }
+            *reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + (int64_t)grow * N + col) = v;
           } else {
-            __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(out) + (int64_t)grow * N + col;
-            if (vec) {
-              const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-              *reinterpret_cast<uint2*>(o) =
-                  make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-            } else {
-              o[0] = __float2bfloat16_rn(v.x);
-              if (left > 1) o[1] = __float2bfloat16_rn(v.y);
-              if (left > 2) o[2] = __float2bfloat16_rn(v.z);
-              if (left > 3) o[3] = __float2bfloat16_rn(v.w);
-            }
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+            *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(out) + (int64_t)grow * N + col) =
+                make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
           }
         }
         if constexpr (OUT == OUT_DACT) {
@@ -491,11 +545,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             sum.w += __shfl_xor_sync(0xffffffffu, sum.w, o);
           }
           if (rl == 0 && left > 0) {
-            float* o = colsum + (int64_t)(row0 / 32) * N + col;
-            o[0] = sum.x;
-            if (left > 1) o[1] = sum.y;
-            if (left > 2) o[2] = sum.z;
-            if (left > 3) o[3] = sum.w;
+            *reinterpret_cast<float4*>(colsum + (int64_t)(row0 / 32) * N + col) = sum;
           }
         }
         __syncwarp();
