@@ -3,6 +3,8 @@
 // 128-byte-swizzle layout that TMA and the tensor core read, accumulators in tensor memory.
 #pragma once
 
+#include <stddef.h>
+
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -80,12 +82,16 @@ constexpr uint32_t FWD_BYTES = X_BYTES + 2 * SLOT_BYTES + V3_BYTES;   // X, weig
 constexpr uint32_t ACC2 = 256, ACC3 = 16;                  // tensor-memory columns of the second and third products
 
 struct FwdRing {
-  uint64_t full[3], empty[3], xready, gready[2], acc1f, acc2f, acc3f, biasf[2], cplf[4];
-  float sb[2][2 * 256 + 8];                                // biases of a layer: first, second, third product
+  uint64_t full[3], empty[3], xready, gready[2], acc1f, acc2f, acc3f, biasf[2], cplf[4], drained;
+  alignas(16) float sb[2][2 * 256 + 8];                    // biases of a layer: first, second, third product (bulk copies)
   float s_new[4][FM], s_log[4][FM];                        // the rows' transformed coordinates and log scales
   uint32_t tmem_slot;
+  uint32_t fills[3];                                       // the producer's, once it has stopped: weight slots, V3, biases
   int abort_flag;
 };
+
+static_assert(offsetof(FwdRing, sb) % 16 == 0 && sizeof(FwdRing::sb[0]) % 16 == 0 && alignof(FwdRing) == 16,
+              "bulk copies start on 16 bytes");
 
 struct FwdWeights {
   const CUtensorMap *v1, *v2, *v3;
@@ -111,6 +117,7 @@ __device__ __forceinline__ uint32_t fwd_begin(FwdRing& rg) {
     mbar_init(su32(&rg.acc2f), 1);
     mbar_init(su32(&rg.acc3f), 1);
     for (int q = 0; q < 4; ++q) mbar_init(su32(&rg.cplf[q]), 4);
+    mbar_init(su32(&rg.drained), 1);
     rg.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -126,19 +133,40 @@ __device__ __forceinline__ uint32_t fwd_begin(FwdRing& rg) {
   return rg.tmem_slot;
 }
 
-// Records a given-up wait in *status and frees the tensor memory; all threads.
+// ring_drain of two slots filled in turn, n fills so far.
+__device__ __forceinline__ void pair_drain(const uint64_t* full, uint32_t n, uint32_t limit) {
+  ring_drain(full, 2, n & 1u, ((n >> 1) & 1u) ^ 1u, limit);
+}
+
+// Lets the copies and products in flight end; all threads (a call: the registers it would take are
+// those of the row warps' loops).
+static __device__ __noinline__ void fwd_drain(FwdRing& rg) {
+  if (threadIdx.x >> 5 == 0) {
+    pair_drain(rg.full, rg.fills[0], F_WAIT);
+    ring_drain(rg.full + 2, 1, 0u, (rg.fills[1] & 1u) ^ 1u, F_WAIT);   // one slot
+    pair_drain(rg.biasf, rg.fills[2], F_WAIT);
+  }
+  if (threadIdx.x >> 5 == 1) mma_drain(&rg.drained, F_WAIT);
+  __syncthreads();
+}
+
+// Records a given-up wait in *status, lets what is in flight end then, and frees the tensor memory;
+// all threads.
 __device__ __forceinline__ void fwd_end(FwdRing& rg, uint32_t tmem, int* status) {
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (threadIdx.x == 0 && *(volatile int*)&rg.abort_flag) atomicExch(status, 1);
+  if (*(volatile int*)&rg.abort_flag) {
+    if (threadIdx.x == 0) atomicExch(status, 1);
+    fwd_drain(rg);
+  }
   if (threadIdx.x >> 5 == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
 
 __device__ __forceinline__ void fwd_produce(FwdRing& rg, const FwdWeights& w, uint32_t sw) {
   const int lane = threadIdx.x & 31, H = w.H, NP = 2 + H / 128;   // weight parts per layer
-  uint32_t it = 0, li = 0;
+  uint32_t it = 0, li = 0, thirds = 0, biases = 0;
   bool ok = true;
   for (int t = blockIdx.x; t < w.tiles && ok; t += gridDim.x)
     for (int n = 0; n < w.K && ok; ++n, ++li)
@@ -175,8 +203,15 @@ __device__ __forceinline__ void fwd_produce(FwdRing& rg, const FwdWeights& w, ui
         }
         __syncwarp();
         it += !last;
+        thirds += last;
+        biases += p == 0;
       }
-  if (!ok && lane == 0) atomicExch(&rg.abort_flag, 1);
+  if (lane == 0) {
+    rg.fills[0] = it;
+    rg.fills[1] = thirds;
+    rg.fills[2] = biases;
+    if (!ok) atomicExch(&rg.abort_flag, 1);
+  }
 }
 
 __device__ __forceinline__ void fwd_multiply(FwdRing& rg, const FwdWeights& w, uint32_t tmem, uint32_t sx, uint32_t sw) {
@@ -256,6 +291,12 @@ __device__ __forceinline__ bool row_wait(uint64_t* bar, uint32_t parity) {
   const bool got = mbar_wait(su32(bar), parity, F_WAIT);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   return __all_sync(0xffffffffu, got);
+}
+// The same, false as well when another warp has given up (the flag as one vote of the warp).
+__device__ __forceinline__ bool row_wait(uint64_t* bar, uint32_t parity, const int* abort_flag) {
+  const bool got = mbar_wait(su32(bar), parity, F_WAIT);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  return !__any_sync(0xffffffffu, !got || *(volatile const int*)abort_flag != 0);
 }
 
 // bias + ReLU of the 32 accumulator columns from `at` on (bias: theirs), written over the first

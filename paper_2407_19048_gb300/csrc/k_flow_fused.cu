@@ -23,8 +23,8 @@
 // warps and biases by every thread from L2, a layer took 9200: 20,000 draws of 16 layers
 // 163 us, now 122 (157 tiles on 152 SMs, two rounds; A from tensor memory 147, biases staged
 // 134, four warps a quarter and 256-column MMAs with the fragment-shaped drain 122).
-// Every mbarrier wait is bounded; on expiry the CTA records a status, stops and frees its
-// tensor memory.
+// Every mbarrier wait is bounded; on expiry the CTA records a status, stops, lets its copies and
+// products in flight end and frees its tensor memory.
 #include "flow_tile.cuh"
 #include "pdl.cuh"
 
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
         proxy_fence();
         row_arrive(&rg.xready);
         const float* bl = rg.sb[li & 1u];
-        if (!(ok = row_wait(&rg.biasf[li & 1u], (li >> 1) & 1u) && !*(volatile int*)&rg.abort_flag)) break;
+        if (!(ok = row_wait(&rg.biasf[li & 1u], (li >> 1) & 1u, &rg.abort_flag))) break;
         uint32_t w[2][8];
         if (!(ok = row_wait(&rg.acc1f, li & 1u))) break;
         for (int rd = 0; rd < NR; ++rd) {                      // chunk 4 rd + h of 32 columns

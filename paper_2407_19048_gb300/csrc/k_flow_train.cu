@@ -140,7 +140,7 @@ __device__ __forceinline__ int64_t mask_at(int l, int64_t p, int64_t P, int chun
 
 // Barriers, tensor memory and the weight ring of both kernels.
 struct Ring {
-  uint64_t full[2], empty[2], in_ready, gready[2], acc1f[2], acc2f[2], acc3f;
+  uint64_t full[2], empty[2], in_ready, gready[2], acc1f[2], acc2f[2], acc3f, drained;
 };
 
 __device__ __forceinline__ void ring_init(Ring* r, int* abort_flag) {
@@ -153,6 +153,7 @@ __device__ __forceinline__ void ring_init(Ring* r, int* abort_flag) {
   }
   mbar_init(su32(&r->in_ready), 8);
   mbar_init(su32(&r->acc3f), 1);
+  mbar_init(su32(&r->drained), 1);
   *abort_flag = 0;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -163,13 +164,7 @@ __device__ __forceinline__ bool wait_mma(uint64_t* bar, uint32_t parity) {   // 
   return got;
 }
 
-// A row warp's wait (all lanes) and arrival (its shared-memory writes made visible to the
-// tensor core and to TMA).
-__device__ __forceinline__ bool wait_rows(uint64_t* bar, uint32_t parity, const int* abort_flag) {
-  const bool got = mbar_wait(su32(bar), parity, F_WAIT);
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  return __all_sync(0xffffffffu, got) && !*(volatile const int*)abort_flag;
-}
+// A row warp's arrival (its shared-memory writes made visible to the tensor core and to TMA).
 __device__ __forceinline__ void arrive_rows(uint64_t* bar) {
   proxy_fence();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -271,7 +266,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1)
         // buffer: the second chunk of the last layer's g2 here, g1 and the first of g2 below
         if (save && l < K - 1 && NR > 1) keep(w[1], 4 + h, l + 1, &s2_map, a.m2);
         const float* bl = rg.sb[li & 1u];
-        if (!(ok = row_wait(&rg.biasf[li & 1u], (li >> 1) & 1u) && !*(volatile int*)&rg.abort_flag)) break;
+        if (!(ok = row_wait(&rg.biasf[li & 1u], (li >> 1) & 1u, &rg.abort_flag))) break;
         if (!(ok = row_wait(&rg.acc1f, li & 1u))) break;
 #pragma unroll
         for (int rd = 0; rd < 2; ++rd) {
@@ -380,7 +375,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
                     const __grid_constant__ CUtensorMap s2_map, BackwardArgs a) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) Ring rg;
-  __shared__ uint32_t tmem_slot;
+  __shared__ uint32_t tmem_slot, fills;                    // (the producer's, once it has stopped)
   __shared__ int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t base = (su32(smem_raw) + 1023u) & ~1023u;
@@ -432,7 +427,10 @@ __global__ void __launch_bounds__(F_THREADS, 1)
           }
           __syncwarp();
         }
-    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
+    if (lane == 0) {
+      fills = it;
+      if (!ok) atomicExch(&abort_flag, 1);
+    }
   } else if (warp == 1) {
     uint32_t it = 0, li = 0;
     bool ok = true;
@@ -582,7 +580,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
           arrive_rows(&rg.in_ready);                           // (it has read the last layer's dX)
         }
         for (int rd = 0; rd < NR && ok; ++rd) {
-          if (!(ok = wait_rows(&rg.acc1f[rd], li & 1u, &abort_flag))) break;
+          if (!(ok = row_wait(&rg.acc1f[rd], li & 1u, &abort_flag))) break;
           const int c = 2 * rd + h;
           if (lane == 0) tma_store_wait_read();                // the last layer's dZ1 has been read
           __syncwarp();
@@ -592,7 +590,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
           sums();
         }
         for (int rd = 0; rd < NR && ok; ++rd) {
-          if (!(ok = wait_rows(&rg.acc2f[rd], li & 1u, &abort_flag))) break;
+          if (!(ok = row_wait(&rg.acc2f[rd], li & 1u, &abort_flag))) break;
           const int c = 2 * rd + h;
           if (lane == 0) tma_store_wait_read();                // dZ2 has been read
           __syncwarp();
@@ -606,7 +604,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
           load8(a.xs + (at + a.n) * 8, w);
           load8(a.o + (at + a.n) * 8, o);
         }
-        if (!(ok = wait_rows(&rg.acc3f, li & 1u, &abort_flag))) break;
+        if (!(ok = row_wait(&rg.acc3f, li & 1u, &abort_flag))) break;
         uint32_t raw[32];
         tmem_ld32_async(lane_addr + 32u * h, raw);
         if (h == 0) {
@@ -651,7 +649,12 @@ __global__ void __launch_bounds__(F_THREADS, 1)
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (threadIdx.x == 0 && *(volatile int*)&abort_flag) atomicExch(&g_train_status, 1);
+  if (*(volatile int*)&abort_flag) {
+    if (threadIdx.x == 0) atomicExch(&g_train_status, 1);
+    if (warp == 0) pair_drain(rg.full, fills, F_WAIT);
+    if (warp == 1) mma_drain(&rg.drained, F_WAIT);
+    __syncthreads();
+  }
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }

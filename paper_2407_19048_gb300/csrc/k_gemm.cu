@@ -15,8 +15,8 @@
 //   store C, while the next tile accumulates.  Eight draining warps keep the fused
 //   epilogue (bias, activation, conversion, stores) off the critical path of products
 //   with a short K, where it, not the MMA, sets the time per tile.
-// Every mbarrier wait is bounded: on expiry the CTA records a status, stops storing,
-// frees its tensor memory and returns.
+// Every mbarrier wait is bounded: on expiry the CTA records a status, stops storing, lets its
+// copies and products in flight end (bounded again), frees its tensor memory and returns.
 //
 // Wide tiles (MW = 2, large products): a CTA computes a 256 x 256 tile of C as two
 // M 128 x N 256 products that share each B tile, from three 64 KiB stages (A 256 x 64 in
@@ -262,8 +262,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   constexpr uint32_t TMEM_COLS = TL::TMEM_COLS;
   constexpr uint32_t IDESC = idesc_bf16(GM, TN_, A_MN, B_MN);
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], tfull[2], tempty[2];
-  __shared__ uint32_t tmem_slot;
+  __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], tfull[2], tempty[2], drained;
+  __shared__ uint32_t tmem_slot, fill_stage, fill_phase;   // (of the producer's next fill, once it has stopped)
   __shared__ int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t base = (su32(smem_raw) + 1023u) & ~1023u;   // 1024-byte aligned stages
@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       mbar_init(su32(&tfull[a]), 1);
       mbar_init(su32(&tempty[a]), EPI_WARPS);
     }
+    mbar_init(su32(&drained), 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -364,7 +365,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       if (*(volatile int*)&abort_flag) ok = false;
       ok = __all_sync(0xffffffffu, ok);
     }
-    if (!ok && lane == 0) atomicExch(&abort_flag, 1);
+    if (lane == 0) {
+      fill_stage = s;
+      fill_phase = ph;
+      if (!ok) atomicExch(&abort_flag, 1);
+    }
   } else if (warp == 1) {
     uint32_t s = 0, ph = 0, tl = 0;
     bool ok = true;
@@ -559,7 +564,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (threadIdx.x == 0 && *(volatile int*)&abort_flag) atomicExch(&g_gemm_status, 1);
+  if (*(volatile int*)&abort_flag) {
+    if (threadIdx.x == 0) atomicExch(&g_gemm_status, 1);
+    if (warp == 0) ring_drain(full, STAGES, fill_stage, fill_phase, WAIT_POLLS);
+    if (warp == 1) mma_drain(&drained, WAIT_POLLS);
+    __syncthreads();
+  }
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * TMEM_COLS) : "memory");
 }

@@ -152,6 +152,22 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+// After a wait was given up: lets a ring's copies land before the CTA gives its shared memory up.
+// The producer's next fill is of stage `next` and waits for parity `phase` of that stage's
+// "empty" barrier (1 in the first round), so the stages before `next` were last filled in this
+// round, phase ^ 1 of their "full" barriers, and the others in the round before, phase `phase`
+// (which a barrier that has completed no phase passes at once).  A whole warp; bounded.
+template <class Bars>
+__device__ __forceinline__ void ring_drain(const Bars& full, int stages, uint32_t next, uint32_t phase, uint32_t limit) {
+  for (int i = 0; i < stages; ++i) mbar_wait_warp(su32(&full[i]), (uint32_t)i < next ? phase ^ 1u : phase, limit);
+}
+// The same of the MMAs in flight, by the warp that issued them: `bar` (one arrival, unused so far).
+__device__ __forceinline__ void mma_drain(uint64_t* bar, uint32_t limit) {
+  if (elect_one()) mma_commit(su32(bar));
+  __syncwarp();
+  mbar_wait_warp(su32(bar), 0u, limit);
+}
+
 // 32 consecutive FP32 columns of this thread's accumulator row.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   uint32_t r[32];
