@@ -20,7 +20,8 @@ launching stream, with a 256 MiB buffer written between steps (outside the event
 the 1.6 GB output of a step exceeds L2 anyway); barrier + synchronize before and
 after; max over ranks.  Under torchrun each rank is an independent replica on its
 own GPU with its own step counters (weak scaling, no data-path collective).  Rank 0
-prints one JSON line.
+prints one JSON line: the headline with its configuration and bounds, and the main figure of
+every further leg; ``--record PATH`` writes all of the legs' figures to a file.
 """
 import argparse
 import hashlib
@@ -1000,6 +1001,43 @@ def cufft_leg(gwx, torch, sim, wl, fused_ms):
     return res
 
 
+# The main figures of the further legs, as the printed line names them: where they lie in the record.
+LEG_FIGURES = {
+    "hl3_ms": "hl3.ms_per_step", "log_likelihood_ms": "log_likelihood.ms_per_call",
+    "importance_eff_per_s": "log_likelihood.importance.value", "tmarg_ms": "log_likelihood_tmarg.ms_per_call",
+    "tmarg_frac": "log_likelihood_tmarg.roofline.frac", "serving_events_per_s": "serving.events_per_s",
+    "serving_p99_ms": "serving.latency_ms_p99", "gemm_ms": "gemm_bf16.ms", "cublas_ms": "gemm_bf16.cublas_ms",
+    "dense_gelu_ms": "gemm_bf16.dense_bias_gelu_ms", "whiten_ms": "fft_vs_cufft.gwx_whiten_ms",
+    "cufft_whiten_ms": "fft_vs_cufft.cufft_whiten_ms", "flow_step_ms": "flow.train_step_ms",
+    "flow_step_graph_ms": "flow.train_step_graph_ms", "flow_sample_20000_ms": "flow.sample_20000_ms.p50",
+    "flow_skymap_ms": "flow.skymap_20000_ms.64", "flow_ess_per_s": "flow.importance_sampling.flow.ess_per_s",
+    "prior_ess_per_s": "flow.importance_sampling.prior.ess_per_s", "resnet_step_ms": "flow_resnet.step_ms",
+    "conv_forward_ms": "conv1d_stage1.implicit_forward_ms", "conv_backward_ms": "conv1d_stage1.implicit_backward_ms",
+    "padded_b_ms": "padded_grid.definition_b.ms_per_step"}
+
+
+def short_line(record):
+    """The line to print from the whole record: every scalar of the top level, the configuration and the clocks as they
+    are, the figures of the bounds and of the end-to-end loop without their notes, and the legs' main figures.  The
+    record itself runs to 23,000 characters (per-event lists, loss curves), which callers that keep the end of the
+    output cut off at its front, where the value stands."""
+    line = {k: v for k, v in record.items() if not isinstance(v, (dict, list))}
+    for k in ("config", "clocks"):
+        line[k] = record[k]
+    for k, drop in (("roofline", ("kernel", "peak_basis", "launch_shape")), ("e2e", ("path",)),
+                    ("cpu_baseline", ("sample",))):
+        line[k] = record[k] and {n: v for n, v in record[k].items() if n not in drop}
+    legs = {}
+    for name, path in LEG_FIGURES.items():
+        v = record
+        for part in path.split("."):
+            v = v.get(part) if isinstance(v, dict) else None
+        if v is not None:
+            legs[name] = float("%.5g" % v)
+    line["legs"] = legs
+    return line
+
+
 def run_gpu(args, wl):
     import torch
     import torch.distributed as dist
@@ -1137,7 +1175,7 @@ def run_gpu(args, wl):
     if world > 1:
         dist.barrier()
     if rank == 0:
-        line = {
+        record = {
             "metric": "whitened injections/sec", "value": value, "unit": "injections/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * total_s / args.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
@@ -1165,7 +1203,10 @@ def run_gpu(args, wl):
             "padded_grid": padded,
             "wall_s_timed_region": t_wall,
         }
-        print(json.dumps(line), flush=True)
+        if args.record:
+            with open(args.record, "w") as fh:
+                fh.write(json.dumps(record) + "\n")
+        print(json.dumps(short_line(record)), flush=True)
     if world > 1:
         dist.destroy_process_group()
     return 0
@@ -1184,6 +1225,7 @@ def main(argv=None):
     ap.add_argument("--background-every", type=int, default=16,
                     help="regenerate the background and its PSD every this many steps")
     ap.add_argument("--batch", type=int, default=None, help="draws per step (default: the workload's)")
+    ap.add_argument("--record", default=None, metavar="PATH", help="write every leg's figures to this file (JSON)")
     ap.add_argument("--only-step", action="store_true",
                     help="time only the device step (no end-to-end or log-likelihood leg); for profiling")
     ap.add_argument("--only-loglike", default=None, metavar="LO,HI",
