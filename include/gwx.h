@@ -406,14 +406,14 @@ int gwx_dense_bf16(const void* X, const void* W, const float* bias, void* Y, int
  * db sums the FP32 dZ.  dX, dW or db may be NULL to skip it.  M, N, K multiples of 8 in
  * [8, 65535 * 32]; X, W, dX, dW 16-byte aligned, dY, bias, db 4-byte aligned.
  * Workspace: gwx_dense_bf16_backward_workspace(M, N, K) bytes. */
-/* dX and dW alone, from dZ already in bfloat16 [M][N] (16-byte aligned); the same sizes and
- * workspace. */
-int gwx_dense_bf16_backward_dz(const void* dZ16, const void* X, const void* W, int64_t M, int64_t N, int64_t K,
-                               float* dX, float* dW, void* workspace, size_t workspace_bytes, void* stream);
 size_t gwx_dense_bf16_backward_workspace(int64_t M, int64_t N, int64_t K);
 int gwx_dense_bf16_backward(const void* X, const void* W, const float* bias, const float* dY, int64_t M,
                             int64_t N, int64_t K, int act, float* dX, float* dW, float* db,
                             void* workspace, size_t workspace_bytes, void* stream);
+/* dX and dW alone, from dZ already in bfloat16 [M][N] (16-byte aligned); the same sizes and
+ * workspace. */
+int gwx_dense_bf16_backward_dz(const void* dZ16, const void* X, const void* W, int64_t M, int64_t N, int64_t K,
+                               float* dX, float* dW, void* workspace, size_t workspace_bytes, void* stream);
 
 /* ---- learned proposal: the pieces around the dense layers ---------------------------
  * The network trained on the simulated batches (Sec. 4, 5; AdamW) starts as the simplest
@@ -745,14 +745,14 @@ int gwx_mean_time_backward(const float* dm, int64_t B, int T, int C, float* dx, 
  * reported by gwx_device_status. */
 int gwx_conv1d_bf16(const void* x, int64_t B, int64_t T, int C, int k, const void* W, int O, const float* addend,
                     float* z, void* stream);
-/* The same backward from dz already in bfloat16 (16-byte aligned). */
-int gwx_conv1d_bf16_backward_dz(const void* dz16, const void* x, const void* W, int64_t B, int64_t T, int C, int O,
-                                int k, const float* addend, float* dx, float* dW, void* workspace,
-                                size_t workspace_bytes, void* stream);
 size_t gwx_conv1d_bf16_backward_workspace(int64_t B, int64_t T, int C, int O, int k);
 int gwx_conv1d_bf16_backward(const float* dz, const void* x, const void* W, int64_t B, int64_t T, int C, int O, int k,
                              const float* addend, float* dx, float* dW, void* workspace, size_t workspace_bytes,
                              void* stream);
+/* The same backward from dz already in bfloat16 (16-byte aligned). */
+int gwx_conv1d_bf16_backward_dz(const void* dz16, const void* x, const void* W, int64_t B, int64_t T, int C, int O,
+                                int k, const float* addend, float* dx, float* dW, void* workspace,
+                                size_t workspace_bytes, void* stream);
 
 /* ---- sky maps ---------------------------------------------------------------------
  * The paper's inference ends in a sky-localisation map in the HEALPix format (Sec. 5).
