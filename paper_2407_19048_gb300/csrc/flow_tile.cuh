@@ -6,7 +6,6 @@
 #include <stddef.h>
 
 #include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
 #include "gwx_internal.h"
@@ -360,23 +359,11 @@ __device__ __forceinline__ void pack_half(int p, const float* v, uint32_t& w0, u
   }
 }
 
-inline PFN_cuTensorMapEncodeTiled_v12000 encoder() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
-  return fn;
-}
-
 // bfloat16 [layers][rows][cols] with the layers lstride elements apart; boxes of box_cols (64, or
 // 32) columns x box_rows rows x one layer, the row of a box as wide as its swizzle.
 inline bool layer_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int64_t layers, int64_t lstride,
                       uint32_t box_rows, uint32_t box_cols = 64) {
-  auto enc = encoder();
+  auto enc = tensor_map_encoder();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)layers};
   cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)lstride * 2};

@@ -109,7 +109,8 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 cudaError_t launch_dz_rows(const float* dY, const void* Y, int64_t M, int N, void* dZ, float* part, cudaStream_t s) {
   const int64_t units = (M + TT - 1) / TT * ((N + 63) / 64);
-  pdl_launch(k_dz_rows, dim3((unsigned)((units + 7) / 8)), dim3(256), 0, s, dY, reinterpret_cast<const __nv_bfloat16*>(Y), M, N, reinterpret_cast<__nv_bfloat16*>(dZ), part);
+  pdl_launch(k_dz_rows, dim3((unsigned)((units + 7) / 8)), dim3(256), 0, s, dY,
+             reinterpret_cast<const __nv_bfloat16*>(Y), M, N, reinterpret_cast<__nv_bfloat16*>(dZ), part);
   return cudaGetLastError();
 }
 
@@ -151,8 +152,10 @@ cudaError_t launch_dense_backward(const void* X, const void* W, const float* bia
   if ((e = launch_dense_backward_dz(dZ, X, W, M, N, K, dX, dW, kpart, s)) != cudaSuccess) return e;
   if (db) {
     const int slices = colsum_slices(P);
-    pdl_launch(k_colsum, dim3(dim3((unsigned)((N + TT - 1) / TT), (unsigned)slices)), dim3(dim3(TT, TT)), 0, s, part, (int)P, (int)N, part2, slices == 1 ? db : nullptr);
-    if (slices > 1) pdl_launch(k_colsum_finish, dim3((unsigned)((N + 127) / 128)), dim3(128), 0, s, part2, slices, (int)N, db);
+    pdl_launch(k_colsum, dim3((unsigned)((N + TT - 1) / TT), (unsigned)slices), dim3(TT, TT), 0, s, part, (int)P,
+               (int)N, part2, slices == 1 ? db : nullptr);
+    if (slices > 1) pdl_launch(k_colsum_finish, dim3((unsigned)((N + 127) / 128)), dim3(128), 0, s, part2, slices,
+                               (int)N, db);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -393,7 +393,8 @@ int64_t flow_layout(const gwx_flow_shape& sh, int64_t* off) {
 // ---- stage launchers ----
 cudaError_t launch_flow_targets(const double* theta, int64_t B, const double* mean8, const double* scale8, float* x,
                                 cudaStream_t s) {
-  pdl_launch(k_flow_targets, dim3(blocks(B, TGT_ROWS)), dim3(4 * TGT_ROWS), 0, s, theta, B, make_std(mean8, scale8), x);
+  pdl_launch(k_flow_targets, dim3(blocks(B, TGT_ROWS)), dim3(4 * TGT_ROWS), 0, s, theta, B, make_std(mean8, scale8),
+             x);
   return cudaGetLastError();
 }
 
@@ -429,7 +430,8 @@ cudaError_t launch_flow_input_backward(int l, const float* dX, int C, int64_t B,
 }
 
 cudaError_t launch_flow_base(uint64_t seed, uint32_t counter, int64_t row0, int64_t n, float* z, cudaStream_t s) {
-  pdl_launch(k_flow_base, dim3(blocks(4 * n, ROW_NT)), dim3(ROW_NT), 0, s, (uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32), counter, row0, n, z);
+  pdl_launch(k_flow_base, dim3(blocks(4 * n, ROW_NT)), dim3(ROW_NT), 0, s, (uint32_t)(seed & 0xffffffffu),
+             (uint32_t)(seed >> 32), counter, row0, n, z);
   return cudaGetLastError();
 }
 

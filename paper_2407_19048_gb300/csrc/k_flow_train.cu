@@ -731,14 +731,15 @@ cudaError_t run_density(const void* params_bf16, const float* params, const int6
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_flow_density, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DENSITY_SMEM);
   if (e != cudaSuccess) return e;
-  pdl_launch(k_flow_density, dim3(grid), dim3(FWD_THREADS), DENSITY_SMEM, s, m1, m2, m3, stores ? stores[0] : m1, stores ? stores[1] : m1, stores ? stores[2] : m1, a);
+  pdl_launch(k_flow_density, dim3(grid), dim3(FWD_THREADS), DENSITY_SMEM, s, m1, m2, m3, stores ? stores[0] : m1,
+             stores ? stores[1] : m1, stores ? stores[2] : m1, a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-// Widths the fused kernels cover: as the sampling kernel, with the context's gradient in two
-// halves of 32 registers.
+// Widths the fused kernels cover: as the sampling kernel, with the context's gradient in registers, 24
+// columns of it with one warp of a quarter and 40 with the other.
 bool flow_fused_train_supported(int C, int H, int K) { return flow_fused_supported(C, H, K) && C <= 64; }
 
 cudaError_t launch_flow_density(const void* params_bf16, const float* params, const int64_t* off_t, int C, int H, int K,
@@ -850,7 +851,9 @@ cudaError_t launch_flow_train_fused(const void* params_bf16, const float* params
       (e = launch_wgrad(f.dz1, f.X, grads + off_t[6], H, 8 + C, n, f.kpart, s, K, n * H, n * (8 + C), lstride)) !=
           cudaSuccess)
     return e;
-  pdl_launch(k_flow_bias_grads, dim3(dim3((unsigned)(2 * (H / 32) + 1), (unsigned)(K + 1))), dim3(1024), 0, s, f.p1, f.p2, f.p3, b.P, H, K, grads + off_t[7], grads + off_t[9], grads + off_t[11], lstride, f.loss_part, (double)n, loss_mean);
+  pdl_launch(k_flow_bias_grads, dim3((unsigned)(2 * (H / 32) + 1), (unsigned)(K + 1)), dim3(1024), 0, s, f.p1, f.p2,
+             f.p3, b.P, H, K, grads + off_t[7], grads + off_t[9], grads + off_t[11], lstride, f.loss_part, (double)n,
+             loss_mean);
   return cudaGetLastError();
 }
 

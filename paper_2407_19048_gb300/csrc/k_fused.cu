@@ -14,6 +14,7 @@
 
 #include "fft16.cuh"
 #include "fft16r.cuh"
+#include "pdl.cuh"
 #include "tc05.cuh"
 #include "waveform.cuh"
 
@@ -691,17 +692,8 @@ static cudaError_t launch_simulate_lg(const DrawCoef* coef, const float* noise, 
   // The blocks may start once every block of the kernel before has (k_prepare, k_whiten_filter say
   // so at their start) and wait for its end themselves: the launch and their set-up lie under it
   // (64 draws of two detectors 21.7 us a batch without, 20.1 with; whitening 3003 windows 79.9, 76.9).
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, coef, noise, L, offsets, W, Wcap, k_lo, D, B, nd, y);
+  pdl_launch(kern, dim3((unsigned)grid), dim3(NT), smem, s, coef, noise, L, offsets, W, Wcap, k_lo, D, B, nd, y);
+  return cudaGetLastError();
 }
 
 // Whitening of the windows d [B][D][N] with the filter W (Wcap floats allocated): staged

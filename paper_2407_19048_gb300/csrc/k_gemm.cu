@@ -37,7 +37,6 @@
 // pairs: slice s covers K blocks [s kbs, (s + 1) kbs) and stores its FP32 partial product
 // at C + s M N; a second kernel sums the slices in a fixed order (deterministic).
 #include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
 #include "gwx_internal.h"
@@ -574,22 +573,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * TMEM_COLS) : "memory");
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
-  return fn;
-}
-
 // Row-major bfloat16 [groups][rows][cols], groups gstride elements apart, as a 3-D tensor
 // map with boxes of 64 columns x 64 rows (an MN-major operand).
 bool make_map_mn(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, int64_t groups, int64_t gstride) {
-  auto enc = encode_fn();
+  auto enc = tensor_map_encoder();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)groups};
   cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)gstride * 2};
@@ -602,7 +589,7 @@ bool make_map_mn(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, 
 
 // Row-major bfloat16 [rows][K] as a 2-D tensor map with boxes of box_rows x 64.
 bool make_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t K, uint32_t box_rows) {
-  auto enc = encode_fn();
+  auto enc = tensor_map_encoder();
   if (!enc) return false;
   cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)K * 2};
@@ -683,7 +670,9 @@ cudaError_t run_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmCal
   auto kern = k_gemm_bf16<OUT, TN_, OPS, MW>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  pdl_launch(kern, dim3(grid), dim3(GEMM_THREADS), smem, s, ta, tb, c.C, c.bias, c.act, make_work_map(TM, TN, c.group, c.groups), (int)c.M, (int)c.N, (int)c.K, kbs, splits, c.extra, c.colsum, c.groups, c.cstride, c.geo);
+  pdl_launch(kern, dim3(grid), dim3(GEMM_THREADS), smem, s, ta, tb, c.C, c.bias, c.act,
+             make_work_map(TM, TN, c.group, c.groups), (int)c.M, (int)c.N, (int)c.K, kbs, splits, c.extra, c.colsum,
+             c.groups, c.cstride, c.geo);
   return cudaGetLastError();
 }
 
@@ -699,21 +688,20 @@ cudaError_t run_gemm_at(int tn, const CUtensorMap& ta, const CUtensorMap& tb, co
 // Tile width of a product: 256 columns unless the 128 x 256 tiles would leave more than half
 // of the SMs idle (the flow's conditioner products on a few hundred to a few thousand rows),
 // then 128 or 64, so that more CTAs share the work; no wider than N needs (the stem's product
-// has 64 columns).  Split-K products keep 256.
-int gemm_tile_width(int64_t M, int64_t N, int splits, int sms) {
-  if (splits > 1) return GN;
+// has 64 columns).
+int gemm_tile_width(int64_t M, int64_t N, int sms) {
   const int64_t tm = (M + GM - 1) / GM;
   for (int tn : {256, 128})
     if (2 * N > tn && tm * ((N + tn - 1) / tn) * 2 >= sms) return tn;
   return 64;
 }
 
-// Wide 256 x 256 tiles for large products: no split K, a K long enough that the epilogue
+// Wide 256 x 256 tiles for large products: a K long enough that the epilogue
 // (no longer overlapped) is a small part of a tile, at least one full wave of them, and no
 // GELU (its erfc epilogue, unoverlapped, cost more than the wide tiles gained: 0.77 vs
 // 0.73 ms for an 8192^3 dense layer).
-bool gemm_wide(int64_t M, int64_t N, int64_t K, int splits, int act, int sms) {
-  return splits == 1 && K >= 1024 && act != GWX_ACT_GELU && ((M + 255) / 256) * ((N + 255) / 256) >= sms;
+bool gemm_wide(int64_t M, int64_t N, int64_t K, int act, int sms) {
+  return K >= 1024 && act != GWX_ACT_GELU && ((M + 255) / 256) * ((N + 255) / 256) >= sms;
 }
 
 // C = A B^T with A [M][K], B [N][K]; OUT as in the kernel.
@@ -725,12 +713,12 @@ cudaError_t launch_gemm(const void* A, const void* B, GemmCall c, cudaStream_t s
   if (e != cudaSuccess) return e;
   CUtensorMap ta, tb;
   if constexpr (OUT != OUT_DACT) {
-    if (gemm_wide(c.M, c.N, c.K, c.splits, c.act, sms)) {
+    if (gemm_wide(c.M, c.N, c.K, c.act, sms)) {
       if (!make_map(&ta, A, c.M, c.K, 2 * GM) || !make_map(&tb, B, c.N, c.K, 256)) return cudaErrorInvalidValue;
       return run_gemm<OUT, 256, OP_KK, 2>(ta, tb, c, sms, s);
     }
   }
-  const int tn = gemm_tile_width(c.M, c.N, c.splits, sms);
+  const int tn = gemm_tile_width(c.M, c.N, sms);
   if (!make_map(&ta, A, c.M, c.K, GM) || !make_map(&tb, B, c.N, c.K, (uint32_t)tn)) return cudaErrorInvalidValue;
   return run_gemm_at<OUT, OP_KK>(tn, ta, tb, c, sms, s);
 }
@@ -738,7 +726,7 @@ cudaError_t launch_gemm(const void* A, const void* B, GemmCall c, cudaStream_t s
 // Channels-last bfloat16 x [Bn][T][C] as a 3-D tensor map with boxes of 64 channels x
 // box_t times.
 bool make_map_3d(CUtensorMap* map, const void* ptr, int64_t Bn, int64_t T, int64_t C, uint32_t box_t) {
-  auto enc = encode_fn();
+  auto enc = tensor_map_encoder();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)T, (cuuint64_t)Bn};
   cuuint64_t strides[2] = {(cuuint64_t)C * 2, (cuuint64_t)T * C * 2};
@@ -802,7 +790,7 @@ cudaError_t launch_gemm_nn(const void* A, const void* B, float* C, int64_t M, in
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
   CUtensorMap ta, tb;
-  const int tn = gemm_tile_width(M, N, 1, sms);
+  const int tn = gemm_tile_width(M, N, sms);
   if (!make_map(&ta, A, M, K, GM) || !make_map(&tb, B, K, N, GK)) return cudaErrorInvalidValue;
   return run_gemm_at<OUT_F32, OP_NN>(tn, ta, tb, c, sms, s);
 }
@@ -836,9 +824,11 @@ static cudaError_t wgrad_finish(const GemmCall& c, float* C, int64_t cstride, co
   const auto* p = reinterpret_cast<const float4*>(part);
   auto* out = reinterpret_cast<float4*>(C);
   if (c.splits >= 16)
-    pdl_launch(k_split_reduce<8>, dim3(dim3((unsigned)((n4 + 31) / 32), (unsigned)c.groups)), dim3(256), 0, s, p, c.splits, n4, cstride / 4, out);
+    pdl_launch(k_split_reduce<8>, dim3((unsigned)((n4 + 31) / 32), (unsigned)c.groups), dim3(256), 0, s, p, c.splits,
+               n4, cstride / 4, out);
   else
-    pdl_launch(k_split_reduce<1>, dim3(dim3((unsigned)((n4 + 255) / 256), (unsigned)c.groups)), dim3(256), 0, s, p, c.splits, n4, cstride / 4, out);
+    pdl_launch(k_split_reduce<1>, dim3((unsigned)((n4 + 255) / 256), (unsigned)c.groups), dim3(256), 0, s, p,
+               c.splits, n4, cstride / 4, out);
   return cudaGetLastError();
 }
 

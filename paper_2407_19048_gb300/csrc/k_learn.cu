@@ -446,21 +446,14 @@ cudaError_t launch_lag_from_spectrum(const void* Y, int64_t B, int D, int64_t N,
 // Spectra of y into ws, then every column of the flow's feature rows.
 cudaError_t launch_spectral_columns(const float* y, int64_t B, int D, int64_t N, int k_lo, int G, int F_pad, bool cross,
                                     bool lag, void* ws, void* out, cudaStream_t s) {
+  static_assert(GWX_MAX_DET == 4, "a kernel for every number of detectors");
   const int ng = (int)((N / 2 - k_lo) / G), chunks = ng > 0 ? (ng + SC_NT - 1) / SC_NT : 1;
-  if (D > 4) {   // more detectors than a thread holds: a kernel a kind of column
-    cudaError_t e = launch_features(y, B, D, N, k_lo, G, F_pad, ws, out, s);
-    int col = D * ng;
-    if (e == cudaSuccess && cross) {
-      e = launch_cross_from_spectrum(ws, B, D, N, k_lo, G, F_pad, col, out, s);
-      col += D * (D - 1) * ng;
-    }
-    return e == cudaSuccess && lag ? launch_lag_from_spectrum(ws, B, D, N, k_lo, G, F_pad, col, out, s) : e;
-  }
   float2* Y = reinterpret_cast<float2*>(ws);
   const cudaError_t e = launch_rfft_rows(y, B * D, N, Y, s);
   if (e != cudaSuccess || B <= 0) return e;
   auto run = [&](auto kern) {
-    pdl_launch(kern, dim3((unsigned)(B * chunks)), dim3(SC_NT), 0, s, Y, N / 2 + 1, (int)N, k_lo, G, ng, chunks, F_pad, cross, lag, reinterpret_cast<__nv_bfloat16*>(out));
+    pdl_launch(kern, dim3((unsigned)(B * chunks)), dim3(SC_NT), 0, s, Y, N / 2 + 1, (int)N, k_lo, G, ng, chunks,
+               F_pad, cross, lag, reinterpret_cast<__nv_bfloat16*>(out));
     return cudaGetLastError();
   };
   switch (D) {

@@ -951,7 +951,9 @@ bool aligned8(const void* p) { return ((uintptr_t)p & 7u) == 0; }
 cudaError_t launch_im2col(const void* x, int64_t B, int T, int C, int k, int s, int p, int K, void* cols,
                           cudaStream_t st) {
   const int To = (T + 2 * p - k) / s + 1;
-  pdl_launch(k_im2col, dim3(dim3(nblk((int64_t)To * (K / 8), 256), (unsigned)B)), dim3(256), 0, st, reinterpret_cast<const __nv_bfloat16*>(x), T, C, k, s, p, To, K, reinterpret_cast<__nv_bfloat16*>(cols));
+  pdl_launch(k_im2col, dim3(nblk((int64_t)To * (K / 8), 256), (unsigned)B), dim3(256), 0, st,
+             reinterpret_cast<const __nv_bfloat16*>(x), T, C, k, s, p, To, K,
+             reinterpret_cast<__nv_bfloat16*>(cols));
   return cudaGetLastError();
 }
 
@@ -959,7 +961,8 @@ cudaError_t launch_im2col_cf(const float* y, int64_t B, int D, int N, int k, int
                              cudaStream_t st) {
   const int To = (N + 2 * p - k) / s + 1;
   if (K % 8 == 0 && aligned16(cols))
-    pdl_launch(k_im2col_cf8, dim3(dim3(nblk((int64_t)To * (K / 8), 256), (unsigned)B)), dim3(256), 0, st, y, D, N, k, s, p, To, K, reinterpret_cast<__nv_bfloat16*>(cols));
+    pdl_launch(k_im2col_cf8, dim3(nblk((int64_t)To * (K / 8), 256), (unsigned)B), dim3(256), 0, st, y, D, N, k, s, p,
+               To, K, reinterpret_cast<__nv_bfloat16*>(cols));
   else
     k_im2col_cf<<<dim3(nblk((int64_t)To * K, 256), (unsigned)B), 256, 0, st>>>(y, D, N, k, s, p, To, K,
                                                                                reinterpret_cast<__nv_bfloat16*>(cols));
@@ -972,9 +975,9 @@ cudaError_t launch_col2im(const float* dcols, int64_t B, int T, int C, int k, in
   const bool v4 = C % 4 == 0 && K % 4 == 0 && aligned16(dcols) && aligned16(addend) && aligned16(dx);
   const dim3 g4(nblk((int64_t)T * C / 4, 256), (unsigned)B);
   if (v4 && k == 1) {
-    pdl_launch(k_col2im4<1>, dim3(g4), dim3(256), 0, st, dcols, T, C, s, p, To, K, addend, dx);
+    pdl_launch(k_col2im4<1>, g4, dim3(256), 0, st, dcols, T, C, s, p, To, K, addend, dx);
   } else if (v4 && k == 5) {
-    pdl_launch(k_col2im4<5>, dim3(g4), dim3(256), 0, st, dcols, T, C, s, p, To, K, addend, dx);
+    pdl_launch(k_col2im4<5>, g4, dim3(256), 0, st, dcols, T, C, s, p, To, K, addend, dx);
   } else if (v4 && k == 7) {
     k_col2im4<7><<<g4, 256, 0, st>>>(dcols, T, C, s, p, To, K, addend, dx);
   } else {
@@ -991,7 +994,8 @@ cudaError_t launch_group_norm(const float* z, int64_t B, int T, int C, int G, co
   const auto r16 = reinterpret_cast<const __nv_bfloat16*>(res16);
   const auto o16 = reinterpret_cast<__nv_bfloat16*>(out16);
   if (v4 && per_sample_ok(C, G)) {
-    pdl_launch(k_gn_forward_s, dim3((unsigned)B), dim3(GN_NT), 0, st, z, T, C, G, 1.0 / ((double)T * (C / G)), gamma, beta, res32, r16, relu, o16, out32, ms);
+    pdl_launch(k_gn_forward_s, dim3((unsigned)B), dim3(GN_NT), 0, st, z, T, C, G, 1.0 / ((double)T * (C / G)), gamma,
+               beta, res32, r16, relu, o16, out32, ms);
   } else if (v4) {
     k_gn_stats<4><<<(unsigned)(B * G), 256, 0, st>>>(z, T, C, G, ms);
     k_gn_apply<4><<<dim3(nblk((int64_t)T * C / 4, 256), (unsigned)B), 256, 0, st>>>(z, T, C, G, ms, gamma, beta, res32,
@@ -1009,7 +1013,8 @@ static cudaError_t launch_gn_backward(const GnSource& src, const float* z, int64
                                       const float* ms, const float* gamma, void* dz, float* dsum, double* part,
                                       cudaStream_t st) {
   const double inv_n = 1.0 / ((double)T * (C / G));
-  pdl_launch(k_gn_backward_s<SRC, OUT16>, dim3((unsigned)B), dim3(gn_bt(SRC)), 0, st, src, z, T, C, G, inv_n, ms, gamma, dz, dsum, part);
+  pdl_launch(k_gn_backward_s<SRC, OUT16>, dim3((unsigned)B), dim3(gn_bt(SRC)), 0, st, src, z, T, C, G, inv_n, ms,
+             gamma, dz, dsum, part);
   return cudaGetLastError();
 }
 
@@ -1082,7 +1087,8 @@ cudaError_t launch_relu_mask(const float* dy, const void* out, int64_t n, float*
 cudaError_t launch_maxpool(const void* x, int64_t B, int T, int C, void* y, uint8_t* arg, cudaStream_t st) {
   const int To = (T + 2 - 3) / 2 + 1;
   if (C % 8 == 0 && aligned16(x) && aligned16(y) && ((uintptr_t)arg & 7u) == 0) {
-    pdl_launch(k_maxpool8, dim3(dim3(nblk((int64_t)To * C / 8, 256), (unsigned)B)), dim3(256), 0, st, reinterpret_cast<const __nv_bfloat16*>(x), T, C, To, reinterpret_cast<__nv_bfloat16*>(y), arg);
+    pdl_launch(k_maxpool8, dim3(nblk((int64_t)To * C / 8, 256), (unsigned)B), dim3(256), 0, st,
+               reinterpret_cast<const __nv_bfloat16*>(x), T, C, To, reinterpret_cast<__nv_bfloat16*>(y), arg);
     return cudaGetLastError();
   }
   k_maxpool<<<dim3(nblk((int64_t)To * C, 256), (unsigned)B), 256, 0, st>>>(

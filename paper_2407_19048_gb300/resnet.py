@@ -193,11 +193,11 @@ class ResNet1D:
         return buf[off:off + nbytes]
 
     # the gradient a group norm's backward starts from (gwx_group_norm_backward_src)
-    PLAIN, MASK, POOL, MEAN = range(4)
+    MASK, POOL, MEAN = 1, 2, 3
 
-    def _gn_back(self, kind, dy, z, ms, g, out=None, arg=None, want_dsum=False):
-        """(dz, dsum, dgamma, dbeta) of the normalisation of z whose output's gradient is dy
-        (PLAIN), dy [out > 0] (MASK), the max pool's dy routed back and masked (POOL) or the
+    def _gn_back(self, kind, dy, z, ms, g, out, arg=None, want_dsum=False):
+        """(dz, dsum, dgamma, dbeta) of the normalisation of z whose output's gradient is
+        dy [out > 0] (MASK), the max pool's dy routed back and masked (POOL) or the
         mean over time's dy / T masked (MEAN); dsum is that gradient itself (FP32, None unless
         wanted).  dz is bfloat16 where one kernel does it all, else FP32."""
         import torch
@@ -220,10 +220,9 @@ class ResNet1D:
         elif kind == self.POOL:
             dsum = torch.empty((B, T, C), dtype=torch.float32, device=self.dev)
             gwx._check(lib.gwx_maxpool_backward(gwx._ptr(dy), gwx._ptr(arg), B, T, C, gwx._ptr(dsum), st))
-        if kind != self.PLAIN:
-            d = torch.empty_like(dsum)
-            gwx._check(lib.gwx_relu_mask(gwx._ptr(dsum), gwx._ptr(out), d.numel(), gwx._ptr(d), st))
-            dsum = d
+        d = torch.empty_like(dsum)
+        gwx._check(lib.gwx_relu_mask(gwx._ptr(dsum), gwx._ptr(out), d.numel(), gwx._ptr(d), st))
+        dsum = d
         dz = torch.empty_like(z)
         scratch = self._scratch(lib.gwx_group_norm_backward_scratch(B, C, GROUPS))
         gwx._check(lib.gwx_group_norm_backward(gwx._ptr(dsum), gwx._ptr(z), B, T, C, GROUPS, gwx._ptr(ms), gwx._ptr(g),
