@@ -48,9 +48,9 @@ SM_MAX_MHZ_FALLBACK = 2070.0
 # dirty lines is counted and this launch's own L2-resident tail is not), keyed by
 # workload, with the hash of the kernel sources it was measured on.  A workload whose
 # capture does not match the current sources reports null.
-TRAFFIC = {"sweep": {"bytes_per_launch": 8 * 199666944, "B": 8192, "sources_sha1": "f9ebc7abb1a4a9f4ac4043fe683ceee8bbef3a46",
+TRAFFIC = {"sweep": {"bytes_per_launch": 8 * 199703808, "B": 8192, "sources_sha1": "673a2fe948b01e62dd6b1520886d0f38acf32f76",
                     "note": "ncu DRAM read + write of the second of two back-to-back 1024-draw launches of the same "
-                            "geometry (caches not flushed: it pays the first launch's write-back, 199.67 MB), scaled "
+                            "geometry (caches not flushed: it pays the first launch's write-back, 199.70 MB), scaled "
                             "by the draws per launch"}}
 
 

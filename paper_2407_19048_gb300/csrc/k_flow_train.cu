@@ -22,7 +22,7 @@
 // sum).  Latency bound: one tile's chain MMA -> drain -> MMA, 6.4 us a layer of 256 in the
 // density with what it keeps (3.8 without; 6.9 with the operands in shared memory), 7.9 in the
 // backward; a batch of 4096 fills 32 SMs.  As ~370 launches of 3 to 13 us (each layer: input
-// rows, three products, coupling step; backward 17 kernels) the step took 3.04 ms, now 0.45.
+// rows, three products, coupling step; backward 17 kernels) the step took 3.04 ms, now 0.44.
 #include "flow_tile.cuh"
 #include "pdl.cuh"
 #include "sum2.cuh"
@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(F_THREADS, 1)
 
 // Bias gradients of every layer and the mean loss: block (c, l) sums 32 columns' partials
 // (p1, p2, p3: H, H and 8 columns) of layer l, 32 row lanes and then a warp a column, in
-// two-float arithmetic (FP64: 9.8 us for 16 layers of 256 and 128 partials, 6.2 now); the
+// two-float arithmetic (FP64: 9.8 us for 16 layers of 256 and 128 partials, 6.0 now); the
 // extra block (0, K) sums the loss in FP64.
 __global__ void __launch_bounds__(1024) k_flow_bias_grads(const float* p1, const float* p2, const float* p3,
                                                           int64_t P, int H, int K,

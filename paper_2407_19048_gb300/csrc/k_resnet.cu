@@ -202,8 +202,8 @@ __global__ void __launch_bounds__(256) k_gn_stats(const float* __restrict__ z, i
 // flight: every pass first issues its rows' loads (eight, or four of several arrays) and then
 // adds them (a loop of load and add kept one row in flight, 10 us a slab).  (512 windows, stem
 // and two blocks, six normalisations: 337 us as a statistics and an apply kernel forward, now
-// 203; ~700 us backward with the ReLU mask, the FP32 dz and its conversion as passes of their
-// own, now 467.  Slabs staged in shared memory by asynchronous copies, columns split over
+// 201; ~700 us backward with the ReLU mask, the FP32 dz and its conversion as passes of their
+// own, now 458.  Slabs staged in shared memory by asynchronous copies, columns split over
 // blocks, read every array once but left too few threads for the runs: 194 and 504.)
 // Sums: thread (run slice s, row lane l, column quad q) reads runs of 16 rows, rl = 256 / (C / 4)
 // rows apart, of channels 4 q .. 4 q + 3, coalesced float4 loads; FP32 within a run (the
