@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(256) k_gn_stats(const float* __restrict__ z, i
 // adds them (a loop of load and add kept one row in flight, 10 us a slab).  (512 windows, stem
 // and two blocks, six normalisations: 337 us as a statistics and an apply kernel forward, now
 // 201; ~700 us backward with the ReLU mask, the FP32 dz and its conversion as passes of their
-// own, now 458.  Slabs staged in shared memory by asynchronous copies, columns split over
+// own, now 411.  Slabs staged in shared memory by asynchronous copies, columns split over
 // blocks, read every array once but left too few threads for the runs: 194 and 504.)
 // Sums: thread (run slice s, row lane l, column quad q) reads runs of 16 rows, rl = 256 / (C / 4)
 // rows apart, of channels 4 q .. 4 q + 3, coalesced float4 loads; FP32 within a run (the
@@ -383,24 +383,27 @@ template <int SRC>
 __device__ __forceinline__ void gn_load(GnRow<SRC>& r, const GnSource& s, int64_t b, int t, int c, int T, int C) {
   const int64_t i = (b * T + t) * C + c;
   if constexpr (SRC == DY_POOL) {
-    // time t is argument 1 of window t/2 (even t), or 2 of window t/2 and 0 of the next (odd t)
-    // (both loads always, without branches: 193 us where this takes 167)
-    const int to = t / 2;
-    const int64_t o = (b * s.To + to) * C + c;
-    r.v0 = r.v1 = make_float4(0.f, 0.f, 0.f, 0.f);
-    r.a0 = r.a1 = make_uchar4(3, 3, 3, 3);
-    if (to < s.To) {
-      r.v0 = *reinterpret_cast<const float4*>(s.dy + o);
-      r.a0 = *reinterpret_cast<const uchar4*>(s.arg + o);
-    }
-    if ((t & 1) && to + 1 < s.To) {
-      r.v1 = *reinterpret_cast<const float4*>(s.dy + o + C);
-      r.a1 = *reinterpret_cast<const uchar4*>(s.arg + o + C);
-    }
+    // time t is argument 1 of window t/2 (even t), or 2 of window t/2, which there always is, and
+    // 0 of the next (odd t, gn_load_next)
+    const int64_t o = (b * s.To + t / 2) * C + c;
+    r.v1 = make_float4(0.f, 0.f, 0.f, 0.f);
+    r.a1 = make_uchar4(3, 3, 3, 3);
+    r.v0 = *reinterpret_cast<const float4*>(s.dy + o);
+    r.a0 = *reinterpret_cast<const uchar4*>(s.arg + o);
   } else if constexpr (SRC != DY_MEAN) {
     r.v0 = *reinterpret_cast<const float4*>(s.dy + i);
   }
   if constexpr (SRC != DY_PLAIN) r.o = *reinterpret_cast<const uint2*>(s.out + i);
+}
+// The next window's share of an odd time, behind the loads that every row has (between them, a branch a
+// row, the kernel took 163 to 180 us; this order 131; both windows always 193).
+__device__ __forceinline__ void gn_load_next(GnRow<DY_POOL>& r, const GnSource& s, int64_t b, int t, int c, int C) {
+  const int to = t / 2 + 1;
+  if ((t & 1) && to < s.To) {
+    const int64_t o = (b * s.To + to) * C + c;
+    r.v1 = *reinterpret_cast<const float4*>(s.dy + o);
+    r.a1 = *reinterpret_cast<const uchar4*>(s.arg + o);
+  }
 }
 
 template <int SRC>
@@ -462,6 +465,10 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
           const int t = min(t0 + (h + i) * rl, T - 1);
           gn_load<SRC>(r[i], src, b, t, 4 * q4, T, C);
           x[i] = z4[t * cq];
+        }
+        if constexpr (SRC == DY_POOL) {
+#pragma unroll
+          for (int i = 0; i < U; ++i) gn_load_next(r[i], src, b, min(t0 + (h + i) * rl, T - 1), 4 * q4, C);
         }
 #pragma unroll
         for (int i = 0; i < U; ++i) {
@@ -543,6 +550,10 @@ __global__ void __launch_bounds__(gn_bt(SRC), 2) k_gn_backward_s(GnSource src, c
       const int t = min(tb + k * step, T - 1);
       gn_load<SRC>(r[k], src, b, t, 4 * q4, T, C);
       x[k] = ld_stream(z4 + t * cq);
+    }
+    if constexpr (SRC == DY_POOL) {
+#pragma unroll
+      for (int k = 0; k < U; ++k) gn_load_next(r[k], src, b, min(tb + k * step, T - 1), 4 * q4, C);
     }
 #pragma unroll
     for (int k = 0; k < U; ++k) {
